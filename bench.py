@@ -869,7 +869,10 @@ def main():
     props = torch.cuda.get_device_properties(device)
     issue_peak = props.multi_processor_count * 4 * pk["sm_max_mhz"] * 1e6 / 1e9  # Ginst/s
     arb_kern = "sim_arb_kernel" if D <= 32 else "sim_arbw_kernel"
-    staged_run = p.staging == 1 or (p.staging == 0 and p.g.info["stageable"] == 1 and not p.arb)
+    # the library's default stages graphs whose copy takes 16 KB at most and batches of at most 32
+    stage_bytes = 20 * wl.desc.n_ops + 8 * wl.desc.n_edges
+    staged_run = p.staging == 1 or (p.staging == 0 and p.g.info["stageable"] == 1 and not p.arb and
+                                    (stage_bytes <= 16 << 10 or p.n_full <= 32))
     full_kern = "sim_full_staged_kernel" if staged_run else "sim_full_kernel"
     kname = {"full": arb_kern if p.arb else full_kern,
              "inc": "sim_arb_inc_kernel" if p.arb_base else arb_kern if p.arb else "sim_inc_kernel",

@@ -123,9 +123,10 @@ typedef struct gmg_base gmg_base_t; /* opaque; base schedule snapshot for increm
  * lists into shared memory with bulk copies; needs one accelerator type,
  * uniform links, every time below 2^31, at most 32 accelerators and the copy
  * within the CTA's shared memory, else GMG_EINVAL.  GMG_STAGING_L1: 4-warp
- * CTAs read the 64-byte op records through the read-only L1 path.
- * GMG_STAGING_DEFAULT stages wherever staging applies (measured faster on the
- * prefill workload) and takes the L1 path elsewhere; sim_batch_noalloc always
+ * CTAs read the records through the read-only L1 path.
+ * GMG_STAGING_DEFAULT stages graphs whose copy takes 16 KB at most and batches
+ * of at most 32 candidates wherever staging applies (measured faster there) and
+ * takes the L1 path elsewhere; sim_batch_noalloc always
  * takes the L1 path (and refuses GMG_STAGING_SHARED). */
 #define GMG_STAGING_DEFAULT 0
 #define GMG_STAGING_SHARED 1
@@ -172,13 +173,16 @@ typedef struct {
   int32_t uniform_links; /* 1 if every off-diagonal link has the same bw and latency */
   int64_t time_bound;    /* proven upper bound of every simulated time */
   int64_t default_queue_cap;
-  int32_t batched_sweep; /* 1 if the simulation kernels start READY ops in batches (graphs on
-                            more than 32 accelerators whose keys have room for a duration class) */
+  int32_t batched_sweep; /* 1 if the simulation kernels keep the pending ops of this graph in a
+                            pool in shared memory (more than 32 accelerators and keys with 5 bits
+                            of room; with at most 32 accelerators lanes hold them).  Either way
+                            every op whose start the others cannot change starts at once */
   int32_t t32;           /* 1 if the kernels carry times as 32-bit integers (time_bound < 2^31) */
   int32_t stageable;     /* 1 if sim_batch can stage this graph's hot fields in shared memory on
                             the current device (one accelerator type, uniform links, 32-bit times,
                             at most 32 accelerators, and the copy fits beside one warp's areas);
-                            the default then stages, with pure-latency transfers */
+                            the default then stages small graphs and small batches, with
+                            pure-latency transfers */
   int32_t reserved_;
 } gmg_info_t;
 

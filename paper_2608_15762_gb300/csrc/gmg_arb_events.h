@@ -20,6 +20,7 @@ namespace {
 template <class Self, class SimBase>
 struct ArbEvents : SimBase {
   using tm_t = typename SimBase::tm_t;
+  uint64_t rk_reg;  // READY keys: one per lane (kKeyMax = empty), the others in the heap
   __device__ explicit ArbEvents(const SimParams& p) : SimBase(p) {}
   __device__ __forceinline__ const Self& self() const { return *static_cast<const Self*>(this); }
 
@@ -39,12 +40,22 @@ struct ArbEvents : SimBase {
     return true;
   }
 
+  // READY keys go to a free lane's register if there is one, else the heap.
+  __device__ __forceinline__ void push_ready(uint64_t key) {
+    const uint32_t freel = __ballot_sync(kFullMask, rk_reg == kKeyMax);
+    if (freel) {
+      if ((int)lane_id() == __ffs(freel) - 1) rk_reg = key;
+    } else if (!this->q.push(key)) {
+      this->status = GMG_SIM_QUEUE;
+    }
+  }
+
   __device__ __forceinline__ void push_readies(bool rdy, tm_t rj, uint32_t j) {
     uint32_t m = __ballot_sync(kFullMask, rdy);
     while (m) {
       const int src = __ffs(m) - 1;
       m &= m - 1;
-      this->push_ready(__shfl_sync(kFullMask, this->kc.make(rj, kReady, j), src));
+      push_ready(__shfl_sync(kFullMask, this->kc.make(rj, kReady, j), src));
     }
   }
 
@@ -58,9 +69,9 @@ struct ArbEvents : SimBase {
       int32_t* rp = self().refs() + p;
       const int32_t left = *rp - 1;
       *rp = left;
-      const tm_t o = this->holdb[p];
+      const tm_t o = this->holdb()[p];
       h = o > v ? o : v;
-      this->holdb[p] = h;
+      this->holdb()[p] = h;
       last = left == 0;
     }
     this->log_event(last, this->kc.make(h, kFree, p), dp);
@@ -146,10 +157,9 @@ struct ArbEvents : SimBase {
     __syncwarp();
   }
 
-  __device__ void drain(int64_t t_next) {
+  __device__ __forceinline__ void drain(int64_t t_next) {
     generate();
-    this->opn = 0;  // generate() emptied the op log; the base drain's own call is then a no-op
-    SimBase::drain(t_next);
+    this->drain_log(t_next);
   }
 };
 

@@ -82,7 +82,8 @@ struct DevGmg {
                               // consumer of that predecessor (kSibNone / kSibMany)}
   const uint32_t* cons;
   const uint64_t* root_keys;  // READY keys of ops without predecessors, ascending
-  const uint64_t* root_keys_q;// the same keys with the duration class below them (batched sweep)
+  const uint64_t* root_keys_q;// the same as keys of the READY pool (time, op, least duration)
+  const int64_t* bytes;       // [N] output sizes (the op records' field, for the HBM events)
   const int64_t* cap;
   const int64_t* base;
   const int64_t* avail0;
@@ -92,6 +93,9 @@ struct DevGmg {
   int64_t max_iter;           // event-loop iteration cap per candidate
   int32_t n, D, R, nroots;
   int32_t ib;                 // op-id bits of a packed key
+  uint32_t opmask;            // 2^ib - 1
+  int32_t ds;                 // accelerator shift of a log entry (above its key)
+  uint64_t keymask;           // key part of a log entry: 2^ds - 1
   int32_t tb;                 // time bits needed (every time < 2^tb)
   int32_t dev_key;            // 1 if an accelerator id fits above (time, class, op) in 64 bits
   int32_t t32;                // 1 if every time is below 2^31 (the kernels then use int32 times)
@@ -99,13 +103,17 @@ struct DevGmg {
   const int64_t* durt;        // [N*ntypes] duration of op i on type t at i*ntypes + t
   const uint8_t* dtype;       // [D] type of each accelerator
   int32_t uniform;
-  int32_t batch;              // 1: the kernels take READY keys in batches (keys carry kQB class bits)
-  // The hot fields in the compact form a CTA stages into shared memory
-  // (sim_full_staged_kernel); present when stage_ok.
+  int32_t qsh;                // time shift of a READY pool key: ib + qb
+  int32_t qb;                 // bits of the earliest finish in a READY pool key (0, or 6 to kMaxQB)
+  // The hot fields in a compact form, read by the sweep wherever the graph has
+  // it (hot_ok) and staged into shared memory by sim_full_staged_kernel
+  // (stage_ok: also at most 32 accelerators).
   const uint4* st_hot;        // [N] {dur, xq | flags << 29, succ_off | nsucc << 24, pred_off | npred << 24}
   const int32_t* st_rel;      // [N] release
-  int32_t stage_ok;           // 1: 32-bit times, one type, uniform links, lists and sizes fit the fields
+  int32_t hot_ok;             // 1: 32-bit times, one type, uniform links, lists and sizes fit the fields
+  int32_t stage_ok;
   int32_t n_edges;
+  int32_t big_bytes;          // 1: some output has 2^48 bytes or more
   const uint8_t* ws;          // the whole device copy (every array above), for L2 prefetches
   int64_t ws_bytes;
 };
@@ -119,19 +127,23 @@ inline int64_t stage_smem_bytes(int64_t n, int64_t E) {
   return 16 + 16 * n + (4 * n + 15) / 16 * 16 + 2 * ((4 * E + 15) / 16 * 16);
 }
 
-// Resident 4-warp blocks per SM the batched kernels are compiled for (their
-// register budget; compile-time overridable for tuning sweeps).
-#ifndef GMG_BATCH_BLOCKS_PER_SM
-#define GMG_BATCH_BLOCKS_PER_SM 7
+// Resident 4-warp blocks per SM the simulation kernels are compiled for (their
+// register budget).
+constexpr int kBlocksPerSM = 7;
+
+// Slots of the READY pool on more than 32 accelerators (a multiple of 32, at
+// most 256; compile-time overridable for tuning sweeps).
+#ifndef GMG_POOL_WIDE
+#define GMG_POOL_WIDE 160
 #endif
-constexpr int kBatchBlocksPerSM = GMG_BATCH_BLOCKS_PER_SM;
+constexpr int kReadyPoolWide = GMG_POOL_WIDE;
 
 // The staged-GMG kernel's largest CTA (one per SM; 72 registers a thread).
 constexpr int kStageMaxWarps = 28;
 
-// Batched sweep: a READY key is followed by kQB bits holding floor(log2) of a
-// lower bound of the op's duration (31 at most).
-constexpr int kQB = 5;
+// A READY pool key keeps an op's least time from ready to finish in up to kMaxQB
+// bits: a 5-bit exponent and a mantissa.
+constexpr int kMaxQB = 16;
 
 // Packed event key: time << (ib + 2) | class << ib | op.  Classes at equal
 // times: READY (an op's last input arrived) < FREE < ALLOC.
@@ -169,10 +181,10 @@ struct DevBase {
   int64_t* res_creq;     // [R]
   // checkpoints c = 0 .. nck-1
   int64_t* ck_time;      // [nck]  T_c (INT64_MAX = not recorded)
-  int64_t* ck_scalars;   // [nck*8]: qsize, rootptr, score, makespan, vflag, vt, vop<<32|vdev, log size
+  int64_t* ck_scalars;   // [nck*8]: qsize, rootptr, score, drained, vflag, vt, vop<<32|vdev, log size
   int64_t* ck_dev;       // [nck*3*D]: free, live, peak
   int64_t* ck_creq;      // [nck*R]
-  uint64_t* ck_qkey;     // [nck*ckq] READY heap
+  uint64_t* ck_qkey;     // [nck*ckq] READY keys
   uint64_t* ck_mkey;     // [nck*ckm] HBM event log entries
   uint8_t* ck_mdev;      // [nck*ckm] their accelerators (when not inside the entries)
   int32_t nck;
@@ -189,14 +201,16 @@ struct SimParams {
   const uint8_t* place;  // kFull: [K][ld]; kBase: base row
   int64_t ld;
   int32_t K;
+  int32_t pool;          // READY pool slots in shared memory per warp (0: at most 32 accelerators, arbitrated kernels)
+  int32_t pend_cap;      // pending READY keys a candidate may have (else GMG_SIM_QUEUE)
   int32_t qs;            // READY heap slots in shared memory per warp (32m+1, >= 33)
   int32_t qcap;          // READY heap slots per warp
   int32_t ms;            // HBM event log slots in shared memory per warp
   int32_t mcap;          // HBM event log slots per warp
   int32_t sortcap;       // sort area entries per warp (power of two, >= max(32, n_dev))
-  int32_t drain_trigger; // batched sweep: ops started before an HBM-event generation
-  int32_t opcap;         // ops started between HBM-event generations (one at a time), or the
-                         // capacity of the list of started ops (batched: drain_trigger + 32)
+  int32_t drain_trigger; // ops started before an HBM-event generation (sweep of the READY pool)
+  int32_t opcap;         // capacity of the list of started ops (drain_trigger + 32), or the ops started
+                         // between HBM-event generations (arbitrated: one at a time)
   int32_t n_trace;
   const int32_t* trace_k;
   const int32_t* move_off;
@@ -207,7 +221,6 @@ struct SimParams {
   int32_t dev_bytes;     // shared bytes of accelerator state per warp
   int32_t stage_bytes;   // shared bytes of the staged GMG copy (sim_full_staged_kernel), else 0
   int32_t no_side;       // 1: no side bytes in shared memory (the accelerator is inside the log entry)
-  int32_t pad_;
   // byte offsets inside a slot (off_pk < 0: the peaks are in shared memory)
   int64_t off_f, off_hold, off_bits, off_creq, off_qk, off_mk, off_md, off_row, off_pk;
   // Incremental candidates: the next candidate a warp takes (zeroed before

@@ -57,8 +57,8 @@ namespace {
 // kMode: kFull (sim_batch), kBase (the arbitrated base snapshot: records
 // ready and finish times and checkpoints), kInc (candidates resumed from it).
 template <bool kT32, bool kTypes, int kMode = kFull>
-struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT32, kTypes>> {
-  using Base = ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT32, kTypes>>;
+struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT32, kTypes, false>> {
+  using Base = ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT32, kTypes, false>>;
   using tm_t = typename Base::tm_t;
   using U = typename std::make_unsigned<tm_t>::type;
   using Base::g;
@@ -70,11 +70,12 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
   using Base::drop_hold;
   using Base::generate;
   using Base::push_readies;
-  static constexpr tm_t kNever = (tm_t)(~(U)0 >> 1);
+  using Base::kNever;
+  using Base::sl;
+  using Base::warp_min_t;
   const ArbParams& A;
   // The warp's scratch slot and shared area; the arrays in them are found
   // from the launch parameters' offsets when used (registers are scarce).
-  uint8_t* sl;
   uint8_t* sm;       // [0, 128): busy links (32 words); then the queue heads if shared
   int32_t nx;        // intents arrived so far
   int32_t xev;       // transfer events handled (loop guard)
@@ -108,24 +109,19 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
   }
   __device__ __forceinline__ uint32_t* lbits() const { return reinterpret_cast<uint32_t*>(sm); }
 
-  __device__ __forceinline__ tm_t warp_min_t(tm_t v) const {
-    if (kT32) return (tm_t)__reduce_min_sync(kFullMask, (int)v);
-    return (tm_t)warp_min_u64((uint64_t)v);  // times are >= 0
-  }
-
   __device__ __forceinline__ void refresh_done() { td_c = warp_min_t(xd); }
   __device__ __forceinline__ void refresh_intent() {
     ik_c = warp_min_u64(fh >= 0 ? (((uint64_t)(U)fa << g.ib) | (uint32_t)fh) : kKeyMax);
   }
 
-  __device__ void setup_arb(int64_t slot, uint8_t* smem_warp) {
-    sl = P.scratch + slot * P.slot_bytes;
+  __device__ void setup_arb(uint8_t* smem_warp) {
     sm = smem_warp;
   }
 
   __device__ void reset_arb() {
     const unsigned lane = lane_id();
     this->reset_common();
+    this->rk_reg = kKeyMax;
     uint4* c4 = reinterpret_cast<uint4*>(cnt());
     int32_t* qh = qhead();
     int32_t* qt = qtail();
@@ -167,16 +163,13 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     if (lane == 0) {
       this->fbuf[i] = f;
       if (cs.w & kReqSink)
-        atomicMax(reinterpret_cast<unsigned long long*>(this->creq + (int32_t)cs.z), (unsigned long long)f);
+        atomicMax(reinterpret_cast<unsigned long long*>(this->creq() + (int32_t)cs.z), (unsigned long long)f);
       if (kMode == kBase) P.base.rb[i] = r;
       this->oplog[this->opn] = i;
     }
     ++this->opn;
     if (cs.w & kScored) this->score += (int64_t)f;
-    if (kMode == kBase) {
-      this->makespan = f > this->makespan ? f : this->makespan;
-      ++this->readypops;
-    }
+    if (kMode == kBase) ++this->readypops;
     if (kMode == kInc && r >= this->T0) ++this->nev;
     __syncwarp();
     uint32_t remote = 0u;
@@ -196,7 +189,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     remote = __reduce_or_sync(kFullMask, remote);
     if (lane == 0) {
       refs()[i] = 1 + __popc(remote);
-      this->holdb[i] = f;
+      this->holdb()[i] = f;
       if (remote) rmask()[i] = remote;
     }
     if (remote && (int)lane == d) {
@@ -382,16 +375,18 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
           break;
         }
         if (td == tx) transfer_done(__ffs(__ballot_sync(kFullMask, xd == td)) - 1, td);
-        else intents_arrive((uint32_t)(ik & this->kc.mask));
+        else intents_arrive((uint32_t)(ik & g.opmask));
         if (kMode == kBase) this->last_t = tx;
         arb_due = true;
         t_arb = tx;
         if (status) break;
         continue;
       }
-      if (nk == kKeyMax) break;
-      if (kMode == kBase) arb_checkpoint(nk);
-      if (this->opn >= P.opcap) drain(this->kc.time(nk));
+      if (kMode == kBase && nk != kKeyMax) arb_checkpoint(nk);
+      if (nk == kKeyMax || this->opn >= P.opcap) {  // the only copy of this code: it is large
+        drain(nk == kKeyMax ? kI64Max : this->kc.time(nk));
+        if (nk == kKeyMax || status) break;
+      }
       if (nk == rm) {
         if (this->rk_reg == rm) this->rk_reg = kKeyMax;
       } else if (nk == rk) {
@@ -409,7 +404,6 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
       start_op(this->kc.op(nk), (tm_t)this->kc.time(nk));
       if (status) break;
     }
-    if (!status) drain(kI64Max);
   }
 
   // -------------------------------------------------------------------------
@@ -427,7 +421,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     if (this->kc.time(next_key) <= (int64_t)this->last_t) return;
     generate();  // the simulation checkpoint then finds no started op left to generate
     const int c = this->ck;
-    this->maybe_checkpoint(next_key);
+    this->maybe_checkpoint(this->kc.time(next_key), this->rk_reg);
     if (this->ck > c && B.ck_time[c] != kI64Max) save_arb(c);
   }
 
@@ -447,7 +441,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     warp_copy16<16>(a + K.off_refs, refs(), 4 * n);
     warp_copy16<16>(a + K.off_rmask, rmask(), 4 * n);
     warp_copy16<16>(a + K.off_nextop, nextop(), 4 * n);
-    warp_copy16<16>(a + K.off_hold, this->holdb, 8 * n);
+    warp_copy16<16>(a + K.off_hold, this->holdb(), 8 * n);
     warp_copy16<16>(a + K.off_xent, xent(), 4 * (int64_t)nx);
     warp_copy16<16>(a + K.off_xnext, xnext(), 4 * (int64_t)nx);
     for (int x = lane; x < g.D * g.D; x += 32) {
@@ -504,10 +498,10 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     warp_copy16(nextop(), a + K.off_nextop, 4 * n);
     if (kT32) {
       narrow_times(rmax(), reinterpret_cast<const int64_t*>(a + K.off_rmax), g.n);
-      narrow_times(this->holdb, reinterpret_cast<const int64_t*>(a + K.off_hold), g.n);
+      narrow_times(this->holdb(), reinterpret_cast<const int64_t*>(a + K.off_hold), g.n);
     } else {
       warp_copy16(rmax(), a + K.off_rmax, 8 * n);
-      warp_copy16(this->holdb, a + K.off_hold, 8 * n);
+      warp_copy16(this->holdb(), a + K.off_hold, 8 * n);
     }
     const int64_t* w = reinterpret_cast<const int64_t*>(a + K.off_warp);
     nx = (int32_t)w[0];
@@ -693,16 +687,16 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     const int64_t* sc = B.ck_scalars + (int64_t)c * 8;
     const int qsz = (int)sc[0];
     const int msz = (int)sc[7];
-    if (qsz + nm > this->q.cap || msz + nm > this->log.cap) {
+    if (qsz + nm > P.qcap || msz + nm > P.mcap) {
       this->write_invalid(k, GMG_SIM_QUEUE);
       return;
     }
     // the simulation state of checkpoint c
     this->Tc = (tm_t)B.ck_time[c];
+    this->drained = (tm_t)sc[3];
     this->rootptr = (int)sc[1];
     this->load_root();
     this->score = sc[2];
-    this->makespan = (tm_t)sc[3];
     this->vflag = (int32_t)sc[4];
     this->vt = sc[5];
     this->vop = (int32_t)(sc[6] >> 32);
@@ -715,7 +709,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     this->rk_reg = kKeyMax;
     this->opn = 0;
     this->dv.load(B.ck_dev + (int64_t)c * 3 * g.D);
-    for (int r = lane; r < g.R; r += 32) this->creq[r] = B.ck_creq[(int64_t)c * g.R + r];
+    for (int r = lane; r < g.R; r += 32) this->creq()[r] = B.ck_creq[(int64_t)c * g.R + r];
     this->fill_fin();
     restore_arb(c);
     // READY keys, except those of moved ops (recomputed below)
@@ -740,7 +734,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
       bool keep = v;
       if (v && this->kc.cls(e) == kFree) {
         const uint32_t op = this->kc.op(e);
-        const int dev = (int)(e >> this->ds);
+        const int dev = (int)(e >> g.ds);
         if (dev == B.row[op]) {
           const XqSucc xs = op_xqsucc(g.ops, op);
           for (uint32_t u = 0; u < xs.nsucc && keep; ++u) {
@@ -808,7 +802,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
         if (lane == 0) {
           rmask()[p] = rc;
           refs()[p] = holds;
-          this->holdb[p] = fp;
+          this->holdb()[p] = fp;
         }
         __syncwarp();
         fifo_set(p, dp, rc != 0u);
@@ -832,7 +826,7 @@ __global__ void __launch_bounds__(128, 7) sim_arb_kernel(const __grid_constant__
   const int64_t nslots = (int64_t)gridDim.x * (blockDim.x >> 5);
   ArbSim<kT32, kTypes> S(A);
   setup_slot(S, A.P, wib, slot, smem);
-  S.setup_arb(slot, smem + A.smem_std + (size_t)wib * A.smem_arb);
+  S.setup_arb(smem + A.smem_std + (size_t)wib * A.smem_arb);
   for (int64_t k = slot; k < A.P.K; k += nslots) {
     S.row = A.P.place + k * A.P.ld;
     if (A.pre_status) {
@@ -859,7 +853,7 @@ __global__ void __launch_bounds__(32) sim_arb_base_kernel(const __grid_constant_
   extern __shared__ __align__(16) uint8_t smem[];
   ArbSim<false, kTypes, kBase> S(A);
   setup_slot(S, A.P, 0, 0, smem);
-  S.setup_arb(0, smem + A.smem_std);
+  S.setup_arb(smem + A.smem_std);
   const DevBase& B = A.P.base;
   const unsigned lane = lane_id();
   warp_prefetch_l2(A.P.g.ws, A.P.g.ws_bytes);
@@ -882,15 +876,16 @@ __global__ void __launch_bounds__(32) sim_arb_base_kernel(const __grid_constant_
   if (S.status != GMG_SIM_OK) return;
   int32_t miss = 0;
   for (int r = lane; r < S.g.R; r += 32) {
-    const int64_t c = S.creq[r];
+    const int64_t c = S.creq()[r];
     B.res_creq[r] = c;
     miss += c > __ldg(S.g.deadline + r) ? 1 : 0;
   }
   miss = (int32_t)__reduce_add_sync(kFullMask, (unsigned)miss);
   S.dv.write_peak(B.res_peak);
+  const int64_t makespan = S.dv.max_busy(S.g);
   if (lane == 0) {
     int64_t* rs = B.res_scalars;
-    rs[0] = S.makespan;
+    rs[0] = makespan;
     rs[1] = S.vflag ? kI64Max : S.score;
     rs[2] = S.vflag;
     rs[3] = S.vop;
@@ -909,7 +904,7 @@ __global__ void __launch_bounds__(128, 7) sim_arb_inc_kernel(const __grid_consta
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
   ArbSim<kT32, kTypes, kInc> S(A);
   setup_slot(S, A.P, wib, slot, smem);
-  S.setup_arb(slot, smem + A.smem_std + (size_t)wib * A.smem_arb);
+  S.setup_arb(smem + A.smem_std + (size_t)wib * A.smem_arb);
   S.rb = A.P.base.rb;
   S.fb = A.P.base.fb;
   uint8_t* crow = A.P.scratch + slot * A.P.slot_bytes + A.P.off_row;

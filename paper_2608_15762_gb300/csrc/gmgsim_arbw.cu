@@ -33,8 +33,8 @@ namespace gsim {
 namespace {
 
 template <bool kT32, bool kTypes>
-struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, kTypes>> {
-  using Base = ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, kTypes>>;
+struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, kTypes, false>> {
+  using Base = ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, kTypes, false>>;
   using tm_t = typename Base::tm_t;
   using U = typename std::make_unsigned<tm_t>::type;
   using Base::g;
@@ -46,9 +46,10 @@ struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, 
   using Base::drop_hold;
   using Base::generate;
   using Base::push_readies;
-  static constexpr tm_t kNever = (tm_t)(~(U)0 >> 1);
+  using Base::kNever;
+  using Base::sl;
+  using Base::warp_min_t;
   const ArbWParams& A;
-  uint8_t* sl;       // the warp's scratch slot
   uint32_t* sb;      // shared [W] busy senders
   uint32_t* rb;      // shared [W] busy receivers
   uint32_t* ps;      // shared [W] sources with a pending intent
@@ -82,10 +83,6 @@ struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, 
   __device__ __forceinline__ uint32_t* pm() const { return at<uint32_t>(A.off_pm); }
   __device__ __forceinline__ uint32_t* lb() const { return at<uint32_t>(A.off_lb); }
 
-  __device__ __forceinline__ tm_t warp_min_t(tm_t v) const {
-    if (kT32) return (tm_t)__reduce_min_sync(kFullMask, (int)v);
-    return (tm_t)warp_min_u64((uint64_t)v);  // times are >= 0
-  }
   static __device__ __forceinline__ bool bit(const uint32_t* s, int i) { return (s[i >> 5] >> (i & 31)) & 1u; }
 
   // The tables hold at most 256 accelerators, eight per lane: each lane loads
@@ -133,8 +130,7 @@ struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, 
     ik_c = warp_min_u64(k);
   }
 
-  __device__ void setup_arb(int64_t slot, uint8_t* smem_warp) {
-    sl = P.scratch + slot * P.slot_bytes;
+  __device__ void setup_arb(uint8_t* smem_warp) {
     uint32_t* w = reinterpret_cast<uint32_t*>(smem_warp);
     sb = w;
     rb = w + 8;
@@ -146,6 +142,7 @@ struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, 
     const unsigned lane = lane_id();
     const int D = g.D, W = A.words;
     this->reset_common();
+    this->rk_reg = kKeyMax;
     uint4* c4 = reinterpret_cast<uint4*>(cnt());
     const int nv = (int)((4 * (size_t)g.n + 15) / 16);
     for (int x = lane; x < nv; x += 32) c4[x] = make_uint4(0u, 0u, 0u, 0u);
@@ -211,7 +208,7 @@ struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, 
     if (lane == 0) {
       this->fbuf[i] = f;
       if (cs.w & kReqSink)
-        atomicMax(reinterpret_cast<unsigned long long*>(this->creq + (int32_t)cs.z), (unsigned long long)f);
+        atomicMax(reinterpret_cast<unsigned long long*>(this->creq() + (int32_t)cs.z), (unsigned long long)f);
       this->oplog[this->opn] = i;
     }
     ++this->opn;
@@ -232,7 +229,7 @@ struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, 
     const int nrem = remote_set(i, d);
     if (lane == 0) {
       refs()[i] = 1 + nrem;
-      this->holdb[i] = f;
+      this->holdb()[i] = f;
       if (nrem) {
         if (fh()[d] < 0) {
           fh()[d] = (int32_t)i;
@@ -442,15 +439,17 @@ struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, 
         if (td == tx) {
           transfer_done(td_src, td);
         } else {
-          intents_arrive((uint32_t)(ik & this->kc.mask));
+          intents_arrive((uint32_t)(ik & g.opmask));
         }
         arb_due = true;
         t_arb = tx;
         if (status) break;
         continue;
       }
-      if (nk == kKeyMax) break;
-      if (this->opn >= P.opcap) drain(this->kc.time(nk));
+      if (nk == kKeyMax || this->opn >= P.opcap) {  // the only copy of this code: it is large
+        drain(nk == kKeyMax ? kI64Max : this->kc.time(nk));
+        if (nk == kKeyMax || status) break;
+      }
       if (nk == rm) {
         if (this->rk_reg == rm) this->rk_reg = kKeyMax;
       } else if (nk == rk) {
@@ -467,7 +466,6 @@ struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes>, Sim<false, kFull, true, kT32, 
       start_op(this->kc.op(nk), (tm_t)this->kc.time(nk));
       if (status) break;
     }
-    if (!status) drain(kI64Max);
   }
 };
 
@@ -479,7 +477,7 @@ __global__ void __launch_bounds__(128, 6) sim_arbw_kernel(const __grid_constant_
   const int64_t nslots = (int64_t)gridDim.x * (blockDim.x >> 5);
   ArbWSim<kT32, kTypes> S(A);
   setup_slot(S, A.P, wib, slot, smem);
-  S.setup_arb(slot, smem + A.smem_std + (size_t)wib * A.smem_arb);
+  S.setup_arb(smem + A.smem_std + (size_t)wib * A.smem_arb);
   for (int64_t k = slot; k < A.P.K; k += nslots) {
     S.row = A.P.place + k * A.P.ld;
     if (A.pre_status) {

@@ -7,13 +7,13 @@ namespace {
 // ---------------------------------------------------------------------------
 // sim_batch: K full placements.
 // ---------------------------------------------------------------------------
-template <bool kReg, bool kKey, bool kT32, bool kTypes, bool kBatch>
-__global__ void __launch_bounds__(128, kBatch ? kBatchBlocksPerSM : 7) sim_full_kernel(const __grid_constant__ SimParams P) {
+template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
+__global__ void __launch_bounds__(128, kBlocksPerSM) sim_full_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
   const int64_t nslots = (int64_t)gridDim.x * (blockDim.x >> 5);
-  Sim<kReg, kFull, kKey, kT32, kTypes, kBatch> S(P);
+  Sim<kNarrow, kFull, kKey, kT32, kTypes, true, kHot> S(P);
   setup_slot(S, P, wib, slot, smem);
   for (int64_t k = slot; k < P.K; k += nslots) {
     S.row = P.place + k * P.ld;
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(32 * kStageMaxWarps, 1) sim_full_staged_kernel
   const int64_t nw = blockDim.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * nw + wib;
   const int64_t nslots = (int64_t)gridDim.x * nw;
-  Sim<true, kFull, true, true, false, false, true> S(P);
+  Sim<true, kFull, true, true, false, true, kHotShared> S(P);
   setup_slot(S, P, wib, slot, smem + P.stage_bytes);
   S.sh_hot = reinterpret_cast<const uint4*>(s_hot);
   S.sh_rel = reinterpret_cast<const int32_t*>(s_rel);
@@ -124,22 +124,24 @@ cudaError_t launch_full_staged(const SimParams& P, int grid, int block, size_t s
   return cudaLaunchKernel((const void*)sim_full_staged_kernel, dim3(grid), dim3(block), args, smem, st);
 }
 
-// Instances by (accelerator state in registers, accelerator id in the event
-// key, 32-bit times, accelerator types, batched sweep).  32-bit times are only
-// chosen with the accelerator id in the key; the batched sweep only with
-// accelerator state in shared memory and the id in the key.
-template <bool R, bool K, bool T32, bool B>
-const void* full_ptr5(bool types) {
-  return types ? (const void*)sim_full_kernel<R, K, T32, true, B> : (const void*)sim_full_kernel<R, K, T32, false, B>;
+// Instances by (at most 32 accelerators, accelerator id in the event key,
+// 32-bit times, accelerator types; compact records wherever the graph has
+// them).  32-bit times are only chosen with the accelerator id in the key,
+// compact records only with 32-bit times.
+template <bool N, bool K, bool T32>
+const void* full_ptr(bool types) {
+  return types ? (const void*)sim_full_kernel<N, K, T32, true, kHotNone>
+               : (const void*)sim_full_kernel<N, K, T32, false, kHotNone>;
 }
-const void* full_kernel_ptr(bool reg, bool key, bool t32, bool types, bool batch) {
-  if (reg) {
-    if (!key) return full_ptr5<true, false, false, false>(types);
-    return t32 ? full_ptr5<true, true, true, false>(types) : full_ptr5<true, true, false, false>(types);
-  }
-  if (!key) return full_ptr5<false, false, false, false>(types);
-  if (batch) return t32 ? full_ptr5<false, true, true, true>(types) : full_ptr5<false, true, false, true>(types);
-  return t32 ? full_ptr5<false, true, true, false>(types) : full_ptr5<false, true, false, false>(types);
+template <bool N>
+const void* full_ptr_n(bool key, bool t32, bool types, bool hot) {
+  if (!key) return full_ptr<N, false, false>(types);
+  if (hot) return (const void*)sim_full_kernel<N, true, true, false, kHotGlobal>;
+  return t32 ? full_ptr<N, true, true>(types) : full_ptr<N, true, false>(types);
+}
+const void* full_kernel_ptr(const DevGmg& g) {
+  const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
+  return g.D <= 32 ? full_ptr_n<true>(key, t32, types, hot) : full_ptr_n<false>(key, t32, types, hot);
 }
 
 }  // namespace gsim

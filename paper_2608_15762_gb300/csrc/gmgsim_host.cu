@@ -17,13 +17,13 @@
 namespace gsim {
 // launchers (gmgsim_kernels.cu)
 size_t select_rank_bytes();
-const void* full_kernel_ptr(bool reg, bool key, bool t32, bool types, bool batch);
-const void* inc_kernel_ptr(bool reg, bool key, bool t32, bool types, bool batch);
+const void* full_kernel_ptr(const DevGmg& g);
+const void* inc_kernel_ptr(const DevGmg& g);
 const void* full_staged_kernel_ptr();
-cudaError_t launch_full(bool reg, const SimParams& P, int grid, int block, size_t smem, cudaStream_t st);
+cudaError_t launch_full(const SimParams& P, int grid, int block, size_t smem, cudaStream_t st);
 cudaError_t launch_full_staged(const SimParams& P, int grid, int block, size_t smem, cudaStream_t st);
-cudaError_t launch_inc(bool reg, const SimParams& P, int grid, int block, size_t smem, cudaStream_t st);
-cudaError_t launch_base(bool reg, const SimParams& P, size_t smem, cudaStream_t st);
+cudaError_t launch_inc(const SimParams& P, int grid, int block, size_t smem, cudaStream_t st);
+cudaError_t launch_base(const SimParams& P, size_t smem, cudaStream_t st);
 cudaError_t set_smem_limits(int smem);
 cudaError_t launch_select(const int32_t* status, const int32_t* viol, const int64_t* score,
                           const int32_t* miss, int32_t K, int32_t mode, void* tmp, int nparts,
@@ -37,26 +37,13 @@ namespace {
 constexpr int64_t kI64Max = 0x7fffffffffffffffll;
 constexpr int kMaxOpsLog2 = 28;          // op ids must fit the packed key
 constexpr int kDefaultWarpsPerBlock = 4;
-constexpr int kSharedQueueEntries = 97;  // 1 + 32 * 3: root, its children, two more groups
-// The batched sweep's sizes (compile-time overridable for tuning sweeps).
-#ifndef GMG_BATCH_QUEUE_SHARED
-#define GMG_BATCH_QUEUE_SHARED 161  // 1 + 32 * 5 (with the log below: 28 warps per SM at 256 accelerators)
-#endif
-#ifndef GMG_BATCH_OPS_PER_GENERATION
-#define GMG_BATCH_OPS_PER_GENERATION 24
-#endif
-#ifndef GMG_BATCH_LOG_SHARED
-#define GMG_BATCH_LOG_SHARED 128
-#endif
-constexpr int kSharedQueueEntriesBatch = GMG_BATCH_QUEUE_SHARED;
-constexpr int kBatchOpsPerGeneration = GMG_BATCH_OPS_PER_GENERATION;
-constexpr int kSharedLogEntriesBatch = GMG_BATCH_LOG_SHARED;
+constexpr int kSharedQueueEntries = 97;  // arbitrated kernels: 1 + 32 * 3: root, its children, two more groups
+constexpr int kSharedOverflowEntries = 33;  // behind the READY pool: the root and its children
 constexpr int64_t kDefaultQueueCap = 1 << 16;
-constexpr int kSharedLogEntries = 192;
+constexpr int kSharedLogEntries = 192, kSharedLogEntriesWide = 112;
 constexpr int64_t kDefaultLogCap = 1 << 17;
 constexpr int kSortCap = 128;             // power of two; raised to n_dev's power of two
 constexpr int kOpsPerGeneration = 24;     // ~85 HBM events per generation (prefill graphs)
-constexpr int kBatchMinDevices = 33;      // the batched sweep serves graphs on more accelerators
 constexpr int kCheckpoints = 256;
 constexpr int kArbCheckpoints = 64;       // arbitrated bases also keep ~32 bytes per op per checkpoint
 constexpr int kCheckpointQueue = 4096;
@@ -65,7 +52,7 @@ constexpr int kCheckpointLog = 8192;
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Layout {
-  size_t off_ops, off_succ, off_pred, off_sib, off_cons, off_roots, off_roots_q, off_cap, off_base, off_avail,
+  size_t off_ops, off_succ, off_pred, off_sib, off_cons, off_roots, off_roots_q, off_bytes, off_cap, off_base, off_avail,
       off_dl, off_links, off_durt, off_dtype, off_linkid, off_st_hot, off_st_rel, total;
 };
 
@@ -125,6 +112,7 @@ void plan(Built& b) {
   L.off_cons = take(4 * (size_t)b.Ec);
   L.off_roots = take(8 * (size_t)b.nroots);
   L.off_roots_q = take(8 * (size_t)b.nroots);
+  L.off_bytes = take(8 * (size_t)b.n);
   L.off_cap = take(8 * (size_t)b.D);
   L.off_base = take(8 * (size_t)b.D);
   L.off_avail = take(8 * (size_t)b.D);
@@ -479,7 +467,6 @@ struct gmg_base {
 namespace {
 
 struct Launch {
-  bool reg;
   int wpb, grid;
   size_t smem;
   int64_t slots;
@@ -499,43 +486,47 @@ int log_cap(const gmg* g, const sim_opts_t* o) {
 
 size_t smem_per_warp(const SimParams& P) {
   const size_t side = P.no_side ? 0 : 1;
-  return align_up((size_t)P.qs * 8 + (size_t)P.ms * (8 + side) + (size_t)P.sortcap * (8 + side) + (size_t)P.opcap * 4,
+  return align_up((size_t)P.pool * 9 + (size_t)P.qs * 8 + (size_t)P.ms * (8 + side) + (size_t)P.sortcap * (8 + side) + (size_t)P.opcap * 4,
                   16) +
          (size_t)P.dev_bytes;
 }
 
-// Shared bytes of accelerator state per warp: live bytes; peaks unless they
-// are kept in global scratch (more than 32 accelerators); free times (of
-// tbytes each) unless lanes hold them in registers (at most 32).
-int dev_smem_bytes(int D, size_t tbytes) {
-  const bool reg = D <= 32;
-  return (int)align_up((size_t)D * 8 + (reg ? (size_t)D * 8 : 0) + (reg ? 0 : (size_t)D * tbytes), 16);
+// Shared bytes of accelerator state per warp: live bytes; peaks and a drain's
+// sums, or (more than 32 accelerators: the peaks are in global scratch) a bit
+// set of the accelerators whose order matters; free times (of
+// tbytes each) unless lanes hold them in registers (the arbitrated kernels of
+// at most 32).
+int dev_smem_bytes(int D, size_t tbytes, bool pool) {
+  const bool narrow = D <= 32;
+  return (int)align_up((size_t)D * 8 + (narrow ? (size_t)D * 72 : 32) + (narrow && !pool ? 0 : (size_t)D * tbytes), 16);
 }
 
 bool g_smem_set = false;
 
-// Slot layout and grid for K candidates of kind `inc` (sweep: the graph's
-// batched sweep if it has one; the arbitrated kernels take keys one at a time).
-int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& L, bool sweep_batch = true) {
+// Slot layout and grid for K candidates of kind `inc` (pool: the READY pool's
+// sweep; the arbitrated kernels take keys one at a time).
+int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& L, bool pool = true) {
   const DevGmg& G = g->dg;
-  const bool batch = G.batch && sweep_batch;
-  L.reg = G.D <= 32;
+  const bool narrow = G.D <= 32;
   L.wpb = (o && o->warps_per_block > 0) ? o->warps_per_block : kDefaultWarpsPerBlock;
   if (L.wpb > 4) return GMG_EINVAL;
   SimParams& P = L.P;
   std::memset(&P, 0, sizeof(P));
   P.g = G;
-  P.qcap = queue_cap(g, o);
-  P.qs = batch ? kSharedQueueEntriesBatch : kSharedQueueEntries;  // >= 33 (the root's children are
-                                                                     // always in shared memory)
+  P.pool = pool && !narrow ? kReadyPoolWide : 0;
+  // pending keys beyond one per lane; the pool's heap has room for one more
+  // (Sim::run puts a pool key there when the next root finds the pool full)
+  P.qcap = queue_cap(g, o) + (pool ? 1 : 0);
+  P.pend_cap = 32 + queue_cap(g, o);
+  P.qs = pool ? kSharedOverflowEntries : kSharedQueueEntries;
   P.mcap = log_cap(g, o);
-  P.ms = batch ? kSharedLogEntriesBatch : kSharedLogEntries;
+  P.ms = narrow || !pool ? kSharedLogEntries : kSharedLogEntriesWide;
   P.sortcap = kSortCap;
   while (P.sortcap < G.D) P.sortcap <<= 1;
-  P.drain_trigger = batch ? kBatchOpsPerGeneration : kOpsPerGeneration;
-  P.opcap = batch ? kBatchOpsPerGeneration + 32 : kOpsPerGeneration;
-  P.dev_bytes = dev_smem_bytes(G.D, G.t32 ? 4 : 8);
-  P.no_side = batch ? 1 : 0;  // the batched sweep keeps the accelerator inside the entry
+  P.drain_trigger = kOpsPerGeneration;
+  P.opcap = pool ? kOpsPerGeneration + 32 : kOpsPerGeneration;
+  P.dev_bytes = dev_smem_bytes(G.D, G.t32 ? 4 : 8, pool);
+  P.no_side = pool && G.dev_key ? 1 : 0;  // the accelerator is inside the log entry
   L.smem = (size_t)L.wpb * smem_per_warp(P);
   size_t o2 = 0;
   auto take = [&](size_t bytes) {
@@ -553,7 +544,7 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
   P.off_mk = take(8 * (size_t)mspill);
   P.off_md = take((size_t)mspill);
   P.off_row = take(inc ? (size_t)align_up(std::max(G.n, 1), 16) : 0);
-  P.off_pk = L.reg ? -1 : take(8 * (size_t)G.D);
+  P.off_pk = narrow ? -1 : take(8 * (size_t)G.D);
   P.slot_bytes = (int64_t)o2;
   const int sms = device_sms();
   if (sms <= 0) return GMG_ECUDA;
@@ -562,18 +553,17 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
     SimParams big = P;
     big.g.D = 256;
     big.sortcap = 256;
-    big.opcap = std::max(kOpsPerGeneration, kBatchOpsPerGeneration + 32);
-    big.qs = std::max(kSharedQueueEntries, kSharedQueueEntriesBatch);
-    big.ms = std::max(kSharedLogEntries, kSharedLogEntriesBatch);
-    big.dev_bytes = 24 * 256;
+    big.pool = kReadyPoolWide;
+    big.opcap = kOpsPerGeneration + 32;
+    big.qs = std::max(kSharedQueueEntries, kSharedOverflowEntries);
+    big.ms = std::max(kSharedLogEntries, kSharedLogEntriesWide);
+    big.dev_bytes = 32 + 24 * 256;
     big.no_side = 0;
     if (set_smem_limits(4 * (int)smem_per_warp(big)) != cudaSuccess) return GMG_ECUDA;
     g_smem_set = true;
   }
   int bps = 0;
-  const bool types = G.ntypes >= 2;
-  const void* fn = inc ? inc_kernel_ptr(L.reg, G.dev_key != 0, G.t32 != 0, types, batch)
-                       : full_kernel_ptr(L.reg, G.dev_key != 0, G.t32 != 0, types, batch);
+  const void* fn = inc ? inc_kernel_ptr(G) : full_kernel_ptr(G);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, 32 * L.wpb, L.smem) != cudaSuccess)
     return GMG_ECUDA;
   bps = std::max(bps, 1);
@@ -607,6 +597,8 @@ bool staged(const sim_opts_t* o) { return o && o->gmg_staging == GMG_STAGING_SHA
 bool l1_path(const sim_opts_t* o) { return o && o->gmg_staging == GMG_STAGING_L1; }
 
 bool g_stage_smem_set = false;
+constexpr int64_t kStageSmallBytes = 16 << 10;
+constexpr int kStageFewCandidates = 32;
 
 // sim_batch with the GMG staged in shared memory: one CTA per SM with as many
 // warps (up to kStageMaxWarps) as fit beside the staged copy.
@@ -645,11 +637,17 @@ int plan_staged(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L) {
 
 // Full placements with pure-latency transfers: the staged-GMG kernel when the
 // caller asks for it (an error if it cannot serve the graph) or by default
-// when it can, else the L1 path.  *stg tells which.
+// for small graphs and few candidates, else the L1 path.  *stg tells which.
 int plan_full(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, bool* stg) {
   *stg = false;
   if (l1_path(o)) return plan_launch(g, K, o, false, L);
-  const int rc = plan_staged(g, K, o, L);
+  // With compact records on both paths, staging pays where the copy leaves the
+  // L1 cache to the candidates' own arrays (prefill graph, N = 3088, a 90 KB
+  // copy: 1.82 against 1.84 ms for 14 candidates, 1.85 against 1.79 ms for 64,
+  // 3.58 against 3.23 ms for 4,096; the 50-op graph, 2 KB: 65.1 against 67.2 us
+  // for 256, 92 against 99 us for 4,096).
+  const bool small = stage_smem_bytes(g->dg.n, g->dg.n_edges) <= kStageSmallBytes || K <= kStageFewCandidates;
+  const int rc = staged(o) || small ? plan_staged(g, K, o, L) : GMG_EINVAL;
   if (rc == GMG_OK) {
     *stg = true;
     return GMG_OK;
@@ -829,14 +827,14 @@ int plan_base(const gmg* g, const sim_opts_t* o, BasePlan& B) {
   int rc = B.arb ? plan_arb(g, 1, o, L, B.A, kBase) : plan_launch(g, 1, o, false, L);
   if (rc) return rc;
   L.wpb = 1;
-  L.P.dev_bytes = dev_smem_bytes(G.D, 8);  // the base snapshot keeps 64-bit times
+  if (B.arb) L.P.dev_bytes = dev_smem_bytes(G.D, 8, false);  // the arbitrated base keeps 64-bit times
   L.smem = smem_per_warp(L.P);
   if (B.arb) {
     B.A.smem_std = (int64_t)L.smem;
     L.smem += (size_t)B.A.smem_arb;
   }
   B.nck = B.arb ? kArbCheckpoints : kCheckpoints;
-  B.ckq = std::min(L.P.qcap, kCheckpointQueue);
+  B.ckq = std::min(L.P.pend_cap - 32, kCheckpointQueue);
   B.ckm = std::min(L.P.mcap, kCheckpointLog);
   B.ld = (int)align_up(std::max(G.n, 1), 16);
   B.stride = std::max(1, G.n / (B.nck - 1));
@@ -932,26 +930,40 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   }
   put(L.off_cons, b.cons.data(), 4 * b.cons.size());
   put(L.off_roots, b.roots.data(), 8 * b.roots.size());
-  // The batched sweep: graphs on more accelerators than a warp has lanes
-  // (accelerator state in shared memory) whose READY keys have room for the
-  // duration class; its root keys carry the class of the op's shortest
-  // duration over the accelerator types.
+  // Root keys of the READY pool: the earliest finish from the op's shortest
+  // duration over the accelerator types (the encoding of ReadyCodec).
   int tb = 1;
   while (tb < 62 && (int64_t(1) << tb) <= b.time_bound) ++tb;
   const bool dev_key = tb + b.ib + 2 + 8 <= 63;
-  const bool batch = b.D >= kBatchMinDevices && dev_key && tb + b.ib + 2 + kQB <= 63;
-  if (batch) {
+  int qb = std::min(kMaxQB, 63 - (tb + b.ib));
+  if (qb < 6) qb = 0;
+  {
     std::vector<uint64_t> rq(b.roots.size());
     for (size_t r = 0; r < b.roots.size(); ++r) {
       const uint32_t i = (uint32_t)(b.roots[r] & ((uint64_t(1) << b.ib) - 1));
       int64_t lo = b.ops[i].dur;
       if (b.T)
         for (int t = 0; t < b.T; ++t) lo = std::min(lo, b.durt[(size_t)i * b.T + t]);
-      uint32_t q = 0;
-      while (q < 31 && (int64_t(2) << q) <= lo) ++q;
-      rq[r] = (b.roots[r] << kQB) | q;
+      uint64_t q = 0;
+      if (qb) {
+        const int m = qb - 5;
+        const uint32_t x = (uint32_t)std::min<int64_t>(lo, 0x7fffffff);
+        int e = 0;
+        while ((x >> e) >> m) ++e;
+        q = ((uint64_t)e << m) | (x >> e);
+      }
+      rq[r] = ((uint64_t)b.ops[i].release << (b.ib + qb)) | ((uint64_t)i << qb) | q;
     }
     put(L.off_roots_q, rq.data(), 8 * rq.size());
+  }
+  int64_t most_bytes = 0;
+  {
+    std::vector<int64_t> bytes(b.n);
+    for (int i = 0; i < b.n; ++i) {
+      bytes[i] = b.ops[i].bytes;
+      most_bytes = std::max(most_bytes, bytes[i]);
+    }
+    put(L.off_bytes, bytes.data(), 8 * bytes.size());
   }
   put(L.off_cap, b.cap.data(), 8 * b.cap.size());
   put(L.off_base, b.base.data(), 8 * b.base.size());
@@ -982,6 +994,8 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   G.cons = reinterpret_cast<const uint32_t*>(w + L.off_cons);
   G.root_keys = reinterpret_cast<const uint64_t*>(w + L.off_roots);
   G.root_keys_q = reinterpret_cast<const uint64_t*>(w + L.off_roots_q);
+  G.bytes = reinterpret_cast<const int64_t*>(w + L.off_bytes);
+  G.big_bytes = most_bytes >= (int64_t(1) << 48) ? 1 : 0;
   G.cap = reinterpret_cast<const int64_t*>(w + L.off_cap);
   G.base = reinterpret_cast<const int64_t*>(w + L.off_base);
   G.avail0 = reinterpret_cast<const int64_t*>(w + L.off_avail);
@@ -998,8 +1012,12 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   G.nroots = b.nroots;
   G.ib = b.ib;
   G.tb = tb;
+  G.opmask = (uint32_t)((uint64_t(1) << b.ib) - 1);
+  G.ds = b.ib + 2 + tb;
+  G.keymask = dev_key ? (uint64_t(1) << G.ds) - 1 : ~uint64_t(0);
+  G.qsh = b.ib + qb;
   G.dev_key = dev_key ? 1 : 0;
-  G.batch = batch ? 1 : 0;
+  G.qb = qb;
   G.st_hot = reinterpret_cast<const uint4*>(w + L.off_st_hot);
   G.st_rel = reinterpret_cast<const int32_t*>(w + L.off_st_rel);
   G.n_edges = b.E;
@@ -1008,7 +1026,8 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   // every time < 2^tb fits int32; the 32-bit instances also take the
   // accelerator id from the event key
   G.t32 = (G.tb <= 31 && G.dev_key) ? 1 : 0;
-  G.stage_ok = (b.stage_ready && G.t32 && G.D <= 32) ? 1 : 0;
+  G.hot_ok = (b.stage_ready && G.t32) ? 1 : 0;
+  G.stage_ok = (G.hot_ok && G.D <= 32) ? 1 : 0;
   G.uniform = b.uniform ? 1 : 0;
   gmg_info_t& I = g->info;
   std::memset(&I, 0, sizeof(I));
@@ -1027,7 +1046,7 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   g->xfer_bound = b.xfer_bound;
   g->shared_links = b.shared_links ? 1 : 0;
   I.default_queue_cap = std::min<int64_t>(b.queue_bound, kDefaultQueueCap);
-  I.batched_sweep = G.batch;
+  I.batched_sweep = b.D > 32 && dev_key && tb + b.ib + 2 + 5 <= 63 ? 1 : 0;
   I.t32 = G.t32;
   // staged only where the copy also fits beside a warp's areas on this device
   I.stageable = 0;
@@ -1085,7 +1104,7 @@ int sim_batch(const gmg_t* g, const uint8_t* d_place, int32_t K, int32_t ld, con
   const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   cudaError_t e = arb ? launch_arb_any(g, L, Q, nullptr, st)
                       : stg ? launch_full_staged(P, L.grid, 32 * L.wpb, L.smem, st)
-                            : launch_full(L.reg, P, L.grid, 32 * L.wpb, L.smem, st);
+                            : launch_full(P, L.grid, 32 * L.wpb, L.smem, st);
   return e == cudaSuccess ? GMG_OK : GMG_ECUDA;
 }
 
@@ -1162,7 +1181,7 @@ extern "C" int sim_batch_noalloc(const gmg_t* g, const uint8_t* d_place, int32_t
   P.K = K;
   P.scratch = scratch;
   const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const cudaError_t e = arb ? launch_arb_any(g, L, Q, nullptr, st) : launch_full(L.reg, P, L.grid, 32 * L.wpb, L.smem, st);
+  const cudaError_t e = arb ? launch_arb_any(g, L, Q, nullptr, st) : launch_full(P, L.grid, 32 * L.wpb, L.smem, st);
   return e == cudaSuccess ? GMG_OK : GMG_ECUDA;
 }
 
@@ -1231,7 +1250,7 @@ int base_create(const gmg_t* g, const uint8_t* d_base_place, const sim_opts_t* o
     b->ck = A.ck;
     e = launch_arb_base(g->dg.ntypes >= 2, A, B.L.smem, reinterpret_cast<cudaStream_t>(stream));
   } else {
-    e = launch_base(B.L.reg, P, B.L.smem, reinterpret_cast<cudaStream_t>(stream));
+    e = launch_base(P, B.L.smem, reinterpret_cast<cudaStream_t>(stream));
   }
   if (e != cudaSuccess) {
     delete b;
@@ -1367,7 +1386,7 @@ int sim_incremental(const gmg_t* g, const gmg_base_t* b, const int32_t* d_move_o
   P.move_off = d_move_off;
   P.move_op = d_move_op;
   P.move_dev = d_move_dev;
-  cudaError_t e = launch_inc(L.reg, P, L.grid, 32 * L.wpb, L.smem, reinterpret_cast<cudaStream_t>(stream));
+  cudaError_t e = launch_inc(P, L.grid, 32 * L.wpb, L.smem, reinterpret_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? GMG_OK : GMG_ECUDA;
 }
 

@@ -8,19 +8,19 @@ namespace {
 // ---------------------------------------------------------------------------
 // sim_incremental: K move lists against the base.
 // ---------------------------------------------------------------------------
-template <bool kReg, bool kKey, bool kT32, bool kTypes, bool kBatch>
-__device__ void regen(Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>& S, uint32_t p);
+template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
+__device__ void regen(Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>& S, uint32_t p);
 
-template <bool kReg, bool kKey, bool kT32, bool kTypes, bool kBatch>
-__device__ void inc_candidate(Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>& S, const SimParams& P, int64_t k, uint8_t* crow) {
-  using tm_t = typename Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>::tm_t;
+template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
+__device__ void inc_candidate(Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>& S, const SimParams& P, int64_t k, uint8_t* crow) {
+  using tm_t = typename Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>::tm_t;
   const DevGmg& g = S.g;
   const DevBase& B = P.base;
   const unsigned lane = lane_id();
   const int32_t m0 = P.move_off[k], m1 = P.move_off[k + 1];
   const int32_t nm = m1 - m0;
   const int words = (g.n + 31) >> 5;
-  for (int w = lane; w < words; w += 32) S.bits[w] = 0u;
+  for (int w = lane; w < words; w += 32) S.bits()[w] = 0u;
   __syncwarp();
   // Validate the move list; duplicates are found with the (zeroed) bitmap.
   bool bad_range = false, dup = false;
@@ -31,7 +31,7 @@ __device__ void inc_candidate(Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>& S, co
       bad_range = true;
     } else {
       const uint32_t b = 1u << (op & 31);
-      if (atomicOr(&S.bits[op >> 5], b) & b) dup = true;
+      if (atomicOr(&S.bits()[op >> 5], b) & b) dup = true;
     }
   }
   bad_range = __any_sync(kFullMask, bad_range);
@@ -108,16 +108,16 @@ __device__ void inc_candidate(Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>& S, co
   const int64_t* sc = B.ck_scalars + (int64_t)c * 8;
   const int qsz = (int)sc[0];
   const int msz = (int)sc[7];
-  if (qsz > S.q.cap || msz > S.log.cap) {
+  if (qsz > P.pend_cap - 32 || msz > P.mcap) {
     S.write_invalid(k, GMG_SIM_QUEUE);
     return;
   }
   // Restore the simulator state of checkpoint c.
   S.Tc = (tm_t)B.ck_time[c];
+  S.drained = (tm_t)sc[3];
   S.rootptr = (int)sc[1];
   S.load_root();
-  S.score = sc[2];
-  S.makespan = (tm_t)sc[3];
+  S.score = lane == 0 ? sc[2] : 0;  // lanes add up their ops' finishes
   S.vflag = (int32_t)sc[4];
   S.vt = sc[5];
   S.vop = (int32_t)(sc[6] >> 32);
@@ -127,15 +127,16 @@ __device__ void inc_candidate(Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>& S, co
   S.readypops = 0;
   S.last_t = -1;
   S.status = GMG_SIM_OK;
-  S.rk_reg = kKeyMax;
   S.opn = 0;
   S.dv.load(B.ck_dev + (int64_t)c * 3 * g.D);
-  for (int r = lane; r < g.R; r += 32) S.creq[r] = B.ck_creq[(int64_t)c * g.R + r];
+  for (int r = lane; r < g.R; r += 32) S.creq()[r] = B.ck_creq[(int64_t)c * g.R + r];
   // ops started before T_c are those with base ready time < T_c: they keep
   // their base finish; the others start with no finish time
   S.fill_fin();
-  // READY keys at T_c; a moved op's key is recomputed (its inputs' transfer
+  // READY keys at T_c (the pool first, the others to the heap); a moved op's key is recomputed (its inputs' transfer
   // times change; its predecessors all finished before T_c).
+  constexpr int kHeld = kNarrow ? 32 : kReadyPoolWide;
+  if constexpr (kNarrow) S.pd.r = S.pd.e = Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>::kNever;
   for (int x = lane; x < qsz; x += 32) {
     uint64_t key = B.ck_qkey[(int64_t)c * B.ckq + x];
     const uint32_t op = S.rq.op(key);
@@ -151,11 +152,14 @@ __device__ void inc_candidate(Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>& S, co
         if (dp != dx) a += S.xfer(dp, dx, op_durbytes(g.ops, p).y, op_xqsucc(g.ops, p).xq);
         rx = a > rx ? a : rx;
       }
-      key = S.rq.make(rx, op, kBatch ? dur_class(S.dur_of(op, dx, op_durbytes(g.ops, op).x)) : 0u);
+      key = S.rq.make((tm_t)rx, op, (tm_t)S.dur_of(op, dx, op_durbytes(g.ops, op).x));
     }
-    *S.q.kp(x) = key;
+    if (x >= kHeld) *S.q.kp(x - kHeld) = key;
+    else if constexpr (kNarrow) S.hold_op((tm_t)S.rq.time(key), op);
+    else S.pool[x] = key;
   }
-  S.q.size = qsz;
+  S.q.size = qsz > kHeld ? qsz - kHeld : 0;
+  if constexpr (!kNarrow) S.empty_pool(qsz < kHeld ? qsz : kHeld);
   // Logged HBM events at T_c, except those of an op p with a moved
   // successor: the receiving accelerators and last consumers of p's output
   // changed (its receive allocations and releases all happen at times
@@ -172,7 +176,7 @@ __device__ void inc_candidate(Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>& S, co
       if (!kKey) dv8 = B.ck_mdev[(int64_t)c * B.ckm + idx];
       keep = true;
       const uint32_t cls = S.kc.cls(e), op = S.kc.op(e);
-      const int dev = kKey ? (int)(e >> S.ds) : (int)dv8;
+      const int dev = kKey ? (int)(e >> g.ds) : (int)dv8;
       const uint4 ls = op_lists(g.ops, op);
       bool moved_succ = false;
       for (uint32_t u = 0; u < ls.y && !moved_succ; ++u) {
@@ -241,8 +245,8 @@ __device__ void inc_candidate(Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>& S, co
 // placement: receive copies on every remote accelerator of its successors
 // (allocated at f_p), and the releases that are already determined because
 // every listed consumer on that accelerator has finished.
-template <bool kReg, bool kKey, bool kT32, bool kTypes, bool kBatch>
-__device__ void regen(Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>& S, uint32_t p) {
+template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
+__device__ void regen(Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>& S, uint32_t p) {
   const DevGmg& g = S.g;
   const unsigned lane = lane_id();
   const int64_t fp = S.fb[p];
@@ -311,12 +315,12 @@ __device__ void regen(Sim<kReg, kInc, kKey, kT32, kTypes, kBatch>& S, uint32_t p
   S.log_event(lane == 0, S.kc.make(m > hm ? m : hm, kFree, p), dp);
 }
 
-template <bool kReg, bool kKey, bool kT32, bool kTypes, bool kBatch>
-__global__ void __launch_bounds__(128, kBatch ? kBatchBlocksPerSM : 7) sim_inc_kernel(const __grid_constant__ SimParams P) {
+template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
+__global__ void __launch_bounds__(128, kBlocksPerSM) sim_inc_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
-  Sim<kReg, kInc, kKey, kT32, kTypes, kBatch> S(P);
+  Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot> S(P);
   setup_slot(S, P, wib, slot, smem);
   S.rb = P.base.rb;
   S.fb = P.base.fb;
@@ -326,22 +330,24 @@ __global__ void __launch_bounds__(128, kBatch ? kBatchBlocksPerSM : 7) sim_inc_k
 
 }  // namespace
 
-// Instances by (accelerator state in registers, accelerator id in the event
-// key, 32-bit times, accelerator types, batched sweep).  32-bit times are only
-// chosen with the accelerator id in the key; the batched sweep only with
-// accelerator state in shared memory and the id in the key.
-template <bool R, bool K, bool T32, bool B>
-const void* inc_ptr5(bool types) {
-  return types ? (const void*)sim_inc_kernel<R, K, T32, true, B> : (const void*)sim_inc_kernel<R, K, T32, false, B>;
+// Instances by (at most 32 accelerators, accelerator id in the event key,
+// 32-bit times, accelerator types; compact records wherever the graph has
+// them).  32-bit times are only chosen with the accelerator id in the key,
+// compact records only with 32-bit times.
+template <bool N, bool K, bool T32>
+const void* inc_ptr(bool types) {
+  return types ? (const void*)sim_inc_kernel<N, K, T32, true, kHotNone>
+               : (const void*)sim_inc_kernel<N, K, T32, false, kHotNone>;
 }
-const void* inc_kernel_ptr(bool reg, bool key, bool t32, bool types, bool batch) {
-  if (reg) {
-    if (!key) return inc_ptr5<true, false, false, false>(types);
-    return t32 ? inc_ptr5<true, true, true, false>(types) : inc_ptr5<true, true, false, false>(types);
-  }
-  if (!key) return inc_ptr5<false, false, false, false>(types);
-  if (batch) return t32 ? inc_ptr5<false, true, true, true>(types) : inc_ptr5<false, true, false, true>(types);
-  return t32 ? inc_ptr5<false, true, true, false>(types) : inc_ptr5<false, true, false, false>(types);
+template <bool N>
+const void* inc_ptr_n(bool key, bool t32, bool types, bool hot) {
+  if (!key) return inc_ptr<N, false, false>(types);
+  if (hot) return (const void*)sim_inc_kernel<N, true, true, false, kHotGlobal>;
+  return t32 ? inc_ptr<N, true, true>(types) : inc_ptr<N, true, false>(types);
+}
+const void* inc_kernel_ptr(const DevGmg& g) {
+  const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
+  return g.D <= 32 ? inc_ptr_n<true>(key, t32, types, hot) : inc_ptr_n<false>(key, t32, types, hot);
 }
 
 }  // namespace gsim

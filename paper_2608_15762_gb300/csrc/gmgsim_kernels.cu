@@ -8,10 +8,10 @@ namespace {
 // ---------------------------------------------------------------------------
 // base_create: simulate the base placement once, recording resume points.
 // ---------------------------------------------------------------------------
-template <bool kReg, bool kKey, bool kTypes, bool kBatch>
-__global__ void __launch_bounds__(32) sim_base_kernel(const __grid_constant__ SimParams P) {
+template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
+__global__ void __launch_bounds__(32, 1) sim_base_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
-  Sim<kReg, kBase, kKey, false, kTypes, kBatch> S(P);
+  Sim<kNarrow, kBase, kKey, kT32, kTypes, true, kHot> S(P);
   setup_slot(S, P, 0, 0, smem);
   const DevBase& B = P.base;
   const unsigned lane = lane_id();
@@ -20,7 +20,6 @@ __global__ void __launch_bounds__(32) sim_base_kernel(const __grid_constant__ Si
   for (int c = lane * 16; c < B.ld; c += 512)
     *reinterpret_cast<uint4*>(B.row + c) = *reinterpret_cast<const uint4*>(P.place + c);
   for (int c = lane; c < B.nck; c += 32) B.ck_time[c] = kI64Max;
-  S.fbuf = B.fb;
   S.row = P.place;
   __syncwarp();
   if (S.row_has_bad_device(P.place)) {
@@ -31,22 +30,24 @@ __global__ void __launch_bounds__(32) sim_base_kernel(const __grid_constant__ Si
   S.ck = 0;
   S.next_ck = 0;
   // checkpoint 0: the initial state, valid for every resume time >= 0
-  S.maybe_checkpoint(S.rq.make(0, 0u, 0u));
+  S.maybe_checkpoint(0);
   S.run();
   if (lane == 0) B.status[0] = S.status;
   if (S.status != GMG_SIM_OK) return;
   int32_t miss = 0;
   for (int r = lane; r < S.g.R; r += 32) {
-    const int64_t c = S.creq[r];
+    const int64_t c = S.creq()[r];
     B.res_creq[r] = c;
     miss += c > __ldg(S.g.deadline + r) ? 1 : 0;
   }
   miss = (int32_t)__reduce_add_sync(kFullMask, (unsigned)miss);
   S.dv.write_peak(B.res_peak);
+  const int64_t makespan = S.dv.max_busy(S.g);
+  const int64_t score = warp_sum_i64(S.score);
   if (lane == 0) {
     int64_t* rs = B.res_scalars;
-    rs[0] = S.makespan;
-    rs[1] = S.vflag ? kI64Max : S.score;
+    rs[0] = makespan;
+    rs[1] = S.vflag ? kI64Max : score;
     rs[2] = S.vflag;
     rs[3] = S.vop;
     rs[4] = S.vdev;
@@ -133,32 +134,43 @@ __global__ void __launch_bounds__(256) select_final_kernel(const Rank* part, int
 // ---------------------------------------------------------------------------
 size_t select_rank_bytes() { return sizeof(Rank); }
 
-const void* full_kernel_ptr(bool reg, bool key, bool t32, bool types, bool batch);  // gmgsim_full.cu
-const void* inc_kernel_ptr(bool reg, bool key, bool t32, bool types, bool batch);   // gmgsim_inc.cu
+const void* full_kernel_ptr(const DevGmg& g);  // gmgsim_full.cu
+const void* inc_kernel_ptr(const DevGmg& g);   // gmgsim_inc.cu
 
-template <bool R, bool K, bool B>
-const void* base_ptr4(bool types) {
-  return types ? (const void*)sim_base_kernel<R, K, true, B> : (const void*)sim_base_kernel<R, K, false, B>;
+// Instances by (at most 32 accelerators, accelerator id in the event key,
+// 32-bit times, accelerator types; compact records wherever the graph has
+// them).  32-bit times are only chosen with the accelerator id in the key,
+// compact records only with 32-bit times.
+template <bool N, bool K, bool T32>
+const void* base_ptr(bool types) {
+  return types ? (const void*)sim_base_kernel<N, K, T32, true, kHotNone>
+               : (const void*)sim_base_kernel<N, K, T32, false, kHotNone>;
 }
-const void* base_kernel_ptr(bool reg, bool key, bool types, bool batch) {
-  if (reg) return key ? base_ptr4<true, true, false>(types) : base_ptr4<true, false, false>(types);
-  if (!key) return base_ptr4<false, false, false>(types);
-  return batch ? base_ptr4<false, true, true>(types) : base_ptr4<false, true, false>(types);
+template <bool N>
+const void* base_ptr_n(bool key, bool t32, bool types, bool hot) {
+  if (!key) return base_ptr<N, false, false>(types);
+  if (hot) return (const void*)sim_base_kernel<N, true, true, false, kHotGlobal>;
+  return t32 ? base_ptr<N, true, true>(types) : base_ptr<N, true, false>(types);
+}
+const void* base_kernel_ptr(const DevGmg& g) {
+  const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
+  return g.D <= 32 ? base_ptr_n<true>(key, t32, types, hot) : base_ptr_n<false>(key, t32, types, hot);
 }
 
 cudaError_t set_smem_limits(int smem) {
-  for (int r = 0; r < 2; ++r)
-    for (int k = 0; k < 2; ++k)
-      for (int t = 0; t < 2; ++t)
-        for (int y = 0; y < 2; ++y)
-          for (int b = 0; b < 2; ++b) {
-            const void* fns[] = {full_kernel_ptr(r, k, t, y, b), inc_kernel_ptr(r, k, t, y, b),
-                                 base_kernel_ptr(r, k, y, b)};
-            for (const void* f : fns) {
-              const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-              if (e != cudaSuccess) return e;
-            }
-          }
+  DevGmg g{};
+  for (int c = 0; c < 32; ++c) {
+    g.D = c & 1 ? 32 : 33;
+    g.dev_key = (c >> 1) & 1;
+    g.t32 = (c >> 2) & 1;
+    g.ntypes = c & 8 ? 2 : 0;
+    g.hot_ok = (c >> 4) & 1;
+    const void* fns[] = {full_kernel_ptr(g), inc_kernel_ptr(g), base_kernel_ptr(g)};
+    for (const void* f : fns) {
+      const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (e != cudaSuccess) return e;
+    }
+  }
   return cudaSuccess;
 }
 
@@ -170,18 +182,19 @@ static cudaError_t launch_ptr(const void* fn, const SimParams& P, int grid, int 
   return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, st);
 }
 
-cudaError_t launch_full(bool reg, const SimParams& P, int grid, int block, size_t smem, cudaStream_t st) {
-  return launch_ptr(full_kernel_ptr(reg, P.g.dev_key != 0, P.g.t32 != 0, P.g.ntypes >= 2, P.g.batch != 0), P, grid,
-                    block, smem, st);
+cudaError_t launch_full(const SimParams& P, int grid, int block, size_t smem, cudaStream_t st) {
+  return launch_ptr(full_kernel_ptr(P.g), P, grid, block,
+                    smem, st);
 }
 
-cudaError_t launch_inc(bool reg, const SimParams& P, int grid, int block, size_t smem, cudaStream_t st) {
-  return launch_ptr(inc_kernel_ptr(reg, P.g.dev_key != 0, P.g.t32 != 0, P.g.ntypes >= 2, P.g.batch != 0), P, grid,
-                    block, smem, st);
+cudaError_t launch_inc(const SimParams& P, int grid, int block, size_t smem, cudaStream_t st) {
+  return launch_ptr(inc_kernel_ptr(P.g), P, grid, block,
+                    smem, st);
 }
 
-cudaError_t launch_base(bool reg, const SimParams& P, size_t smem, cudaStream_t st) {
-  return launch_ptr(base_kernel_ptr(reg, P.g.dev_key != 0, P.g.ntypes >= 2, P.g.batch != 0), P, 1, 32, smem, st);
+cudaError_t launch_base(const SimParams& P, size_t smem, cudaStream_t st) {
+  return launch_ptr(base_kernel_ptr(P.g), P, 1, 32, smem,
+                    st);
 }
 
 cudaError_t launch_select(const int32_t* status, const int32_t* viol, const int64_t* score,

@@ -17,10 +17,13 @@
 //                  of a successor at f_i (Recv before Send, Sec. 3.5.2), each
 //                  released by its last listed consumer there (Sec. 3.3.2).
 //
-// READY keys live in a warp-cooperative 32-ary min-heap: the 32 children of
-// a node are compared by the 32 lanes at once (one coalesced load, two
-// redux.sync), so a pop costs log32(size) warp steps.  Ops without
-// predecessors never enter it: their keys are pre-sorted on the host.
+// READY keys are taken many at a time (Sim::run): every pending key carries a
+// lower bound of its op's finish, and all pending keys with a ready time below
+// the smallest of these bounds are started together, one op per lane -- nothing
+// that they make ready can precede any of them.  Pending keys sit in a pool of
+// 32 or more slots in shared memory; what does not fit goes to a
+// warp-cooperative 32-ary min-heap.  Ops without predecessors enter the pool
+// when they are due: their keys are pre-sorted on the host.
 //
 // HBM events are appended to a per-warp log in O(1).  Every event produced
 // while handling READY(r, .) happens at a time >= r, so once the next READY
@@ -144,43 +147,48 @@ __device__ __forceinline__ uint4 op_cons(const OpRec* ops, uint32_t i) {
   return __ldg(reinterpret_cast<const uint4*>(ops + i) + 3);  // cons_off, ncons, req, flags
 }
 
+// The codecs' parameters stay in the launch parameters (constant bank).
 struct KeyCodec {
-  int ib;
-  uint64_t mask;
+  const DevGmg& g;
   template <typename TM>
   __device__ __forceinline__ uint64_t make(TM t, uint32_t cls, uint32_t op) const {
     using U = typename std::make_unsigned<TM>::type;
-    return ((uint64_t)(U)t << (ib + 2)) | ((uint64_t)cls << ib) | (uint64_t)op;
+    return ((uint64_t)(U)t << (g.ib + 2)) | ((uint64_t)cls << g.ib) | (uint64_t)op;
   }
-  __device__ __forceinline__ int64_t time(uint64_t k) const { return (int64_t)(k >> (ib + 2)); }
-  __device__ __forceinline__ uint64_t time_floor(int64_t t) const { return (uint64_t)t << (ib + 2); }
-  __device__ __forceinline__ uint32_t cls(uint64_t k) const { return (uint32_t)(k >> ib) & 3u; }
-  __device__ __forceinline__ uint32_t op(uint64_t k) const { return (uint32_t)(k & mask); }
+  __device__ __forceinline__ int64_t time(uint64_t k) const { return (int64_t)(k >> (g.ib + 2)); }
+  __device__ __forceinline__ uint64_t time_floor(int64_t t) const { return (uint64_t)t << (g.ib + 2); }
+  __device__ __forceinline__ uint32_t cls(uint64_t k) const { return (uint32_t)(k >> g.ib) & 3u; }
+  __device__ __forceinline__ uint32_t op(uint64_t k) const { return (uint32_t)k & g.opmask; }
 };
 
-// READY keys as queued: the KeyCodec key with class READY, shifted up by qb
-// bits that hold the op's duration class (floor(log2) of a lower bound of its
-// duration) in the batched sweep; qb = 0 otherwise (then equal to the
-// KeyCodec key).  The class bits sit below the op id, so they never change
-// the order of two keys.
+// READY keys of the pool: time, op id, then qb bits that hold how far the op's
+// finish is from its ready time at least (floating point, rounded down: qb - 5
+// bits of mantissa below a 5-bit exponent; qb = 0 where the key has no room,
+// then the distance is taken as 1).  These bits are the lowest, so they never
+// change the order of two keys.
 struct ReadyCodec {
-  int ib, qb;
-  uint64_t mask;
-  template <typename TM>
-  __device__ __forceinline__ uint64_t make(TM t, uint32_t op, uint32_t q) const {
-    using U = typename std::make_unsigned<TM>::type;
-    return ((((uint64_t)(U)t << (ib + 2)) | (uint64_t)op) << qb) | (qb ? (uint64_t)q : 0ull);
+  const DevGmg& g;
+  __device__ __forceinline__ uint32_t enc(uint32_t x) const {  // x >= 1
+    const int m = g.qb - 5;
+    const int e = max(0, 32 - m - __clz(x));
+    return ((uint32_t)e << m) | (x >> e);
   }
-  __device__ __forceinline__ int64_t time(uint64_t k) const { return (int64_t)(k >> (ib + 2 + qb)); }
-  __device__ __forceinline__ uint32_t op(uint64_t k) const { return (uint32_t)((k >> qb) & mask); }
-  __device__ __forceinline__ uint32_t q(uint64_t k) const { return (uint32_t)k & ((1u << qb) - 1u); }
+  template <typename TM>
+  __device__ __forceinline__ uint64_t make(TM t, uint32_t op, TM least) const {
+    using U = typename std::make_unsigned<TM>::type;
+    const uint32_t x = sizeof(TM) > 4 && least > (TM)0x7fffffff ? 0x7fffffffu : (uint32_t)least;
+    return ((uint64_t)(U)t << g.qsh) | ((uint64_t)op << g.qb) | (g.qb ? enc(x) : 0u);
+  }
+  __device__ __forceinline__ int64_t time(uint64_t k) const { return (int64_t)(k >> g.qsh); }
+  __device__ __forceinline__ uint32_t op(uint64_t k) const { return (uint32_t)(k >> g.qb) & g.opmask; }
+  // The earliest finish of the key's op.
+  __device__ __forceinline__ int64_t bound(uint64_t k) const {
+    if (g.qb == 0) return time(k) + 1;
+    const int m = g.qb - 5;
+    const uint32_t q = (uint32_t)k & ((1u << g.qb) - 1u);
+    return time(k) + (int64_t)((q & ((1u << m) - 1u)) << (q >> m));
+  }
 };
-
-// floor(log2(dur)) for dur >= 1, at most 31: 2^class is a lower bound of dur.
-__device__ __forceinline__ uint32_t dur_class(int64_t dur) {
-  const uint32_t c = 63u - (uint32_t)__clzll((unsigned long long)dur);
-  return c < 31u ? c : 31u;
-}
 
 __device__ __forceinline__ int64_t warp_sum_i64(int64_t v) {
 #pragma unroll
@@ -195,11 +203,14 @@ __device__ __forceinline__ int64_t warp_sum_i64(int64_t v) {
 // arguments; lane 0 performs the stores.
 // ---------------------------------------------------------------------------
 struct ReadyHeap {
+  const SimParams& P;
   uint64_t* sk;
-  uint64_t* gk;
-  int qs, cap, size;
+  uint8_t* sl;  // the warp's scratch slot
+  int size;
 
-  __device__ __forceinline__ uint64_t* kp(int i) const { return i < qs ? sk + i : gk + (i - qs); }
+  __device__ __forceinline__ uint64_t* kp(int i) const {
+    return i < P.qs ? sk + i : reinterpret_cast<uint64_t*>(sl + P.off_qk) + (i - P.qs);
+  }
   __device__ __forceinline__ uint64_t top() const { return size > 0 ? sk[0] : kKeyMax; }
 
   __device__ void sift_down(int pos, uint64_t x) {
@@ -220,24 +231,6 @@ struct ReadyHeap {
     __syncwarp();
   }
 
-  // The same as sift_down while every slot in use is in shared memory.
-  __device__ void sift_down_shared(int pos, uint64_t x) {
-    const unsigned lane = lane_id();
-    while (true) {
-      const int c0 = pos * 32 + 1;
-      if (c0 >= size) break;
-      const int idx = c0 + (int)lane;
-      const uint64_t ck = idx < size ? sk[idx] : kKeyMax;
-      const uint64_t m = warp_min_u64(ck);
-      if (m >= x) break;
-      const int src = __ffs(__ballot_sync(kFullMask, ck == m)) - 1;
-      if (lane == 0) sk[pos] = m;
-      pos = c0 + src;
-    }
-    if (lane == 0) sk[pos] = x;
-    __syncwarp();
-  }
-
   __device__ void pop() {
     const int n = --size;
     if (n == 0) return;
@@ -245,39 +238,8 @@ struct ReadyHeap {
     sift_down(0, x);
   }
 
-  // pop / push with a branch for a heap held entirely in shared memory (the
-  // batched sweep's larger shared part makes that the common case)
-  __device__ void pop_fast() {
-    const int n = --size;
-    if (n == 0) return;
-    if (n < qs) {
-      sift_down_shared(0, sk[n]);
-      return;
-    }
-    const uint64_t x = *kp(n);
-    sift_down(0, x);
-  }
-
-  __device__ bool push_fast(uint64_t key) {
-    if (size >= cap) return false;
-    if (size < qs) {
-      int pos = size++;
-      while (pos > 0) {
-        const int par = (pos - 1) >> 5;
-        const uint64_t pk = sk[par];
-        if (pk <= key) break;
-        if (lane_id() == 0) sk[pos] = pk;
-        pos = par;
-      }
-      if (lane_id() == 0) sk[pos] = key;
-      __syncwarp();
-      return true;
-    }
-    return push(key);
-  }
-
   __device__ bool push(uint64_t key) {
-    if (size >= cap) return false;
+    if (size >= P.qcap) return false;
     int pos = size++;
     while (pos > 0) {
       const int par = (pos - 1) >> 5;
@@ -302,53 +264,62 @@ struct ReadyHeap {
 };
 
 // ---------------------------------------------------------------------------
-// HBM event log: unordered 8-byte entries -- (accelerator << ds) | key when
+// HBM event log: unordered 8-byte entries -- (accelerator << g.ds) | key when
 // the accelerator id fits above the key, else the key with the accelerator
 // in a side byte array.  Slots [0, ms) are in shared memory, the rest in
 // global scratch.
 // ---------------------------------------------------------------------------
 struct MemLog {
+  const SimParams& P;
   uint64_t* sk;
   uint8_t* sd;
-  uint64_t* gk;
-  uint8_t* gd;
-  int ms, cap, n;
+  uint8_t* sl;  // the warp's scratch slot
+  int n;
 
-  __device__ __forceinline__ uint64_t* kp(int i) const { return i < ms ? sk + i : gk + (i - ms); }
-  __device__ __forceinline__ uint8_t* dp(int i) const { return i < ms ? sd + i : gd + (i - ms); }
+  __device__ __forceinline__ uint64_t* kp(int i) const {
+    return i < P.ms ? sk + i : reinterpret_cast<uint64_t*>(sl + P.off_mk) + (i - P.ms);
+  }
+  __device__ __forceinline__ uint8_t* dp(int i) const { return i < P.ms ? sd + i : sl + P.off_md + (i - P.ms); }
 };
 
 // ---------------------------------------------------------------------------
-// Per-accelerator state.  Free times: with at most 32 accelerators lane d
-// holds accelerator d's in a register, else a shared array of the kernel's
-// time type.  Live bytes: a shared array (the drain updates it a batch at a
-// time).  Peak bytes: a shared array, or with more than 32 accelerators an
-// array in the warp's global scratch (only raised by atomicMax and read at
-// the end, so its latency is never waited on).
+// Per-accelerator state.  Free times: a shared array of the kernel's time
+// type, or (kReg: the arbitrated kernel of at most 32 accelerators, which takes
+// keys one at a time) accelerator d's in a register of lane d.  Live bytes: a
+// shared array (the drain updates it a batch at a time).  Peak bytes: a shared
+// array, or with more than 32 accelerators (!kPkShared) an array in the warp's
+// global scratch (only raised by atomicMax and read at the end, so its latency
+// is never waited on).
 // ---------------------------------------------------------------------------
-template <bool kReg, typename TM>
+template <bool kReg, bool kPkShared, typename TM>
 struct Devices {
   TM fr_reg;
   TM* fr;       // shared [D] (when !kReg)
   int64_t* lv;  // shared [D]
   int64_t* pk;  // [D], shared or global
+  uint32_t* acc;   // shared [16 * D], zero between drains (kPkShared)
+  uint32_t* over;  // shared [8] (!kPkShared)
   int D;
   __device__ void setup(const DevGmg& g, uint8_t* sm, int64_t* pk_global) {
     D = g.D;
-    lv = reinterpret_cast<int64_t*>(sm);
-    if (kReg) {  // peaks in shared memory (a compile-time fact for these instances)
-      pk = lv + D;
-      fr = nullptr;
+    if (kPkShared) {  // sums of a drain by accelerator, else a bit set of accelerators
+      acc = reinterpret_cast<uint32_t*>(sm);
+      sm += 64 * (size_t)D;
     } else {
-      pk = pk_global;
-      fr = reinterpret_cast<TM*>(lv + D);
+      over = reinterpret_cast<uint32_t*>(sm);
+      sm += 32;
     }
+    lv = reinterpret_cast<int64_t*>(sm);
+    pk = kPkShared ? lv + D : pk_global;  // a compile-time fact of the instance
+    fr = kReg ? nullptr : reinterpret_cast<TM*>(lv + (kPkShared ? 2 * D : D));
   }
   __device__ void reset(const DevGmg& g) {
     const unsigned l = lane_id();
     for (int d = l; d < D; d += 32) {
       lv[d] = g.base[d];
       pk[d] = g.base[d];
+      if (kPkShared)
+        for (int w = 0; w < 4; ++w) reinterpret_cast<uint4*>(acc)[4 * d + w] = make_uint4(0u, 0u, 0u, 0u);
       if (!kReg) fr[d] = (TM)g.avail0[d];
     }
     if (kReg) fr_reg = l < (unsigned)D ? (TM)g.avail0[l] : (TM)0;
@@ -399,6 +370,8 @@ struct Devices {
       if (!kReg) fr[d] = (TM)src[d];
       lv[d] = src[D + d];
       pk[d] = src[2 * D + d];
+      if (kPkShared)
+        for (int w = 0; w < 4; ++w) reinterpret_cast<uint4*>(acc)[4 * d + w] = make_uint4(0u, 0u, 0u, 0u);
     }
     if (kReg) fr_reg = l < (unsigned)D ? (TM)src[l] : (TM)0;
     __syncwarp();
@@ -414,19 +387,21 @@ struct Devices {
     return (int64_t)warp_max_u64(m);
   }
   __device__ void write_peak(int64_t* dst) const {
-    for (int d = lane_id(); d < D; d += 32) dst[d] = pk[d];
+    for (int d = lane_id(); d < D; d += 32) dst[d] = kPkShared ? pk[d] : __ldcg(pk + d);
   }
 };
 
-// Shared-memory carve-up per warp: READY heap head, event-log head, sort
+// Shared-memory carve-up per warp: READY pool, heap head, event-log head, sort
 // area, accelerator state.
 struct WarpSmem {
+  uint64_t* pool;   // [pool]
   uint32_t* oplog;  // [opcap]
   uint64_t* heap;   // [qs]
   uint64_t* logk;   // [ms]
-  uint64_t* sortk;  // [sortcap]
+  uint64_t* sortk;  // [P.sortcap]
   uint8_t* logd;    // [ms]
-  uint8_t* sortd;   // [sortcap]
+  uint8_t* sortd;   // [P.sortcap]
+  uint8_t* fstk;    // [pool]
   uint8_t* dev;     // accelerator state (P.dev_bytes)
 };
 
@@ -436,17 +411,19 @@ __device__ __forceinline__ WarpSmem carve_smem(uint8_t* smem, const SimParams& P
   // the side bytes (accelerator of a log entry) are left out where the
   // accelerator is inside the entry and shared memory is tight (P.no_side)
   const size_t side = P.no_side ? 0 : 1;
-  const size_t head = align16((size_t)P.qs * 8 + (size_t)P.ms * (8 + side) + (size_t)P.sortcap * (8 + side) +
-                              (size_t)P.opcap * 4);
+  const size_t head = align16((size_t)P.pool * 9 + (size_t)P.qs * 8 + (size_t)P.ms * (8 + side) +
+                              (size_t)P.sortcap * (8 + side) + (size_t)P.opcap * 4);
   const size_t per = head + (size_t)P.dev_bytes;
   uint8_t* b = smem + per * wib;
   WarpSmem w;
-  w.heap = reinterpret_cast<uint64_t*>(b);
+  w.pool = reinterpret_cast<uint64_t*>(b);
+  w.heap = w.pool + P.pool;
   w.logk = w.heap + P.qs;
   w.sortk = w.logk + P.ms;
   w.logd = reinterpret_cast<uint8_t*>(w.sortk + P.sortcap);
   w.sortd = w.logd + P.ms * side;
   w.oplog = reinterpret_cast<uint32_t*>(w.sortd + P.sortcap * side);
+  w.fstk = reinterpret_cast<uint8_t*>(w.oplog + P.opcap);
   w.dev = b + head;
   return w;
 }
@@ -458,38 +435,50 @@ __device__ __forceinline__ WarpSmem carve_smem(uint8_t* smem, const SimParams& P
 // start, finish, free and arrival times are carried as int32 (bytes, scores
 // and outputs stay int64).
 // kTypes: the graph has several accelerator types (durations per (type, op)).
-// kBatch: the batched sweep (run_batched), for accelerator state in shared
-// memory with the accelerator id in the event key.
-// kStage: the hot fields of the GMG (durations, transfer sizes, flags, both
-// CSR lists, releases) are read from the CTA's shared-memory copy (staged by
-// sim_full_staged_kernel) when starting ops and testing successors.
-template <bool kReg, int kMode, bool kKey, bool kT32 = false, bool kTypes = false, bool kBatch = false,
-          bool kStage = false>
+// kNarrow: at most 32 accelerators.
+// kPool: the READY pool and its sweep (run) -- every pure-latency kernel; the
+// arbitrated simulators, which take one event at a time, bring their own loop
+// and READY queue (gmg_arb_events.h).
+// kHot: the sweep reads compact 16-byte records (duration, transfer time, flags,
+// both CSR lists) instead of the 64-byte ones -- kHotGlobal through the
+// read-only path, kHotShared from the CTA's shared-memory copy (staged by
+// sim_full_staged_kernel).
+constexpr int kHotNone = 0, kHotGlobal = 1, kHotShared = 2;
+template <bool kNarrow, int kMode, bool kKey, bool kT32 = false, bool kTypes = false, bool kPool = true,
+          int kHot = kHotNone>
 struct Sim {
-  static_assert(!(kT32 && kMode == kBase), "the base snapshot keeps 64-bit times");
-  static_assert(!kBatch || (!kReg && kKey), "the batched sweep keeps accelerator state in shared memory");
-  static_assert(!kStage || (kMode == kFull && kT32 && !kTypes && !kBatch), "staged GMG: 32-bit, one type");
+  static_assert(kHot == kHotNone || (kT32 && !kTypes && kPool), "compact records: 32-bit times, one type");
   using tm_t = typename std::conditional<kT32, int32_t, int64_t>::type;
   const SimParams& P;
   const DevGmg& g;
-  KeyCodec kc;      // HBM log entries (and READY keys when qb = 0)
-  ReadyCodec rq;    // READY keys
-  ReadyHeap q;      // READY keys beyond the register tier
-  uint64_t rk_reg;  // register tier: one READY key per lane (kKeyMax = empty)
+  static constexpr int kSlots = kReadyPoolWide / 32;  // pool slots per lane (more than 32 accelerators)
+  static constexpr tm_t kNever = (tm_t)(~(typename std::make_unsigned<tm_t>::type)0 >> 1);
+  struct Pending {
+    tm_t r, e, dur;  // ready time, earliest finish (both kNever: empty), duration
+    uint32_t op;
+    int d;           // its accelerator
+  };
+  KeyCodec kc;      // HBM log entries (and the arbitrated simulators' READY keys)
+  ReadyCodec rq;    // READY keys of the pool
+  ReadyHeap q;      // READY keys beyond the pool (the lanes)
+  Pending pd;       // at most 32 accelerators: this lane's pending op
+  uint64_t* pool;   // more: shared [32 * kSlots], pending READY keys (kKeyMax = empty)
+  uint8_t* fstk;    // shared [32 * kSlots]: the empty slots, a stack of nfree
+  int nfree;
   MemLog log;
   uint64_t* sortk;
   uint8_t* sortd;
-  int sortcap;
+  static constexpr int kWindows = 4;
+  tm_t drained;     // every event before this time is applied, none after it
   uint32_t* oplog;  // ops started since the last HBM-event generation
   int opn;
-  int ds;           // accelerator shift of a log entry
-  uint64_t lowmask; // key part of a log entry
-  Devices<kReg, tm_t> dv;
+  Devices<kNarrow && !kPool, kNarrow, tm_t> dv;
   const uint8_t* row;
-  tm_t* fbuf;       // finish times (scratch; the base's own array in kBase)
-  tm_t* holdb;      // latest outgoing arrival of each op's output (scratch)
-  uint32_t* bits;
-  int64_t* creq;
+  tm_t* fbuf;       // finish times (scratch)
+  uint8_t* sl;      // the warp's scratch slot (the less used arrays in it are found from the launch parameters)
+  __device__ __forceinline__ tm_t* holdb() const { return reinterpret_cast<tm_t*>(sl + P.off_hold); }  // [N] latest outgoing arrival of the op's output
+  __device__ __forceinline__ uint32_t* bits() const { return reinterpret_cast<uint32_t*>(sl + P.off_bits); }
+  __device__ __forceinline__ int64_t* creq() const { return reinterpret_cast<int64_t*>(sl + P.off_creq); }
   // incremental resume
   const int64_t* rb;
   const int64_t* fb;
@@ -497,33 +486,26 @@ struct Sim {
   // running results
   int rootptr;
   uint64_t rkey;    // root_keys[rootptr], kKeyMax past the end
-  int64_t score, nev, readypops;
+  int64_t score, nev;   // with the pool each lane's share, summed at the end
+  int64_t readypops;
   int32_t iters;        // ops started (loop guard; the event count of a full run)
-  tm_t makespan, last_t;  // running values, kept in base mode only (checkpoints)
+  tm_t last_t;          // latest READY time handled, kept in base mode only (checkpoints)
   int32_t vflag, vop, vdev, status;
   int64_t vt;
   // base checkpoints
   int ck, next_ck;
-  // staged GMG (kStage): shared copies
+  // staged GMG (kHotShared): shared copies
   const uint4* sh_hot;      // per op {dur, xq | flags << 29, succ_off | nsucc << 24, pred_off | npred << 24}
   const int32_t* sh_rel;    // per op release
   const uint32_t* sh_succ;  // successor lists
   const uint32_t* sh_pred;  // predecessor lists (hold bits included)
 
-  __device__ Sim(const SimParams& p) : P(p), g(p.g) {
-    kc.ib = g.ib;
-    kc.mask = (1ull << g.ib) - 1ull;
-    rq.ib = g.ib;
-    rq.mask = kc.mask;
-    rq.qb = kBatch ? kQB : 0;
-    ds = g.ib + 2 + g.tb;
-    lowmask = kKey ? (1ull << ds) - 1ull : kKeyMax;
-  }
+  __device__ Sim(const SimParams& p) : P(p), g(p.g), kc{p.g}, rq{p.g}, q{p}, log{p} {}
+  __device__ __forceinline__ uint64_t lowmask() const { return kKey ? g.keymask : kKeyMax; }  // key of a log entry
 
-  // Started ops are those with a finish time (every finish time is >= 1;
-  // the finish array is zeroed per candidate; the batched sweep marks an op
-  // whose READY key is queued with -1).
-  __device__ __forceinline__ bool popped(uint32_t x) const { return fin(x) > 0; }
+  // Started ops are those with a finish time: every finish time is >= 1, the
+  // finish array is zeroed per candidate, and the sweep marks a join whose READY
+  // key is queued with -1.
   // The low 32 bits of a base-snapshot time (little-endian int64).
   static __device__ __forceinline__ tm_t base_time(const int64_t* a, uint32_t x) {
     if (kT32) return (tm_t)__ldg(reinterpret_cast<const int32_t*>(a) + 2 * (size_t)x);
@@ -571,37 +553,33 @@ struct Sim {
   }
 
 
-  __device__ __forceinline__ void load_root() {
-    rkey = rootptr < g.nroots ? __ldg((kBatch ? g.root_keys_q : g.root_keys) + rootptr) : kKeyMax;
+  __device__ __forceinline__ tm_t warp_min_t(tm_t v) const {
+    if (kT32) return (tm_t)__reduce_min_sync(kFullMask, (int)v);
+    return (tm_t)warp_min_u64((uint64_t)v);  // times are >= 0
   }
 
-  // READY keys go to a free lane's register if there is one, else the heap.
-  __device__ __forceinline__ void push_ready(uint64_t key) {
-    const uint32_t freel = __ballot_sync(kFullMask, rk_reg == kKeyMax);
-    if (freel) {
-      if ((int)lane_id() == __ffs(freel) - 1) rk_reg = key;
-    } else if (!(kBatch ? q.push_fast(key) : q.push(key))) {
-      status = GMG_SIM_QUEUE;
-    }
+  __device__ __forceinline__ void load_root() {
+    rkey = rootptr < g.nroots ? __ldg((kPool ? g.root_keys_q : g.root_keys) + rootptr) : kKeyMax;
   }
+
   // Every lane with `want` logs (key, dev).  Uniform call.
   __device__ __forceinline__ void log_event(bool want, uint64_t key, int dev) {
     const uint32_t b = __ballot_sync(kFullMask, want);
     const int cnt = __popc(b);
     const int pos = log.n + __popc(b & lanes_below());
-    if (kKey && log.n + 32 <= log.ms) {
+    if (kKey && log.n + 32 <= P.ms) {
       // fast path: every lane's slot is in shared memory
-      if (want) log.sk[pos] = ((uint64_t)(dev & 0xff) << ds) | key;
+      if (want) log.sk[pos] = ((uint64_t)(dev & 0xff) << g.ds) | key;
       log.n += cnt;
       return;
     }
     if (cnt == 0 || status) return;
-    if (log.n + cnt > log.cap) {
+    if (log.n + cnt > P.mcap) {
       status = GMG_SIM_QUEUE;
       return;
     }
     if (want) {
-      *log.kp(pos) = kKey ? (((uint64_t)(dev & 0xff) << ds) | key) : key;
+      *log.kp(pos) = kKey ? (((uint64_t)(dev & 0xff) << g.ds) | key) : key;
       if (!kKey) *log.dp(pos) = (uint8_t)dev;
     }
     log.n += cnt;
@@ -646,15 +624,19 @@ struct Sim {
   __device__ void reset_common() {
     const unsigned lane = lane_id();
     zero_fin();
-    for (int r = lane; r < g.R; r += 32) creq[r] = 0;
+    for (int r = lane; r < g.R; r += 32) creq()[r] = 0;
     dv.reset(g);
     q.size = 0;
-    rk_reg = kKeyMax;
+    if constexpr (kPool) {
+      if constexpr (kNarrow) pd.r = pd.e = kNever;
+      else empty_pool(0);
+    }
     log.n = 0;
+    drained = 0;
     opn = 0;
     rootptr = 0;
     load_root();
-    score = makespan = 0;
+    score = 0;
     iters = nev = readypops = 0;
     last_t = -1;
     vflag = 0;
@@ -662,142 +644,6 @@ struct Sim {
     vt = -1;
     status = GMG_SIM_OK;
     __syncwarp();
-  }
-
-  // -------------------------------------------------------------------------
-  // READY(r, i): start op i (Sec. 3.3.2/3.3.3), record it for HBM-event
-  // generation, and push the successors it makes ready.
-  // -------------------------------------------------------------------------
-  __device__ void start_op(uint32_t i, tm_t r) {
-    if constexpr (kStage) {
-      start_op_staged(i, r);
-      return;
-    }
-    const unsigned lane = lane_id();
-    const longlong2 db = op_durbytes(g.ops, i);
-    const XqSucc xs = op_xqsucc(g.ops, i);
-    const uint4 cs = op_cons(g.ops, i);
-    const int64_t bytes = db.y, xq = xs.xq;
-    const uint32_t succ_off = xs.succ_off, nsucc = xs.nsucc;
-    const uint32_t flags = cs.w;
-    const int d = row[i];
-    const tm_t dur = (tm_t)dur_of(i, d, db.x);
-    const tm_t fd = dv.get_free(d);
-    const tm_t s = r > fd ? r : fd;
-    const tm_t f = s + dur;
-    dv.set_free(d, f);
-    if (lane == 0) {
-      fbuf[i] = f;
-      if (flags & kReqSink)
-        atomicMax(reinterpret_cast<unsigned long long*>(creq + (int32_t)cs.z), (unsigned long long)f);
-      if (kMode == kBase) P.base.rb[i] = r;
-      oplog[opn] = i;
-    }
-    ++opn;
-    if (flags & kScored) score += (int64_t)f;
-    if (kMode == kBase) makespan = f > makespan ? f : makespan;
-    if (kMode == kInc && r >= T0) ++nev;
-    if (kMode == kBase) ++readypops;
-    __syncwarp();
-
-    // Successors: a successor is ready once every predecessor has finished;
-    // its ready time is the latest arrival over all of them.
-    for (uint32_t c0 = 0; c0 < nsucc; c0 += 32) {
-      const uint32_t t = c0 + lane;
-      uint32_t j = 0;
-      tm_t rj = 0;
-      bool rdy = false;
-      if (t < nsucc) {
-        j = __ldg(g.succ + succ_off + t);
-        const int dj = row[j];
-        tm_t arr = f;
-        if (dj != d) arr = f + xfer(d, dj, bytes, xq);
-        const RelPred jp = op_relpred(g.ops, j);
-        const tm_t rel = (tm_t)jp.rel;
-        rj = rel > arr ? rel : arr;
-        rdy = true;
-        if (jp.npred > 1) {
-          for (uint32_t k = 0; k < jp.npred; ++k) {
-            const uint32_t p = __ldg(g.pred + jp.pred_off + k) & kIdMask;
-            if (p == i) continue;
-            tm_t a = fin(p);
-            if (a <= 0) {  // not started yet
-              rdy = false;
-              break;
-            }
-            const int dp = row[p];
-            if (dp != dj) a += xfer(dp, dj, op_durbytes(g.ops, p).y, op_xqsucc(g.ops, p).xq);
-            rj = a > rj ? a : rj;
-          }
-        }
-      }
-      uint32_t m = __ballot_sync(kFullMask, rdy);
-      while (m) {
-        const int src = __ffs(m) - 1;
-        m &= m - 1;
-        push_ready(__shfl_sync(kFullMask, kc.make(rj, kReady, j), src));
-      }
-    }
-  }
-
-  // start_op with the hot fields from the CTA's staged copy of the GMG (the
-  // links are uniform: a transfer takes xq + lat0).
-  __device__ void start_op_staged(uint32_t i, tm_t r) {
-    const unsigned lane = lane_id();
-    const uint4 h = sh_hot[i];
-    const uint32_t flags = h.y >> 29;
-    const tm_t xq = (tm_t)(h.y & 0x1fffffffu);
-    const uint32_t succ_off = h.z & 0xffffffu, nsucc = h.z >> 24;
-    const int d = row[i];
-    const tm_t fd = dv.get_free(d);
-    const tm_t s = r > fd ? r : fd;
-    const tm_t f = s + (tm_t)(int32_t)h.x;
-    dv.set_free(d, f);
-    if (lane == 0) {
-      fbuf[i] = f;
-      if (flags & kReqSink)
-        atomicMax(reinterpret_cast<unsigned long long*>(creq + (int32_t)op_cons(g.ops, i).z), (unsigned long long)f);
-      oplog[opn] = i;
-    }
-    ++opn;
-    if (flags & kScored) score += (int64_t)f;
-    __syncwarp();
-    const tm_t lat = (tm_t)g.lat0;
-    for (uint32_t c0 = 0; c0 < nsucc; c0 += 32) {
-      const uint32_t t = c0 + lane;
-      uint32_t j = 0;
-      tm_t rj = 0;
-      bool rdy = false;
-      if (t < nsucc) {
-        j = sh_succ[succ_off + t];
-        const int dj = row[j];
-        const tm_t arr = dj != d ? f + xq + lat : f;
-        const uint32_t po = sh_hot[j].w;
-        const uint32_t npred = po >> 24, pred_off = po & 0xffffffu;
-        const tm_t rel = (tm_t)sh_rel[j];
-        rj = rel > arr ? rel : arr;
-        rdy = true;
-        if (npred > 1) {
-          for (uint32_t k = 0; k < npred; ++k) {
-            const uint32_t p = sh_pred[pred_off + k] & kIdMask;
-            if (p == i) continue;
-            tm_t a = fin(p);
-            if (a <= 0) {  // not started yet
-              rdy = false;
-              break;
-            }
-            if (row[p] != dj) a += (tm_t)(sh_hot[p].y & 0x1fffffffu) + lat;
-            rj = a > rj ? a : rj;
-          }
-        }
-      }
-      uint32_t m = __ballot_sync(kFullMask, rdy);
-      while (m) {
-        const int src = __ffs(m) - 1;
-        m &= m - 1;
-        push_ready(__shfl_sync(kFullMask, kc.make(rj, kReady, j), src));
-      }
-    }
   }
 
   // -------------------------------------------------------------------------
@@ -811,124 +657,214 @@ struct Sim {
   // producer's outgoing arrivals).  Ops on one accelerator finish in the
   // order they start, so "last consumer here" compares finish times and can
   // be decided any time after the op started.
+  //
+  // Bounded by the chain of dependent loads (record, list entries, placement
+  // and finish times of the ops on them): the first two entries of both lists
+  // -- all that most ops have -- are loaded side by side, one level after the
+  // other, and a lane's events are written together.
   // -------------------------------------------------------------------------
+
+  // One event of this lane in the making: appended by log_lanes.
+  __device__ __forceinline__ uint64_t entry(tm_t t, uint32_t cls, uint32_t op, int dev) const {
+    const uint64_t k = kc.make(t, cls, op);
+    return kKey ? ((uint64_t)(dev & 0xff) << g.ds) | k : k;
+  }
+  template <int kMax>
+  __device__ __forceinline__ void log_lanes(const uint64_t (&ev)[kMax], const int (&dev)[kMax], uint32_t want) {
+    const unsigned lane = lane_id();
+    const int c = __popc(want);
+    int at = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFullMask, at, o);
+      if ((int)lane >= o) at += y;
+    }
+    const int total = __shfl_sync(kFullMask, at, 31);
+    at += log.n - c;
+    if (log.n + total <= P.ms) {
+#pragma unroll
+      for (int x = 0; x < kMax; ++x)
+        if ((want >> x) & 1u) {
+          log.sk[at] = ev[x];
+          if (!kKey) log.sd[at] = (uint8_t)dev[x];
+          ++at;
+        }
+    } else {
+      if (status) return;
+      if (log.n + total > P.mcap) {
+        status = GMG_SIM_QUEUE;
+        return;
+      }
+#pragma unroll
+      for (int x = 0; x < kMax; ++x)
+        if ((want >> x) & 1u) {
+          *log.kp(at) = ev[x];
+          if (!kKey) *log.dp(at) = (uint8_t)dev[x];
+          ++at;
+        }
+    }
+    log.n += total;
+  }
+
+  // Whether op x (ending at f on d) is the last listed consumer on d of its
+  // predecessor: ps is the predecessor's entry in x's list.
+  __device__ __forceinline__ bool releases(uint32_t x, int d, tm_t f, const uint2 ps) const {
+    if (!(ps.x & kHoldBit)) return false;
+    const uint32_t sb = ps.y;
+    if (sb == kSibNone) return true;
+    if (sb != kSibMany) {
+      if (row[sb & ~kSibLater] != d) return true;
+      if (sb & kSibLater) return false;  // the other consumer finishes later
+      const tm_t fs = fin(sb);
+      return fs > 0 && fs < f;
+    }
+    const uint32_t p = ps.x & kIdMask;
+    const XqSucc px = op_xqsucc(g.ops, p);
+    const uint4 pcs = op_cons(g.ops, p);
+    const bool all = (pcs.w & kAllCons) != 0;
+    const uint32_t* lst = all ? g.succ + px.succ_off : g.cons + pcs.x;
+    const uint32_t nl = all ? px.nsucc : pcs.y;
+    for (uint32_t w = 0; w < nl; ++w) {
+      const uint32_t c = __ldg(lst + w);
+      const tm_t fc = c != x ? fin(c) : 0;
+      if (c != x && row[c] == d && !(fc > 0 && fc < f)) return false;
+    }
+    return true;
+  }
+  // When p's copy on d that an op ending at f there releases is freed (p's own
+  // copy: not before its outgoing arrivals, recorded when p's events were
+  // generated; p started before this op).
+  __device__ __forceinline__ tm_t freed_at(uint32_t p, int d, tm_t f) const {
+    if (row[p] != d) return f;
+    const tm_t h = (kMode == kInc && base_time(rb, p) < Tc) ? lane_hold(p, fin(p), d) : holdb()[p];
+    return h > f ? h : f;
+  }
+  // A listed consumer of x on accelerator e?
+  __device__ __forceinline__ bool consumer_on(const uint4& cs, int e) const {
+    for (uint32_t w = 0; w < cs.y; ++w)
+      if (row[__ldg(g.cons + cs.x + w)] == e) return true;
+    return false;
+  }
+
   __device__ void generate() {
     const unsigned lane = lane_id();
     for (int c0 = 0; c0 < opn; c0 += 32) {
       const int idx = c0 + (int)lane;
       const bool v = idx < opn;
       const uint32_t x = v ? oplog[idx] : 0u;
-      longlong2 db = make_longlong2(0, 0), rx = make_longlong2(0, 0);
-      uint4 ls = make_uint4(0, 0, 0, 0), cs = make_uint4(0, 0, 0, 0);
+      Start s;
+      s.nsucc = 0;
+      s.flags = kAllCons;
+      s.dur = s.xq = 0;
+      s.bytes = 0;
+      s.succ_off = 0;
+      uint32_t pred_off = 0, npred = 0;
       int d = 0;
       tm_t f = 0;
       if (v) {
-        db = op_durbytes(g.ops, x);
-        const XqSucc xs = op_xqsucc(g.ops, x);
-        const RelPred rp = op_relpred(g.ops, x);
-        rx = make_longlong2(rp.rel, xs.xq);
-        ls = make_uint4(xs.succ_off, xs.nsucc, rp.pred_off, rp.npred);
-        cs = op_cons(g.ops, x);
         d = row[x];
         f = fbuf[x];
+        if constexpr (kHot != kHotNone) {
+          const uint4 h = hot(x);
+          s.dur = (tm_t)h.x;
+          s.xq = (tm_t)(h.y & 0x1fffffffu);
+          s.flags = h.y >> 29;
+          s.succ_off = h.z & 0xffffffu;
+          s.nsucc = h.z >> 24;
+          pred_off = h.w & 0xffffffu;
+          npred = h.w >> 24;
+        } else {
+          s = start_of(x, d);
+          const RelPred rp = op_relpred(g.ops, x);
+          pred_off = rp.pred_off;
+          npred = rp.npred;
+        }
       }
-      const int64_t bytes = db.y, xq = rx.y;
-      const bool allcons = (cs.w & kAllCons) != 0;
-      log_event(v, kc.make(f - (tm_t)dur_of(x, d, db.x), kAlloc, x), d);
+      // list entries, then what they point at, side by side
+      int du[2] = {d, d};
+      uint2 ps[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        if ((uint32_t)u < npred) ps[u] = __ldg(g.predsib + pred_off + u);
+        if ((uint32_t)u < s.nsucc) du[u] = row[succ_at(s.succ_off + u)];
+      }
+      const bool all = (s.flags & kAllCons) != 0;
+      uint64_t ev[6];
+      int dev[6];
+      uint32_t want = v ? 1u : 0u;
+      dev[0] = d;
+      ev[0] = entry(f - s.dur, kAlloc, x, d);
       // receive copies, one per distinct remote accelerator
       tm_t hold = f;
       bool localc = false;
-      const uint32_t nsx = ls.y;
-      const uint32_t maxs = __reduce_max_sync(kFullMask, nsx);
-      const bool anyexp = __any_sync(kFullMask, v && !allcons);
-      for (uint32_t u = 0; u < maxs; ++u) {
-        bool want = false, nocons = false;
-        int du = 0;
-        tm_t arr = f;
-        if (u < nsx) {
-          du = row[__ldg(g.succ + ls.x + u)];
-          if (du == d) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        dev[1 + u] = du[u];
+        ev[1 + u] = entry(f, kAlloc, x, du[u]);
+        if ((uint32_t)u < s.nsucc) {
+          if (du[u] == d) {
             localc = true;
-          } else {
-            want = true;
-            for (uint32_t w = 0; w < u; ++w)
-              if (row[__ldg(g.succ + ls.x + w)] == du) {
-                want = false;
-                break;
-              }
-          }
-          if (want) {
-            arr = f + xfer(d, du, bytes, xq);
-            hold = arr > hold ? arr : hold;
-            if (!allcons) {
-              nocons = true;
-              for (uint32_t w = 0; w < cs.y; ++w)
-                if (row[__ldg(g.cons + cs.x + w)] == du) {
-                  nocons = false;
-                  break;
-                }
-            }
+          } else if (u == 0 || du[1] != du[0]) {
+            want |= 2u << u;
+            const tm_t a = f + (kHot != kHotNone ? s.xq + (tm_t)g.lat0 : xfer(d, du[u], s.bytes, s.xq));
+            hold = a > hold ? a : hold;
           }
         }
-        log_event(want, kc.make(f, kAlloc, x), du);
-        if (anyexp) log_event(nocons, kc.make(arr, kFree, x), du);
       }
-      if (v && !allcons) {
-        localc = false;
-        for (uint32_t w = 0; w < cs.y; ++w)
-          if (row[__ldg(g.cons + cs.x + w)] == d) {
-            localc = true;
-            break;
+      if (__any_sync(kFullMask, s.nsucc > 2u || !all)) {
+        // longer lists, and copies that nobody listed holds
+        const uint32_t maxs = __reduce_max_sync(kFullMask, s.nsucc);
+        const uint4 cs = v && !all ? op_cons(g.ops, x) : make_uint4(0u, 0u, 0u, 0u);
+        for (uint32_t u = 0; u < maxs; ++u) {
+          bool first = false;
+          int e = d;
+          tm_t a = f;
+          if (u < s.nsucc) {
+            e = row[succ_at(s.succ_off + u)];
+            first = e != d;
+            localc = localc || e == d;
+            for (uint32_t w = 0; w < u && first; ++w) first = row[succ_at(s.succ_off + w)] != e;
+            if (first) {
+              a = f + (kHot != kHotNone ? s.xq + (tm_t)g.lat0 : xfer(d, e, s.bytes, s.xq));
+              hold = a > hold ? a : hold;
+            }
           }
+          if (u >= 2u) log_event(first, kc.make(f, kAlloc, x), e);
+          log_event(first && !all && !consumer_on(cs, e), kc.make(a, kFree, x), e);
+        }
+        if (v && !all) localc = consumer_on(cs, d);
       }
-      log_event(v && !localc, kc.make(hold, kFree, x), d);
-      if (v) holdb[x] = hold;
+      if (v && !localc) want |= 8u;
+      dev[3] = d;
+      ev[3] = entry(hold, kFree, x, d);
+      if (v) holdb()[x] = hold;
       __syncwarp();
       // releases of the inputs this op holds
-      const uint32_t npx = ls.w;
-      const uint32_t maxp = __reduce_max_sync(kFullMask, npx);
-      for (uint32_t u = 0; u < maxp; ++u) {
-        bool rel = false;
-        tm_t T = f;
-        uint32_t p = 0;
-        if (u < npx) {
-          const uint2 ps = __ldg(g.predsib + ls.z + u);
-          p = ps.x & kIdMask;
-          if (ps.x & kHoldBit) {
-            const uint32_t sb = ps.y;
-            if (sb == kSibNone) {
-              rel = true;
-            } else if (sb != kSibMany && (sb & kSibLater)) {
-              rel = row[sb & ~kSibLater] != d;  // the other consumer finishes later
-            } else if (sb != kSibMany) {
-              const tm_t fs = fin(sb);
-              rel = !(row[sb] == d && !(fs > 0 && fs < f));
-            } else {
-              const XqSucc px = op_xqsucc(g.ops, p);
-              const uint4 pls = make_uint4(px.succ_off, px.nsucc, 0u, 0u);
-              const uint4 pcs = op_cons(g.ops, p);
-              const bool all = (pcs.w & kAllCons) != 0;
-              const uint32_t* lst = all ? g.succ + pls.x : g.cons + pcs.x;
-              const uint32_t nl = all ? pls.y : pcs.y;
-              rel = true;
-              for (uint32_t w = 0; w < nl; ++w) {
-                const uint32_t c = __ldg(lst + w);
-                const tm_t fc = c != x ? fin(c) : 0;
-                if (c != x && row[c] == d && !(fc > 0 && fc < f)) {
-                  rel = false;
-                  break;
-                }
-              }
-            }
-            if (rel && row[p] == d) {
-              // p's own copy: not before its outgoing arrivals (recorded when
-              // p's events were generated; p started before this op)
-              const tm_t h = (kMode == kInc && base_time(rb, p) < Tc) ? lane_hold(p, fin(p), d) : holdb[p];
-              T = h > T ? h : T;
-            }
-          }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint32_t p = ps[u].x & kIdMask;
+        dev[4 + u] = d;
+        ev[4 + u] = 0;
+        if (releases(x, d, f, ps[u])) {
+          want |= 16u << u;
+          ev[4 + u] = entry(freed_at(p, d, f), kFree, p, d);
         }
-        log_event(rel, kc.make(T, kFree, p), d);
+      }
+      log_lanes<6>(ev, dev, want);
+      if (__any_sync(kFullMask, npred > 2u)) {
+        const uint32_t maxp = __reduce_max_sync(kFullMask, npred);
+        for (uint32_t u = 2; u < maxp; ++u) {
+          bool rel = false;
+          tm_t t = f;
+          uint32_t p = 0;
+          if (u < npred) {
+            const uint2 e = __ldg(g.predsib + pred_off + u);
+            p = e.x & kIdMask;
+            rel = releases(x, d, f, e);
+            if (rel) t = freed_at(p, d, f);
+          }
+          log_event(rel, kc.make(t, kFree, p), d);
+        }
       }
     }
     opn = 0;
@@ -941,7 +877,7 @@ struct Sim {
       const uint64_t k = sortk[e];
       const int dev = sortd[e];
       const uint32_t op = kc.op(k);
-      const int64_t b = op_durbytes(g.ops, op).y;
+      const int64_t b = __ldg(g.bytes + op);
       if (kc.cls(k) == kFree) {
         dv.release(dev, b);
       } else if (dv.alloc(dev, b, __ldg(g.cap + dev))) {
@@ -966,12 +902,12 @@ struct Sim {
   __device__ __forceinline__ void apply_chunk(uint64_t key, bool v, uint64_t& vmin) {
     const unsigned lane = lane_id();
     const uint64_t tmask = (1ull << g.tb) - 1ull;
-    const int dev = v ? (int)(key >> ds) : -1 - (int)lane;
-    const uint32_t op = (uint32_t)(key & kc.mask);
+    const int dev = v ? (int)(key >> g.ds) : -1 - (int)lane;
+    const uint32_t op = (uint32_t)(key & g.opmask);
     const bool isalloc = v && kc.cls(key) == kAlloc;
     int64_t delta = 0;
     if (v) {
-      const int64_t b = op_durbytes(g.ops, op).y;
+      const int64_t b = __ldg(g.bytes + op);
       delta = isalloc ? b : -b;
     }
     int64_t s = delta;
@@ -991,7 +927,8 @@ struct Sim {
     const uint64_t cm = warp_min_u64(vk);
     vmin = cm < vmin ? cm : vmin;
     __syncwarp();
-    if (isalloc)  // live bytes are never negative
+    // live bytes are never negative; in shared memory most do not raise the peak
+    if (isalloc && (!kNarrow || live > dv.pk[dev]))
       atomicMax(reinterpret_cast<unsigned long long*>(dv.pk + dev), (unsigned long long)live);
     if (last) dv.lv[dev] = live;
     __syncwarp();
@@ -1003,7 +940,7 @@ struct Sim {
     if (!vflag && vmin != kKeyMax) {
       vflag = 1;
       vt = (int64_t)(vmin >> (g.ib + 8));
-      vop = (int32_t)((vmin >> 8) & kc.mask);
+      vop = (int32_t)((vmin >> 8) & g.opmask);
       vdev = (int32_t)(vmin & 0xffu);
     }
   }
@@ -1018,72 +955,167 @@ struct Sim {
     settle_violation(vmin);
   }
 
-  // Bitonic sort of 32*E keys held in registers: lane l holds elements
-  // l + 32 e.  Pairs 32 or more apart meet inside a lane, closer pairs via
-  // shfl_xor.  Fully unrolled.
-  template <int E>
-  static __device__ __forceinline__ void reg_bitonic(uint64_t (&a)[E]) {
-    const int lane = (int)lane_id();
-#pragma unroll
-    for (int k = 2; k <= 32 * E; k <<= 1) {
-#pragma unroll
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        if (j >= 32) {
-#pragma unroll
-          for (int e = 0; e < E; ++e) {
-            const int e2 = e ^ (j >> 5);
-            if (e2 > e) {
-              const bool asc = ((lane + 32 * e) & k) == 0;
-              const uint64_t x = a[e], y = a[e2];
-              const bool sw = asc ? (x > y) : (x < y);
-              a[e] = sw ? y : x;
-              a[e2] = sw ? x : y;
-            }
-          }
-        } else {
-#pragma unroll
-          for (int e = 0; e < E; ++e) {
-            const uint64_t o = __shfl_xor_sync(kFullMask, a[e], j);
-            const bool keep_min = ((lane & j) == 0) == (((lane + 32 * e) & k) == 0);
-            a[e] = (keep_min == (o < a[e])) ? o : a[e];
-          }
-        }
-      }
+  // Sort and apply m extracted events of accelerators whose order matters.
+  // may_violate: one of them may exceed its capacity -- then equal times are
+  // told apart by op id (the whole entry is the sort key), else the order of
+  // equal times of one kind does not matter and 32 bits hold the key.
+  __device__ __forceinline__ void apply_ordered(int m, bool may_violate, tm_t span) {
+    constexpr int kDevBits = kNarrow ? 5 : 8;
+    if (!may_violate && m <= 32 && (span >> (32 - kDevBits - 6)) == 0) {
+      apply_short(m);
+    } else {
+      sort_area(m);
+      apply_segmented(m);
     }
   }
 
-  template <int E>
-  __device__ __forceinline__ void sort_apply_regs_e(int m) {
+  // m <= 32 events, none of which exceeds a capacity: sorted in registers by
+  // (accelerator, time since the last drain, frees first, position) in 32 bits,
+  // then a prefix sum of the byte changes, less its value where the
+  // accelerator's events begin, gives the live bytes after each.  (A bitonic
+  // network over the 64-bit entries takes three times the instructions.)
+  __device__ __forceinline__ void apply_short(int m) {
+    constexpr int kDevBits = kNarrow ? 5 : 8;
     const int lane = (int)lane_id();
-    uint64_t a[E];
+    const bool v = lane < m;
+    uint32_t a = 0xffffffffu;
+    int64_t delta = 0;
+    if (v) {
+      const uint64_t x = sortk[lane];
+      const bool al = kc.cls(x) == kAlloc;
+      const tm_t t = (tm_t)((x & lowmask()) >> (g.ib + 2)) - drained;
+      delta = __ldg(g.bytes + (uint32_t)(x & g.opmask));
+      if (!al) delta = -delta;
+      a = ((uint32_t)(x >> g.ds) << (32 - kDevBits)) | ((uint32_t)t << 6) | (al ? 32u : 0u) | (uint32_t)lane;
+    }
 #pragma unroll
-    for (int e = 0; e < E; ++e) a[e] = lane + 32 * e < m ? sortk[lane + 32 * e] : kKeyMax;
-    reg_bitonic<E>(a);
-    uint64_t vmin = kKeyMax;
+    for (int k = 2; k <= 32; k <<= 1) {
 #pragma unroll
-    for (int e = 0; e < E; ++e) apply_chunk(a[e], lane + 32 * e < m, vmin);
-    settle_violation(vmin);
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        const uint32_t o = __shfl_xor_sync(kFullMask, a, j);
+        const bool keep_min = ((lane & j) == 0) == ((lane & k) == 0);
+        a = keep_min ? (o < a ? o : a) : (o < a ? a : o);
+      }
+    }
+    delta = __shfl_sync(kFullMask, delta, (int)(a & 31u));
+    if (!v) delta = 0;
+    const int dev = v ? (int)(a >> (32 - kDevBits)) : -1 - lane;
+    int64_t s = delta;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(kFullMask, s, o);
+      if (lane >= o) s += y;
+    }
+    const int dl = __shfl_up_sync(kFullMask, dev, 1), dr = __shfl_down_sync(kFullMask, dev, 1);
+    const uint32_t heads = __ballot_sync(kFullMask, lane == 0 || dl != dev);
+    const int head = 31 - __clz(heads & (lanes_below() | (1u << lane)));
+    const int64_t before = __shfl_sync(kFullMask, s - delta, head);
+    const int64_t live = (v ? dv.lv[dev] : 0) + s - before;
+    __syncwarp();
+    if (v && (a & 32u) && (!kNarrow || live > dv.pk[dev]))
+      atomicMax(reinterpret_cast<unsigned long long*>(dv.pk + dev), (unsigned long long)live);
+    if (v && (lane == 31 || dr != dev)) dv.lv[dev] = live;
+    __syncwarp();
   }
 
-  // Sort and apply m <= 32 extracted events in registers.  (Wider register
-  // networks sort faster but their unrolled code -- each inlining its own
-  // copies of the segmented apply -- overflowed the instruction cache: larger
-  // drains go through the shared-memory sort.)
-  __device__ void sort_apply_regs(int m) { sort_apply_regs_e<1>(m); }
+  // Apply the m events just extracted.  Their order matters only on an
+  // accelerator whose peak they can raise (without a violation so far the peak
+  // is within the capacity).  An upper bound of its live bytes is cheap: with at
+  // most 32 accelerators extract() has summed up what is allocated and freed on
+  // each in every quarter of the time since the last drain, and within a quarter
+  // the live bytes are at most those at its start plus all its allocations; with
+  // more (few events each) the whole drain is one such interval.  Everywhere
+  // else the sums are enough.
+  __device__ __forceinline__ void apply_due(int m, tm_t span) {
+    const unsigned lane = lane_id();
+    uint32_t fail = 0u;
+    bool viol = false;
+    if constexpr (kNarrow) {
+      if (g.big_bytes) {  // not summed: the 24-bit halves would not hold the sizes
+        apply_ordered(m, true, span);
+        return;
+      }
+      bool over = false;
+      if ((int)lane < g.D) {
+        uint4* q4 = reinterpret_cast<uint4*>(dv.acc) + kWindows * lane;
+        const int64_t l0 = dv.lv[lane], peak = dv.pk[lane];
+        int64_t l = l0, top = 0;
+#pragma unroll
+        for (int w = 0; w < kWindows; ++w) {
+          const uint4 x = q4[w];
+          q4[w] = make_uint4(0u, 0u, 0u, 0u);
+          const int64_t most = l + (int64_t)(((uint64_t)x.y << 24) + x.x);
+          top = most > top ? most : top;
+          l = most - (int64_t)(((uint64_t)x.w << 24) + x.z);
+        }
+        over = top > peak;
+        if (!over) dv.lv[lane] = l;
+        else viol = top > __ldg(g.cap + lane);
+      }
+      fail = __ballot_sync(kFullMask, over);
+      if (fail == 0u) return;
+    } else {
+      // extract() has added the allocations to the live bytes
+      if (lane < 8u) dv.over[lane] = 0u;
+      __syncwarp();
+      for (int c0 = 0; c0 < m; c0 += 32) {
+        const int idx = c0 + (int)lane;
+        if (idx < m) {
+          const uint64_t e = sortk[idx];
+          const int dev = (int)(e >> g.ds);
+          if (kc.cls(e) == kAlloc && dv.lv[dev] > __ldcg(dv.pk + dev)) {
+            atomicOr(dv.over + (dev >> 5), 1u << (dev & 31));
+            viol = viol || dv.lv[dev] > __ldg(g.cap + dev);
+          }
+        }
+      }
+      __syncwarp();
+    }
+    viol = __any_sync(kFullMask, viol);
+    // the other accelerators' events leave; with more than 32 accelerators
+    // their frees are applied, and where the order matters the allocations are
+    // taken back
+    int keep = 0;
+    for (int c0 = 0; c0 < m; c0 += 32) {
+      const int idx = c0 + (int)lane;
+      const bool v = idx < m;
+      const uint64_t e = v ? sortk[idx] : 0ull;
+      const int dev = (int)(e >> g.ds);
+      bool k;
+      if constexpr (kNarrow) {
+        k = v && ((fail >> dev) & 1u);
+      } else {
+        k = v && ((dv.over[dev >> 5] >> (dev & 31)) & 1u);
+        if (v && k == (kc.cls(e) == kAlloc))
+          atomicAdd(reinterpret_cast<unsigned long long*>(dv.lv + dev),
+                    (unsigned long long)-__ldg(g.bytes + (uint32_t)(e & g.opmask)));
+      }
+      const uint32_t bk = __ballot_sync(kFullMask, k);
+      if (k) sortk[keep + __popc(bk & lanes_below())] = e;  // at most idx: in place
+      keep += __popc(bk);
+      __syncwarp();
+    }
+    if (keep) apply_ordered(keep, viol, span);
+  }
 
   __device__ int count_below(uint64_t kmax) const {
     int c = 0;
     for (int c0 = 0; c0 < log.n; c0 += 32) {
       const int idx = c0 + (int)lane_id();
-      const bool take = idx < log.n && (*log.kp(idx) & lowmask) < kmax;
+      const bool take = idx < log.n && (*log.kp(idx) & lowmask()) < kmax;
       c += __popc(__ballot_sync(kFullMask, take));
     }
     return c;
   }
 
   // Move the logged events whose key part is < kmax to the sort area (their
-  // number is known to fit) and compact the rest; returns their number.
-  __device__ int extract(uint64_t kmax) {
+  // number is known to fit) and compact the rest; returns their number.  Sums
+  // them up for apply_due on the way: with at most 32 accelerators what is
+  // allocated and freed per accelerator and quarter of the time since the last
+  // drain (quarters of 2^wsh), each as sums of the low 24 and of the higher 24
+  // bits of the sizes (32-bit shared atomics; at most 256 events), with more the
+  // allocations into the live bytes.
+  __device__ int extract(uint64_t kmax, int wsh) {
     const unsigned lane = lane_id();
     const bool side = !kKey;
     int m = 0, keep = 0;
@@ -1094,7 +1126,7 @@ struct Sim {
       uint64_t e = kKeyMax;
       uint8_t dv8 = 0;
       if (v) {
-        if (idx < log.ms) {
+        if (idx < P.ms) {
           e = log.sk[idx];
           if (side) dv8 = log.sd[idx];
         } else {
@@ -1102,13 +1134,29 @@ struct Sim {
           if (side) dv8 = *log.dp(idx);
         }
       }
-      const bool take = v && (e & lowmask) < kmax;
+      const bool take = v && (e & lowmask()) < kmax;
       const uint32_t bt = __ballot_sync(kFullMask, take);
       const uint32_t bk = __ballot_sync(kFullMask, v && !take);
       if (take) {
         const int pos = m + __popc(bt & lanes_below());
         sortk[pos] = e;
         if (side) sortd[pos] = dv8;
+        if constexpr (kKey) {
+          const uint64_t b = (uint64_t)__ldg(g.bytes + (uint32_t)(e & g.opmask));
+          const bool al = kc.cls(e) == kAlloc;
+          const int dev = (int)(e >> g.ds);
+          if constexpr (kNarrow) {
+            const tm_t t = (tm_t)((e & lowmask()) >> (g.ib + 2)) - drained;
+            const int w = min((int)(t >> wsh), kWindows - 1);
+            uint32_t* a = dv.acc + 4 * (kWindows * dev + w) + (al ? 0 : 2);
+            if (!g.big_bytes) {
+              atomicAdd(a, (uint32_t)b & 0xffffffu);
+              atomicAdd(a + 1, (uint32_t)(b >> 24));
+            }
+          } else if (al) {
+            atomicAdd(reinterpret_cast<unsigned long long*>(dv.lv + dev), (unsigned long long)b);
+          }
+        }
       } else if (v) {
         const int pos = keep + __popc(bk & lanes_below());  // pos <= idx: in place
         *log.kp(pos) = e;
@@ -1154,254 +1202,640 @@ struct Sim {
   }
 
   // Apply every logged event that can no longer be preceded (time < t_next).
-  __device__ void drain(int64_t t_next) {
+  __device__ __forceinline__ void drain(int64_t t_next) {
     generate();
+    drain_log(t_next);
+  }
+  __device__ __forceinline__ void drain_log(int64_t t_next) {
     const uint64_t lim = t_next == kI64Max ? kKeyMax : kc.time_floor(t_next);
+    // the time since the last drain, and quarters of it (the last drain of all
+    // has one interval)
+    const tm_t span = t_next == kI64Max ? kNever : (tm_t)t_next - drained;
+    int wsh = 8 * (int)sizeof(tm_t) - 1;
+    if (span < ((tm_t)1 << 30)) wsh = max(0, 32 - __clz((uint32_t)span) - 2);
     while (log.n > 0) {
       uint64_t kmax = lim;
-      if (log.n > sortcap) {
+      if (log.n > P.sortcap) {
         const int due = count_below(lim);
         if (due == 0) break;
-        if (due > sortcap) {
+        if (due > P.sortcap) {
           // Rare: more due events than the sort area.  Bisect a key bound
-          // with at most sortcap events below it (at most n_dev <= sortcap
+          // with at most P.sortcap events below it (at most n_dev <= P.sortcap
           // events share a key part).
           uint64_t lo = kKeyMax;
           for (int c0 = 0; c0 < log.n; c0 += 32) {
             const int idx = c0 + (int)lane_id();
-            const uint64_t kk = idx < log.n ? (*log.kp(idx) & lowmask) : kKeyMax;
+            const uint64_t kk = idx < log.n ? (*log.kp(idx) & lowmask()) : kKeyMax;
             lo = kk < lo ? kk : lo;
           }
-          lo = warp_min_u64(lo) + 1;  // 1 <= count_below(lo) <= sortcap
-          uint64_t hi = lim;          // count_below(hi) > sortcap
+          lo = warp_min_u64(lo) + 1;  // 1 <= count_below(lo) <= P.sortcap
+          uint64_t hi = lim;          // count_below(hi) > P.sortcap
           while (hi - lo > 1) {
             const uint64_t mid = lo + (hi - lo) / 2;
-            if (count_below(mid) <= sortcap) lo = mid;
+            if (count_below(mid) <= P.sortcap) lo = mid;
             else hi = mid;
           }
           kmax = lo;
         }
       }
-      const int m = extract(kmax);
+      const int m = extract(kmax, wsh);
       if (m == 0) break;
-      if (kKey && m <= 32) {
-        sort_apply_regs(m);
+      if (kKey) {
+        apply_due(m, span);
       } else {
         sort_area(m);
-        if (kKey) apply_segmented(m);
-        else apply_serial(m);
+        apply_serial(m);
       }
       if (kmax == lim) break;
     }
+    drained = (tm_t)t_next;
   }
 
-  __device__ void maybe_checkpoint(uint64_t next_key);
-
-  // The event loop (Sec. 3.3.3).
-  __device__ void run() {
-    if (status) return;
-    if constexpr (kBatch) {
-      run_batched();
-      return;
-    }
-    while (true) {
-      const uint64_t top = q.top();
-      const uint64_t rm = warp_min_u64(rk_reg);
-      const uint64_t rk = rkey;
-      uint64_t nk = rk < top ? rk : top;
-      nk = rm < nk ? rm : nk;
-      if (kMode == kBase) maybe_checkpoint(nk);
-      if (nk == kKeyMax) break;
-      if (opn >= P.opcap) drain(kc.time(nk));
-      if (nk == rm) {
-        if (rk_reg == rm) rk_reg = kKeyMax;  // keys are unique
-      } else if (nk == rk) {
-        ++rootptr;
-        load_root();
-      } else {
-        __syncwarp();
-        q.pop();
-      }
-      if (++iters > (int32_t)g.max_iter) {
-        status = GMG_SIM_LOOP;
-        break;
-      }
-      const tm_t t = (tm_t)kc.time(nk);
-      if (kMode == kBase) last_t = t;
-      start_op(kc.op(nk), t);
-      if (status) break;
-    }
-    if (!status) drain(kI64Max);
-  }
+  __device__ void maybe_checkpoint(int64_t next_t, uint64_t held = kKeyMax);
 
   // -------------------------------------------------------------------------
-  // Batched sweep: the keys are taken in the same order as by run(), but
-  // consecutive keys are handled together, one op per lane.  Key k_m joins
-  // the batch k_1 < ... < k_{m-1} while time(k_m) < min_l (time(k_l) +
-  // 2^class(k_l)).  Every key pushed while handling k_l is at least
-  // (f_l, READY, .) with f_l >= r_l + dur_l >= r_l + 2^class(k_l) > r_m, so
-  // nothing a batch pushes can precede one of its keys: handling them
-  // together, each accelerator's ops in key order, gives the starts of
-  // handling them one at a time.  (Many tenants on many accelerators keep
-  // about a dozen keys per batch; the dependent loads of a batch's ops then
-  // overlap instead of following each other.)
+  // The event loop (Sec. 3.3.3), many READY keys at a time.  Let lim be the
+  // smallest earliest finish over every pending key.  A key pushed later is the
+  // successor of a pending op (or of one that such an op makes ready), so its
+  // ready time is >= lim: the pending keys with a time below lim are exactly the
+  // next ones in key order, and none of them can make an op ready that precedes
+  // another of them.  They are started together, one op per lane, each
+  // accelerator's ops in key order, which gives the starts of handling them one
+  // at a time.  An op's earliest finish is max(ready time, its accelerator's
+  // free time when it was queued) + duration: free times only grow.
+  //
+  // What bounds the sweep is the chain of dependent instructions and loads per
+  // op (record, successors, their placement and predecessors) and, one key at a
+  // time, the extraction of the minimum; a batch pays each once for all its ops
+  // and finds its keys with one reduction.
   // -------------------------------------------------------------------------
-  __device__ __forceinline__ uint64_t peek(uint64_t& rm) const {
+  __device__ __forceinline__ uint64_t outside_min() const {
     const uint64_t top = q.top();
-    rm = warp_min_u64(rk_reg);
-    const uint64_t nk = rkey < top ? rkey : top;
-    return rm < nk ? rm : nk;
+    return rkey < top ? rkey : top;
   }
-  __device__ __forceinline__ void take(uint64_t nk, uint64_t rm) {
-    if (nk == rm) {
-      if (rk_reg == rm) rk_reg = kKeyMax;  // keys are unique
-    } else if (nk == rkey) {
+  __device__ __forceinline__ tm_t key_time(uint64_t k) const { return k == kKeyMax ? kNever : (tm_t)rq.time(k); }
+  // Removes the smallest key outside the pool (root list or heap).
+  __device__ __forceinline__ void take_outside(uint64_t x) {
+    if (x == rkey) {
       ++rootptr;
       load_root();
     } else {
       __syncwarp();
-      q.pop_fast();
+      q.pop();
     }
   }
-  // An op whose inputs several ops of one batch complete is queued once: the
-  // first lane to mark its (zero) finish time with -1 queues it.
-  __device__ __forceinline__ bool claim(uint32_t j) {
-    if (kT32) return atomicCAS(reinterpret_cast<int*>(fbuf + j), 0, -1) == 0;
-    return atomicCAS(reinterpret_cast<unsigned long long*>(fbuf + j), 0ull, ~0ull) == 0ull;
+  __device__ void run() {
+    if (status) return;
+    if constexpr (kNarrow) run_narrow();
+    else run_wide();
   }
 
-  __device__ void run_batched() {
-    const unsigned lane = lane_id();
-    while (true) {
-      uint64_t rm;
-      uint64_t nk = peek(rm);
-      if (kMode == kBase) maybe_checkpoint(nk);
-      if (nk == kKeyMax) break;
-      if (opn >= P.drain_trigger) drain(rq.time(nk));
-      uint64_t mine = kKeyMax;
-      int m = 0;
-      int64_t lim = 0;
-      while (true) {
-        const int64_t t = rq.time(nk);
-        const bool from_reg = nk == rm;
-        take(nk, rm);
-        if ((int)lane == m) mine = nk;
-        const int64_t e = t + ((int64_t)1 << rq.q(nk));
-        lim = (m == 0 || e < lim) ? e : lim;
-        if (kMode == kBase) last_t = (tm_t)t;
-        if (++m == 32) break;
-        // the register tier's minimum only changes when its key was taken
-        if (from_reg) rm = warp_min_u64(rk_reg);
-        const uint64_t top = q.top();
-        nk = rkey < top ? rkey : top;
-        nk = rm < nk ? rm : nk;
-        if (nk == kKeyMax || rq.time(nk) >= lim) break;
-      }
-      iters += m;
-      if (iters > (int32_t)g.max_iter) {
-        status = GMG_SIM_LOOP;
-        break;
-      }
-      start_batch(mine, m);
-      if (status) break;
-    }
-    if (!status) drain(kI64Max);
+  // What starting an op needs of its record, and the record of a successor.
+  struct Start {
+    tm_t dur, xq;
+    int64_t bytes;
+    uint32_t succ_off, nsucc, flags;
+    int32_t req;
+  };
+  __device__ __forceinline__ uint4 hot(uint32_t i) const { return kHot == kHotShared ? sh_hot[i] : __ldg(g.st_hot + i); }
+  __device__ __forceinline__ uint32_t succ_at(uint32_t k) const {
+    return kHot == kHotShared ? sh_succ[k] : __ldg(g.succ + k);
   }
-
-  // Start the batch's ops (lane b < m holds key b), record them for HBM-event
-  // generation, and queue the successors they make ready.
-  __device__ void start_batch(uint64_t key, int m) {
-    const unsigned lane = lane_id();
-    const bool v = (int)lane < m;
-    uint32_t i = 0, succ_off = 0, nsucc = 0, flags = 0;
-    int32_t req = 0;
-    int d = 0;
-    tm_t r = 0, f = 0, dur = 0;
-    int64_t bytes = 0, xq = 0;
-    if (v) {
-      i = rq.op(key);
-      r = (tm_t)rq.time(key);
+  __device__ __forceinline__ uint32_t pred_at(uint32_t k) const {
+    return (kHot == kHotShared ? sh_pred[k] : __ldg(g.pred + k)) & kIdMask;
+  }
+  __device__ __forceinline__ Start start_of(uint32_t i, int d) const {
+    Start s;
+    if constexpr (kHot != kHotNone) {
+      const uint4 h = hot(i);
+      s.dur = (tm_t)h.x;
+      s.xq = (tm_t)(h.y & 0x1fffffffu);
+      s.flags = h.y >> 29;
+      s.succ_off = h.z & 0xffffffu;
+      s.nsucc = h.z >> 24;
+      s.bytes = 0;
+      s.req = 0;  // read when the op ends a request
+    } else {
       const longlong2 db = op_durbytes(g.ops, i);
       const XqSucc xs = op_xqsucc(g.ops, i);
       const uint4 cs = op_cons(g.ops, i);
-      bytes = db.y;
-      xq = xs.xq;
-      succ_off = xs.succ_off;
-      nsucc = xs.nsucc;
-      req = (int32_t)cs.z;
-      flags = cs.w;
-      d = row[i];
-      dur = (tm_t)dur_of(i, d, db.x);
+      s.bytes = db.y;
+      s.xq = (tm_t)xs.xq;
+      s.succ_off = xs.succ_off;
+      s.nsucc = xs.nsucc;
+      s.req = (int32_t)cs.z;
+      s.flags = cs.w;
+      s.dur = (tm_t)dur_of(i, d, db.x);
     }
-    // every accelerator starts its ops of the batch in key (= lane) order
-    bool todo = v;
-    while (__any_sync(kFullMask, todo)) {
-      const uint32_t grp = __match_any_sync(kFullMask, todo ? (uint32_t)d : 256u + lane);
-      if (todo && __ffs(grp) - 1 == (int)lane) {
-        const tm_t fd = dv.fr[d];
-        const tm_t s = r > fd ? r : fd;
-        f = s + dur;
+    return s;
+  }
+  // The time that p's output takes to dj (p on dp, another accelerator).
+  __device__ __forceinline__ tm_t sends(uint32_t p, int dp, int dj) const {
+    if constexpr (kHot != kHotNone) return (tm_t)(hot(p).y & 0x1fffffffu) + (tm_t)g.lat0;
+    return xfer(dp, dj, op_durbytes(g.ops, p).y, op_xqsucc(g.ops, p).xq);
+  }
+
+  // The op started by this lane (i on d, ending at f) reaches its successor j:
+  // ready once every predecessor has started, at the latest arrival over all of
+  // them (Sec. 3.3.2).
+  struct Reached {
+    uint32_t j;
+    int d;
+    tm_t r, dur;
+    bool rdy, join;
+  };
+  __device__ __forceinline__ Reached reach(uint32_t i, int d, tm_t f, const Start& s, uint32_t u) const {
+    Reached x;
+    x.j = succ_at(s.succ_off + u);
+    x.d = row[x.j];
+    uint32_t npred, pred_off;
+    if constexpr (kHot != kHotNone) {
+      const uint4 h = hot(x.j);
+      x.dur = (tm_t)h.x;
+      npred = h.w >> 24;
+      pred_off = h.w & 0xffffffu;
+      x.r = (tm_t)(kHot == kHotShared ? sh_rel[x.j] : __ldg(g.st_rel + x.j));
+    } else {
+      const RelPred jp = op_relpred(g.ops, x.j);
+      x.dur = (tm_t)dur_of(x.j, x.d, op_durbytes(g.ops, x.j).x);
+      npred = jp.npred;
+      pred_off = jp.pred_off;
+      x.r = (tm_t)jp.rel;
+    }
+    tm_t arr = f;
+    if (x.d != d) arr += kHot != kHotNone ? s.xq + (tm_t)g.lat0 : xfer(d, x.d, s.bytes, s.xq);
+    x.r = x.r > arr ? x.r : arr;
+    x.rdy = true;
+    x.join = npred > 1;
+    if (npred == 2u) {  // one other predecessor: its loads side by side
+      const tm_t fj = fin(x.j);  // nonzero: queued already, by another lane of this batch
+      const uint32_t p0 = pred_at(pred_off), p1 = pred_at(pred_off + 1u);
+      const uint32_t p = p0 == i ? p1 : p0;
+      const tm_t a = fin(p);
+      const int dp = row[p];
+      const tm_t b = a + (dp != x.d ? sends(p, dp, x.d) : (tm_t)0);
+      x.rdy = a > 0 && fj == 0;
+      x.r = b > x.r ? b : x.r;
+    } else if (x.join) {
+      const tm_t fj = fin(x.j);
+      for (uint32_t t = 0; t < npred; ++t) {
+        const uint32_t p = pred_at(pred_off + t);
+        if (p == i) continue;
+        tm_t a = fin(p);
+        const int dp = row[p];
+        if (a <= 0) {
+          x.rdy = false;
+          break;
+        }
+        if (dp != x.d) a += sends(p, dp, x.d);
+        x.r = a > x.r ? a : x.r;
+      }
+      x.rdy = x.rdy && fj == 0;
+    }
+    return x;
+  }
+  // A join whose inputs several lanes complete is queued once.  Uniform call.
+  __device__ __forceinline__ void claim(Reached& x) {
+    const uint32_t jm = __ballot_sync(kFullMask, x.rdy && x.join);
+    if (jm == 0u) return;
+    if (jm & (jm - 1u)) {
+      const uint32_t grp = __match_any_sync(kFullMask, x.rdy && x.join ? x.j : ~lane_id());
+      if (x.join && __ffs(grp) - 1 != (int)lane_id()) x.rdy = false;
+    }
+    if (x.rdy && x.join) fbuf[x.j] = (tm_t)-1;
+    __syncwarp();
+  }
+  // Op i of this lane started, ready at r and ending at f (act: the lanes that
+  // started one).  Uniform call.
+  __device__ __forceinline__ void record(bool v, uint32_t act, uint32_t i, tm_t r, tm_t f, const Start& s) {
+    if (v) {
+      fbuf[i] = f;
+      if (s.flags & kReqSink) {
+        const int32_t req = kHot != kHotNone ? (int32_t)op_cons(g.ops, i).z : s.req;
+        atomicMax(reinterpret_cast<unsigned long long*>(creq() + req), (unsigned long long)f);
+      }
+      if (kMode == kBase) {
+        P.base.rb[i] = r;
+        P.base.fb[i] = f;
+      }
+      oplog[opn + __popc(act & lanes_below())] = i;
+      if (s.flags & kScored) score += (int64_t)f;
+      if (kMode == kInc && r >= T0) ++nev;
+    }
+    opn += __popc(act);
+    if (kMode == kBase) {
+      const tm_t lt = (tm_t)warp_max_u64(v ? (uint64_t)r : 0ull);
+      last_t = lt > last_t ? lt : last_t;
+      readypops += __popc(act);
+    }
+  }
+  __device__ __forceinline__ bool count_started(int m) {
+    iters += m;
+    if (iters <= (int32_t)g.max_iter) return true;
+    status = GMG_SIM_LOOP;
+    return false;
+  }
+
+  // ---- at most 32 accelerators: one pending op per lane, in registers -------
+  __device__ __forceinline__ void hold_op(tm_t r, uint32_t op) {
+    pd.r = r;
+    pd.op = op;
+    pd.d = row[op];
+    if constexpr (kHot != kHotNone) pd.dur = (tm_t)hot(op).x;
+    else pd.dur = (tm_t)dur_of(op, pd.d, op_durbytes(g.ops, op).x);
+    pd.e = earliest(r, pd.d, pd.dur);
+  }
+  __device__ __forceinline__ tm_t earliest(tm_t r, int d, tm_t dur) const {
+    const tm_t fd = dv.fr[d];
+    return (r > fd ? r : fd) + dur;
+  }
+  __device__ __forceinline__ uint64_t held_key() const {
+    return pd.r == kNever ? kKeyMax : rq.make(pd.r, pd.op, (tm_t)(pd.e - pd.r));
+  }
+  __device__ __forceinline__ bool precedes(tm_t ra, uint32_t ia, tm_t rb_, uint32_t ib_) const {
+    return ra < rb_ || (ra == rb_ && ia < ib_);
+  }
+
+  __device__ void run_narrow() {
+    const unsigned lane = lane_id();
+    uint64_t xk = outside_min();  // the smallest key outside the lanes, and its time
+    tm_t xr = key_time(xk);
+    while (true) {
+      if (kMode == kBase && readypops >= next_ck) {
+        const tm_t t = warp_min_t(pd.r);
+        const tm_t tn = t < xr ? t : xr;
+        if (tn != kNever) maybe_checkpoint((int64_t)tn, held_key());
+      }
+      tm_t lim = warp_min_t(pd.e);
+      const bool end = lim == kNever && xr == kNever;
+      if (end || opn >= P.drain_trigger) {  // the only copy of this code: it is large
+        const tm_t t = warp_min_t(pd.r);
+        drain(end ? kI64Max : (int64_t)(t < xr ? t : xr));
+        if (end || status) break;
+      }
+      bool act;
+      if (xr < lim) {
+        // keys outside the lanes are due (rare: every root once, the heap only
+        // after the lanes were all taken): they come into empty lanes
+        uint32_t fm = __ballot_sync(kFullMask, pd.r == kNever);
+        bool fresh = false;
+        while (fm && xr < lim) {
+          const int dst = __ffs(fm) - 1;
+          fm &= fm - 1u;
+          if ((int)lane == dst) {
+            pd.r = xr;
+            pd.op = rq.op(xk);
+            fresh = true;
+          }
+          take_outside(xk);
+          xk = outside_min();
+          xr = key_time(xk);
+        }
+        if (fresh) hold_op(pd.r, pd.op);
+        lim = warp_min_t(pd.e);
+        act = pd.r < lim;
+        if (xr < lim) {
+          // no empty lane: only keys before the next outside one; if there is
+          // none it changes places with the last key of the lanes
+          act = act && precedes(pd.r, pd.op, xr, rq.op(xk));
+          if (!__any_sync(kFullMask, act)) {
+            const uint64_t mine = held_key();
+            const uint64_t last = warp_max_u64(mine);
+            const uint64_t x = xk;
+            take_outside(x);
+            q.push(last);  // the heap keeps one entry beyond its limit for this
+            act = mine == last;
+            if (act) hold_op((tm_t)rq.time(x), rq.op(x));
+            xk = outside_min();
+            xr = key_time(xk);
+          }
+        }
+      } else {
+        act = pd.r < lim;
+      }
+      const uint32_t b = __ballot_sync(kFullMask, act);
+      const int m = __popc(b);
+      if (!count_started(m)) break;
+      const uint32_t i = pd.op;
+      const int d = pd.d;
+      const tm_t r = pd.r;
+      Start s;
+      s.nsucc = 0;
+      s.flags = 0;
+      tm_t f = 0, fd = 0;
+      if (act) {
+        s = start_of(i, d);
+        fd = dv.fr[d];
+      }
+      // every accelerator starts its ops of the batch in key order
+      if (m > 1 && __popc(__reduce_or_sync(kFullMask, act ? 1u << d : 0u)) < m) {
+        int ord = 0;
+        for (uint32_t o = b; o; o &= o - 1u) {
+          const int src = __ffs(o) - 1;
+          const tm_t ro = __shfl_sync(kFullMask, r, src);
+          const uint32_t io = __shfl_sync(kFullMask, i, src);
+          const int dd = __shfl_sync(kFullMask, d, src);
+          ord += act && dd == d && precedes(ro, io, r, i) ? 1 : 0;
+        }
+        const int last = (int)__reduce_max_sync(kFullMask, (unsigned)ord);
+        for (int t = 0; t < last; ++t) {
+          if (act && ord == t) {
+            f = earliest(r, d, pd.dur);
+            dv.fr[d] = f;
+          }
+          __syncwarp();
+        }
+        act = act && ord == last;  // the others have theirs
+        if (act) fd = dv.fr[d];
+      }
+      if (act) {
+        f = (r > fd ? r : fd) + pd.dur;
         dv.fr[d] = f;
-        todo = false;
+      }
+      const bool v = (b >> lane) & 1u;
+      record(v, b, i, r, f, s);
+      if (v) pd.r = pd.e = kNever;
+      __syncwarp();
+      // successors: a lane's first ready one stays in the lane, further ones go
+      // to empty lanes
+      for (uint32_t u = 0; __any_sync(kFullMask, u < s.nsucc); ++u) {
+        Reached x;
+        x.rdy = x.join = false;
+        x.j = 0;
+        x.d = 0;
+        x.r = x.dur = 0;
+        if (u < s.nsucc) x = reach(i, d, f, s, u);
+        claim(x);
+        tm_t e = kNever;
+        if (x.rdy) {
+          e = earliest(x.r, x.d, x.dur);
+          if (pd.r == kNever) {
+            pd.r = x.r;
+            pd.e = e;
+            pd.dur = x.dur;
+            pd.op = x.j;
+            pd.d = x.d;
+            x.rdy = false;
+          }
+        }
+        uint32_t more = __ballot_sync(kFullMask, x.rdy);
+        while (more) {
+          const int src = __ffs(more) - 1;
+          more &= more - 1u;
+          const uint32_t fm = __ballot_sync(kFullMask, pd.r == kNever);
+          const tm_t xr_ = __shfl_sync(kFullMask, x.r, src), xe = __shfl_sync(kFullMask, e, src),
+                     xd = __shfl_sync(kFullMask, x.dur, src);
+          const uint32_t xj = __shfl_sync(kFullMask, x.j, src);
+          const int xdev = __shfl_sync(kFullMask, x.d, src);
+          if (fm) {
+            if ((int)lane == __ffs(fm) - 1) {
+              pd.r = xr_;
+              pd.e = xe;
+              pd.dur = xd;
+              pd.op = xj;
+              pd.d = xdev;
+            }
+          } else {
+            if (32 + q.size >= P.pend_cap || !q.push(rq.make(xr_, xj, (tm_t)(xe - xr_)))) status = GMG_SIM_QUEUE;
+            xk = outside_min();
+            xr = key_time(xk);
+          }
+        }
+      }
+      if (status) break;
+    }
+  }
+
+  // ---- more accelerators: pending ops as keys in a pool in shared memory -----
+
+  // Slots [from, 32 * kSlots) are empty.
+  __device__ void empty_pool(int from) {
+    for (int x = (int)lane_id(); x < 32 * kSlots; x += 32) {
+      if (x >= from) pool[x] = kKeyMax;
+      fstk[x] = (uint8_t)(32 * kSlots - 1 - x);
+    }
+    nfree = 32 * kSlots - from;
+    __syncwarp();
+  }
+  __device__ __forceinline__ uint64_t pool_min() const {
+    uint64_t m = kKeyMax;
+#pragma unroll
+    for (int s = 0; s < kSlots; ++s) {
+      const uint64_t k = pool[32 * s + lane_id()];
+      m = k < m ? k : m;
+    }
+    return warp_min_u64(m);
+  }
+  __device__ __forceinline__ uint64_t next_key() const {
+    const uint64_t m = pool_min(), x = outside_min();
+    return m < x ? m : x;
+  }
+
+  __device__ void run_wide() {
+    const unsigned lane = lane_id();
+    while (true) {
+      if (kMode == kBase && readypops >= next_ck) {
+        const uint64_t nk = next_key();
+        if (nk != kKeyMax) maybe_checkpoint(rq.time(nk));
+      }
+      const bool end = nfree == 32 * kSlots && outside_min() == kKeyMax;
+      if (end || opn >= P.drain_trigger) {  // the only copy of this code: it is large
+        drain(end ? kI64Max : rq.time(next_key()));
+        if (end || status) break;
+      }
+      uint64_t k[kSlots];
+      tm_t lim = kNever;
+#pragma unroll
+      for (int s = 0; s < kSlots; ++s) {
+        k[s] = pool[32 * s + lane];
+        const tm_t e = k[s] == kKeyMax ? kNever : (tm_t)rq.bound(k[s]);
+        lim = e < lim ? e : lim;
+      }
+      lim = warp_min_t(lim);
+      // keys outside the pool that are due come in (rare: the roots once each,
+      // the heap only after the pool was full)
+      uint64_t x = outside_min();
+      uint64_t kb = kKeyMax;  // keys below kb are started
+      if (key_time(x) < lim) {
+        __syncwarp();
+        while (key_time(x) < lim) {
+          int slot;
+          if (nfree > 0) {
+            slot = fstk[--nfree];
+            take_outside(x);
+          } else {
+            // full: x waits unless it is the next key of all; it then changes
+            // places with the pool's last key
+            if (x > pool_min()) {
+              kb = x;
+              break;
+            }
+            uint64_t mx = 0;
+            int ms = 0;
+#pragma unroll
+            for (int s = 0; s < kSlots; ++s) {
+              const uint64_t y = pool[32 * s + lane];
+              if (y > mx) {
+                mx = y;
+                ms = 32 * s + (int)lane;
+              }
+            }
+            const uint64_t last = warp_max_u64(mx);
+            slot = __shfl_sync(kFullMask, ms, __ffs(__ballot_sync(kFullMask, mx == last)) - 1);
+            take_outside(x);
+            q.push(last);  // the heap keeps one entry beyond its limit for this
+          }
+          if (lane == 0) pool[slot] = x;
+          __syncwarp();
+          const tm_t e = (tm_t)rq.bound(x);
+          lim = e < lim ? e : lim;
+          x = outside_min();
+        }
+#pragma unroll
+        for (int s = 0; s < kSlots; ++s) k[s] = pool[32 * s + lane];
+      }
+      const uint64_t lb = (uint64_t)lim << g.qsh;
+      kb = lb < kb ? lb : kb;
+      int m = 0;
+      uint32_t b[kSlots];
+#pragma unroll
+      for (int s = 0; s < kSlots; ++s) {
+        b[s] = __ballot_sync(kFullMask, k[s] < kb);
+        m += __popc(b[s]);
+      }
+      if (m > 32) {
+        // more keys than lanes: a bound with 16 to 32 keys below it (or at
+        // least one)
+        uint64_t lo = pool_min() + 1, hi = kb;
+        m = 0;
+        while (m < 16 && hi - lo > 1) {
+          const uint64_t mid = lo + (hi - lo) / 2;
+          int c = 0;
+#pragma unroll
+          for (int s = 0; s < kSlots; ++s) c += __popc(__ballot_sync(kFullMask, k[s] < mid));
+          if (c <= 32) {
+            lo = mid;
+            m = c;
+          } else {
+            hi = mid;
+          }
+        }
+        m = 0;
+#pragma unroll
+        for (int s = 0; s < kSlots; ++s) {
+          b[s] = __ballot_sync(kFullMask, k[s] < lo);
+          m += __popc(b[s]);
+        }
+      }
+      // one key per lane, through the sort area (free between drains)
+      int at = 0;
+      __syncwarp();
+#pragma unroll
+      for (int s = 0; s < kSlots; ++s) {
+        if ((b[s] >> lane) & 1u) {
+          const int pos = at + __popc(b[s] & lanes_below());
+          sortk[pos] = k[s];
+          reinterpret_cast<uint32_t*>(sortk + 32)[pos] = (uint32_t)(32 * s) + lane;
+        }
+        at += __popc(b[s]);
+      }
+      __syncwarp();
+      uint64_t key = kKeyMax;
+      int slot = 0;
+      if ((int)lane < m) {
+        key = sortk[lane];
+        slot = (int)reinterpret_cast<const uint32_t*>(sortk + 32)[lane];
+      }
+      if (!count_started(m)) break;
+      start_batch(key, slot, m);
+      if (status) break;
+    }
+  }
+
+  // Start the batch's ops (lanes below m: a key and the pool slot that it came
+  // from), record them for HBM-event generation, and queue the successors they
+  // make ready.
+  __device__ __forceinline__ void start_batch(uint64_t key, int slot, int m) {
+    const unsigned lane = lane_id();
+    const bool v = key != kKeyMax;
+    const uint32_t i = rq.op(key);
+    const tm_t r = (tm_t)rq.time(key);
+    int d = 0;
+    tm_t f = 0;
+    Start s;
+    s.nsucc = 0;
+    s.flags = 0;
+    s.dur = 0;
+    if (v) {
+      d = row[i];
+      s = start_of(i, d);
+    }
+    // every accelerator starts its ops of the batch in key order
+    int ord = 0, maxord = 0;
+    if (m > 1) {
+      const uint32_t grp = __match_any_sync(kFullMask, v ? (uint32_t)d : 256u + lane);
+      uint32_t o = grp & ~(1u << lane);
+      while (__any_sync(kFullMask, o != 0u)) {
+        const uint64_t ok = __shfl_sync(kFullMask, key, o ? __ffs(o) - 1 : (int)lane);
+        if (ok < key) ++ord;
+        o &= o - 1u;
+        maxord = 1;
+      }
+      if (maxord) maxord = (int)__reduce_max_sync(kFullMask, (unsigned)ord);
+    }
+    for (int t = 0; t <= maxord; ++t) {
+      if (v && ord == t) {
+        f = earliest(r, d, s.dur);
+        dv.fr[d] = f;
       }
       __syncwarp();
     }
-    if (v) {
-      fbuf[i] = f;
-      if (flags & kReqSink)
-        atomicMax(reinterpret_cast<unsigned long long*>(creq + req), (unsigned long long)f);
-      if (kMode == kBase) P.base.rb[i] = r;
-      oplog[opn + (int)lane] = i;
-    }
-    opn += m;
-    score += warp_sum_i64((v && (flags & kScored)) ? (int64_t)f : 0);
-    if (kMode == kBase) {
-      const tm_t mk = (tm_t)warp_max_u64(v ? (uint64_t)f : 0ull);
-      makespan = mk > makespan ? mk : makespan;
-      readypops += m;
-    }
-    if (kMode == kInc) nev += __popc(__ballot_sync(kFullMask, v && r >= T0));
+    record(v, __ballot_sync(kFullMask, v), i, r, f, s);
     __syncwarp();
-    // successors: ready once every predecessor has started; ready time = the
-    // latest arrival over all of them (Sec. 3.3.2)
-    const uint32_t maxs = __reduce_max_sync(kFullMask, nsucc);
-    for (uint32_t u = 0; u < maxs; ++u) {
-      uint32_t j = 0, qj = 0;
-      tm_t rj = 0;
-      bool rdy = false;
-      if (u < nsucc) {
-        j = __ldg(g.succ + succ_off + u);
-        const int dj = row[j];
-        tm_t arr = f;
-        if (dj != d) arr = f + xfer(d, dj, bytes, xq);
-        const RelPred jp = op_relpred(g.ops, j);
-        qj = dur_class(dur_of(j, dj, op_durbytes(g.ops, j).x));
-        const tm_t rel = (tm_t)jp.rel;
-        rj = rel > arr ? rel : arr;
-        rdy = true;
-        if (jp.npred > 1) {
-          for (uint32_t k = 0; k < jp.npred; ++k) {
-            const uint32_t p = __ldg(g.pred + jp.pred_off + k) & kIdMask;
-            if (p == i) continue;
-            tm_t a = fin(p);
-            if (a <= 0) {  // not started yet
-              rdy = false;
-              break;
-            }
-            const int dp = row[p];
-            if (dp != dj) a += xfer(dp, dj, op_durbytes(g.ops, p).y, op_xqsucc(g.ops, p).xq);
-            rj = a > rj ? a : rj;
-          }
-          if (rdy) rdy = claim(j);
+    // successors: a lane's first ready one takes its own slot, further ones
+    // take empty slots
+    bool kept = false;
+    for (uint32_t u = 0; __any_sync(kFullMask, u < s.nsucc); ++u) {
+      Reached x;
+      x.rdy = x.join = false;
+      x.j = 0;
+      x.d = 0;
+      x.r = x.dur = 0;
+      if (u < s.nsucc) x = reach(i, d, f, s, u);
+      claim(x);
+      uint64_t nk = kKeyMax;
+      if (x.rdy) {
+        nk = rq.make(x.r, x.j, (tm_t)(earliest(x.r, x.d, x.dur) - x.r));
+        if (!kept) {
+          pool[slot] = nk;
+          kept = true;
+          x.rdy = false;
         }
       }
-      uint32_t bm = __ballot_sync(kFullMask, rdy);
-      while (bm) {
-        const int src = __ffs(bm) - 1;
-        bm &= bm - 1;
-        push_ready(__shfl_sync(kFullMask, rq.make(rj, j, qj), src));
+      const uint32_t more = __ballot_sync(kFullMask, x.rdy);
+      if (more) {
+        const int c = __popc(more), have = nfree < c ? nfree : c;
+        const int rank = __popc(more & lanes_below());
+        if (x.rdy && rank < have) pool[fstk[nfree - 1 - rank]] = nk;
+        nfree -= have;
+        uint32_t rest = __ballot_sync(kFullMask, x.rdy && rank >= have);
+        while (rest) {
+          const int src = __ffs(rest) - 1;
+          rest &= rest - 1;
+          if (!q.push(__shfl_sync(kFullMask, nk, src))) status = GMG_SIM_QUEUE;
+        }
+        if (32 * kSlots - nfree + q.size > P.pend_cap) status = GMG_SIM_QUEUE;
+        __syncwarp();
       }
     }
+    const bool gone = v && !kept;
+    const uint32_t gm = __ballot_sync(kFullMask, gone);
+    if (gone) {
+      pool[slot] = kKeyMax;
+      fstk[nfree + __popc(gm & lanes_below())] = (uint8_t)slot;
+    }
+    nfree += __popc(gm);
+    __syncwarp();
   }
 
   __device__ void write_invalid(int64_t k, int32_t st) {
@@ -1446,7 +1880,7 @@ struct Sim {
     const unsigned lane = lane_id();
     int32_t miss = 0;
     for (int r = lane; r < g.R; r += 32) {
-      const int64_t c = creq[r];
+      const int64_t c = creq()[r];
       miss += c > __ldg(g.deadline + r) ? 1 : 0;
       if (o.req_done) o.req_done[k * g.R + r] = c;
     }
@@ -1456,16 +1890,18 @@ struct Sim {
     // the accelerators that ran an op (an op finishes after its accelerator's
     // initial availability).
     const int64_t mk = dv.max_busy(g);
+    const int64_t sc = kPool ? warp_sum_i64(score) : score;
+    const int64_t ne = kMode == kFull ? (int64_t)iters : kPool ? warp_sum_i64(nev) : nev;
     if (lane == 0) {
       o.makespan[k] = mk;
-      o.score[k] = vflag ? kI64Max : score;
+      o.score[k] = vflag ? kI64Max : sc;
       o.status[k] = GMG_SIM_OK;
       o.viol_flag[k] = vflag;
       o.viol_op[k] = vop;
       o.viol_dev[k] = vdev;
       o.viol_time[k] = vt;
       o.sla_miss[k] = miss;
-      o.events[k] = kMode == kFull ? (int64_t)iters : nev;
+      o.events[k] = ne;
     }
     const int ts = trace_slot(k);
     if (ts >= 0)
@@ -1501,39 +1937,52 @@ struct Sim {
 };
 
 // Base-mode checkpoint: at a time boundary T_c (nothing at the next key's
-// time handled yet), save the complete simulator state -- accelerator state,
+// time next_t handled yet), save the complete simulator state -- accelerator state,
 // READY heap, event log, partial results; the ops started by then are those
 // with base ready time < T_c.  An incremental candidate whose resume time T0
 // is >= T_c restarts there.
-template <bool kReg, int kMode, bool kKey, bool kT32, bool kTypes, bool kBatch, bool kStage>
-__device__ void Sim<kReg, kMode, kKey, kT32, kTypes, kBatch, kStage>::maybe_checkpoint(uint64_t next_key) {
+template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, bool kPool, int kHot>
+__device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kPool, kHot>::maybe_checkpoint(int64_t tn, uint64_t held) {
   if (kMode != kBase) return;
   const DevBase& B = P.base;
-  if (next_key == kKeyMax || ck >= B.nck || readypops < next_ck) return;
-  const int64_t tn = rq.time(next_key);
-  if (tn <= last_t) return;
+  if (ck >= B.nck || readypops < next_ck) return;
+  if (tn <= (int64_t)last_t) return;
   const unsigned lane = lane_id();
   generate();
-  const bool hasreg = rk_reg != kKeyMax;
-  const uint32_t regm = __ballot_sync(kFullMask, hasreg);
-  const int nready = q.size + __popc(regm);
+  // the pool's keys (or the keys that the lanes hold) follow the heap's
+  constexpr bool kPooled = kPool && !kNarrow;
+  const uint32_t hm = __ballot_sync(kFullMask, held != kKeyMax);
+  const int nready = q.size + (kPooled ? 32 * kSlots - nfree : __popc(hm));
   if (nready <= B.ckq && log.n <= B.ckm) {
     int64_t* sc = B.ck_scalars + (int64_t)ck * 8;
-    if (hasreg) B.ck_qkey[(int64_t)ck * B.ckq + q.size + __popc(regm & lanes_below())] = rk_reg;
+    uint64_t* qk = B.ck_qkey + (int64_t)ck * B.ckq;
+    if (kPooled) {
+      int at = q.size;
+#pragma unroll
+      for (int s = 0; s < kSlots; ++s) {
+        const uint64_t k = pool[32 * s + lane];
+        const uint32_t b = __ballot_sync(kFullMask, k != kKeyMax);
+        if (k != kKeyMax) qk[at + __popc(b & lanes_below())] = k;
+        at += __popc(b);
+      }
+    } else if (held != kKeyMax) {
+      qk[q.size + __popc(hm & lanes_below())] = held;
+    }
+    const int64_t total = kPool ? warp_sum_i64(score) : score;
     if (lane == 0) {
       B.ck_time[ck] = tn;
       sc[0] = nready;
       sc[1] = rootptr;
-      sc[2] = score;
-      sc[3] = makespan;
+      sc[2] = total;
+      sc[3] = (int64_t)drained;
       sc[4] = vflag;
       sc[5] = vt;
       sc[6] = ((int64_t)vop << 32) | (uint32_t)vdev;
       sc[7] = log.n;
     }
     dv.save(B.ck_dev + (int64_t)ck * 3 * g.D);
-    for (int r = lane; r < g.R; r += 32) B.ck_creq[(int64_t)ck * g.R + r] = creq[r];
-    for (int x = lane; x < q.size; x += 32) B.ck_qkey[(int64_t)ck * B.ckq + x] = *q.kp(x);
+    for (int r = lane; r < g.R; r += 32) B.ck_creq[(int64_t)ck * g.R + r] = creq()[r];
+    for (int x = lane; x < q.size; x += 32) qk[x] = *q.kp(x);
     for (int x = lane; x < log.n; x += 32) {
       B.ck_mkey[(int64_t)ck * B.ckm + x] = *log.kp(x);
       if (!kKey) B.ck_mdev[(int64_t)ck * B.ckm + x] = *log.dp(x);
@@ -1546,33 +1995,28 @@ __device__ void Sim<kReg, kMode, kKey, kT32, kTypes, kBatch, kStage>::maybe_chec
   __syncwarp();
 }
 
-template <bool kReg, int kMode, bool kKey, bool kT32, bool kTypes, bool kBatch, bool kStage>
-__device__ void setup_slot(Sim<kReg, kMode, kKey, kT32, kTypes, kBatch, kStage>& S, const SimParams& P, unsigned wib,
+template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, bool kPool, int kHot>
+__device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kPool, kHot>& S, const SimParams& P, unsigned wib,
                            int64_t slot, uint8_t* smem) {
   uint8_t* sl = P.scratch + slot * P.slot_bytes;
   const WarpSmem w = carve_smem(smem, P, wib);
+  S.pool = w.pool;
+  S.fstk = w.fstk;
+  S.nfree = 0;
   S.q.sk = w.heap;
-  S.q.gk = reinterpret_cast<uint64_t*>(sl + P.off_qk);
-  S.q.qs = P.qs;
-  S.q.cap = P.qcap;
+  S.q.sl = sl;
+  S.log.sl = sl;
   S.q.size = 0;
   S.log.sk = w.logk;
   S.log.sd = w.logd;
-  S.log.gk = reinterpret_cast<uint64_t*>(sl + P.off_mk);
-  S.log.gd = sl + P.off_md;
-  S.log.ms = P.ms;
-  S.log.cap = P.mcap;
   S.log.n = 0;
   S.sortk = w.sortk;
   S.sortd = w.sortd;
   S.oplog = w.oplog;
   S.opn = 0;
-  S.sortcap = P.sortcap;
-  using tm_t = typename Sim<kReg, kMode, kKey, kT32, kTypes, kBatch, kStage>::tm_t;
+  using tm_t = typename Sim<kNarrow, kMode, kKey, kT32, kTypes, kPool, kHot>::tm_t;
   S.fbuf = reinterpret_cast<tm_t*>(sl + P.off_f);
-  S.holdb = reinterpret_cast<tm_t*>(sl + P.off_hold);
-  S.bits = reinterpret_cast<uint32_t*>(sl + P.off_bits);
-  S.creq = reinterpret_cast<int64_t*>(sl + P.off_creq);
+  S.sl = sl;
   S.dv.setup(P.g, w.dev, P.off_pk >= 0 ? reinterpret_cast<int64_t*>(sl + P.off_pk) : nullptr);
   S.T0 = -1;
   S.Tc = 0;

@@ -1,0 +1,98 @@
+"""GPU parity of the sweep of pending READY ops and of the HBM accounting where
+they can go wrong: more pending ops than lanes or pool slots, more startable ops
+than lanes, equal times, batches that share accelerators, capacities that bind,
+sizes beyond 48 bits, 64-bit times; against the oracle, bit for bit."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from gpu_common import compare, oracle_rows, torch_place  # noqa: E402
+from helpers import mk  # noqa: E402
+from oracle import oracle as O  # noqa: E402
+from paper_2608_15762_gb300 import gmgsim as G  # noqa: E402
+from paper_2608_15762_gb300 import workloads as W  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2608_15762_gb300 import build
+    build.build()
+    assert torch.cuda.is_available()
+
+
+def _chains(seed, chains, length, D, dur_hi=20, bytes_lo=1, bytes_hi=1 << 20, cap=None, release_hi=0, fan=1):
+    """Independent chains; with fan > 1 every op feeds `fan` ops of the next
+    level of its chain and one op joins them."""
+    g = np.random.default_rng(seed)
+    preds, rel = [], []
+    for c in range(chains):
+        last = []
+        r = int(g.integers(0, release_hi + 1))
+        for _ in range(length):
+            first = len(preds)
+            preds.append(last)
+            rel.append(r if not last else 0)
+            if fan > 1:
+                for _ in range(fan):
+                    preds.append([first])
+                    rel.append(0)
+                preds.append(list(range(first + 1, first + 1 + fan)))
+                rel.append(0)
+            last = [len(preds) - 1]
+    n = len(preds)
+    return mk(preds, g.integers(1, dur_hi + 1, n), g.integers(bytes_lo, bytes_hi + 1, n), n_dev=D, bw=1000, lat=2,
+              release=rel, req_id=[0] * n, deadline=[1000], cap=None if cap is None else [cap] * D)
+
+
+def _rows(seed, K, n, D):
+    rows = np.zeros((K, W.placement_ld(n)), np.uint8)
+    rows[:, :n] = np.random.default_rng(seed).integers(0, D, (K, n))
+    rows[-1, :n] = 0
+    return rows
+
+
+@pytest.mark.parametrize("D", [1, 2, 8, 32, 33, 256])
+@pytest.mark.parametrize("kw", [
+    dict(chains=33, length=6),                                   # one more chain than lanes
+    dict(chains=161, length=4),                                  # one more than pool slots
+    dict(chains=400, length=2, dur_hi=1),                        # lockstep: every op startable at once
+    dict(chains=70, length=5, release_hi=60, dur_hi=4),          # roots that come in while the pool is full
+    dict(chains=9, length=4, fan=5),                             # joins, long lists
+    dict(chains=20, length=6, bytes_lo=1 << 18, cap=6 << 20),    # capacities that bind
+    dict(chains=5, length=5, bytes_lo=1 << 48, bytes_hi=1 << 50),  # sizes beyond 48 bits
+    dict(chains=30, length=6, dur_hi=1 << 29),                   # 64-bit times
+])
+def test_pending_ops_and_accounting(D, kw):
+    d = _chains(7, D=D, **kw)
+    rows = _rows(8, 13, d.n_ops, D)
+    g = G.gmg_create(d)
+    tk = torch.tensor([0, 12], dtype=torch.int32, device="cuda")
+    out = G.sim_batch(g, torch_place(rows), req_done=True, trace_k=tk)
+    base = rows[0, :d.n_ops].copy()
+    mv = W.random_moves(9, 40, base, D, max_moves=5)
+    b = G.base_create(g, torch.from_numpy(base).cuda())
+    inc = G.sim_incremental(g, b, *G.moves_to_device(mv, "cuda"), req_done=True)
+    torch.cuda.synchronize()
+    got = out.to_numpy()
+    compare(got, *oracle_rows(d, rows))
+    for slot, k in enumerate((0, 12)):
+        r = O.simulate(d, rows[k])
+        assert np.array_equal(got["trace_start"][slot], r["start"])
+        assert np.array_equal(got["trace_finish"][slot], r["finish"])
+    compare(inc.to_numpy(), *O.incremental_batch(d, base, mv))
+
+
+@pytest.mark.parametrize("K", [32, 33])
+def test_default_staging_rule_gives_the_same(K):
+    """The staged copy and the L1 path on the two sides of the default's line."""
+    wl = W.config2()
+    rows = wl.full_rows(range(K))
+    g = G.gmg_create(wl.desc)
+    outs = [G.sim_batch(g, torch_place(rows), req_done=True, gmg_staging=m)
+            for m in (G.GMG_STAGING_DEFAULT, G.GMG_STAGING_SHARED, G.GMG_STAGING_L1)]
+    torch.cuda.synchronize()
+    for o in outs:
+        compare(o.to_numpy(), *oracle_rows(wl.desc, rows))
