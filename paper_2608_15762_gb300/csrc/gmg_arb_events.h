@@ -17,148 +17,197 @@
 namespace gsim {
 namespace {
 
+constexpr int kArrivals = kArbArrivals;
+
 template <class Self, class SimBase>
 struct ArbEvents : SimBase {
   using tm_t = typename SimBase::tm_t;
-  uint64_t rk_reg;  // READY keys: one per lane (kKeyMax = empty), the others in the heap
   __device__ explicit ArbEvents(const SimParams& p) : SimBase(p) {}
   __device__ __forceinline__ const Self& self() const { return *static_cast<const Self*>(this); }
 
-  // One more input of op j present at time a (per lane); true if it was the
-  // last, with its ready time in rj.
-  __device__ __forceinline__ bool add_input(uint32_t j, tm_t a, tm_t& rj) const {
+  // One more input of op j (on accelerator d) present at time a (per lane);
+  // ready if it was the last.
+  __device__ __forceinline__ typename SimBase::Reached add_input(uint32_t j, int d, tm_t a) const {
+    typename SimBase::Reached x;
+    x.j = j;
+    x.d = d;
+    x.join = false;
     int32_t* cp = self().cnt() + j;
     tm_t* mp = self().rmax() + j;
-    const int32_t c = *cp + 1;
-    *cp = c;
-    const tm_t m = c == 1 ? a : (*mp > a ? *mp : a);
-    *mp = m;
-    const RelPred jp = op_relpred(this->g.ops, j);
-    if ((uint32_t)c != jp.npred) return false;
-    const tm_t rel = (tm_t)jp.rel;
-    rj = rel > m ? rel : m;
-    return true;
+    uint32_t npred;
+    if constexpr (SimBase::kCompact) {
+      const uint4 h = this->hot(j);
+      x.dur = (tm_t)h.x;
+      npred = h.w >> 24;
+      x.r = (tm_t)__ldg(this->g.st_rel + j);
+    } else {
+      const RelPred jp = op_relpred(this->g.ops, j);
+      x.dur = (tm_t)this->dur_of(j, d, op_durbytes(this->g.ops, j).x);
+      npred = jp.npred;
+      x.r = (tm_t)jp.rel;
+    }
+    tm_t m = a;
+    x.rdy = npred == 1u;
+    if (npred > 1u) {
+      const int32_t c = *cp + 1;
+      const tm_t o = *mp;
+      m = c > 1 && o > a ? o : a;
+      *cp = c;
+      *mp = m;
+      x.rdy = (uint32_t)c == npred;
+    }
+    x.r = x.r > m ? x.r : m;
+    return x;
   }
 
-  // READY keys go to a free lane's register if there is one, else the heap.
-  __device__ __forceinline__ void push_ready(uint64_t key) {
-    const uint32_t freel = __ballot_sync(kFullMask, rk_reg == kKeyMax);
-    if (freel) {
-      if ((int)lane_id() == __ffs(freel) - 1) rk_reg = key;
-    } else if (!this->q.push(key)) {
-      this->status = GMG_SIM_QUEUE;
-    }
-  }
-
-  __device__ __forceinline__ void push_readies(bool rdy, tm_t rj, uint32_t j) {
-    uint32_t m = __ballot_sync(kFullMask, rdy);
-    while (m) {
-      const int src = __ffs(m) - 1;
-      m &= m - 1;
-      push_ready(__shfl_sync(kFullMask, this->kc.make(rj, kReady, j), src));
-    }
-  }
-
-  // One hold on op p's own copy (on accelerator dp) ends at time v (per
-  // lane; `want`: this lane releases one).  Logs the copy's release when it
-  // was the last hold.
-  __device__ __forceinline__ void drop_hold(bool want, uint32_t p, tm_t v, int dp) {
-    bool last = false;
-    tm_t h = v;
-    if (want) {
-      int32_t* rp = self().refs() + p;
-      const int32_t left = *rp - 1;
-      *rp = left;
-      const tm_t o = this->holdb()[p];
-      h = o > v ? o : v;
-      this->holdb()[p] = h;
-      last = left == 0;
-    }
-    this->log_event(last, this->kc.make(h, kFree, p), dp);
+  // One hold on op p's own copy ends at time v (per lane); true if it was the
+  // last: the copy is then released at h.
+  __device__ __forceinline__ bool drop_hold(uint32_t p, tm_t v, tm_t& h) {
+    int32_t* rp = self().refs() + p;
+    const tm_t o = this->holdb()[p];
+    const int32_t left = *rp - 1;
+    *rp = left;
+    h = o > v ? o : v;
+    this->holdb()[p] = h;
+    return left == 0;
   }
 
   // HBM events of the ops started since the last generation, one op per
   // lane: the own copy allocated at s; the op's local hold on its own copy
   // ends at f if no listed consumer is local; every held input whose last
   // local listed consumer this op is gets released at f (a receive copy) or
-  // loses its local hold (the producer's own copy).
-  __device__ void generate() {
+  // loses its local hold (the producer's own copy).  One op ends the local hold
+  // on a copy, so no two lanes touch the same one.  Loads side by side as in the
+  // pure-latency simulation.
+  __device__ __forceinline__ void generate() {
     const unsigned lane = lane_id();
     for (int c0 = 0; c0 < this->opn; c0 += 32) {
       const int idx = c0 + (int)lane;
       const bool v = idx < this->opn;
       const uint32_t x = v ? this->oplog[idx] : 0u;
-      longlong2 db = make_longlong2(0, 0);
-      uint4 ls = make_uint4(0, 0, 0, 0), cs = make_uint4(0, 0, 0, 0);
+      typename SimBase::Start s;
+      s.nsucc = 0;
+      s.flags = kAllCons;
+      s.dur = 0;
+      s.succ_off = 0;
+      uint32_t pred_off = 0, npred = 0;
       int d = 0;
       tm_t f = 0;
       if (v) {
-        db = op_durbytes(this->g.ops, x);
-        ls = op_lists(this->g.ops, x);
-        cs = op_cons(this->g.ops, x);
         d = this->row[x];
         f = this->fbuf[x];
-      }
-      this->log_event(v, this->kc.make(f - (tm_t)this->dur_of(x, d, db.x), kAlloc, x), d);
-      bool localc = false;
-      if (v) {
-        const bool all = (cs.w & kAllCons) != 0;
-        const uint32_t* lst = all ? this->g.succ + ls.x : this->g.cons + cs.x;
-        const uint32_t nl = all ? ls.y : cs.y;
-        for (uint32_t w = 0; w < nl; ++w)
-          if (this->row[__ldg(lst + w)] == d) {
-            localc = true;
-            break;
-          }
-      }
-      drop_hold(v && !localc, x, f, d);
-      __syncwarp();
-      const uint32_t npx = ls.w;
-      const uint32_t maxp = __reduce_max_sync(kFullMask, npx);
-      for (uint32_t u = 0; u < maxp; ++u) {
-        bool rel = false;
-        uint32_t p = 0;
-        if (u < npx) {
-          const uint2 ps = __ldg(this->g.predsib + ls.z + u);
-          p = ps.x & kIdMask;
-          if (ps.x & kHoldBit) {
-            const uint32_t sb = ps.y;
-            if (sb == kSibNone) {
-              rel = true;
-            } else if (sb != kSibMany && (sb & kSibLater)) {
-              rel = this->row[sb & ~kSibLater] != d;  // the other consumer finishes later
-            } else if (sb != kSibMany) {
-              const tm_t fs = this->fin(sb);
-              rel = !(this->row[sb] == d && !(fs > 0 && fs < f));
-            } else {
-              const XqSucc px = op_xqsucc(this->g.ops, p);
-              const uint4 pcs = op_cons(this->g.ops, p);
-              const bool all = (pcs.w & kAllCons) != 0;
-              const uint32_t* lst = all ? this->g.succ + px.succ_off : this->g.cons + pcs.x;
-              const uint32_t nl = all ? px.nsucc : pcs.y;
-              rel = true;
-              for (uint32_t w = 0; w < nl; ++w) {
-                const uint32_t c = __ldg(lst + w);
-                const tm_t fc = c != x ? this->fin(c) : 0;
-                if (c != x && this->row[c] == d && !(fc > 0 && fc < f)) {
-                  rel = false;
-                  break;
-                }
-              }
-            }
-          }
+        if constexpr (SimBase::kCompact) {
+          const uint4 h = this->hot(x);
+          s.dur = (tm_t)h.x;
+          s.flags = h.y >> 29;
+          s.succ_off = h.z & 0xffffffu;
+          s.nsucc = h.z >> 24;
+          pred_off = h.w & 0xffffffu;
+          npred = h.w >> 24;
+        } else {
+          s = this->start_of(x, d);
+          const RelPred rp = op_relpred(this->g.ops, x);
+          pred_off = rp.pred_off;
+          npred = rp.npred;
         }
-        const bool own = rel && this->row[p] == d;
-        this->log_event(rel && !own, this->kc.make(f, kFree, p), d);
-        drop_hold(own, p, f, d);
+      }
+      bool localc = false;
+      uint2 ps[2] = {make_uint2(0u, 0u), make_uint2(0u, 0u)};
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        if ((uint32_t)u < npred) ps[u] = __ldg(this->g.predsib + pred_off + u);
+        if ((uint32_t)u < s.nsucc) localc = localc || this->row[this->succ_at(s.succ_off + u)] == d;
+      }
+      if (!(s.flags & kAllCons)) {
+        localc = this->consumer_on(op_cons(this->g.ops, x), d);
+      } else {
+        for (uint32_t u = 2; u < s.nsucc && !localc; ++u) localc = this->row[this->succ_at(s.succ_off + u)] == d;
+      }
+      uint64_t ev[4];
+      int dev[4] = {d, d, d, d};
+      uint32_t want = v ? 1u : 0u;
+      ev[0] = this->entry(f - s.dur, kAlloc, x, d);
+      tm_t h = f;
+      if (v && !localc && drop_hold(x, f, h)) want |= 2u;
+      ev[1] = this->entry(h, kFree, x, d);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint32_t p = ps[u].x & kIdMask;
+        tm_t t = f;
+        if (this->releases(x, d, f, ps[u]) && (this->row[p] != d || drop_hold(p, f, t))) want |= 4u << u;
+        ev[2 + u] = this->entry(t, kFree, p, d);
+      }
+      this->template log_lanes<4>(ev, dev, want);
+      if (__any_sync(kFullMask, npred > 2u)) {
+        const uint32_t maxp = __reduce_max_sync(kFullMask, npred);
+        for (uint32_t u = 2; u < maxp; ++u) {
+          bool rel = false;
+          tm_t t = f;
+          uint32_t p = 0;
+          if (u < npred) {
+            const uint2 e = __ldg(this->g.predsib + pred_off + u);
+            p = e.x & kIdMask;
+            rel = this->releases(x, d, f, e) && (this->row[p] != d || drop_hold(p, f, t));
+          }
+          this->log_event(rel, this->kc.make(t, kFree, p), d);
+        }
       }
     }
     this->opn = 0;
     __syncwarp();
   }
 
+  // Transfers that arrived since the last generation wait in a list (dlog: the
+  // producer and the destination; dtime; drained before it has no room for 32 more),
+  // so that what they end is looked up for
+  // all of them at once, one per lane: one hold on the sender's copy; the receive
+  // copy is released on arrival if no listed consumer is there.
+  uint32_t* dlog;  // shared [kArrivals]
+  tm_t* dtime;     // shared [kArrivals]
+  int dn;
+  template <int kDevBits>
+  __device__ __forceinline__ void log_arrival(uint32_t p, int e, tm_t t) {
+    if (lane_id() == 0) {
+      dlog[dn] = (p << kDevBits) | (uint32_t)e;
+      dtime[dn] = t;
+    }
+    ++dn;
+  }
+  template <int kDevBits>
+  __device__ __forceinline__ void arrivals() {
+    const unsigned lane = lane_id();
+    __syncwarp();
+    for (int c0 = 0; c0 < dn; c0 += 32) {
+      const int idx = c0 + (int)lane;
+      const bool v = idx < dn;
+      const uint32_t x = v ? dlog[idx] : 0u;
+      const uint32_t p = x >> kDevBits;
+      const int e = (int)(x & ((1u << kDevBits) - 1u));
+      const tm_t t = v ? dtime[idx] : 0;
+      const uint4 cs = v ? op_cons(this->g.ops, p) : make_uint4(0u, 0u, 0u, kAllCons);
+      const int dp = v ? this->row[p] : 0;
+      uint32_t want = v && !(cs.w & kAllCons) && !this->consumer_on(cs, e) ? 1u : 0u;
+      // transfers of one producer one after the other
+      const uint32_t grp = __match_any_sync(kFullMask, v ? p : ~lane);
+      const int ord = __popc(grp & lanes_below());
+      const int last = (int)__reduce_max_sync(kFullMask, (unsigned)ord);
+      tm_t h = 0;
+      for (int r = 0; r <= last; ++r) {
+        if (v && ord == r && drop_hold(p, t, h)) want |= 2u;
+        __syncwarp();
+      }
+      const uint64_t ev[2] = {this->entry(t, kFree, p, e), this->entry(h, kFree, p, dp)};
+      const int dev[2] = {e, dp};
+      this->template log_lanes<2>(ev, dev, want);
+    }
+    dn = 0;
+    __syncwarp();
+  }
+
+  template <int kDevBits>
   __device__ __forceinline__ void drain(int64_t t_next) {
     generate();
+    arrivals<kDevBits>();
     this->drain_log(t_next);
   }
 };

@@ -81,8 +81,7 @@ struct DevGmg {
   const uint2* predsib;       // per predecessor entry: {pred | hold bit, the other listed
                               // consumer of that predecessor (kSibNone / kSibMany)}
   const uint32_t* cons;
-  const uint64_t* root_keys;  // READY keys of ops without predecessors, ascending
-  const uint64_t* root_keys_q;// the same as keys of the READY pool (time, op, least duration)
+  const uint64_t* root_keys;  // READY keys of ops without predecessors (time, op, least duration), ascending
   const int64_t* bytes;       // [N] output sizes (the op records' field, for the HBM events)
   const int64_t* cap;
   const int64_t* base;
@@ -148,6 +147,10 @@ constexpr int kMaxQB = 16;
 // Packed event key: time << (ib + 2) | class << ib | op.  Classes at equal
 // times: READY (an op's last input arrived) < FREE < ALLOC.
 constexpr uint32_t kReady = 0, kFree = 1, kAlloc = 2;
+
+// Completed transfers that an arbitrated simulation keeps for its next
+// event generation.
+constexpr int kArbArrivals = 64;
 
 // Candidate simulation modes.
 enum Mode : int { kFull = 0, kInc = 1, kBase = 2 };

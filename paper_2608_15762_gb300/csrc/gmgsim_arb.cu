@@ -56,208 +56,139 @@ namespace {
 
 // kMode: kFull (sim_batch), kBase (the arbitrated base snapshot: records
 // ready and finish times and checkpoints), kInc (candidates resumed from it).
-template <bool kT32, bool kTypes, int kMode = kFull>
-struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT32, kTypes, false>> {
-  using Base = ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT32, kTypes, false>>;
+template <bool kT32, bool kTypes, int kMode = kFull, int kHot = kHotNone>
+struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode, kHot>, Sim<true, kMode, true, kT32, kTypes, kHot>> {
+  using Base = ArbEvents<ArbSim<kT32, kTypes, kMode, kHot>, Sim<true, kMode, true, kT32, kTypes, kHot>>;
   using tm_t = typename Base::tm_t;
-  using U = typename std::make_unsigned<tm_t>::type;
+  using Reached = typename Base::Reached;
+  using Outside = typename Base::Outside;
+  using Batch = typename Base::Batch;
   using Base::g;
   using Base::P;
+  using Base::pd;
   using Base::row;
   using Base::status;
   using Base::add_input;
-  using Base::drain;
-  using Base::drop_hold;
+  using Base::arrivals;
   using Base::generate;
-  using Base::push_readies;
   using Base::kNever;
+  using Base::place;
   using Base::sl;
   using Base::warp_min_t;
+  static constexpr int kDevBits = 5;
   const ArbParams& A;
-  // The warp's scratch slot and shared area; the arrays in them are found
-  // from the launch parameters' offsets when used (registers are scarce).
-  uint8_t* sm;       // [0, 128): busy links (32 words); then the queue heads if shared
-  int32_t nx;        // intents arrived so far
-  int32_t xev;       // transfer events handled (loop guard)
-  uint32_t sendm, recvm;  // accelerators whose sending / receiving endpoint is busy
-  // lane a: accelerator a's transfer state
-  uint32_t pm;       // destinations with a pending intent from a
-  tm_t xd;           // completion of the transfer a is sending (kNever: none)
-  uint32_t xdp;      // its producer
-  int xde;           // its destination
-  int32_t fh, ft;    // FIFO of started ops with remote successors (-1: empty)
-  tm_t fa;           // finish time of the FIFO head (kNever: empty)
-  bool arb_due;
-  tm_t t_arb;
-  tm_t td_c;         // next DONE time (warp minimum of xd), kept current
-  uint64_t ik_c;     // next INTENT key (time << ib | op), kept current
+  // The warp's shared area: busy links (32 words), then the arrivals waiting for
+  // the next generation (gmg_arb_events.h).
+  uint8_t* sm;
+  int32_t xev;     // transfer events handled (loop guard)
+  uint32_t recvm;  // accelerators whose receiving endpoint is busy
+  // lane a: accelerator a's side of the transfers
+  tm_t xd;         // completion of the transfer a is sending (kNever: none)
+  uint32_t xdp;    // its producer << 5 | its destination
+  // a's started ops with remote successors that are not all on their way yet, in
+  // finish order (linked through nextop): those whose intents have arrived from
+  // ah to al, the coming ones from uh to lt (-1: none; lt is the last of both)
+  int32_t ah, uh;
+  tm_t fu;         // finish time of uh (kNever: none)
+  // (al, lt, the destinations left of ah and its finish time, used on changes
+  // only, are the lane's words in the shared area: registers are scarce)
+  __device__ __forceinline__ int32_t& al() const { return reinterpret_cast<int32_t*>(sm + 128)[lane_id()]; }
+  __device__ __forceinline__ int32_t& lt() const { return reinterpret_cast<int32_t*>(sm + 256)[lane_id()]; }
+  __device__ __forceinline__ uint32_t& hm() const { return reinterpret_cast<uint32_t*>(sm + 384)[lane_id()]; }
+  __device__ __forceinline__ tm_t& hf() const { return reinterpret_cast<tm_t*>(sm + 512)[lane_id()]; }
 
   __device__ ArbSim(const ArbParams& a) : Base(a.P), A(a) {}
 
   template <typename T>
   __device__ __forceinline__ T* at(int64_t off) const { return reinterpret_cast<T*>(sl + off); }
-  __device__ __forceinline__ int32_t* cnt() const { return at<int32_t>(A.off_cnt); }      // [N] inputs present
+  __device__ __forceinline__ int32_t* cnt() const { return at<int32_t>(A.off_cnt); }      // [N] inputs present (joins)
   __device__ __forceinline__ tm_t* rmax() const { return at<tm_t>(A.off_rmax); }          // [N] latest arrival
   __device__ __forceinline__ int32_t* refs() const { return at<int32_t>(A.off_refs); }    // [N] holds left
-  __device__ __forceinline__ uint32_t* rmask() const { return at<uint32_t>(A.off_rmask); }  // [N] remote accs
-  __device__ __forceinline__ int32_t* nextop() const { return at<int32_t>(A.off_nextop); }  // [N] FIFO link
-  __device__ __forceinline__ uint32_t* xent() const { return at<uint32_t>(A.off_xent); }  // [xcap] p << 5 | e
-  __device__ __forceinline__ int32_t* xnext() const { return at<int32_t>(A.off_xnext); }  // [xcap]
-  __device__ __forceinline__ int32_t* qtail() const { return at<int32_t>(A.off_qtail); }  // [D*D]
-  __device__ __forceinline__ int32_t* qhead() const {                                      // [D*D]
-    return A.heads_shared ? reinterpret_cast<int32_t*>(sm + 128) : at<int32_t>(A.off_qhead);
-  }
+  __device__ __forceinline__ uint32_t* rmask() const { return at<uint32_t>(A.off_rmask); }  // [N] destinations left
+  __device__ __forceinline__ int32_t* nextop() const { return at<int32_t>(A.off_nextop); }  // [N] list link
   __device__ __forceinline__ uint32_t* lbits() const { return reinterpret_cast<uint32_t*>(sm); }
-
-  __device__ __forceinline__ void refresh_done() { td_c = warp_min_t(xd); }
-  __device__ __forceinline__ void refresh_intent() {
-    ik_c = warp_min_u64(fh >= 0 ? (((uint64_t)(U)fa << g.ib) | (uint32_t)fh) : kKeyMax);
-  }
 
   __device__ void setup_arb(uint8_t* smem_warp) {
     sm = smem_warp;
+    this->dtime = reinterpret_cast<tm_t*>(sm + 768);
+    this->dlog = reinterpret_cast<uint32_t*>(sm + 768 + 8 * kArrivals);
   }
 
   __device__ void reset_arb() {
     const unsigned lane = lane_id();
     this->reset_common();
-    this->rk_reg = kKeyMax;
     uint4* c4 = reinterpret_cast<uint4*>(cnt());
-    int32_t* qh = qhead();
-    int32_t* qt = qtail();
     const int nv = (int)((4 * (size_t)g.n + 15) / 16);
     for (int x = lane; x < nv; x += 32) c4[x] = make_uint4(0u, 0u, 0u, 0u);
-    for (int x = lane; x < g.D * g.D; x += 32) {
-      qh[x] = -1;
-      qt[x] = -1;
-    }
     lbits()[lane] = 0u;
-    nx = 0;
+    this->dn = 0;
     xev = 0;
-    sendm = recvm = pm = 0u;
+    recvm = 0u;
     xd = kNever;
     xdp = 0u;
-    xde = 0;
-    fh = ft = -1;
-    fa = kNever;
-    arb_due = false;
-    t_arb = 0;
-    td_c = kNever;
-    ik_c = kKeyMax;
+    ah = uh = -1;
+    al() = lt() = -1;
+    fu = kNever;
     __syncwarp();
   }
 
-  // READY(r, i): start op i; local successors get this input; if some
-  // successor is remote, i joins its accelerator's FIFO of coming intents.
-  __device__ void start_op(uint32_t i, tm_t r) {
-    const unsigned lane = lane_id();
-    const longlong2 db = op_durbytes(g.ops, i);
-    const XqSucc xs = op_xqsucc(g.ops, i);
-    const uint4 cs = op_cons(g.ops, i);
-    const int d = row[i];
-    const tm_t dur = (tm_t)this->dur_of(i, d, db.x);
-    const tm_t fd = this->dv.get_free(d);
-    const tm_t s = r > fd ? r : fd;
-    const tm_t f = s + dur;
-    this->dv.set_free(d, f);
-    if (lane == 0) {
-      this->fbuf[i] = f;
-      if (cs.w & kReqSink)
-        atomicMax(reinterpret_cast<unsigned long long*>(this->creq() + (int32_t)cs.z), (unsigned long long)f);
-      if (kMode == kBase) P.base.rb[i] = r;
-      this->oplog[this->opn] = i;
+  // Lane a: op p, ending at f, joins the end of a's list.
+  __device__ __forceinline__ void append(uint32_t p, tm_t f) {
+    if (lt() >= 0) nextop()[lt()] = (int32_t)p;
+    if (uh < 0) {
+      uh = (int32_t)p;
+      fu = f;
     }
-    ++this->opn;
-    if (cs.w & kScored) this->score += (int64_t)f;
-    if (kMode == kBase) ++this->readypops;
-    if (kMode == kInc && r >= this->T0) ++this->nev;
-    __syncwarp();
+    lt() = (int32_t)p;
+  }
+
+  // READY ops: start them; local successors get this input; an op with remote
+  // successors joins its accelerator's list.
+  __device__ __forceinline__ void start_ops(Batch& B, Outside& o) {
+    const unsigned lane = lane_id();
     uint32_t remote = 0u;
-    for (uint32_t c0 = 0; c0 < xs.nsucc; c0 += 32) {
-      const uint32_t t = c0 + lane;
-      uint32_t j = 0;
-      tm_t rj = 0;
-      bool rdy = false;
-      if (t < xs.nsucc) {
-        j = __ldg(g.succ + xs.succ_off + t);
-        const int dj = row[j];
-        if (dj == d) rdy = add_input(j, f, rj);
-        else remote |= 1u << dj;
+    // ops of one accelerator (which may feed one local successor) in turn
+    for (int t = 0; t <= B.last; ++t) {
+      const uint32_t ns = B.ord == t ? B.s.nsucc : 0u;
+      for (uint32_t u = 0; __any_sync(kFullMask, u < ns); ++u) {
+        Reached x;
+        x.rdy = x.join = false;
+        x.j = 0;
+        x.d = 0;
+        x.r = x.dur = 0;
+        if (u < ns) {
+          const uint32_t j = this->succ_at(B.s.succ_off + u);
+          const int dj = row[j];
+          if (dj == B.d) x = add_input(j, dj, B.f);
+          else remote |= 1u << dj;
+        }
+        place(x, o);
       }
-      push_readies(rdy, rj, j);
+      __syncwarp();
     }
-    remote = __reduce_or_sync(kFullMask, remote);
-    if (lane == 0) {
-      refs()[i] = 1 + __popc(remote);
-      this->holdb()[i] = f;
-      if (remote) rmask()[i] = remote;
+    if (B.v) {
+      refs()[B.i] = 1 + __popc(remote);
+      this->holdb()[B.i] = B.f;
+      if (remote) rmask()[B.i] = remote;
     }
-    if (remote && (int)lane == d) {
-      if (fh < 0) {
-        fh = (int32_t)i;
-        fa = f;
-      } else {
-        nextop()[ft] = (int32_t)i;
+    const uint32_t rem = __ballot_sync(kFullMask, B.v && remote);
+    for (int t = 0; t <= B.last; ++t)
+      for (uint32_t m = B.last ? __ballot_sync(kFullMask, ((rem >> lane) & 1u) && B.ord == t) : rem; m; m &= m - 1u) {
+        const int src = __ffs(m) - 1;
+        const uint32_t p = __shfl_sync(kFullMask, B.i, src);
+        const tm_t f = __shfl_sync(kFullMask, B.f, src);
+        if ((int)lane == __shfl_sync(kFullMask, B.d, src)) append(p, f);
       }
-      ft = (int32_t)i;
-    }
     __syncwarp();
-    if (remote) refresh_intent();
-  }
-
-  // The intents of the earliest FIFO head arrive: one per remote
-  // accelerator, numbered in destination order.
-  __device__ void intents_arrive(uint32_t p) {
-    const unsigned lane = lane_id();
-    const int a = row[p];
-    const uint32_t R = rmask()[p];
-    if (nx + __popc(R) > A.xcap) {
-      status = GMG_SIM_QUEUE;
-      return;
-    }
-    if (lane == 0) {
-      uint32_t* xe = xent();
-      int32_t* xn = xnext();
-      int32_t* qh = qhead();
-      int32_t* qt = qtail();
-      uint32_t r = R;
-      while (r) {
-        const int e = __ffs(r) - 1;
-        r &= r - 1;
-        const int32_t x = nx++;
-        const int pair = a * g.D + e;
-        xe[x] = (p << 5) | (uint32_t)e;
-        xn[x] = -1;
-        const int32_t tl = qt[pair];
-        if (tl >= 0) xn[tl] = x;
-        else qh[pair] = x;
-        qt[pair] = x;
-      }
-    } else {
-      nx += __popc(R);
-    }
-    if ((int)lane == a) {
-      pm |= R;
-      if (fh == ft) {
-        fh = ft = -1;
-        fa = kNever;
-      } else {
-        fh = nextop()[fh];
-        fa = this->fin((uint32_t)fh);
-      }
-    }
-    __syncwarp();
-    refresh_intent();
   }
 
   // The transfer sent by lane src completes at time t.
-  __device__ void transfer_done(int src, tm_t t) {
+  __device__ __forceinline__ void transfer_done(int src, tm_t t, Outside& o) {
     const unsigned lane = lane_id();
-    const uint32_t p = __shfl_sync(kFullMask, xdp, src);
-    const int e = __shfl_sync(kFullMask, xde, src);
+    const uint32_t pe = __shfl_sync(kFullMask, xdp, src);
+    const uint32_t p = pe >> kDevBits;
+    const int e = (int)(pe & 31u);
     if ((int)lane == src) xd = kNever;
-    refresh_done();
-    sendm &= ~(1u << src);
     recvm &= ~(1u << e);
     if (A.shared_links) {
       const uint32_t lid = __ldg(A.link + src * g.D + e);
@@ -265,163 +196,201 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
       __syncwarp();
     }
     // p's successors on e have this input now
-    const XqSucc xs = op_xqsucc(g.ops, p);
-    for (uint32_t c0 = 0; c0 < xs.nsucc; c0 += 32) {
+    uint32_t off, ns;
+    if constexpr (kHot != kHotNone) {
+      const uint4 h = this->hot(p);
+      off = h.z & 0xffffffu;
+      ns = h.z >> 24;
+    } else {
+      const XqSucc xs = op_xqsucc(g.ops, p);
+      off = xs.succ_off;
+      ns = xs.nsucc;
+    }
+    for (uint32_t c0 = 0; c0 < ns; c0 += 32) {
       const uint32_t u = c0 + lane;
-      uint32_t j = 0;
-      tm_t rj = 0;
-      bool rdy = false;
-      if (u < xs.nsucc) {
-        j = __ldg(g.succ + xs.succ_off + u);
-        if (row[j] == e) rdy = add_input(j, t, rj);
+      Reached x;
+      x.rdy = x.join = false;
+      x.j = 0;
+      x.d = 0;
+      x.r = x.dur = 0;
+      if (u < ns) {
+        const uint32_t j = this->succ_at(off + u);
+        if (row[j] == e) x = add_input(j, e, t);
       }
-      push_readies(rdy, rj, j);
+      place(x, o);
     }
     __syncwarp();
-    // the receive copy: released on arrival if no listed consumer is on e
-    const uint4 cs = op_cons(g.ops, p);
-    bool here = (cs.w & kAllCons) != 0;  // the successors there are consumers
-    if (!here) {
-      bool f = false;
-      for (uint32_t u = lane; u < cs.y; u += 32) f |= row[__ldg(g.cons + cs.x + u)] == e;
-      here = __any_sync(kFullMask, f);
-    }
-    this->log_event(lane == 0 && !here, this->kc.make(t, kFree, p), e);
-    // the sender's copy: one hold fewer
-    drop_hold(lane == 0, p, t, src);
+    this->template log_arrival<kDevBits>(p, e, t);
   }
 
-  // Start every pending intent whose endpoints and link are free, in order.
-  __device__ void arbitrate(tm_t t) {
+  // Start every pending intent whose endpoints and link are free, in (intent
+  // time, producer, destination) order: each free accelerator offers the first
+  // destination that it can send to of the first op in its list that has one, and
+  // a warp minimum over (finish time, op) picks the next to start.  An offer
+  // stands until its destination (or, with shared links, anything) is taken.
+  __device__ __forceinline__ void arbitrate(tm_t t) {
     const int lane = (int)lane_id();
     const int D = g.D;
     const bool links = A.shared_links != 0;
-    bool started = false;
+    int32_t cp = -1, prev = -1;  // the op offered, the one before it in the list
+    uint32_t cm = 0u;            // its destinations left
+    tm_t cf = kNever;
+    int ce = 0;
+    bool scan = xd == kNever && ah >= 0;
     while (true) {
-      uint32_t best = 0xffffffffu;
-      int be = 0;
-      if (lane < D && !((sendm >> lane) & 1u)) {
-        uint32_t c = pm & ~recvm;
-        while (c) {
-          const int e = __ffs(c) - 1;
-          c &= c - 1;
+      if (scan) {
+        cp = ah;
+        cm = hm();
+        cf = hf();
+        prev = -1;
+        for (int32_t guard = 0;; ++guard) {
+          uint32_t c = cm & ~recvm;
           if (links) {
-            const uint32_t lid = __ldg(A.link + lane * D + e);
-            if ((lbits()[lid >> 5] >> (lid & 31u)) & 1u) continue;
+            uint32_t ok = 0u;
+            while (c) {
+              const int e = __ffs(c) - 1;
+              c &= c - 1u;
+              const uint32_t lid = __ldg(A.link + lane * D + e);
+              if (!((lbits()[lid >> 5] >> (lid & 31u)) & 1u)) {
+                ok = 1u << e;
+                break;
+              }
+            }
+            c = ok;
           }
-          const uint32_t h = (uint32_t)qhead()[lane * D + e];
-          if (h < best) {
-            best = h;
-            be = e;
+          if (c) {
+            ce = __ffs(c) - 1;
+            break;
           }
+          if (cp == al() || guard > g.n) {
+            cp = -1;
+            break;
+          }
+          prev = cp;
+          cp = nextop()[cp];
+          cm = rmask()[cp];
+          cf = this->fin((uint32_t)cp);
         }
       }
-      const uint32_t m = __reduce_min_sync(kFullMask, best);
-      if (m == 0xffffffffu) break;
-      started = true;
-      const int src = __ffs(__ballot_sync(kFullMask, best == m)) - 1;
-      const int e = __shfl_sync(kFullMask, be, src);
-      const uint32_t p = xent()[m] >> 5;
-      const int32_t nxt = xnext()[m];
-      const int pair = src * D + e;
-      __syncwarp();
-      if (lane == 0) {
-        qhead()[pair] = nxt;
-        if (nxt < 0) qtail()[pair] = -1;
-        if (links) {
-          const uint32_t lid = __ldg(A.link + pair);
-          lbits()[lid >> 5] |= 1u << (lid & 31u);
-        }
-      }
-      if (nxt < 0 && lane == src) pm &= ~(1u << e);
-      sendm |= 1u << src;
+      const uint64_t key = cp >= 0 ? ((uint64_t)cf << g.ib) | (uint32_t)cp : kKeyMax;
+      const uint64_t best = warp_min_u64(key);
+      if (best == kKeyMax) break;
+      const int src = __ffs(__ballot_sync(kFullMask, key == best)) - 1;
+      const int e = __shfl_sync(kFullMask, ce, src);
+      const uint32_t p = (uint32_t)best & g.opmask;
+      const tm_t done = t + this->sends(p, src, e);
       recvm |= 1u << e;
-      const tm_t done = t + this->xfer(src, e, op_durbytes(g.ops, p).y, op_xqsucc(g.ops, p).xq);
+      if (links) {
+        const uint32_t lid = __ldg(A.link + src * D + e);
+        if (lane == 0) lbits()[lid >> 5] |= 1u << (lid & 31u);
+        __syncwarp();
+      }
       if (lane == src) {
         xd = done;
-        xdp = p;
-        xde = e;
+        xdp = (p << kDevBits) | (uint32_t)e;
+        const uint32_t left = cm & ~(1u << e);
+        if (left) {
+          rmask()[p] = left;
+          if (cp == ah) hm() = left;
+        } else {  // leaves the list
+          const bool tail = cp == lt();
+          const int32_t nx = tail ? -1 : nextop()[cp];
+          if (cp == ah) {
+            ah = cp == al() ? -1 : nx;
+            if (ah >= 0) {
+              hm() = rmask()[ah];
+              hf() = this->fin((uint32_t)ah);
+            } else {
+              al() = -1;
+            }
+          } else {
+            if (!tail) nextop()[prev] = nx;
+            if (cp == al()) al() = prev;
+          }
+          if (tail) lt() = prev;
+        }
       }
+      scan = cp >= 0 && lane != src && (links || ce == e);
+      if (lane == src) cp = -1;
       __syncwarp();
       this->log_event(lane == 0, this->kc.make(t, kAlloc, p), e);
     }
-    if (started) refresh_done();
   }
 
-  // The event loop: transfer events, then the arbiter once the last event of
-  // a time is handled, then READY keys.
+  // The event loop: transfer events at a time (completions, then new intents,
+  // then the arbiter), then the READY ops before the next one that the others
+  // cannot delay.
   __device__ void run() {
     if (status) return;
+    const unsigned lane = lane_id();
     const int32_t xlim = A.xcap + g.n + 2;
+    Outside o;
+    this->look_outside(o);
     while (true) {
-      const tm_t td = td_c;
-      const uint64_t ik = ik_c;
-      const tm_t ti = ik == kKeyMax ? kNever : (tm_t)(ik >> g.ib);
+      const tm_t td = warp_min_t(xd), ti = warp_min_t(fu);
       const tm_t tx = td < ti ? td : ti;
-      if (arb_due && tx > t_arb) {
-        arbitrate(t_arb);
-        arb_due = false;
-        if (status) break;
-        continue;
+      tm_t lim = warp_min_t(pd.e);
+      const bool end = lim == kNever && o.r == kNever && tx == kNever;
+      // (at most 32 transfers complete at one time)
+      if (end || this->opn >= P.drain_trigger || this->dn > kArrivals - 32) {  // the only copy of this code
+        const tm_t r = warp_min_t(pd.r);
+        tm_t tn = r < o.r ? r : o.r;
+        tn = tx < tn ? tx : tn;
+        this->template drain<kDevBits>(end ? kI64Max : (int64_t)tn);
+        if (end || status) break;
       }
-      const uint64_t top = this->q.top();
-      const uint64_t rm = warp_min_u64(this->rk_reg);
-      const uint64_t rk = this->rkey;
-      uint64_t nk = rk < top ? rk : top;
-      nk = rm < nk ? rm : nk;
-      if (tx != kNever && (nk == kKeyMax || (int64_t)tx <= this->kc.time(nk))) {
-        if (++xev > xlim) {
+      lim = lim < tx ? lim : tx;
+      const bool act = this->starts(lim, tx, o);
+      if (__any_sync(kFullMask, act)) {
+        if (kMode == kBase && this->readypops >= this->next_ck) arb_checkpoint(o);
+        Batch B;
+        if (!this->start_held(act, B)) break;
+        start_ops(B, o);
+      } else {
+        uint32_t dm = __ballot_sync(kFullMask, xd == tx);
+        const bool arrives = fu == tx;
+        const int events = __popc(dm) + __popc(__ballot_sync(kFullMask, arrives));
+        xev += events;
+        if (xev > xlim || events == 0) {
           status = GMG_SIM_LOOP;
           break;
         }
-        if (td == tx) transfer_done(__ffs(__ballot_sync(kFullMask, xd == td)) - 1, td);
-        else intents_arrive((uint32_t)(ik & g.opmask));
+        for (; dm; dm &= dm - 1u) transfer_done(__ffs(dm) - 1, tx, o);
+        if (arrives) {
+          if (ah < 0) {
+            ah = uh;
+            hm() = rmask()[uh];
+            hf() = tx;
+          }
+          al() = uh;
+          uh = uh == lt() ? -1 : nextop()[uh];
+          fu = uh < 0 ? kNever : this->fin((uint32_t)uh);
+        }
+        arbitrate(tx);
         if (kMode == kBase) this->last_t = tx;
-        arb_due = true;
-        t_arb = tx;
-        if (status) break;
-        continue;
       }
-      if (kMode == kBase && nk != kKeyMax) arb_checkpoint(nk);
-      if (nk == kKeyMax || this->opn >= P.opcap) {  // the only copy of this code: it is large
-        drain(nk == kKeyMax ? kI64Max : this->kc.time(nk));
-        if (nk == kKeyMax || status) break;
-      }
-      if (nk == rm) {
-        if (this->rk_reg == rm) this->rk_reg = kKeyMax;
-      } else if (nk == rk) {
-        ++this->rootptr;
-        this->load_root();
-      } else {
-        __syncwarp();
-        this->q.pop();
-      }
-      if (++this->iters > (int32_t)g.max_iter) {
-        status = GMG_SIM_LOOP;
-        break;
-      }
-      if (kMode == kBase) this->last_t = (tm_t)this->kc.time(nk);
-      start_op(this->kc.op(nk), (tm_t)this->kc.time(nk));
       if (status) break;
     }
   }
 
   // -------------------------------------------------------------------------
-  // Arbitrated base snapshot.  A checkpoint is taken right before a READY key
-  // whose time T_c is past every event handled so far: every transfer event
-  // and arbitration before T_c is done (transfer events at a time come before
-  // READY keys at that time, and the arbiter runs before the next later
-  // event), nothing at T_c or later is.  The simulation part is the base
-  // snapshot's (Sim::maybe_checkpoint, after this simulator's own event
-  // generation); the arbiter's part goes to the checkpoint's arena.
+  // Arbitrated base snapshot.  A checkpoint is taken right before READY ops
+  // whose smallest time T_c is past every event handled so far: every transfer
+  // event and arbitration before T_c is done (transfer events at a time come
+  // before READY ops at that time), nothing at T_c or later is.  The simulation
+  // part is the base snapshot's (Sim::maybe_checkpoint, after this simulator's
+  // own event generation); the arbiter's part goes to the checkpoint's arena.
   // -------------------------------------------------------------------------
-  __device__ void arb_checkpoint(uint64_t next_key) {
+  __device__ void arb_checkpoint(const Outside& o) {
     const DevBase& B = P.base;
     if (this->ck >= B.nck || this->readypops < this->next_ck) return;
-    if (this->kc.time(next_key) <= (int64_t)this->last_t) return;
+    const tm_t r = warp_min_t(pd.r);
+    const tm_t tn = r < o.r ? r : o.r;
+    if (tn <= this->last_t) return;
     generate();  // the simulation checkpoint then finds no started op left to generate
+    this->template arrivals<kDevBits>();
     const int c = this->ck;
-    this->maybe_checkpoint(this->kc.time(next_key), this->rk_reg);
+    this->maybe_checkpoint((int64_t)tn, this->held_key());
     if (this->ck > c && B.ck_time[c] != kI64Max) save_arb(c);
   }
 
@@ -442,28 +411,20 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     warp_copy16<16>(a + K.off_rmask, rmask(), 4 * n);
     warp_copy16<16>(a + K.off_nextop, nextop(), 4 * n);
     warp_copy16<16>(a + K.off_hold, this->holdb(), 8 * n);
-    warp_copy16<16>(a + K.off_xent, xent(), 4 * (int64_t)nx);
-    warp_copy16<16>(a + K.off_xnext, xnext(), 4 * (int64_t)nx);
-    for (int x = lane; x < g.D * g.D; x += 32) {
-      reinterpret_cast<int32_t*>(a + K.off_qhead)[x] = qhead()[x];
-      reinterpret_cast<int32_t*>(a + K.off_qtail)[x] = qtail()[x];
-    }
     int64_t* ls = reinterpret_cast<int64_t*>(a + K.off_lanes) + 7 * lane;
-    ls[0] = pm;
-    ls[1] = (int64_t)xd;
-    ls[2] = xdp;
-    ls[3] = xde;
-    ls[4] = fh;
-    ls[5] = ft;
-    ls[6] = (int64_t)fa;
+    ls[0] = (int64_t)xd;
+    ls[1] = xdp;
+    ls[2] = ah;
+    ls[3] = al();
+    ls[4] = uh;
+    ls[5] = lt();
+    ls[6] = (int64_t)fu;
     int64_t* w = reinterpret_cast<int64_t*>(a + K.off_warp);
     if (lane == 0) {
-      w[0] = nx;
-      w[1] = xev;
-      w[2] = sendm;
-      w[3] = recvm;
+      w[0] = xev;
+      w[1] = recvm;
     }
-    reinterpret_cast<uint32_t*>(w + 4)[lane] = lbits()[lane];
+    reinterpret_cast<uint32_t*>(w + 2)[lane] = lbits()[lane];
     __syncwarp();
   }
 
@@ -504,28 +465,23 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
       warp_copy16(this->holdb(), a + K.off_hold, 8 * n);
     }
     const int64_t* w = reinterpret_cast<const int64_t*>(a + K.off_warp);
-    nx = (int32_t)w[0];
-    xev = (int32_t)w[1];
-    sendm = (uint32_t)w[2];
-    recvm = (uint32_t)w[3];
-    lbits()[lane] = reinterpret_cast<const uint32_t*>(w + 4)[lane];
-    warp_copy16(xent(), a + K.off_xent, 4 * (int64_t)nx);
-    warp_copy16(xnext(), a + K.off_xnext, 4 * (int64_t)nx);
-    for (int x = lane; x < g.D * g.D; x += 32) {
-      qhead()[x] = reinterpret_cast<const int32_t*>(a + K.off_qhead)[x];
-      qtail()[x] = reinterpret_cast<const int32_t*>(a + K.off_qtail)[x];
-    }
+    xev = (int32_t)w[0];
+    recvm = (uint32_t)w[1];
+    lbits()[lane] = reinterpret_cast<const uint32_t*>(w + 2)[lane];
     const int64_t* ls = reinterpret_cast<const int64_t*>(a + K.off_lanes) + 7 * lane;
-    pm = (uint32_t)ls[0];
-    xd = narrow_time(ls[1]);
-    xdp = (uint32_t)ls[2];
-    xde = (int)ls[3];
-    fh = (int32_t)ls[4];
-    ft = (int32_t)ls[5];
-    fa = narrow_time(ls[6]);
-    arb_due = false;
-    t_arb = 0;
+    xd = narrow_time(ls[0]);
+    xdp = (uint32_t)ls[1];
+    ah = (int32_t)ls[2];
+    al() = (int32_t)ls[3];
+    uh = (int32_t)ls[4];
+    lt() = (int32_t)ls[5];
+    fu = narrow_time(ls[6]);
+    this->dn = 0;
     __syncwarp();
+    // an op whose intents have arrived finished before T0: the moves change
+    // nothing about it
+    hm() = ah >= 0 ? rmask()[ah] : 0u;
+    hf() = ah >= 0 ? this->fin((uint32_t)ah) : kNever;
   }
 
   // Remote accelerators of p's successors under placement rw (uniform).
@@ -553,18 +509,17 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     return __any_sync(kFullMask, f);
   }
 
-  // Op p (started before the resume point, finishing at or after it) in the
-  // FIFO of coming intents of its accelerator d, kept in finish order: insert
-  // (want) or remove.  The list runs from the head to the tail through
-  // nextop (the tail's link is not kept).  Uniform call; lane d owns the head
-  // and tail.
-  __device__ void fifo_set(uint32_t p, int d, bool want) {
+  // Op p (started before the resume point, finishing at or after it) among the
+  // coming ones of its accelerator d's list, kept in finish order: insert
+  // (want) or remove.  Uniform call; lane d owns the list's ends.
+  __device__ void list_set(uint32_t p, int d, bool want) {
     const unsigned lane = lane_id();
-    int32_t h = __shfl_sync(kFullMask, fh, d);
-    int32_t t = __shfl_sync(kFullMask, ft, d);
+    const int32_t a = __shfl_sync(kFullMask, al(), d);  // the link of the last arrived op leads to the first coming one
+    int32_t h = __shfl_sync(kFullMask, uh, d);
+    int32_t t = __shfl_sync(kFullMask, lt(), d);
     int32_t* nxp = nextop();
     const tm_t fp = this->fin(p);
-    int32_t prev = -1, cur = h;
+    int32_t prev = a, cur = h;
     bool found = false;
     for (int guard = 0; cur >= 0 && guard <= g.n; ++guard) {
       if (cur == (int32_t)p) {
@@ -576,24 +531,25 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
       cur = cur == t ? -1 : nxp[cur];
     }
     if (want == found) return;
+    const bool first = cur == h;  // (also with no coming op)
     if (want) {  // link p between prev and cur
       if (lane == 0) {
         nxp[p] = cur;
         if (prev >= 0) nxp[prev] = (int32_t)p;
       }
-      if (prev < 0) h = (int32_t)p;
+      if (first) h = (int32_t)p;
       if (cur < 0) t = (int32_t)p;
     } else {  // unlink p (cur == p)
       const int32_t after = (int32_t)p == t ? -1 : nxp[p];
       if (lane == 0 && prev >= 0) nxp[prev] = after;
-      if (prev < 0) h = after;
+      if (first) h = after;
       if (t == (int32_t)p) t = prev;
     }
     __syncwarp();
     if ((int)lane == d) {
-      fh = h;
-      ft = h < 0 ? -1 : t;
-      fa = h < 0 ? kNever : this->fin((uint32_t)h);
+      uh = h;
+      lt() = t;
+      fu = h < 0 ? kNever : this->fin((uint32_t)h);
     }
     __syncwarp();
   }
@@ -606,7 +562,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
   // remote one has finished) and its READY key; and for every predecessor p
   // of a moved op that started before T_c (it finishes at or after T0, so
   // none of its intents, transfers or receive buffers exist yet): its remote
-  // set, the holds on its copy, its place in its accelerator's FIFO of coming
+  // set, the holds on its copy, its place in its accelerator's list of coming
   // intents, and whether its copy's release is already logged.
   __device__ void inc_candidate(int64_t k, uint8_t* crow) {
     const DevBase& B = P.base;
@@ -687,7 +643,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     const int64_t* sc = B.ck_scalars + (int64_t)c * 8;
     const int qsz = (int)sc[0];
     const int msz = (int)sc[7];
-    if (qsz + nm > P.qcap || msz + nm > P.mcap) {
+    if (qsz + nm > P.pend_cap - 32 || msz + nm > P.mcap) {
       this->write_invalid(k, GMG_SIM_QUEUE);
       return;
     }
@@ -696,7 +652,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     this->drained = (tm_t)sc[3];
     this->rootptr = (int)sc[1];
     this->load_root();
-    this->score = sc[2];
+    this->score = lane == 0 ? sc[2] : 0;  // lanes add up their ops' finishes
     this->vflag = (int32_t)sc[4];
     this->vt = sc[5];
     this->vop = (int32_t)(sc[6] >> 32);
@@ -706,22 +662,28 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
     this->readypops = 0;
     this->last_t = -1;
     status = GMG_SIM_OK;
-    this->rk_reg = kKeyMax;
+    pd.r = pd.e = kNever;
     this->opn = 0;
     this->dv.load(B.ck_dev + (int64_t)c * 3 * g.D);
     for (int r = lane; r < g.R; r += 32) this->creq()[r] = B.ck_creq[(int64_t)c * g.R + r];
     this->fill_fin();
     restore_arb(c);
-    // READY keys, except those of moved ops (recomputed below)
+    // READY keys, except those of moved ops (recomputed below): the lanes' go
+    // through the sort area (free between drains), the others to the heap
+    auto queue = [&](int n, uint64_t key) {
+      if (n < 32) this->sortk[n] = key;
+      else *this->q.kp(n - 32) = key;
+    };
     int nq = 0;
     for (int c0 = 0; c0 < qsz; c0 += 32) {
       const int x = c0 + (int)lane;
       const bool v = x < qsz;
       const uint64_t key = v ? B.ck_qkey[(int64_t)c * B.ckq + x] : 0ull;
-      const uint32_t op = this->kc.op(key);
-      const bool keep = v && crow[op] == B.row[op];
+      const uint32_t op = this->rq.op(key);
+      // (a moved op without predecessors keeps its ready time)
+      const bool keep = v && (crow[op] == B.row[op] || op_relpred(g.ops, op).npred == 0u);
       const uint32_t bal = __ballot_sync(kFullMask, keep);
-      if (keep) *this->q.kp(nq + __popc(bal & lanes_below())) = key;
+      if (keep) queue(nq + __popc(bal & lanes_below()), key);
       nq += __popc(bal);
     }
     // logged HBM events, except the release of a moved op's predecessor's own
@@ -774,7 +736,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
       if (rp.npred > 0 && (uint32_t)cx == rp.npred) {
         const tm_t rel = (tm_t)rp.rel;
         const tm_t rj = rel > (tm_t)rx ? rel : (tm_t)rx;
-        if (lane == 0) *this->q.kp(nq) = this->kc.make(rj, kReady, x);
+        if (lane == 0) queue(nq, this->rq.make(rj, x, (tm_t)1));
         ++nq;
       }
       // started predecessors: remote set, holds, FIFO, own copy's release;
@@ -805,26 +767,29 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode>, Sim<true, kMode, true, kT
           this->holdb()[p] = fp;
         }
         __syncwarp();
-        fifo_set(p, dp, rc != 0u);
+        list_set(p, dp, rc != 0u);
         this->log_event(lane == 0 && holds == 0, this->kc.make(fp, kFree, p), dp);
       }
     }
-    this->q.size = nq;
+    __syncwarp();
+    if ((int)lane < nq && lane < 32u) {
+      const uint64_t key = this->sortk[lane];
+      this->hold_op((tm_t)this->rq.time(key), this->rq.op(key));
+    }
+    this->q.size = nq > 32 ? nq - 32 : 0;
     this->q.heapify();
-    refresh_done();
-    refresh_intent();
     run();
     this->finish(k);
   }
 };
 
-template <bool kT32, bool kTypes>
+template <bool kT32, bool kTypes, int kHot>
 __global__ void __launch_bounds__(128, 7) sim_arb_kernel(const __grid_constant__ ArbParams A) {
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
   const int64_t nslots = (int64_t)gridDim.x * (blockDim.x >> 5);
-  ArbSim<kT32, kTypes> S(A);
+  ArbSim<kT32, kTypes, kFull, kHot> S(A);
   setup_slot(S, A.P, wib, slot, smem);
   S.setup_arb(smem + A.smem_std + (size_t)wib * A.smem_arb);
   for (int64_t k = slot; k < A.P.K; k += nslots) {
@@ -849,7 +814,7 @@ __global__ void __launch_bounds__(128, 7) sim_arb_kernel(const __grid_constant__
 // The arbitrated base snapshot: the base placement simulated once (64-bit
 // times) with checkpoints of the simulation and the arbiter.
 template <bool kTypes>
-__global__ void __launch_bounds__(32) sim_arb_base_kernel(const __grid_constant__ ArbParams A) {
+__global__ void __launch_bounds__(32, 1) sim_arb_base_kernel(const __grid_constant__ ArbParams A) {
   extern __shared__ __align__(16) uint8_t smem[];
   ArbSim<false, kTypes, kBase> S(A);
   setup_slot(S, A.P, 0, 0, smem);
@@ -860,7 +825,6 @@ __global__ void __launch_bounds__(32) sim_arb_base_kernel(const __grid_constant_
   for (int c = lane * 16; c < B.ld; c += 512)
     *reinterpret_cast<uint4*>(B.row + c) = *reinterpret_cast<const uint4*>(A.P.place + c);
   for (int c = lane; c < B.nck; c += 32) B.ck_time[c] = kI64Max;
-  S.fbuf = B.fb;
   S.row = A.P.place;
   __syncwarp();
   if (S.row_has_bad_device(A.P.place)) {
@@ -870,7 +834,10 @@ __global__ void __launch_bounds__(32) sim_arb_base_kernel(const __grid_constant_
   S.reset_arb();
   S.ck = 0;
   S.next_ck = 0;
-  S.arb_checkpoint(S.kc.make(0, kReady, 0));  // checkpoint 0: the initial state
+  {  // checkpoint 0: the initial state
+    const typename ArbSim<false, kTypes, kBase>::Outside none{kKeyMax, 0};
+    S.arb_checkpoint(none);
+  }
   S.run();
   if (lane == 0) B.status[0] = S.status;
   if (S.status != GMG_SIM_OK) return;
@@ -883,10 +850,11 @@ __global__ void __launch_bounds__(32) sim_arb_base_kernel(const __grid_constant_
   miss = (int32_t)__reduce_add_sync(kFullMask, (unsigned)miss);
   S.dv.write_peak(B.res_peak);
   const int64_t makespan = S.dv.max_busy(S.g);
+  const int64_t score = warp_sum_i64(S.score);
   if (lane == 0) {
     int64_t* rs = B.res_scalars;
     rs[0] = makespan;
-    rs[1] = S.vflag ? kI64Max : S.score;
+    rs[1] = S.vflag ? kI64Max : score;
     rs[2] = S.vflag;
     rs[3] = S.vop;
     rs[4] = S.vdev;
@@ -897,12 +865,12 @@ __global__ void __launch_bounds__(32) sim_arb_base_kernel(const __grid_constant_
 }
 
 // Incremental candidates resumed from the arbitrated base snapshot.
-template <bool kT32, bool kTypes>
+template <bool kT32, bool kTypes, int kHot>
 __global__ void __launch_bounds__(128, 7) sim_arb_inc_kernel(const __grid_constant__ ArbParams A) {
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
-  ArbSim<kT32, kTypes, kInc> S(A);
+  ArbSim<kT32, kTypes, kInc, kHot> S(A);
   setup_slot(S, A.P, wib, slot, smem);
   S.setup_arb(smem + A.smem_std + (size_t)wib * A.smem_arb);
   S.rb = A.P.base.rb;
@@ -961,24 +929,24 @@ cudaError_t launch_expand_moves(const uint8_t* base_row, const int32_t* base_sta
   return cudaGetLastError();
 }
 
-const void* arb_kernel_ptr(bool t32, bool types) {
-  if (t32) return types ? (const void*)sim_arb_kernel<true, true> : (const void*)sim_arb_kernel<true, false>;
-  return types ? (const void*)sim_arb_kernel<false, true> : (const void*)sim_arb_kernel<false, false>;
-}
-
-cudaError_t launch_arb(bool t32, bool types, const ArbParams& A, int grid, int block, size_t smem,
-                       cudaStream_t st) {
-  void* args[] = {const_cast<ArbParams*>(&A)};
-  return cudaLaunchKernel(arb_kernel_ptr(t32, types), dim3(grid), dim3(block), args, smem, st);
-}
-
+// Instances by (32-bit times, accelerator types; compact records wherever the
+// graph has them).
+#define ARB_PTR(kernel)                                                       \
+  if (G.hot_ok) return (const void*)kernel<true, false, kHotGlobal>;          \
+  if (G.t32)                                                                  \
+    return G.ntypes >= 2 ? (const void*)kernel<true, true, kHotNone>          \
+                         : (const void*)kernel<true, false, kHotNone>;        \
+  return G.ntypes >= 2 ? (const void*)kernel<false, true, kHotNone> : (const void*)kernel<false, false, kHotNone>
+const void* arb_kernel_ptr(const DevGmg& G) { ARB_PTR(sim_arb_kernel); }
+const void* arb_inc_kernel_ptr(const DevGmg& G) { ARB_PTR(sim_arb_inc_kernel); }
+#undef ARB_PTR
 const void* arb_base_kernel_ptr(bool types) {
   return types ? (const void*)sim_arb_base_kernel<true> : (const void*)sim_arb_base_kernel<false>;
 }
 
-const void* arb_inc_kernel_ptr(bool t32, bool types) {
-  if (t32) return types ? (const void*)sim_arb_inc_kernel<true, true> : (const void*)sim_arb_inc_kernel<true, false>;
-  return types ? (const void*)sim_arb_inc_kernel<false, true> : (const void*)sim_arb_inc_kernel<false, false>;
+cudaError_t launch_arb(const ArbParams& A, int grid, int block, size_t smem, cudaStream_t st) {
+  void* args[] = {const_cast<ArbParams*>(&A)};
+  return cudaLaunchKernel(arb_kernel_ptr(A.P.g), dim3(grid), dim3(block), args, smem, st);
 }
 
 cudaError_t launch_arb_base(bool types, const ArbParams& A, size_t smem, cudaStream_t st) {
@@ -986,10 +954,9 @@ cudaError_t launch_arb_base(bool types, const ArbParams& A, size_t smem, cudaStr
   return cudaLaunchKernel(arb_base_kernel_ptr(types), dim3(1), dim3(32), args, smem, st);
 }
 
-cudaError_t launch_arb_inc(bool t32, bool types, const ArbParams& A, int grid, int block, size_t smem,
-                           cudaStream_t st) {
+cudaError_t launch_arb_inc(const ArbParams& A, int grid, int block, size_t smem, cudaStream_t st) {
   void* args[] = {const_cast<ArbParams*>(&A)};
-  return cudaLaunchKernel(arb_inc_kernel_ptr(t32, types), dim3(grid), dim3(block), args, smem, st);
+  return cudaLaunchKernel(arb_inc_kernel_ptr(A.P.g), dim3(grid), dim3(block), args, smem, st);
 }
 
 }  // namespace gsim

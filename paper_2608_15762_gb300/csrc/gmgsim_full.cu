@@ -13,7 +13,7 @@ __global__ void __launch_bounds__(128, kBlocksPerSM) sim_full_kernel(const __gri
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
   const int64_t nslots = (int64_t)gridDim.x * (blockDim.x >> 5);
-  Sim<kNarrow, kFull, kKey, kT32, kTypes, true, kHot> S(P);
+  Sim<kNarrow, kFull, kKey, kT32, kTypes, kHot> S(P);
   setup_slot(S, P, wib, slot, smem);
   for (int64_t k = slot; k < P.K; k += nslots) {
     S.row = P.place + k * P.ld;
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(32 * kStageMaxWarps, 1) sim_full_staged_kernel
   const int64_t nw = blockDim.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * nw + wib;
   const int64_t nslots = (int64_t)gridDim.x * nw;
-  Sim<true, kFull, true, true, false, true, kHotShared> S(P);
+  Sim<true, kFull, true, true, false, kHotShared> S(P);
   setup_slot(S, P, wib, slot, smem + P.stage_bytes);
   S.sh_hot = reinterpret_cast<const uint4*>(s_hot);
   S.sh_rel = reinterpret_cast<const int32_t*>(s_rel);

@@ -37,7 +37,6 @@ namespace {
 constexpr int64_t kI64Max = 0x7fffffffffffffffll;
 constexpr int kMaxOpsLog2 = 28;          // op ids must fit the packed key
 constexpr int kDefaultWarpsPerBlock = 4;
-constexpr int kSharedQueueEntries = 97;  // arbitrated kernels: 1 + 32 * 3: root, its children, two more groups
 constexpr int kSharedOverflowEntries = 33;  // behind the READY pool: the root and its children
 constexpr int64_t kDefaultQueueCap = 1 << 16;
 constexpr int kSharedLogEntries = 192, kSharedLogEntriesWide = 112;
@@ -52,7 +51,7 @@ constexpr int kCheckpointLog = 8192;
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Layout {
-  size_t off_ops, off_succ, off_pred, off_sib, off_cons, off_roots, off_roots_q, off_bytes, off_cap, off_base, off_avail,
+  size_t off_ops, off_succ, off_pred, off_sib, off_cons, off_roots, off_bytes, off_cap, off_base, off_avail,
       off_dl, off_links, off_durt, off_dtype, off_linkid, off_st_hot, off_st_rel, total;
 };
 
@@ -111,7 +110,6 @@ void plan(Built& b) {
   L.off_sib = take(8 * (size_t)b.E);
   L.off_cons = take(4 * (size_t)b.Ec);
   L.off_roots = take(8 * (size_t)b.nroots);
-  L.off_roots_q = take(8 * (size_t)b.nroots);
   L.off_bytes = take(8 * (size_t)b.n);
   L.off_cap = take(8 * (size_t)b.D);
   L.off_base = take(8 * (size_t)b.D);
@@ -493,19 +491,16 @@ size_t smem_per_warp(const SimParams& P) {
 
 // Shared bytes of accelerator state per warp: live bytes; peaks and a drain's
 // sums, or (more than 32 accelerators: the peaks are in global scratch) a bit
-// set of the accelerators whose order matters; free times (of
-// tbytes each) unless lanes hold them in registers (the arbitrated kernels of
-// at most 32).
-int dev_smem_bytes(int D, size_t tbytes, bool pool) {
+// set of the accelerators whose order matters; free times (of tbytes each).
+int dev_smem_bytes(int D, size_t tbytes) {
   const bool narrow = D <= 32;
-  return (int)align_up((size_t)D * 8 + (narrow ? (size_t)D * 72 : 32) + (narrow && !pool ? 0 : (size_t)D * tbytes), 16);
+  return (int)align_up((size_t)D * 8 + (narrow ? (size_t)D * 72 : 32) + (size_t)D * tbytes, 16);
 }
 
 bool g_smem_set = false;
 
-// Slot layout and grid for K candidates of kind `inc` (pool: the READY pool's
-// sweep; the arbitrated kernels take keys one at a time).
-int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& L, bool pool = true) {
+// Slot layout and grid for K candidates of kind `inc`.
+int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& L) {
   const DevGmg& G = g->dg;
   const bool narrow = G.D <= 32;
   L.wpb = (o && o->warps_per_block > 0) ? o->warps_per_block : kDefaultWarpsPerBlock;
@@ -513,20 +508,20 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
   SimParams& P = L.P;
   std::memset(&P, 0, sizeof(P));
   P.g = G;
-  P.pool = pool && !narrow ? kReadyPoolWide : 0;
-  // pending keys beyond one per lane; the pool's heap has room for one more
-  // (Sim::run puts a pool key there when the next root finds the pool full)
-  P.qcap = queue_cap(g, o) + (pool ? 1 : 0);
+  P.pool = narrow ? 0 : kReadyPoolWide;
+  // pending keys beyond one per lane; the heap has room for one more (a pool key
+  // goes there when the next root finds the pool full)
+  P.qcap = queue_cap(g, o) + 1;
   P.pend_cap = 32 + queue_cap(g, o);
-  P.qs = pool ? kSharedOverflowEntries : kSharedQueueEntries;
+  P.qs = kSharedOverflowEntries;
   P.mcap = log_cap(g, o);
-  P.ms = narrow || !pool ? kSharedLogEntries : kSharedLogEntriesWide;
+  P.ms = narrow ? kSharedLogEntries : kSharedLogEntriesWide;
   P.sortcap = kSortCap;
   while (P.sortcap < G.D) P.sortcap <<= 1;
   P.drain_trigger = kOpsPerGeneration;
-  P.opcap = pool ? kOpsPerGeneration + 32 : kOpsPerGeneration;
-  P.dev_bytes = dev_smem_bytes(G.D, G.t32 ? 4 : 8, pool);
-  P.no_side = pool && G.dev_key ? 1 : 0;  // the accelerator is inside the log entry
+  P.opcap = kOpsPerGeneration + 32;
+  P.dev_bytes = dev_smem_bytes(G.D, G.t32 ? 4 : 8);
+  P.no_side = G.dev_key ? 1 : 0;  // the accelerator is inside the log entry
   L.smem = (size_t)L.wpb * smem_per_warp(P);
   size_t o2 = 0;
   auto take = [&](size_t bytes) {
@@ -555,7 +550,6 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
     big.sortcap = 256;
     big.pool = kReadyPoolWide;
     big.opcap = kOpsPerGeneration + 32;
-    big.qs = std::max(kSharedQueueEntries, kSharedOverflowEntries);
     big.ms = std::max(kSharedLogEntries, kSharedLogEntriesWide);
     big.dev_bytes = 32 + 24 * 256;
     big.no_side = 0;
@@ -689,7 +683,7 @@ int plan_arb(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbParams&
   if (!G.dev_key || G.n >= (1 << 27)) return GMG_ERANGE;
   const int64_t xcap = std::max<int64_t>(g->xfer_bound, 1);
   if (xcap > (int64_t(1) << 29)) return GMG_ERANGE;
-  int rc = plan_launch(g, K, o, mode == kInc, L, false);
+  int rc = plan_launch(g, K, o, mode == kInc, L);
   if (rc) return rc;
   std::memset(&A, 0, sizeof(A));
   SimParams& P = L.P;
@@ -701,26 +695,20 @@ int plan_arb(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbParams&
   };
   A.xcap = (int32_t)xcap;
   A.shared_links = g->shared_links;
-  A.heads_shared = G.D <= 16 ? 1 : 0;
-  const size_t n = (size_t)G.n, DD = (size_t)G.D * G.D;
+  const size_t n = (size_t)G.n;
   A.off_cnt = take(4 * n);
   A.off_rmax = take((G.t32 && mode != kBase ? 4 : 8) * n);
   A.off_refs = take(4 * n);
   A.off_rmask = take(4 * n);
   A.off_nextop = take(4 * n);
-  A.off_xent = take(4 * (size_t)xcap);
-  A.off_xnext = take(4 * (size_t)xcap);
-  A.off_qhead = take(A.heads_shared ? 0 : 4 * DD);
-  A.off_qtail = take(4 * DD);
   P.slot_bytes = (int64_t)o2;
-  A.smem_arb = (int32_t)align_up(128 + (A.heads_shared ? 4 * DD : 0), 16);
+  A.smem_arb = 768 + 12 * kArbArrivals;  // busy links, lanes' words; arrivals to look up
   A.smem_std = (int64_t)L.smem;
   L.smem += (size_t)L.wpb * (size_t)A.smem_arb;
   const int sms = device_sms();
   if (sms <= 0) return GMG_ECUDA;
   int bps = 0;
-  const void* fn = mode == kInc ? arb_inc_kernel_ptr(G.t32 != 0, G.ntypes >= 2)
-                                : arb_kernel_ptr(G.t32 != 0, G.ntypes >= 2);
+  const void* fn = mode == kInc ? arb_inc_kernel_ptr(G) : arb_kernel_ptr(G);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, 32 * L.wpb, L.smem) != cudaSuccess)
     return GMG_ECUDA;
   bps = std::max(bps, 1);
@@ -731,6 +719,8 @@ int plan_arb(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbParams&
   return GMG_OK;
 }
 
+bool g_arbw_smem_set = false;
+
 // Arbitrated transfers on 33..256 accelerators: per-accelerator transfer
 // state in tables.  Op ids below 2^24 (an intent packs op << 8 | destination).
 int plan_arbw(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbWParams& A) {
@@ -739,10 +729,12 @@ int plan_arbw(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbWParam
   if (!G.dev_key || G.n >= (1 << 24)) return GMG_ERANGE;
   const int64_t xcap = std::max<int64_t>(g->xfer_bound, 1);
   if (xcap > (int64_t(1) << 29)) return GMG_ERANGE;
-  int rc = plan_launch(g, K, o, false, L, false);
+  int rc = plan_launch(g, K, o, false, L);
   if (rc) return rc;
   std::memset(&A, 0, sizeof(A));
   SimParams& P = L.P;
+  P.pool = 0;  // lanes hold the pending ops
+  L.smem = (size_t)L.wpb * smem_per_warp(P);
   size_t o2 = (size_t)P.slot_bytes;
   auto take = [&](size_t bytes) {
     const size_t at = o2;
@@ -752,31 +744,27 @@ int plan_arbw(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbWParam
   const size_t n = (size_t)G.n, D = (size_t)G.D, DD = D * D, tsz = G.t32 ? 4 : 8;
   A.xcap = (int32_t)xcap;
   A.shared_links = g->shared_links;
-  A.words = (int32_t)((D + 31) / 32);
   A.off_cnt = take(4 * n);
   A.off_rmax = take(tsz * n);
   A.off_refs = take(4 * n);
   A.off_nextop = take(4 * n);
-  A.off_xent = take(4 * (size_t)xcap);
-  A.off_xnext = take(4 * (size_t)xcap);
-  A.off_qhead = take(4 * DD);
-  A.off_qtail = take(4 * DD);
-  A.off_xd = take(tsz * D);
-  A.off_xp = take(4 * D);
-  A.off_xe = take(4 * D);
-  A.off_fh = take(4 * D);
-  A.off_ft = take(4 * D);
-  A.off_fa = take(tsz * D);
-  A.off_pm = take(4 * D * (size_t)A.words);
-  A.off_lb = take(4 * ((DD + 31) / 32));
+  A.off_xent = take(4 * (size_t)std::max(G.n_edges, 1));  // an entry per (op, distinct destination) at most
+  A.off_xnext = take(4 * (size_t)std::max(G.n_edges, 1));
+  A.off_lb = take(g->shared_links ? 4 * ((DD + 31) / 32) : 0);
   P.slot_bytes = (int64_t)o2;
-  A.smem_arb = 128;  // four 8-word bit sets
+  // per accelerator two times and five words; busy receivers; arrivals to look up
+  A.smem_arb = (int32_t)align_up((2 * tsz + 20) * D + 32 + (4 + tsz) * kArbArrivals, 16);
   A.smem_std = (int64_t)L.smem;
   L.smem += (size_t)L.wpb * (size_t)A.smem_arb;
+  if (!g_arbw_smem_set) {
+    // a block of four warps on 256 accelerators asks for most
+    if (set_arbw_smem_limit() != cudaSuccess) return GMG_ECUDA;
+    g_arbw_smem_set = true;
+  }
   const int sms = device_sms();
   if (sms <= 0) return GMG_ECUDA;
   int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, arbw_kernel_ptr(G.t32 != 0, G.ntypes >= 2), 32 * L.wpb,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, arbw_kernel_ptr(G), 32 * L.wpb,
                                                     L.smem) != cudaSuccess)
     return GMG_ECUDA;
   bps = std::max(bps, 1);
@@ -803,11 +791,11 @@ cudaError_t launch_arb_any(const gmg* g, Launch& L, ArbPlan& Q, const int32_t* p
   if (Q.wide) {
     Q.AW.P = L.P;
     Q.AW.pre_status = pre_status;
-    return launch_arbw(g->dg.t32 != 0, g->dg.ntypes >= 2, Q.AW, L.grid, 32 * L.wpb, L.smem, st);
+    return launch_arbw(Q.AW, L.grid, 32 * L.wpb, L.smem, st);
   }
   Q.A.P = L.P;
   Q.A.pre_status = pre_status;
-  return launch_arb(g->dg.t32 != 0, g->dg.ntypes >= 2, Q.A, L.grid, 32 * L.wpb, L.smem, st);
+  return launch_arb(Q.A, L.grid, 32 * L.wpb, L.smem, st);
 }
 
 
@@ -827,7 +815,7 @@ int plan_base(const gmg* g, const sim_opts_t* o, BasePlan& B) {
   int rc = B.arb ? plan_arb(g, 1, o, L, B.A, kBase) : plan_launch(g, 1, o, false, L);
   if (rc) return rc;
   L.wpb = 1;
-  if (B.arb) L.P.dev_bytes = dev_smem_bytes(G.D, 8, false);  // the arbitrated base keeps 64-bit times
+  if (B.arb) L.P.dev_bytes = dev_smem_bytes(G.D, 8);  // the arbitrated base keeps 64-bit times
   L.smem = smem_per_warp(L.P);
   if (B.arb) {
     B.A.smem_std = (int64_t)L.smem;
@@ -861,7 +849,7 @@ int plan_base(const gmg* g, const sim_opts_t* o, BasePlan& B) {
   B.off_arena = 0;
   if (B.arb) {
     // one arena per checkpoint: the arbiter's per-op arrays (times as int64),
-    // intents, pair queues, lane and warp state
+    // lane and warp state
     ArbCk& K = B.A.ck;
     size_t a = 0;
     auto at = [&](size_t bytes) {
@@ -869,19 +857,15 @@ int plan_base(const gmg* g, const sim_opts_t* o, BasePlan& B) {
       a = align_up(a + std::max<size_t>(bytes, 1), 256);
       return (int64_t)r;
     };
-    const size_t n = (size_t)G.n, DD = (size_t)G.D * G.D, xc = (size_t)B.A.xcap;
+    const size_t n = (size_t)G.n;
     K.off_cnt = at(4 * n);
     K.off_rmax = at(8 * n);
     K.off_refs = at(4 * n);
     K.off_rmask = at(4 * n);
     K.off_nextop = at(4 * n);
     K.off_hold = at(8 * n);
-    K.off_xent = at(4 * xc);
-    K.off_xnext = at(4 * xc);
-    K.off_qhead = at(4 * DD);
-    K.off_qtail = at(4 * DD);
     K.off_lanes = at(7 * 8 * 32);
-    K.off_warp = at(4 * 8 + 32 * 4);
+    K.off_warp = at(8 * 2 + 32 * 4);
     K.bytes = (int64_t)a;
     B.off_arena = take((size_t)K.bytes * B.nck);
   }
@@ -929,7 +913,6 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
     put(L.off_sib, ps.data(), 4 * ps.size());
   }
   put(L.off_cons, b.cons.data(), 4 * b.cons.size());
-  put(L.off_roots, b.roots.data(), 8 * b.roots.size());
   // Root keys of the READY pool: the earliest finish from the op's shortest
   // duration over the accelerator types (the encoding of ReadyCodec).
   int tb = 1;
@@ -954,7 +937,7 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
       }
       rq[r] = ((uint64_t)b.ops[i].release << (b.ib + qb)) | ((uint64_t)i << qb) | q;
     }
-    put(L.off_roots_q, rq.data(), 8 * rq.size());
+    put(L.off_roots, rq.data(), 8 * rq.size());
   }
   int64_t most_bytes = 0;
   {
@@ -993,7 +976,6 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   G.predsib = reinterpret_cast<const uint2*>(w + L.off_sib);
   G.cons = reinterpret_cast<const uint32_t*>(w + L.off_cons);
   G.root_keys = reinterpret_cast<const uint64_t*>(w + L.off_roots);
-  G.root_keys_q = reinterpret_cast<const uint64_t*>(w + L.off_roots_q);
   G.bytes = reinterpret_cast<const int64_t*>(w + L.off_bytes);
   G.big_bytes = most_bytes >= (int64_t(1) << 48) ? 1 : 0;
   G.cap = reinterpret_cast<const int64_t*>(w + L.off_cap);
@@ -1337,7 +1319,7 @@ int sim_incremental(const gmg_t* g, const gmg_base_t* b, const int32_t* d_move_o
     A.P = P;
     A.ck = b->ck;
     A.pre_status = nullptr;
-    return launch_arb_inc(g->dg.t32 != 0, g->dg.ntypes >= 2, A, L.grid, 32 * L.wpb, L.smem,
+    return launch_arb_inc(A, L.grid, 32 * L.wpb, L.smem,
                           reinterpret_cast<cudaStream_t>(stream)) == cudaSuccess
                ? GMG_OK
                : GMG_ECUDA;

@@ -9,11 +9,11 @@ namespace {
 // sim_incremental: K move lists against the base.
 // ---------------------------------------------------------------------------
 template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
-__device__ void regen(Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>& S, uint32_t p);
+__device__ void regen(Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>& S, uint32_t p);
 
 template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
-__device__ void inc_candidate(Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>& S, const SimParams& P, int64_t k, uint8_t* crow) {
-  using tm_t = typename Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>::tm_t;
+__device__ void inc_candidate(Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>& S, const SimParams& P, int64_t k, uint8_t* crow) {
+  using tm_t = typename Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>::tm_t;
   const DevGmg& g = S.g;
   const DevBase& B = P.base;
   const unsigned lane = lane_id();
@@ -136,7 +136,7 @@ __device__ void inc_candidate(Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>
   // READY keys at T_c (the pool first, the others to the heap); a moved op's key is recomputed (its inputs' transfer
   // times change; its predecessors all finished before T_c).
   constexpr int kHeld = kNarrow ? 32 : kReadyPoolWide;
-  if constexpr (kNarrow) S.pd.r = S.pd.e = Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>::kNever;
+  if constexpr (kNarrow) S.pd.r = S.pd.e = Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>::kNever;
   for (int x = lane; x < qsz; x += 32) {
     uint64_t key = B.ck_qkey[(int64_t)c * B.ckq + x];
     const uint32_t op = S.rq.op(key);
@@ -246,7 +246,7 @@ __device__ void inc_candidate(Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>
 // (allocated at f_p), and the releases that are already determined because
 // every listed consumer on that accelerator has finished.
 template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
-__device__ void regen(Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot>& S, uint32_t p) {
+__device__ void regen(Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>& S, uint32_t p) {
   const DevGmg& g = S.g;
   const unsigned lane = lane_id();
   const int64_t fp = S.fb[p];
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(128, kBlocksPerSM) sim_inc_kernel(const __grid
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
-  Sim<kNarrow, kInc, kKey, kT32, kTypes, true, kHot> S(P);
+  Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot> S(P);
   setup_slot(S, P, wib, slot, smem);
   S.rb = P.base.rb;
   S.fb = P.base.fb;

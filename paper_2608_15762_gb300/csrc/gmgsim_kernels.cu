@@ -11,7 +11,7 @@ namespace {
 template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
 __global__ void __launch_bounds__(32, 1) sim_base_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
-  Sim<kNarrow, kBase, kKey, kT32, kTypes, true, kHot> S(P);
+  Sim<kNarrow, kBase, kKey, kT32, kTypes, kHot> S(P);
   setup_slot(S, P, 0, 0, smem);
   const DevBase& B = P.base;
   const unsigned lane = lane_id();

@@ -284,17 +284,14 @@ struct MemLog {
 
 // ---------------------------------------------------------------------------
 // Per-accelerator state.  Free times: a shared array of the kernel's time
-// type, or (kReg: the arbitrated kernel of at most 32 accelerators, which takes
-// keys one at a time) accelerator d's in a register of lane d.  Live bytes: a
-// shared array (the drain updates it a batch at a time).  Peak bytes: a shared
-// array, or with more than 32 accelerators (!kPkShared) an array in the warp's
-// global scratch (only raised by atomicMax and read at the end, so its latency
-// is never waited on).
+// type.  Live bytes: a shared array (the drain updates it a batch at a time).
+// Peak bytes: a shared array, or with more than 32 accelerators (!kPkShared) an
+// array in the warp's global scratch (only raised by atomicMax and read where an
+// allocation may exceed it).
 // ---------------------------------------------------------------------------
-template <bool kReg, bool kPkShared, typename TM>
+template <bool kPkShared, typename TM>
 struct Devices {
-  TM fr_reg;
-  TM* fr;       // shared [D] (when !kReg)
+  TM* fr;       // shared [D]
   int64_t* lv;  // shared [D]
   int64_t* pk;  // [D], shared or global
   uint32_t* acc;   // shared [16 * D], zero between drains (kPkShared)
@@ -311,7 +308,7 @@ struct Devices {
     }
     lv = reinterpret_cast<int64_t*>(sm);
     pk = kPkShared ? lv + D : pk_global;  // a compile-time fact of the instance
-    fr = kReg ? nullptr : reinterpret_cast<TM*>(lv + (kPkShared ? 2 * D : D));
+    fr = reinterpret_cast<TM*>(lv + (kPkShared ? 2 * D : D));
   }
   __device__ void reset(const DevGmg& g) {
     const unsigned l = lane_id();
@@ -320,22 +317,9 @@ struct Devices {
       pk[d] = g.base[d];
       if (kPkShared)
         for (int w = 0; w < 4; ++w) reinterpret_cast<uint4*>(acc)[4 * d + w] = make_uint4(0u, 0u, 0u, 0u);
-      if (!kReg) fr[d] = (TM)g.avail0[d];
+      fr[d] = (TM)g.avail0[d];
     }
-    if (kReg) fr_reg = l < (unsigned)D ? (TM)g.avail0[l] : (TM)0;
     __syncwarp();
-  }
-  __device__ __forceinline__ TM get_free(int d) const {
-    if (kReg) return __shfl_sync(kFullMask, fr_reg, d);
-    return fr[d];
-  }
-  __device__ __forceinline__ void set_free(int d, TM v) {
-    if (kReg) {
-      if ((int)lane_id() == d) fr_reg = v;
-    } else {
-      __syncwarp();
-      if (lane_id() == 0) fr[d] = v;
-    }
   }
   // One event at a time (used when accelerator ids do not fit in the sort key).
   __device__ __forceinline__ bool alloc(int d, int64_t b, int64_t cap) {
@@ -358,22 +342,20 @@ struct Devices {
   __device__ void save(int64_t* dst) const {
     const unsigned l = lane_id();
     for (int d = l; d < D; d += 32) {
-      if (!kReg) dst[d] = (int64_t)fr[d];
+      dst[d] = (int64_t)fr[d];
       dst[D + d] = lv[d];
       dst[2 * D + d] = pk[d];
     }
-    if (kReg && l < (unsigned)D) dst[l] = (int64_t)fr_reg;
   }
   __device__ void load(const int64_t* src) {
     const unsigned l = lane_id();
     for (int d = l; d < D; d += 32) {
-      if (!kReg) fr[d] = (TM)src[d];
+      fr[d] = (TM)src[d];
       lv[d] = src[D + d];
       pk[d] = src[2 * D + d];
       if (kPkShared)
         for (int w = 0; w < 4; ++w) reinterpret_cast<uint4*>(acc)[4 * d + w] = make_uint4(0u, 0u, 0u, 0u);
     }
-    if (kReg) fr_reg = l < (unsigned)D ? (TM)src[l] : (TM)0;
     __syncwarp();
   }
   // Largest final free time over the accelerators whose free time moved past
@@ -381,7 +363,7 @@ struct Devices {
   __device__ int64_t max_busy(const DevGmg& g) const {
     uint64_t m = 0;
     for (int d = lane_id(); d < D; d += 32) {
-      const int64_t f = kReg ? (int64_t)fr_reg : (int64_t)fr[d];
+      const int64_t f = (int64_t)fr[d];
       if (f > g.avail0[d]) m = (uint64_t)f > m ? (uint64_t)f : m;
     }
     return (int64_t)warp_max_u64(m);
@@ -436,22 +418,23 @@ __device__ __forceinline__ WarpSmem carve_smem(uint8_t* smem, const SimParams& P
 // and outputs stay int64).
 // kTypes: the graph has several accelerator types (durations per (type, op)).
 // kNarrow: at most 32 accelerators.
-// kPool: the READY pool and its sweep (run) -- every pure-latency kernel; the
-// arbitrated simulators, which take one event at a time, bring their own loop
-// and READY queue (gmg_arb_events.h).
+// kPool: pending READY ops are keys in a pool in shared memory (the pure-latency
+// kernels of more than 32 accelerators, where more ops are pending than a warp
+// has lanes), else each lane holds one.
 // kHot: the sweep reads compact 16-byte records (duration, transfer time, flags,
 // both CSR lists) instead of the 64-byte ones -- kHotGlobal through the
 // read-only path, kHotShared from the CTA's shared-memory copy (staged by
 // sim_full_staged_kernel).
 constexpr int kHotNone = 0, kHotGlobal = 1, kHotShared = 2;
-template <bool kNarrow, int kMode, bool kKey, bool kT32 = false, bool kTypes = false, bool kPool = true,
-          int kHot = kHotNone>
+template <bool kNarrow, int kMode, bool kKey, bool kT32 = false, bool kTypes = false, int kHot = kHotNone,
+          bool kPool = !kNarrow>
 struct Sim {
-  static_assert(kHot == kHotNone || (kT32 && !kTypes && kPool), "compact records: 32-bit times, one type");
+  static_assert(kHot == kHotNone || (kT32 && !kTypes), "compact records: 32-bit times, one type");
   using tm_t = typename std::conditional<kT32, int32_t, int64_t>::type;
   const SimParams& P;
   const DevGmg& g;
-  static constexpr int kSlots = kReadyPoolWide / 32;  // pool slots per lane (more than 32 accelerators)
+  static constexpr int kSlots = kReadyPoolWide / 32;  // pool slots per lane (kPool)
+  static constexpr bool kCompact = kHot != kHotNone;
   static constexpr tm_t kNever = (tm_t)(~(typename std::make_unsigned<tm_t>::type)0 >> 1);
   struct Pending {
     tm_t r, e, dur;  // ready time, earliest finish (both kNever: empty), duration
@@ -461,8 +444,8 @@ struct Sim {
   KeyCodec kc;      // HBM log entries (and the arbitrated simulators' READY keys)
   ReadyCodec rq;    // READY keys of the pool
   ReadyHeap q;      // READY keys beyond the pool (the lanes)
-  Pending pd;       // at most 32 accelerators: this lane's pending op
-  uint64_t* pool;   // more: shared [32 * kSlots], pending READY keys (kKeyMax = empty)
+  Pending pd;       // !kPool: this lane's pending op
+  uint64_t* pool;   // kPool: shared [32 * kSlots], pending READY keys (kKeyMax = empty)
   uint8_t* fstk;    // shared [32 * kSlots]: the empty slots, a stack of nfree
   int nfree;
   MemLog log;
@@ -472,7 +455,7 @@ struct Sim {
   tm_t drained;     // every event before this time is applied, none after it
   uint32_t* oplog;  // ops started since the last HBM-event generation
   int opn;
-  Devices<kNarrow && !kPool, kNarrow, tm_t> dv;
+  Devices<kNarrow, tm_t> dv;
   const uint8_t* row;
   tm_t* fbuf;       // finish times (scratch)
   uint8_t* sl;      // the warp's scratch slot (the less used arrays in it are found from the launch parameters)
@@ -486,7 +469,7 @@ struct Sim {
   // running results
   int rootptr;
   uint64_t rkey;    // root_keys[rootptr], kKeyMax past the end
-  int64_t score, nev;   // with the pool each lane's share, summed at the end
+  int64_t score, nev;   // each lane's share, summed at the end
   int64_t readypops;
   int32_t iters;        // ops started (loop guard; the event count of a full run)
   tm_t last_t;          // latest READY time handled, kept in base mode only (checkpoints)
@@ -559,7 +542,7 @@ struct Sim {
   }
 
   __device__ __forceinline__ void load_root() {
-    rkey = rootptr < g.nroots ? __ldg((kPool ? g.root_keys_q : g.root_keys) + rootptr) : kKeyMax;
+    rkey = rootptr < g.nroots ? __ldg(g.root_keys + rootptr) : kKeyMax;
   }
 
   // Every lane with `want` logs (key, dev).  Uniform call.
@@ -627,10 +610,8 @@ struct Sim {
     for (int r = lane; r < g.R; r += 32) creq()[r] = 0;
     dv.reset(g);
     q.size = 0;
-    if constexpr (kPool) {
-      if constexpr (kNarrow) pd.r = pd.e = kNever;
-      else empty_pool(0);
-    }
+    if constexpr (kPool) empty_pool(0);
+    else pd.r = pd.e = kNever;
     log.n = 0;
     drained = 0;
     opn = 0;
@@ -1286,8 +1267,8 @@ struct Sim {
   }
   __device__ void run() {
     if (status) return;
-    if constexpr (kNarrow) run_narrow();
-    else run_wide();
+    if constexpr (kPool) run_pool();
+    else run_lanes();
   }
 
   // What starting an op needs of its record, and the record of a successor.
@@ -1436,7 +1417,7 @@ struct Sim {
     return false;
   }
 
-  // ---- at most 32 accelerators: one pending op per lane, in registers -------
+  // ---- one pending op per lane, in registers --------------------------------
   __device__ __forceinline__ void hold_op(tm_t r, uint32_t op) {
     pd.r = r;
     pd.op = op;
@@ -1456,157 +1437,198 @@ struct Sim {
     return ra < rb_ || (ra == rb_ && ia < ib_);
   }
 
-  __device__ void run_narrow() {
-    const unsigned lane = lane_id();
-    uint64_t xk = outside_min();  // the smallest key outside the lanes, and its time
-    tm_t xr = key_time(xk);
+  // The smallest key outside the lanes, and its time (kNever: none).
+  struct Outside {
+    uint64_t k;
+    tm_t r;
+  };
+  __device__ __forceinline__ void look_outside(Outside& o) const {
+    o.k = outside_min();
+    o.r = key_time(o.k);
+  }
+
+  // Whether this lane's pending op starts now: those before lim, the smallest
+  // earliest finish (and `until`, a time that no start may pass).  Keys outside
+  // the lanes that are due (rare: every root once, the heap only after the lanes
+  // were all taken) come into empty lanes first.
+  __device__ __forceinline__ bool starts(tm_t lim, tm_t until, Outside& o) {
+    if (o.r >= lim) return pd.r < lim;
+    uint32_t fm = __ballot_sync(kFullMask, pd.r == kNever);
+    bool fresh = false;
+    while (fm && o.r < lim) {
+      const int dst = __ffs(fm) - 1;
+      fm &= fm - 1u;
+      if ((int)lane_id() == dst) {
+        pd.r = o.r;
+        pd.op = rq.op(o.k);
+        fresh = true;
+      }
+      take_outside(o.k);
+      look_outside(o);
+    }
+    if (fresh) hold_op(pd.r, pd.op);
+    lim = warp_min_t(pd.e);
+    lim = lim < until ? lim : until;
+    bool act = pd.r < lim;
+    if (o.r < lim) {
+      // no empty lane: only keys before the next outside one; if there is none
+      // it changes places with the last key of the lanes
+      act = act && precedes(pd.r, pd.op, o.r, rq.op(o.k));
+      if (!__any_sync(kFullMask, act)) {
+        const uint64_t mine = held_key();
+        const uint64_t last = warp_max_u64(mine);
+        const uint64_t x = o.k;
+        take_outside(x);
+        q.push(last);  // the heap keeps one entry beyond its limit for this
+        act = mine == last;
+        if (act) hold_op((tm_t)rq.time(x), rq.op(x));
+        look_outside(o);
+      }
+    }
+    return act;
+  }
+
+  // The ops started together: this lane's (v) and the lanes' (b); ord: its place
+  // among the batch's ops of its accelerator, last: the largest of these.
+  struct Batch {
+    bool v;
+    uint32_t b, i;
+    int d, ord, last;
+    tm_t f;
+    Start s;
+  };
+  // Start the lanes' ops with act; false if the iteration limit is passed.
+  __device__ __forceinline__ bool start_held(bool act, Batch& B) {
+    B.v = act;
+    B.b = __ballot_sync(kFullMask, act);
+    const int m = __popc(B.b);
+    if (!count_started(m)) return false;
+    B.i = pd.op;
+    B.d = pd.d;
+    const tm_t r = pd.r;
+    B.s.nsucc = 0;
+    B.s.flags = 0;
+    B.f = 0;
+    B.ord = B.last = 0;
+    tm_t fd = 0;
+    if (act) {
+      B.s = start_of(B.i, B.d);
+      fd = dv.fr[B.d];
+    }
+    // every accelerator starts its ops of the batch in key order
+    bool shared = false;
+    if (m > 1) {
+      if constexpr (kNarrow) {
+        shared = __popc(__reduce_or_sync(kFullMask, act ? 1u << B.d : 0u)) < m;
+      } else {
+        const uint32_t grp = __match_any_sync(kFullMask, act ? (uint32_t)B.d : 256u + lane_id());
+        shared = __any_sync(kFullMask, (grp & (grp - 1u)) != 0u);
+      }
+    }
+    if (shared) {
+      int ord = 0;
+      for (uint32_t o = B.b; o; o &= o - 1u) {
+        const int src = __ffs(o) - 1;
+        const tm_t ro = __shfl_sync(kFullMask, r, src);
+        const uint32_t io = __shfl_sync(kFullMask, B.i, src);
+        const int dd = __shfl_sync(kFullMask, B.d, src);
+        ord += act && dd == B.d && precedes(ro, io, r, B.i) ? 1 : 0;
+      }
+      const int last = (int)__reduce_max_sync(kFullMask, (unsigned)ord);
+      for (int t = 0; t < last; ++t) {
+        if (act && ord == t) {
+          B.f = earliest(r, B.d, pd.dur);
+          dv.fr[B.d] = B.f;
+        }
+        __syncwarp();
+      }
+      act = act && ord == last;  // the others have theirs
+      if (act) fd = dv.fr[B.d];
+      B.ord = ord;
+      B.last = last;
+    }
+    if (act) {
+      B.f = (r > fd ? r : fd) + pd.dur;
+      dv.fr[B.d] = B.f;
+    }
+    record(B.v, B.b, B.i, r, B.f, B.s);
+    if (B.v) pd.r = pd.e = kNever;
+    __syncwarp();
+    return true;
+  }
+
+  // Ops that became ready (at most one per lane) become pending: in this lane if
+  // it is empty, else in another empty one, else in the heap.
+  __device__ __forceinline__ void place(Reached& x, Outside& o) {
+    tm_t e = kNever;
+    if (x.rdy) {
+      e = earliest(x.r, x.d, x.dur);
+      if (pd.r == kNever) {
+        pd.r = x.r;
+        pd.e = e;
+        pd.dur = x.dur;
+        pd.op = x.j;
+        pd.d = x.d;
+        x.rdy = false;
+      }
+    }
+    uint32_t more = __ballot_sync(kFullMask, x.rdy);
+    while (more) {
+      const int src = __ffs(more) - 1;
+      more &= more - 1u;
+      const uint32_t fm = __ballot_sync(kFullMask, pd.r == kNever);
+      const tm_t r = __shfl_sync(kFullMask, x.r, src), te = __shfl_sync(kFullMask, e, src),
+                 dur = __shfl_sync(kFullMask, x.dur, src);
+      const uint32_t j = __shfl_sync(kFullMask, x.j, src);
+      const int d = __shfl_sync(kFullMask, x.d, src);
+      if (fm) {
+        if ((int)lane_id() == __ffs(fm) - 1) {
+          pd.r = r;
+          pd.e = te;
+          pd.dur = dur;
+          pd.op = j;
+          pd.d = d;
+        }
+      } else {
+        if (32 + q.size >= P.pend_cap || !q.push(rq.make(r, j, (tm_t)(te - r)))) status = GMG_SIM_QUEUE;
+        look_outside(o);
+      }
+    }
+  }
+
+  __device__ void run_lanes() {
+    Outside o;
+    look_outside(o);
     while (true) {
       if (kMode == kBase && readypops >= next_ck) {
         const tm_t t = warp_min_t(pd.r);
-        const tm_t tn = t < xr ? t : xr;
+        const tm_t tn = t < o.r ? t : o.r;
         if (tn != kNever) maybe_checkpoint((int64_t)tn, held_key());
       }
-      tm_t lim = warp_min_t(pd.e);
-      const bool end = lim == kNever && xr == kNever;
+      const tm_t lim = warp_min_t(pd.e);
+      const bool end = lim == kNever && o.r == kNever;
       if (end || opn >= P.drain_trigger) {  // the only copy of this code: it is large
         const tm_t t = warp_min_t(pd.r);
-        drain(end ? kI64Max : (int64_t)(t < xr ? t : xr));
+        drain(end ? kI64Max : (int64_t)(t < o.r ? t : o.r));
         if (end || status) break;
       }
-      bool act;
-      if (xr < lim) {
-        // keys outside the lanes are due (rare: every root once, the heap only
-        // after the lanes were all taken): they come into empty lanes
-        uint32_t fm = __ballot_sync(kFullMask, pd.r == kNever);
-        bool fresh = false;
-        while (fm && xr < lim) {
-          const int dst = __ffs(fm) - 1;
-          fm &= fm - 1u;
-          if ((int)lane == dst) {
-            pd.r = xr;
-            pd.op = rq.op(xk);
-            fresh = true;
-          }
-          take_outside(xk);
-          xk = outside_min();
-          xr = key_time(xk);
-        }
-        if (fresh) hold_op(pd.r, pd.op);
-        lim = warp_min_t(pd.e);
-        act = pd.r < lim;
-        if (xr < lim) {
-          // no empty lane: only keys before the next outside one; if there is
-          // none it changes places with the last key of the lanes
-          act = act && precedes(pd.r, pd.op, xr, rq.op(xk));
-          if (!__any_sync(kFullMask, act)) {
-            const uint64_t mine = held_key();
-            const uint64_t last = warp_max_u64(mine);
-            const uint64_t x = xk;
-            take_outside(x);
-            q.push(last);  // the heap keeps one entry beyond its limit for this
-            act = mine == last;
-            if (act) hold_op((tm_t)rq.time(x), rq.op(x));
-            xk = outside_min();
-            xr = key_time(xk);
-          }
-        }
-      } else {
-        act = pd.r < lim;
-      }
-      const uint32_t b = __ballot_sync(kFullMask, act);
-      const int m = __popc(b);
-      if (!count_started(m)) break;
-      const uint32_t i = pd.op;
-      const int d = pd.d;
-      const tm_t r = pd.r;
-      Start s;
-      s.nsucc = 0;
-      s.flags = 0;
-      tm_t f = 0, fd = 0;
-      if (act) {
-        s = start_of(i, d);
-        fd = dv.fr[d];
-      }
-      // every accelerator starts its ops of the batch in key order
-      if (m > 1 && __popc(__reduce_or_sync(kFullMask, act ? 1u << d : 0u)) < m) {
-        int ord = 0;
-        for (uint32_t o = b; o; o &= o - 1u) {
-          const int src = __ffs(o) - 1;
-          const tm_t ro = __shfl_sync(kFullMask, r, src);
-          const uint32_t io = __shfl_sync(kFullMask, i, src);
-          const int dd = __shfl_sync(kFullMask, d, src);
-          ord += act && dd == d && precedes(ro, io, r, i) ? 1 : 0;
-        }
-        const int last = (int)__reduce_max_sync(kFullMask, (unsigned)ord);
-        for (int t = 0; t < last; ++t) {
-          if (act && ord == t) {
-            f = earliest(r, d, pd.dur);
-            dv.fr[d] = f;
-          }
-          __syncwarp();
-        }
-        act = act && ord == last;  // the others have theirs
-        if (act) fd = dv.fr[d];
-      }
-      if (act) {
-        f = (r > fd ? r : fd) + pd.dur;
-        dv.fr[d] = f;
-      }
-      const bool v = (b >> lane) & 1u;
-      record(v, b, i, r, f, s);
-      if (v) pd.r = pd.e = kNever;
-      __syncwarp();
-      // successors: a lane's first ready one stays in the lane, further ones go
-      // to empty lanes
-      for (uint32_t u = 0; __any_sync(kFullMask, u < s.nsucc); ++u) {
+      Batch B;
+      if (!start_held(starts(lim, kNever, o), B)) break;
+      for (uint32_t u = 0; __any_sync(kFullMask, u < B.s.nsucc); ++u) {
         Reached x;
         x.rdy = x.join = false;
         x.j = 0;
         x.d = 0;
         x.r = x.dur = 0;
-        if (u < s.nsucc) x = reach(i, d, f, s, u);
+        if (u < B.s.nsucc) x = reach(B.i, B.d, B.f, B.s, u);
         claim(x);
-        tm_t e = kNever;
-        if (x.rdy) {
-          e = earliest(x.r, x.d, x.dur);
-          if (pd.r == kNever) {
-            pd.r = x.r;
-            pd.e = e;
-            pd.dur = x.dur;
-            pd.op = x.j;
-            pd.d = x.d;
-            x.rdy = false;
-          }
-        }
-        uint32_t more = __ballot_sync(kFullMask, x.rdy);
-        while (more) {
-          const int src = __ffs(more) - 1;
-          more &= more - 1u;
-          const uint32_t fm = __ballot_sync(kFullMask, pd.r == kNever);
-          const tm_t xr_ = __shfl_sync(kFullMask, x.r, src), xe = __shfl_sync(kFullMask, e, src),
-                     xd = __shfl_sync(kFullMask, x.dur, src);
-          const uint32_t xj = __shfl_sync(kFullMask, x.j, src);
-          const int xdev = __shfl_sync(kFullMask, x.d, src);
-          if (fm) {
-            if ((int)lane == __ffs(fm) - 1) {
-              pd.r = xr_;
-              pd.e = xe;
-              pd.dur = xd;
-              pd.op = xj;
-              pd.d = xdev;
-            }
-          } else {
-            if (32 + q.size >= P.pend_cap || !q.push(rq.make(xr_, xj, (tm_t)(xe - xr_)))) status = GMG_SIM_QUEUE;
-            xk = outside_min();
-            xr = key_time(xk);
-          }
-        }
+        place(x, o);
       }
       if (status) break;
     }
   }
 
-  // ---- more accelerators: pending ops as keys in a pool in shared memory -----
+  // ---- pending ops as keys in a pool in shared memory -------------------------
 
   // Slots [from, 32 * kSlots) are empty.
   __device__ void empty_pool(int from) {
@@ -1631,138 +1653,137 @@ struct Sim {
     return m < x ? m : x;
   }
 
-  __device__ void run_wide() {
+  // The pending ops that start now: those before lim, the smallest earliest finish
+  // (and `until`, a time that no start may pass); returns their number m, and in
+  // the first m lanes their keys and pool slots.
+  __device__ __forceinline__ int startable(tm_t until, uint64_t& key, int& slot) {
     const unsigned lane = lane_id();
-    while (true) {
-      if (kMode == kBase && readypops >= next_ck) {
-        const uint64_t nk = next_key();
-        if (nk != kKeyMax) maybe_checkpoint(rq.time(nk));
-      }
-      const bool end = nfree == 32 * kSlots && outside_min() == kKeyMax;
-      if (end || opn >= P.drain_trigger) {  // the only copy of this code: it is large
-        drain(end ? kI64Max : rq.time(next_key()));
-        if (end || status) break;
-      }
-      uint64_t k[kSlots];
-      tm_t lim = kNever;
+    uint64_t k[kSlots];
+    tm_t lim = kNever;
 #pragma unroll
-      for (int s = 0; s < kSlots; ++s) {
-        k[s] = pool[32 * s + lane];
-        const tm_t e = k[s] == kKeyMax ? kNever : (tm_t)rq.bound(k[s]);
-        lim = e < lim ? e : lim;
-      }
-      lim = warp_min_t(lim);
-      // keys outside the pool that are due come in (rare: the roots once each,
-      // the heap only after the pool was full)
-      uint64_t x = outside_min();
-      uint64_t kb = kKeyMax;  // keys below kb are started
-      if (key_time(x) < lim) {
-        __syncwarp();
-        while (key_time(x) < lim) {
-          int slot;
-          if (nfree > 0) {
-            slot = fstk[--nfree];
-            take_outside(x);
-          } else {
-            // full: x waits unless it is the next key of all; it then changes
-            // places with the pool's last key
-            if (x > pool_min()) {
-              kb = x;
-              break;
-            }
-            uint64_t mx = 0;
-            int ms = 0;
-#pragma unroll
-            for (int s = 0; s < kSlots; ++s) {
-              const uint64_t y = pool[32 * s + lane];
-              if (y > mx) {
-                mx = y;
-                ms = 32 * s + (int)lane;
-              }
-            }
-            const uint64_t last = warp_max_u64(mx);
-            slot = __shfl_sync(kFullMask, ms, __ffs(__ballot_sync(kFullMask, mx == last)) - 1);
-            take_outside(x);
-            q.push(last);  // the heap keeps one entry beyond its limit for this
+    for (int s = 0; s < kSlots; ++s) {
+      k[s] = pool[32 * s + lane];
+      const tm_t e = k[s] == kKeyMax ? kNever : (tm_t)rq.bound(k[s]);
+      lim = e < lim ? e : lim;
+    }
+    lim = warp_min_t(lim);
+    lim = lim < until ? lim : until;
+    // keys outside the pool that are due come in (rare: the roots once each,
+    // the heap only after the pool was full)
+    uint64_t x = outside_min();
+    uint64_t kb = kKeyMax;  // keys below kb are started
+    if (key_time(x) < lim) {
+      __syncwarp();
+      while (key_time(x) < lim) {
+        int slot;
+        if (nfree > 0) {
+          slot = fstk[--nfree];
+          take_outside(x);
+        } else {
+          // full: x waits unless it is the next key of all; it then changes
+          // places with the pool's last key
+          if (x > pool_min()) {
+            kb = x;
+            break;
           }
-          if (lane == 0) pool[slot] = x;
-          __syncwarp();
-          const tm_t e = (tm_t)rq.bound(x);
-          lim = e < lim ? e : lim;
-          x = outside_min();
-        }
+          uint64_t mx = 0;
+          int ms = 0;
 #pragma unroll
-        for (int s = 0; s < kSlots; ++s) k[s] = pool[32 * s + lane];
+          for (int s = 0; s < kSlots; ++s) {
+            const uint64_t y = pool[32 * s + lane];
+            if (y > mx) {
+              mx = y;
+              ms = 32 * s + (int)lane;
+            }
+          }
+          const uint64_t last = warp_max_u64(mx);
+          slot = __shfl_sync(kFullMask, ms, __ffs(__ballot_sync(kFullMask, mx == last)) - 1);
+          take_outside(x);
+          q.push(last);  // the heap keeps one entry beyond its limit for this
+        }
+        if (lane == 0) pool[slot] = x;
+        __syncwarp();
+        const tm_t e = (tm_t)rq.bound(x);
+        lim = e < lim ? e : lim;
+        x = outside_min();
       }
-      const uint64_t lb = (uint64_t)lim << g.qsh;
-      kb = lb < kb ? lb : kb;
-      int m = 0;
-      uint32_t b[kSlots];
+#pragma unroll
+      for (int s = 0; s < kSlots; ++s) k[s] = pool[32 * s + lane];
+    }
+    const uint64_t lb = (uint64_t)lim << g.qsh;
+    kb = lb < kb ? lb : kb;
+    int m = 0;
+    uint32_t b[kSlots];
+#pragma unroll
+    for (int s = 0; s < kSlots; ++s) {
+      b[s] = __ballot_sync(kFullMask, k[s] < kb);
+      m += __popc(b[s]);
+    }
+    if (m > 32) {
+      // more keys than lanes: a bound with 16 to 32 keys below it (or at
+      // least one)
+      uint64_t lo = pool_min() + 1, hi = kb;
+      m = 0;
+      while (m < 16 && hi - lo > 1) {
+        const uint64_t mid = lo + (hi - lo) / 2;
+        int c = 0;
+#pragma unroll
+        for (int s = 0; s < kSlots; ++s) c += __popc(__ballot_sync(kFullMask, k[s] < mid));
+        if (c <= 32) {
+          lo = mid;
+          m = c;
+        } else {
+          hi = mid;
+        }
+      }
+      m = 0;
 #pragma unroll
       for (int s = 0; s < kSlots; ++s) {
-        b[s] = __ballot_sync(kFullMask, k[s] < kb);
+        b[s] = __ballot_sync(kFullMask, k[s] < lo);
         m += __popc(b[s]);
       }
-      if (m > 32) {
-        // more keys than lanes: a bound with 16 to 32 keys below it (or at
-        // least one)
-        uint64_t lo = pool_min() + 1, hi = kb;
-        m = 0;
-        while (m < 16 && hi - lo > 1) {
-          const uint64_t mid = lo + (hi - lo) / 2;
-          int c = 0;
-#pragma unroll
-          for (int s = 0; s < kSlots; ++s) c += __popc(__ballot_sync(kFullMask, k[s] < mid));
-          if (c <= 32) {
-            lo = mid;
-            m = c;
-          } else {
-            hi = mid;
-          }
-        }
-        m = 0;
-#pragma unroll
-        for (int s = 0; s < kSlots; ++s) {
-          b[s] = __ballot_sync(kFullMask, k[s] < lo);
-          m += __popc(b[s]);
-        }
-      }
-      // one key per lane, through the sort area (free between drains)
-      int at = 0;
-      __syncwarp();
-#pragma unroll
-      for (int s = 0; s < kSlots; ++s) {
-        if ((b[s] >> lane) & 1u) {
-          const int pos = at + __popc(b[s] & lanes_below());
-          sortk[pos] = k[s];
-          reinterpret_cast<uint32_t*>(sortk + 32)[pos] = (uint32_t)(32 * s) + lane;
-        }
-        at += __popc(b[s]);
-      }
-      __syncwarp();
-      uint64_t key = kKeyMax;
-      int slot = 0;
-      if ((int)lane < m) {
-        key = sortk[lane];
-        slot = (int)reinterpret_cast<const uint32_t*>(sortk + 32)[lane];
-      }
-      if (!count_started(m)) break;
-      start_batch(key, slot, m);
-      if (status) break;
     }
+    // one key per lane, through the sort area (free between drains)
+    int at = 0;
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < kSlots; ++s) {
+      if ((b[s] >> lane) & 1u) {
+        const int pos = at + __popc(b[s] & lanes_below());
+        sortk[pos] = k[s];
+        reinterpret_cast<uint32_t*>(sortk + 32)[pos] = (uint32_t)(32 * s) + lane;
+      }
+      at += __popc(b[s]);
+    }
+    __syncwarp();
+    key = kKeyMax;
+    slot = 0;
+    if ((int)lane < m) {
+      key = sortk[lane];
+      slot = (int)reinterpret_cast<const uint32_t*>(sortk + 32)[lane];
+    }
+    return m;
   }
 
-  // Start the batch's ops (lanes below m: a key and the pool slot that it came
-  // from), record them for HBM-event generation, and queue the successors they
-  // make ready.
-  __device__ __forceinline__ void start_batch(uint64_t key, int slot, int m) {
+  // The ops started together: this lane's (v), its place among the batch's ops of
+  // its accelerator (ord) and the largest of these.
+  struct WideBatch {
+    bool v;
+    uint32_t i;
+    int d, ord, last;
+    tm_t f;
+    Start s;
+  };
+  // Start the batch's ops (lanes below m: a key) and record them for HBM-event
+  // generation.
+  __device__ __forceinline__ void start_keys(uint64_t key, int m, WideBatch& B) {
     const unsigned lane = lane_id();
     const bool v = key != kKeyMax;
     const uint32_t i = rq.op(key);
     const tm_t r = (tm_t)rq.time(key);
     int d = 0;
     tm_t f = 0;
-    Start s;
+    Start& s = B.s;
     s.nsucc = 0;
     s.flags = 0;
     s.dur = 0;
@@ -1792,16 +1813,74 @@ struct Sim {
     }
     record(v, __ballot_sync(kFullMask, v), i, r, f, s);
     __syncwarp();
-    // successors: a lane's first ready one takes its own slot, further ones
-    // take empty slots
+    B.v = v;
+    B.i = i;
+    B.d = d;
+    B.f = f;
+    B.ord = ord;
+    B.last = maxord;
+  }
+
+  // Keys of ready ops (per lane) to empty slots, or to the heap.
+  __device__ __forceinline__ void spill(bool want, uint64_t nk) {
+    const uint32_t more = __ballot_sync(kFullMask, want);
+    if (more == 0u) return;
+    const int c = __popc(more), have = nfree < c ? nfree : c;
+    const int rank = __popc(more & lanes_below());
+    if (want && rank < have) pool[fstk[nfree - 1 - rank]] = nk;
+    nfree -= have;
+    uint32_t rest = __ballot_sync(kFullMask, want && rank >= have);
+    while (rest) {
+      const int src = __ffs(rest) - 1;
+      rest &= rest - 1;
+      if (!q.push(__shfl_sync(kFullMask, nk, src))) status = GMG_SIM_QUEUE;
+    }
+    if (32 * kSlots - nfree + q.size > P.pend_cap) status = GMG_SIM_QUEUE;
+    __syncwarp();
+  }
+  __device__ __forceinline__ void free_slots(bool gone, int slot) {
+    const uint32_t gm = __ballot_sync(kFullMask, gone);
+    if (gone) {
+      pool[slot] = kKeyMax;
+      fstk[nfree + __popc(gm & lanes_below())] = (uint8_t)slot;
+    }
+    nfree += __popc(gm);
+    __syncwarp();
+  }
+
+  __device__ void run_pool() {
+    while (true) {
+      if (kMode == kBase && readypops >= next_ck) {
+        const uint64_t nk = next_key();
+        if (nk != kKeyMax) maybe_checkpoint(rq.time(nk));
+      }
+      const bool end = nfree == 32 * kSlots && outside_min() == kKeyMax;
+      if (end || opn >= P.drain_trigger) {  // the only copy of this code: it is large
+        drain(end ? kI64Max : rq.time(next_key()));
+        if (end || status) break;
+      }
+      uint64_t key;
+      int slot;
+      const int m = startable(kNever, key, slot);
+      if (!count_started(m)) break;
+      start_batch(key, slot, m);
+      if (status) break;
+    }
+  }
+
+  // Start the batch's ops and queue the successors they make ready: a lane's
+  // first takes its own slot, further ones take empty slots.
+  __device__ __forceinline__ void start_batch(uint64_t key, int slot, int m) {
+    WideBatch B;
+    start_keys(key, m, B);
     bool kept = false;
-    for (uint32_t u = 0; __any_sync(kFullMask, u < s.nsucc); ++u) {
+    for (uint32_t u = 0; __any_sync(kFullMask, u < B.s.nsucc); ++u) {
       Reached x;
       x.rdy = x.join = false;
       x.j = 0;
       x.d = 0;
       x.r = x.dur = 0;
-      if (u < s.nsucc) x = reach(i, d, f, s, u);
+      if (u < B.s.nsucc) x = reach(B.i, B.d, B.f, B.s, u);
       claim(x);
       uint64_t nk = kKeyMax;
       if (x.rdy) {
@@ -1812,30 +1891,9 @@ struct Sim {
           x.rdy = false;
         }
       }
-      const uint32_t more = __ballot_sync(kFullMask, x.rdy);
-      if (more) {
-        const int c = __popc(more), have = nfree < c ? nfree : c;
-        const int rank = __popc(more & lanes_below());
-        if (x.rdy && rank < have) pool[fstk[nfree - 1 - rank]] = nk;
-        nfree -= have;
-        uint32_t rest = __ballot_sync(kFullMask, x.rdy && rank >= have);
-        while (rest) {
-          const int src = __ffs(rest) - 1;
-          rest &= rest - 1;
-          if (!q.push(__shfl_sync(kFullMask, nk, src))) status = GMG_SIM_QUEUE;
-        }
-        if (32 * kSlots - nfree + q.size > P.pend_cap) status = GMG_SIM_QUEUE;
-        __syncwarp();
-      }
+      spill(x.rdy, nk);
     }
-    const bool gone = v && !kept;
-    const uint32_t gm = __ballot_sync(kFullMask, gone);
-    if (gone) {
-      pool[slot] = kKeyMax;
-      fstk[nfree + __popc(gm & lanes_below())] = (uint8_t)slot;
-    }
-    nfree += __popc(gm);
-    __syncwarp();
+    free_slots(B.v && !kept, slot);
   }
 
   __device__ void write_invalid(int64_t k, int32_t st) {
@@ -1890,8 +1948,8 @@ struct Sim {
     // the accelerators that ran an op (an op finishes after its accelerator's
     // initial availability).
     const int64_t mk = dv.max_busy(g);
-    const int64_t sc = kPool ? warp_sum_i64(score) : score;
-    const int64_t ne = kMode == kFull ? (int64_t)iters : kPool ? warp_sum_i64(nev) : nev;
+    const int64_t sc = warp_sum_i64(score);
+    const int64_t ne = kMode == kFull ? (int64_t)iters : warp_sum_i64(nev);
     if (lane == 0) {
       o.makespan[k] = mk;
       o.score[k] = vflag ? kI64Max : sc;
@@ -1941,8 +1999,8 @@ struct Sim {
 // READY heap, event log, partial results; the ops started by then are those
 // with base ready time < T_c.  An incremental candidate whose resume time T0
 // is >= T_c restarts there.
-template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, bool kPool, int kHot>
-__device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kPool, kHot>::maybe_checkpoint(int64_t tn, uint64_t held) {
+template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool>
+__device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool>::maybe_checkpoint(int64_t tn, uint64_t held) {
   if (kMode != kBase) return;
   const DevBase& B = P.base;
   if (ck >= B.nck || readypops < next_ck) return;
@@ -1950,13 +2008,12 @@ __device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kPool, kHot>::maybe_chec
   const unsigned lane = lane_id();
   generate();
   // the pool's keys (or the keys that the lanes hold) follow the heap's
-  constexpr bool kPooled = kPool && !kNarrow;
   const uint32_t hm = __ballot_sync(kFullMask, held != kKeyMax);
-  const int nready = q.size + (kPooled ? 32 * kSlots - nfree : __popc(hm));
+  const int nready = q.size + (kPool ? 32 * kSlots - nfree : __popc(hm));
   if (nready <= B.ckq && log.n <= B.ckm) {
     int64_t* sc = B.ck_scalars + (int64_t)ck * 8;
     uint64_t* qk = B.ck_qkey + (int64_t)ck * B.ckq;
-    if (kPooled) {
+    if (kPool) {
       int at = q.size;
 #pragma unroll
       for (int s = 0; s < kSlots; ++s) {
@@ -1968,7 +2025,7 @@ __device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kPool, kHot>::maybe_chec
     } else if (held != kKeyMax) {
       qk[q.size + __popc(hm & lanes_below())] = held;
     }
-    const int64_t total = kPool ? warp_sum_i64(score) : score;
+    const int64_t total = warp_sum_i64(score);
     if (lane == 0) {
       B.ck_time[ck] = tn;
       sc[0] = nready;
@@ -1995,8 +2052,8 @@ __device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kPool, kHot>::maybe_chec
   __syncwarp();
 }
 
-template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, bool kPool, int kHot>
-__device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kPool, kHot>& S, const SimParams& P, unsigned wib,
+template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool>
+__device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool>& S, const SimParams& P, unsigned wib,
                            int64_t slot, uint8_t* smem) {
   uint8_t* sl = P.scratch + slot * P.slot_bytes;
   const WarpSmem w = carve_smem(smem, P, wib);
@@ -2014,7 +2071,7 @@ __device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kPool, kHot>&
   S.sortd = w.sortd;
   S.oplog = w.oplog;
   S.opn = 0;
-  using tm_t = typename Sim<kNarrow, kMode, kKey, kT32, kTypes, kPool, kHot>::tm_t;
+  using tm_t = typename Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool>::tm_t;
   S.fbuf = reinterpret_cast<tm_t*>(sl + P.off_f);
   S.sl = sl;
   S.dv.setup(P.g, w.dev, P.off_pk >= 0 ? reinterpret_cast<int64_t*>(sl + P.off_pk) : nullptr);

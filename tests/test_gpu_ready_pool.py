@@ -96,3 +96,26 @@ def test_default_staging_rule_gives_the_same(K):
     torch.cuda.synchronize()
     for o in outs:
         compare(o.to_numpy(), *oracle_rows(wl.desc, rows))
+
+
+@pytest.mark.parametrize("D", [2, 32, 33, 256])
+@pytest.mark.parametrize("kw", [
+    dict(chains=300, length=3, dur_hi=1, bytes_lo=4096, bytes_hi=4096),  # transfers that complete together
+    dict(chains=80, length=4, dur_hi=1, release_hi=2, bytes_lo=0, bytes_hi=1 << 12),
+    dict(chains=9, length=4, fan=5),                                       # several destinations per op
+    dict(chains=40, length=4, dur_hi=1 << 29),                             # 64-bit times
+])
+def test_arbitrated_events_at_one_time(D, kw):
+    """More pending ops than lanes, and more completions and intents at one time
+    than are looked up at once."""
+    d = _chains(17, D=D, **kw)
+    rows = _rows(18, 9, d.n_ops, D)
+    g = G.gmg_create(d)
+    out = G.sim_batch(g, torch_place(rows), req_done=True, arbitrated=True)
+    base = rows[0, :d.n_ops].copy()
+    mv = W.random_moves(19, 24, base, D, max_moves=5)
+    b = G.base_create(g, torch.from_numpy(base).cuda(), arbitrated=D <= 32)
+    inc = G.sim_incremental(g, b, *G.moves_to_device(mv, "cuda"), req_done=True, arbitrated=True)
+    torch.cuda.synchronize()
+    compare(out.to_numpy(), *O.simulate_batch(d, rows, arbitrated=True))
+    compare(inc.to_numpy(), *O.incremental_batch(d, base, mv, arbitrated=True), check_events=D > 32)
