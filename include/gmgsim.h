@@ -124,9 +124,10 @@ typedef struct gmg_base gmg_base_t; /* opaque; base schedule snapshot for increm
  * uniform links, every time below 2^31, at most 32 accelerators and the copy
  * within the CTA's shared memory, else GMG_EINVAL.  GMG_STAGING_L1: 4-warp
  * CTAs read the records through the read-only L1 path.
- * GMG_STAGING_DEFAULT stages graphs whose copy takes 16 KB at most and batches
- * of at most 32 candidates wherever staging applies (measured faster there) and
- * takes the L1 path elsewhere; sim_batch_noalloc always
+ * GMG_STAGING_DEFAULT takes the fastest measured: batches of up to about 14
+ * candidates per SM run with two warps per candidate by the L1 path (32-bit
+ * times), larger ones are staged where staging applies and the copy takes 16 KB
+ * at most, and take the L1 path elsewhere; sim_batch_noalloc always
  * takes the L1 path (and refuses GMG_STAGING_SHARED). */
 #define GMG_STAGING_DEFAULT 0
 #define GMG_STAGING_SHARED 1
@@ -181,7 +182,7 @@ typedef struct {
   int32_t stageable;     /* 1 if sim_batch can stage this graph's hot fields in shared memory on
                             the current device (one accelerator type, uniform links, 32-bit times,
                             at most 32 accelerators, and the copy fits beside one warp's areas);
-                            the default then stages small graphs and small batches, with
+                            the default then stages large batches of small graphs, with
                             pure-latency transfers */
   int32_t reserved_;
 } gmg_info_t;

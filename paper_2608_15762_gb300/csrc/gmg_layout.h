@@ -222,6 +222,7 @@ struct SimParams {
   uint8_t* scratch;
   int64_t slot_bytes;    // scratch bytes per warp slot
   int32_t dev_bytes;     // shared bytes of accelerator state per warp
+  int32_t pair_bytes;    // shared bytes that two warps of a candidate hand ops over in, else 0
   int32_t stage_bytes;   // shared bytes of the staged GMG copy (sim_full_staged_kernel), else 0
   int32_t no_side;       // 1: no side bytes in shared memory (the accelerator is inside the log entry)
   // byte offsets inside a slot (off_pk < 0: the peaks are in shared memory)

@@ -664,7 +664,8 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode, kHot>, Sim<true, kMode, tr
     status = GMG_SIM_OK;
     pd.r = pd.e = kNever;
     this->opn = 0;
-    this->dv.load(B.ck_dev + (int64_t)c * 3 * g.D);
+    this->dv.load_free(B.ck_dev + (int64_t)c * 3 * g.D);
+    this->dv.load_bytes(B.ck_dev + (int64_t)c * 3 * g.D);
     for (int r = lane; r < g.R; r += 32) this->creq()[r] = B.ck_creq[(int64_t)c * g.R + r];
     this->fill_fin();
     restore_arb(c);
@@ -839,29 +840,7 @@ __global__ void __launch_bounds__(32, 1) sim_arb_base_kernel(const __grid_consta
     S.arb_checkpoint(none);
   }
   S.run();
-  if (lane == 0) B.status[0] = S.status;
-  if (S.status != GMG_SIM_OK) return;
-  int32_t miss = 0;
-  for (int r = lane; r < S.g.R; r += 32) {
-    const int64_t c = S.creq()[r];
-    B.res_creq[r] = c;
-    miss += c > __ldg(S.g.deadline + r) ? 1 : 0;
-  }
-  miss = (int32_t)__reduce_add_sync(kFullMask, (unsigned)miss);
-  S.dv.write_peak(B.res_peak);
-  const int64_t makespan = S.dv.max_busy(S.g);
-  const int64_t score = warp_sum_i64(S.score);
-  if (lane == 0) {
-    int64_t* rs = B.res_scalars;
-    rs[0] = makespan;
-    rs[1] = S.vflag ? kI64Max : score;
-    rs[2] = S.vflag;
-    rs[3] = S.vop;
-    rs[4] = S.vdev;
-    rs[5] = S.vt;
-    rs[6] = miss;
-    rs[7] = S.ck;
-  }
+  write_base(S, B);
 }
 
 // Incremental candidates resumed from the arbitrated base snapshot.

@@ -27,6 +27,36 @@ __global__ void __launch_bounds__(128, kBlocksPerSM) sim_full_kernel(const __gri
   }
 }
 
+// Few candidates: two warps each, the sweep and the HBM accounting.
+template <bool kNarrow, bool kTypes, int kHot>
+__global__ void __launch_bounds__(64, 2 * kBlocksPerSM) sim_full_pair_kernel(const __grid_constant__ SimParams P) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int64_t slot = blockIdx.x;
+  const int64_t nslots = gridDim.x;
+  if (threadIdx.x < 32u) {
+    Sim<kNarrow, kFull, true, true, kTypes, kHot, !kNarrow, kSweep> S(P);
+    setup_slot(S, P, 0, slot, smem);
+    for (int64_t k = slot; k < P.K; k += nslots) {
+      S.row = P.place + k * P.ld;
+      S.reset_common();
+      if (S.row_has_bad_device(S.row)) S.status = GMG_SIM_BADDEV;
+      S.run();
+      S.hand_end();
+    }
+    leave_pair(S);
+  } else {
+    Sim<kNarrow, kFull, true, true, kTypes, kHot, !kNarrow, kAccount> S(P);
+    setup_slot(S, P, 0, slot, smem);
+    for (int64_t k = slot; k < P.K; k += nslots) {
+      S.row = P.place + k * P.ld;
+      S.reset_common();
+      S.account();
+      S.finish(k);
+      S.done();
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // sim_batch with the GMG staged in shared memory (sim_opts_t.gmg_staging = 1):
 // one CTA per SM of up to kStageMaxWarps warps.  Thread 0 copies the compact
@@ -142,6 +172,18 @@ const void* full_ptr_n(bool key, bool t32, bool types, bool hot) {
 const void* full_kernel_ptr(const DevGmg& g) {
   const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
   return g.D <= 32 ? full_ptr_n<true>(key, t32, types, hot) : full_ptr_n<false>(key, t32, types, hot);
+}
+// Two warps per candidate: graphs with 32-bit times.
+const void* full_pair_kernel_ptr(const DevGmg& g) {
+  const bool types = g.ntypes >= 2;
+  if (g.hot_ok)
+    return g.D <= 32 ? (const void*)sim_full_pair_kernel<true, false, kHotGlobal>
+                     : (const void*)sim_full_pair_kernel<false, false, kHotGlobal>;
+  if (g.D <= 32)
+    return types ? (const void*)sim_full_pair_kernel<true, true, kHotNone>
+                 : (const void*)sim_full_pair_kernel<true, false, kHotNone>;
+  return types ? (const void*)sim_full_pair_kernel<false, true, kHotNone>
+               : (const void*)sim_full_pair_kernel<false, false, kHotNone>;
 }
 
 }  // namespace gsim

@@ -19,11 +19,13 @@ namespace gsim {
 size_t select_rank_bytes();
 const void* full_kernel_ptr(const DevGmg& g);
 const void* inc_kernel_ptr(const DevGmg& g);
+const void* full_pair_kernel_ptr(const DevGmg& g);
+const void* inc_pair_kernel_ptr(const DevGmg& g);
 const void* full_staged_kernel_ptr();
-cudaError_t launch_full(const SimParams& P, int grid, int block, size_t smem, cudaStream_t st);
+cudaError_t launch_full(bool pair, const SimParams& P, int grid, int block, size_t smem, cudaStream_t st);
 cudaError_t launch_full_staged(const SimParams& P, int grid, int block, size_t smem, cudaStream_t st);
-cudaError_t launch_inc(const SimParams& P, int grid, int block, size_t smem, cudaStream_t st);
-cudaError_t launch_base(const SimParams& P, size_t smem, cudaStream_t st);
+cudaError_t launch_inc(bool pair, const SimParams& P, int grid, int block, size_t smem, cudaStream_t st);
+cudaError_t launch_base(bool pair, const SimParams& P, size_t smem, cudaStream_t st);
 cudaError_t set_smem_limits(int smem);
 cudaError_t launch_select(const int32_t* status, const int32_t* viol, const int64_t* score,
                           const int32_t* miss, int32_t K, int32_t mode, void* tmp, int nparts,
@@ -465,6 +467,7 @@ struct gmg_base {
 namespace {
 
 struct Launch {
+  bool pair;    // two warps per candidate (a block of its own)
   int wpb, grid;
   size_t smem;
   int64_t slots;
@@ -486,7 +489,7 @@ size_t smem_per_warp(const SimParams& P) {
   const size_t side = P.no_side ? 0 : 1;
   return align_up((size_t)P.pool * 9 + (size_t)P.qs * 8 + (size_t)P.ms * (8 + side) + (size_t)P.sortcap * (8 + side) + (size_t)P.opcap * 4,
                   16) +
-         (size_t)P.dev_bytes;
+         (size_t)P.dev_bytes + (size_t)P.pair_bytes;
 }
 
 // Shared bytes of accelerator state per warp: live bytes; peaks and a drain's
@@ -497,12 +500,18 @@ int dev_smem_bytes(int D, size_t tbytes) {
   return (int)align_up((size_t)D * 8 + (narrow ? (size_t)D * 72 : 32) + (size_t)D * tbytes, 16);
 }
 
+// Shared bytes that a candidate's two warps hand started ops over in: two
+// messages, the sweep's 48 words on the way from the pool to the lanes, and two
+// lists of ops.
+int pair_bytes(const SimParams& P) { return (int)align_up(2 * 48 + 8 * 48 + 2 * (size_t)P.opcap * 4, 16); }
+
 bool g_smem_set = false;
 
 // Slot layout and grid for K candidates of kind `inc`.
 int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& L) {
   const DevGmg& G = g->dg;
   const bool narrow = G.D <= 32;
+  L.pair = false;
   L.wpb = (o && o->warps_per_block > 0) ? o->warps_per_block : kDefaultWarpsPerBlock;
   if (L.wpb > 4) return GMG_EINVAL;
   SimParams& P = L.P;
@@ -553,6 +562,7 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
     big.ms = std::max(kSharedLogEntries, kSharedLogEntriesWide);
     big.dev_bytes = 32 + 24 * 256;
     big.no_side = 0;
+    big.pair_bytes = pair_bytes(big);
     if (set_smem_limits(4 * (int)smem_per_warp(big)) != cudaSuccess) return GMG_ECUDA;
     g_smem_set = true;
   }
@@ -567,6 +577,39 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
   P.g = G;
   return GMG_OK;
 }
+
+// Two warps per candidate where all candidates fit on the GPU at once that way
+// (and the caller has not set the warps per block): the sweep of a candidate
+// does not wait for its HBM accounting.  Graphs with 32-bit times.
+int plan_pair(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& L) {
+  const DevGmg& G = g->dg;
+  if (!G.t32 || (o && o->warps_per_block > 0)) return GMG_EINVAL;
+  const int rc = plan_launch(g, K, o, inc, L);
+  if (rc) return rc;
+  SimParams& P = L.P;
+  P.pair_bytes = pair_bytes(P);
+  L.pair = true;
+  L.wpb = 1;
+  L.smem = smem_per_warp(P);
+  const int sms = device_sms();
+  if (sms <= 0) return GMG_ECUDA;
+  int bps = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, inc ? inc_pair_kernel_ptr(G) : full_pair_kernel_ptr(G), 64,
+                                                    L.smem) != cudaSuccess)
+    return GMG_ECUDA;
+  if ((int64_t)K > (int64_t)sms * bps) return GMG_EINVAL;
+  // the scratch stays that of one warp per candidate (four to a block): enough
+  L.grid = std::max(K, 1);
+  L.slots = std::max(L.slots, (int64_t)L.grid);
+  return GMG_OK;
+}
+
+// Incremental candidates: two warps each if that holds them all, else one.
+int plan_inc(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L) {
+  const int rc = plan_pair(g, K, o, true, L);
+  return rc == GMG_EINVAL ? plan_launch(g, K, o, true, L) : rc;
+}
+int block_threads(const Launch& L) { return L.pair ? 64 : 32 * L.wpb; }
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
@@ -592,7 +635,6 @@ bool l1_path(const sim_opts_t* o) { return o && o->gmg_staging == GMG_STAGING_L1
 
 bool g_stage_smem_set = false;
 constexpr int64_t kStageSmallBytes = 16 << 10;
-constexpr int kStageFewCandidates = 32;
 
 // sim_batch with the GMG staged in shared memory: one CTA per SM with as many
 // warps (up to kStageMaxWarps) as fit beside the staged copy.
@@ -630,23 +672,25 @@ int plan_staged(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L) {
 }
 
 // Full placements with pure-latency transfers: the staged-GMG kernel when the
-// caller asks for it (an error if it cannot serve the graph) or by default
-// for small graphs and few candidates, else the L1 path.  *stg tells which.
+// caller asks for it (an error if it cannot serve the graph); by default two
+// warps per candidate while all candidates fit at once that way, beyond that the
+// staged kernel for small graphs, whose copy leaves the L1 cache to the
+// candidates' own arrays, else one warp per candidate.  *stg tells which.
+// (Measured, two warps / staged / one warp: the 50-op graph 55 / 65 / 67 us for
+// 256 candidates, - / 90 / 98 us for 4,096; the prefill graph, N = 3088, a 90 KB
+// copy, 1.41 / 1.80 / 1.84 ms for 14, 1.61 / 2.11 / 2.07 ms for 2,048, - / 3.39 /
+// 3.11 ms for 4,096.)
 int plan_full(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, bool* stg) {
   *stg = false;
-  if (l1_path(o)) return plan_launch(g, K, o, false, L);
-  // With compact records on both paths, staging pays where the copy leaves the
-  // L1 cache to the candidates' own arrays (prefill graph, N = 3088, a 90 KB
-  // copy: 1.82 against 1.84 ms for 14 candidates, 1.85 against 1.79 ms for 64,
-  // 3.58 against 3.23 ms for 4,096; the 50-op graph, 2 KB: 65.1 against 67.2 us
-  // for 256, 92 against 99 us for 4,096).
-  const bool small = stage_smem_bytes(g->dg.n, g->dg.n_edges) <= kStageSmallBytes || K <= kStageFewCandidates;
-  const int rc = staged(o) || small ? plan_staged(g, K, o, L) : GMG_EINVAL;
-  if (rc == GMG_OK) {
-    *stg = true;
-    return GMG_OK;
+  if (!staged(o)) {
+    const int rc = plan_pair(g, K, o, false, L);
+    if (rc != GMG_EINVAL) return rc;
   }
-  if (staged(o) || rc != GMG_EINVAL) return rc;
+  if (staged(o) || (!l1_path(o) && stage_smem_bytes(g->dg.n, g->dg.n_edges) <= kStageSmallBytes)) {
+    const int rc = plan_staged(g, K, o, L);
+    *stg = rc == GMG_OK;
+    if (staged(o) || rc != GMG_EINVAL) return rc;
+  }
   return plan_launch(g, K, o, false, L);
 }
 
@@ -816,6 +860,8 @@ int plan_base(const gmg* g, const sim_opts_t* o, BasePlan& B) {
   if (rc) return rc;
   L.wpb = 1;
   if (B.arb) L.P.dev_bytes = dev_smem_bytes(G.D, 8);  // the arbitrated base keeps 64-bit times
+  L.pair = !B.arb && G.t32;
+  if (L.pair) L.P.pair_bytes = pair_bytes(L.P);
   L.smem = smem_per_warp(L.P);
   if (B.arb) {
     B.A.smem_std = (int64_t)L.smem;
@@ -1086,7 +1132,7 @@ int sim_batch(const gmg_t* g, const uint8_t* d_place, int32_t K, int32_t ld, con
   const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   cudaError_t e = arb ? launch_arb_any(g, L, Q, nullptr, st)
                       : stg ? launch_full_staged(P, L.grid, 32 * L.wpb, L.smem, st)
-                            : launch_full(P, L.grid, 32 * L.wpb, L.smem, st);
+                            : launch_full(L.pair, P, L.grid, block_threads(L), L.smem, st);
   return e == cudaSuccess ? GMG_OK : GMG_ECUDA;
 }
 
@@ -1163,7 +1209,8 @@ extern "C" int sim_batch_noalloc(const gmg_t* g, const uint8_t* d_place, int32_t
   P.K = K;
   P.scratch = scratch;
   const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const cudaError_t e = arb ? launch_arb_any(g, L, Q, nullptr, st) : launch_full(P, L.grid, 32 * L.wpb, L.smem, st);
+  const cudaError_t e = arb ? launch_arb_any(g, L, Q, nullptr, st)
+                            : launch_full(false, P, L.grid, 32 * L.wpb, L.smem, st);
   return e == cudaSuccess ? GMG_OK : GMG_ECUDA;
 }
 
@@ -1232,7 +1279,7 @@ int base_create(const gmg_t* g, const uint8_t* d_base_place, const sim_opts_t* o
     b->ck = A.ck;
     e = launch_arb_base(g->dg.ntypes >= 2, A, B.L.smem, reinterpret_cast<cudaStream_t>(stream));
   } else {
-    e = launch_base(P, B.L.smem, reinterpret_cast<cudaStream_t>(stream));
+    e = launch_base(B.L.pair, P, B.L.smem, reinterpret_cast<cudaStream_t>(stream));
   }
   if (e != cudaSuccess) {
     delete b;
@@ -1275,7 +1322,7 @@ size_t inc_scratch_bytes(const gmg_t* g, int32_t K, const sim_opts_t* opts) {
     return need;
   }
   Launch L;
-  if (plan_launch(g, K, opts, true, L)) return 0;
+  if (plan_inc(g, K, opts, L)) return 0;
   return kCounterBytes + (size_t)L.slots * (size_t)L.P.slot_bytes;
 }
 
@@ -1356,7 +1403,7 @@ int sim_incremental(const gmg_t* g, const gmg_base_t* b, const int32_t* d_move_o
                                                                                                 : GMG_ECUDA;
   }
   Launch L;
-  rc = plan_launch(g, K, opts, true, L);
+  rc = plan_inc(g, K, opts, L);
   if (rc) return rc;
   SimParams& P = L.P;
   rc = take_counter(P, d_scratch, scratch_bytes, L, reinterpret_cast<cudaStream_t>(stream));
@@ -1368,7 +1415,7 @@ int sim_incremental(const gmg_t* g, const gmg_base_t* b, const int32_t* d_move_o
   P.move_off = d_move_off;
   P.move_op = d_move_op;
   P.move_dev = d_move_dev;
-  cudaError_t e = launch_inc(P, L.grid, 32 * L.wpb, L.smem, reinterpret_cast<cudaStream_t>(stream));
+  cudaError_t e = launch_inc(L.pair, P, L.grid, block_threads(L), L.smem, reinterpret_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? GMG_OK : GMG_ECUDA;
 }
 

@@ -8,158 +8,29 @@ namespace {
 // ---------------------------------------------------------------------------
 // sim_incremental: K move lists against the base.
 // ---------------------------------------------------------------------------
-template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
-__device__ void regen(Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>& S, uint32_t p);
+template <class S_>
+__device__ void regen(S_& S, uint32_t p);
 
-template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
-__device__ void inc_candidate(Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>& S, const SimParams& P, int64_t k, uint8_t* crow) {
-  using tm_t = typename Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>::tm_t;
+// The accounting's part of resuming candidate k at checkpoint c: the live and
+// peak bytes and the logged HBM events at T_c, repaired for the moves.
+template <class S_>
+__device__ __forceinline__ void resume_accounts(S_& S, const SimParams& P, int64_t k, int c) {
+  constexpr bool kKey = S_::kKeyed;
   const DevGmg& g = S.g;
   const DevBase& B = P.base;
   const unsigned lane = lane_id();
-  const int32_t m0 = P.move_off[k], m1 = P.move_off[k + 1];
-  const int32_t nm = m1 - m0;
-  const int words = (g.n + 31) >> 5;
-  for (int w = lane; w < words; w += 32) S.bits()[w] = 0u;
-  __syncwarp();
-  // Validate the move list; duplicates are found with the (zeroed) bitmap.
-  bool bad_range = false, dup = false;
-  for (int t = lane; t < nm; t += 32) {
-    const int32_t op = P.move_op[m0 + t];
-    const int dvc = P.move_dev[m0 + t];
-    if (op < 0 || op >= g.n || dvc >= g.D) {
-      bad_range = true;
-    } else {
-      const uint32_t b = 1u << (op & 31);
-      if (atomicOr(&S.bits()[op >> 5], b) & b) dup = true;
-    }
-  }
-  bad_range = __any_sync(kFullMask, bad_range);
-  dup = __any_sync(kFullMask, dup);
-  __syncwarp();
-  if (B.status[0] != GMG_SIM_OK) {
-    S.write_invalid(k, GMG_SIM_BADBASE);
-    return;
-  }
-  if (bad_range || dup) {
-    S.write_invalid(k, bad_range ? GMG_SIM_MOVE_RANGE : GMG_SIM_MOVE_DUP);
-    return;
-  }
-  // The candidate's placement = base + moves.
-  warp_copy16(crow, B.row, B.ld);
-  __syncwarp();
-  uint64_t t0 = kKeyMax;
-  for (int t = lane; t < nm; t += 32) {
-    const int32_t op = P.move_op[m0 + t];
-    const uint8_t dvc = P.move_dev[m0 + t];
-    crow[op] = dvc;
-    if (dvc != B.row[op]) {
-      const RelPred rp = op_relpred(g.ops, (uint32_t)op);
-      const uint4 ls = make_uint4(0u, 0u, rp.pred_off, rp.npred);
-      uint64_t tx;
-      if (ls.w == 0) {
-        tx = (uint64_t)rp.rel;
-      } else {
-        tx = kKeyMax;
-        for (uint32_t u = 0; u < ls.w; ++u) {
-          const uint64_t fp = (uint64_t)S.fb[__ldg(g.pred + ls.z + u) & kIdMask];
-          tx = fp < tx ? fp : tx;
-        }
-      }
-      t0 = tx < t0 ? tx : t0;
-    }
-  }
-  t0 = warp_min_u64(t0);
-  __syncwarp();
-  S.row = crow;
-  const DevOut& o = P.out;
-  if (t0 == kKeyMax) {
-    // No effective move: the base results.
-    const int64_t* rs = B.res_scalars;
-    if (lane == 0) {
-      o.makespan[k] = rs[0];
-      o.score[k] = rs[1];
-      o.status[k] = GMG_SIM_OK;
-      o.viol_flag[k] = (int32_t)rs[2];
-      o.viol_op[k] = (int32_t)rs[3];
-      o.viol_dev[k] = (int32_t)rs[4];
-      o.viol_time[k] = rs[5];
-      o.sla_miss[k] = (int32_t)rs[6];
-      o.events[k] = 0;
-    }
-    for (int d = lane; d < g.D; d += 32) o.peak[k * g.D + d] = B.res_peak[d];
-    if (o.req_done)
-      for (int r = lane; r < g.R; r += 32) o.req_done[k * g.R + r] = B.res_creq[r];
-    const int ts = S.trace_slot(k);
-    if (ts >= 0)
-      for (int x = lane; x < g.n; x += 32) {
-        o.trace_finish[(int64_t)ts * g.n + x] = B.fb[x];
-        o.trace_start[(int64_t)ts * g.n + x] =
-            B.fb[x] - S.dur_of((uint32_t)x, B.row[x], op_durbytes(g.ops, (uint32_t)x).x);
-      }
-    return;
-  }
-  S.T0 = (tm_t)t0;
-  // Latest recorded resume point at or before T0.
-  int best = -1;
-  for (int c = lane; c < B.nck; c += 32)
-    if (B.ck_time[c] <= S.T0) best = c;
-  const int c = __reduce_max_sync(kFullMask, best);
+  const uint8_t* crow = S.row;
+  const int32_t m0 = P.move_off[k], nm = P.move_off[k + 1] - m0;
   const int64_t* sc = B.ck_scalars + (int64_t)c * 8;
-  const int qsz = (int)sc[0];
   const int msz = (int)sc[7];
-  if (qsz > P.pend_cap - 32 || msz > P.mcap) {
-    S.write_invalid(k, GMG_SIM_QUEUE);
-    return;
-  }
-  // Restore the simulator state of checkpoint c.
+  using tm_t = typename S_::tm_t;
   S.Tc = (tm_t)B.ck_time[c];
   S.drained = (tm_t)sc[3];
-  S.rootptr = (int)sc[1];
-  S.load_root();
-  S.score = lane == 0 ? sc[2] : 0;  // lanes add up their ops' finishes
   S.vflag = (int32_t)sc[4];
   S.vt = sc[5];
   S.vop = (int32_t)(sc[6] >> 32);
   S.vdev = (int32_t)(sc[6] & 0xffffffff);
-  S.iters = 0;
-  S.nev = 0;
-  S.readypops = 0;
-  S.last_t = -1;
-  S.status = GMG_SIM_OK;
-  S.opn = 0;
-  S.dv.load(B.ck_dev + (int64_t)c * 3 * g.D);
-  for (int r = lane; r < g.R; r += 32) S.creq()[r] = B.ck_creq[(int64_t)c * g.R + r];
-  // ops started before T_c are those with base ready time < T_c: they keep
-  // their base finish; the others start with no finish time
-  S.fill_fin();
-  // READY keys at T_c (the pool first, the others to the heap); a moved op's key is recomputed (its inputs' transfer
-  // times change; its predecessors all finished before T_c).
-  constexpr int kHeld = kNarrow ? 32 : kReadyPoolWide;
-  if constexpr (kNarrow) S.pd.r = S.pd.e = Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>::kNever;
-  for (int x = lane; x < qsz; x += 32) {
-    uint64_t key = B.ck_qkey[(int64_t)c * B.ckq + x];
-    const uint32_t op = S.rq.op(key);
-    if (crow[op] != B.row[op]) {
-      const int dx = crow[op];
-      const RelPred rp = op_relpred(g.ops, op);
-      const uint4 ls = make_uint4(0u, 0u, rp.pred_off, rp.npred);
-      int64_t rx = rp.rel;
-      for (uint32_t u = 0; u < ls.w; ++u) {
-        const uint32_t p = __ldg(g.pred + ls.z + u) & kIdMask;
-        const int dp = crow[p];
-        int64_t a = S.fb[p];
-        if (dp != dx) a += S.xfer(dp, dx, op_durbytes(g.ops, p).y, op_xqsucc(g.ops, p).xq);
-        rx = a > rx ? a : rx;
-      }
-      key = S.rq.make((tm_t)rx, op, (tm_t)S.dur_of(op, dx, op_durbytes(g.ops, op).x));
-    }
-    if (x >= kHeld) *S.q.kp(x - kHeld) = key;
-    else if constexpr (kNarrow) S.hold_op((tm_t)S.rq.time(key), op);
-    else S.pool[x] = key;
-  }
-  S.q.size = qsz > kHeld ? qsz - kHeld : 0;
-  if constexpr (!kNarrow) S.empty_pool(qsz < kHeld ? qsz : kHeld);
+  S.dv.load_bytes(B.ck_dev + (int64_t)c * 3 * g.D);
   // Logged HBM events at T_c, except those of an op p with a moved
   // successor: the receiving accelerators and last consumers of p's output
   // changed (its receive allocations and releases all happen at times
@@ -236,17 +107,165 @@ __device__ void inc_candidate(Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>& S, c
       }
     }
   }
+}
+
+template <class S_>
+__device__ __forceinline__ bool inc_candidate(S_& S, const SimParams& P, int64_t k, uint8_t* crow) {
+  constexpr bool kNarrow = !S_::kPooled;
+  using tm_t = typename S_::tm_t;
+  const DevGmg& g = S.g;
+  const DevBase& B = P.base;
+  const unsigned lane = lane_id();
+  const int32_t m0 = P.move_off[k], m1 = P.move_off[k + 1];
+  const int32_t nm = m1 - m0;
+  const int words = (g.n + 31) >> 5;
+  for (int w = lane; w < words; w += 32) S.bits()[w] = 0u;
+  __syncwarp();
+  // Validate the move list; duplicates are found with the (zeroed) bitmap.
+  bool bad_range = false, dup = false;
+  for (int t = lane; t < nm; t += 32) {
+    const int32_t op = P.move_op[m0 + t];
+    const int dvc = P.move_dev[m0 + t];
+    if (op < 0 || op >= g.n || dvc >= g.D) {
+      bad_range = true;
+    } else {
+      const uint32_t b = 1u << (op & 31);
+      if (atomicOr(&S.bits()[op >> 5], b) & b) dup = true;
+    }
+  }
+  bad_range = __any_sync(kFullMask, bad_range);
+  dup = __any_sync(kFullMask, dup);
+  __syncwarp();
+  if (B.status[0] != GMG_SIM_OK) {
+    S.write_invalid(k, GMG_SIM_BADBASE);
+    return false;
+  }
+  if (bad_range || dup) {
+    S.write_invalid(k, bad_range ? GMG_SIM_MOVE_RANGE : GMG_SIM_MOVE_DUP);
+    return false;
+  }
+  // The candidate's placement = base + moves.
+  warp_copy16(crow, B.row, B.ld);
+  __syncwarp();
+  uint64_t t0 = kKeyMax;
+  for (int t = lane; t < nm; t += 32) {
+    const int32_t op = P.move_op[m0 + t];
+    const uint8_t dvc = P.move_dev[m0 + t];
+    crow[op] = dvc;
+    if (dvc != B.row[op]) {
+      const RelPred rp = op_relpred(g.ops, (uint32_t)op);
+      const uint4 ls = make_uint4(0u, 0u, rp.pred_off, rp.npred);
+      uint64_t tx;
+      if (ls.w == 0) {
+        tx = (uint64_t)rp.rel;
+      } else {
+        tx = kKeyMax;
+        for (uint32_t u = 0; u < ls.w; ++u) {
+          const uint64_t fp = (uint64_t)S.fb[__ldg(g.pred + ls.z + u) & kIdMask];
+          tx = fp < tx ? fp : tx;
+        }
+      }
+      t0 = tx < t0 ? tx : t0;
+    }
+  }
+  t0 = warp_min_u64(t0);
+  __syncwarp();
+  S.row = crow;
+  const DevOut& o = P.out;
+  if (t0 == kKeyMax) {
+    // No effective move: the base results.
+    const int64_t* rs = B.res_scalars;
+    if (lane == 0) {
+      o.makespan[k] = rs[0];
+      o.score[k] = rs[1];
+      o.status[k] = GMG_SIM_OK;
+      o.viol_flag[k] = (int32_t)rs[2];
+      o.viol_op[k] = (int32_t)rs[3];
+      o.viol_dev[k] = (int32_t)rs[4];
+      o.viol_time[k] = rs[5];
+      o.sla_miss[k] = (int32_t)rs[6];
+      o.events[k] = 0;
+    }
+    for (int d = lane; d < g.D; d += 32) o.peak[k * g.D + d] = B.res_peak[d];
+    if (o.req_done)
+      for (int r = lane; r < g.R; r += 32) o.req_done[k * g.R + r] = B.res_creq[r];
+    const int ts = S.trace_slot(k);
+    if (ts >= 0)
+      for (int x = lane; x < g.n; x += 32) {
+        o.trace_finish[(int64_t)ts * g.n + x] = B.fb[x];
+        o.trace_start[(int64_t)ts * g.n + x] =
+            B.fb[x] - S.dur_of((uint32_t)x, B.row[x], op_durbytes(g.ops, (uint32_t)x).x);
+      }
+    return false;
+  }
+  S.T0 = (tm_t)t0;
+  // Latest recorded resume point at or before T0.
+  int best = -1;
+  for (int c = lane; c < B.nck; c += 32)
+    if (B.ck_time[c] <= S.T0) best = c;
+  const int c = __reduce_max_sync(kFullMask, best);
+  const int64_t* sc = B.ck_scalars + (int64_t)c * 8;
+  const int qsz = (int)sc[0];
+  const int msz = (int)sc[7];
+  if (qsz > P.pend_cap - 32 || msz > P.mcap) {
+    S.write_invalid(k, GMG_SIM_QUEUE);
+    return false;
+  }
+  // Restore the simulator state of checkpoint c.
+  S.Tc = (tm_t)B.ck_time[c];
+  S.rootptr = (int)sc[1];
+  S.load_root();
+  S.score = lane == 0 ? sc[2] : 0;  // lanes add up their ops' finishes
+  S.iters = 0;
+  S.nev = 0;
+  S.readypops = 0;
+  S.last_t = -1;
+  S.status = GMG_SIM_OK;
+  S.opn = 0;
+  S.dv.load_free(B.ck_dev + (int64_t)c * 3 * g.D);
+  for (int r = lane; r < g.R; r += 32) S.creq()[r] = B.ck_creq[(int64_t)c * g.R + r];
+  // ops started before T_c are those with base ready time < T_c: they keep
+  // their base finish; the others start with no finish time
+  S.fill_fin();
+  if constexpr (S_::kRoleOf == kSweep) S.hand_over(k, kHandResume, c);
+  // READY keys at T_c (the pool first, the others to the heap); a moved op's key is recomputed (its inputs' transfer
+  // times change; its predecessors all finished before T_c).
+  constexpr int kHeld = kNarrow ? 32 : kReadyPoolWide;
+  if constexpr (kNarrow) S.pd.r = S.pd.e = S_::kNever;
+  for (int x = lane; x < qsz; x += 32) {
+    uint64_t key = B.ck_qkey[(int64_t)c * B.ckq + x];
+    const uint32_t op = S.rq.op(key);
+    if (crow[op] != B.row[op]) {
+      const int dx = crow[op];
+      const RelPred rp = op_relpred(g.ops, op);
+      const uint4 ls = make_uint4(0u, 0u, rp.pred_off, rp.npred);
+      int64_t rx = rp.rel;
+      for (uint32_t u = 0; u < ls.w; ++u) {
+        const uint32_t p = __ldg(g.pred + ls.z + u) & kIdMask;
+        const int dp = crow[p];
+        int64_t a = S.fb[p];
+        if (dp != dx) a += S.xfer(dp, dx, op_durbytes(g.ops, p).y, op_xqsucc(g.ops, p).xq);
+        rx = a > rx ? a : rx;
+      }
+      key = S.rq.make((tm_t)rx, op, (tm_t)S.dur_of(op, dx, op_durbytes(g.ops, op).x));
+    }
+    if (x >= kHeld) *S.q.kp(x - kHeld) = key;
+    else if constexpr (kNarrow) S.hold_op((tm_t)S.rq.time(key), op);
+    else S.pool[x] = key;
+  }
+  S.q.size = qsz > kHeld ? qsz - kHeld : 0;
+  if constexpr (!kNarrow) S.empty_pool(qsz < kHeld ? qsz : kHeld);
   S.q.heapify();
-  S.run();
-  S.finish(k);
+  if constexpr (S_::kRoleOf == kBoth) resume_accounts(S, P, k, c);
+  return true;
 }
 
 // HBM events of op p (finished before the resume point) under the candidate
 // placement: receive copies on every remote accelerator of its successors
 // (allocated at f_p), and the releases that are already determined because
-// every listed consumer on that accelerator has finished.
-template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
-__device__ void regen(Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>& S, uint32_t p) {
+// every listed consumer on that accelerator started before the resume point.
+template <class S_>
+__device__ void regen(S_& S, uint32_t p) {
   const DevGmg& g = S.g;
   const unsigned lane = lane_id();
   const int64_t fp = S.fb[p];
@@ -286,11 +305,11 @@ __device__ void regen(Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>& S, uint32_t 
       for (uint32_t u = 0; u < nl; ++u) {
         const uint32_t c = __ldg(lst + u);
         if (S.row[c] != du) continue;
-        const int64_t fc = S.fin(c);
-        if (fc <= 0) {  // not started yet
+        if (S.rb[c] >= S.Tc) {  // not started by then
           rel = false;
           break;
         }
+        const int64_t fc = S.fb[c];
         tr = fc > tr ? fc : tr;
       }
     }
@@ -304,9 +323,8 @@ __device__ void regen(Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot>& S, uint32_t 
     if (t < nl) {
       const uint32_t c = __ldg(lst + t);
       if (S.row[c] == dp) {
-        const int64_t fc = S.fin(c);
-        if (fc <= 0) pending = true;
-        else mx = (uint64_t)fc > mx ? (uint64_t)fc : mx;
+        if (S.rb[c] >= S.Tc) pending = true;
+        else mx = (uint64_t)S.fb[c] > mx ? (uint64_t)S.fb[c] : mx;
       }
     }
   }
@@ -325,7 +343,49 @@ __global__ void __launch_bounds__(128, kBlocksPerSM) sim_inc_kernel(const __grid
   S.rb = P.base.rb;
   S.fb = P.base.fb;
   uint8_t* crow = P.scratch + slot * P.slot_bytes + P.off_row;
-  for (int64_t k = take_candidate(P.next_k); k < P.K; k = take_candidate(P.next_k)) inc_candidate(S, P, k, crow);
+  for (int64_t k = take_candidate(P.next_k); k < P.K; k = take_candidate(P.next_k)) {
+    if (!inc_candidate(S, P, k, crow)) continue;
+    S.run();
+    S.finish(k);
+  }
+}
+
+// Few candidates: two warps each, the sweep and the HBM accounting.
+template <bool kNarrow, bool kTypes, int kHot>
+__global__ void __launch_bounds__(64, 2 * kBlocksPerSM) sim_inc_pair_kernel(const __grid_constant__ SimParams P) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int64_t slot = blockIdx.x;
+  uint8_t* crow = P.scratch + slot * P.slot_bytes + P.off_row;
+  if (threadIdx.x < 32u) {
+    Sim<kNarrow, kInc, true, true, kTypes, kHot, !kNarrow, kSweep> S(P);
+    setup_slot(S, P, 0, slot, smem);
+    S.rb = P.base.rb;
+    S.fb = P.base.fb;
+    for (int64_t k = take_candidate(P.next_k); k < P.K; k = take_candidate(P.next_k)) {
+      if (!inc_candidate(S, P, k, crow)) continue;  // written; the other warp has not heard of it
+      S.run();
+      S.hand_end();
+    }
+    S.hand_over(0, kHandQuit, 0);
+    leave_pair(S);
+  } else {
+    Sim<kNarrow, kInc, true, true, kTypes, kHot, !kNarrow, kAccount> S(P);
+    setup_slot(S, P, 0, slot, smem);
+    S.rb = P.base.rb;
+    S.fb = P.base.fb;
+    S.row = crow;
+    while (true) {
+      Hand h;
+      if (S.take_hand(h) & kHandQuit) break;
+      S.status = GMG_SIM_OK;
+      S.opn = 0;
+      resume_accounts(S, P, h.t, h.n);
+      S.free_hand();
+      S.account();
+      S.finish(h.t);
+      S.done();
+    }
+  }
 }
 
 }  // namespace
@@ -348,6 +408,18 @@ const void* inc_ptr_n(bool key, bool t32, bool types, bool hot) {
 const void* inc_kernel_ptr(const DevGmg& g) {
   const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
   return g.D <= 32 ? inc_ptr_n<true>(key, t32, types, hot) : inc_ptr_n<false>(key, t32, types, hot);
+}
+// Two warps per candidate: graphs with 32-bit times.
+const void* inc_pair_kernel_ptr(const DevGmg& g) {
+  const bool types = g.ntypes >= 2;
+  if (g.hot_ok)
+    return g.D <= 32 ? (const void*)sim_inc_pair_kernel<true, false, kHotGlobal>
+                     : (const void*)sim_inc_pair_kernel<false, false, kHotGlobal>;
+  if (g.D <= 32)
+    return types ? (const void*)sim_inc_pair_kernel<true, true, kHotNone>
+                 : (const void*)sim_inc_pair_kernel<true, false, kHotNone>;
+  return types ? (const void*)sim_inc_pair_kernel<false, true, kHotNone>
+               : (const void*)sim_inc_pair_kernel<false, false, kHotNone>;
 }
 
 }  // namespace gsim

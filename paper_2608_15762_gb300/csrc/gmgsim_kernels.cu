@@ -8,55 +8,62 @@ namespace {
 // ---------------------------------------------------------------------------
 // base_create: simulate the base placement once, recording resume points.
 // ---------------------------------------------------------------------------
+// The base placement is kept for the candidates.
+__device__ __forceinline__ void copy_base_row(const SimParams& P) {
+  const DevBase& B = P.base;
+  for (int c = (int)lane_id() * 16; c < B.ld; c += 512)
+    *reinterpret_cast<uint4*>(B.row + c) = *reinterpret_cast<const uint4*>(P.place + c);
+  __syncwarp();
+}
+
+template <class S_>
+__device__ __forceinline__ void sweep_base(S_& S, const SimParams& P) {
+  S.row = P.place;
+  S.reset_common();
+  if (S.row_has_bad_device(P.place)) S.status = GMG_SIM_BADDEV;
+  S.ck = 0;
+  S.next_ck = 0;
+  // checkpoint 0: the initial state, valid for every resume time >= 0
+  if (S.status == GMG_SIM_OK) S.maybe_checkpoint(0);
+  S.run();
+}
+
 template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
 __global__ void __launch_bounds__(32, 1) sim_base_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
   Sim<kNarrow, kBase, kKey, kT32, kTypes, kHot> S(P);
   setup_slot(S, P, 0, 0, smem);
-  const DevBase& B = P.base;
-  const unsigned lane = lane_id();
   warp_prefetch_l2(P.g.ws, P.g.ws_bytes);
-  // keep a copy of the base placement for the candidates
-  for (int c = lane * 16; c < B.ld; c += 512)
-    *reinterpret_cast<uint4*>(B.row + c) = *reinterpret_cast<const uint4*>(P.place + c);
-  for (int c = lane; c < B.nck; c += 32) B.ck_time[c] = kI64Max;
-  S.row = P.place;
+  copy_base_row(P);
+  for (int c = lane_id(); c < P.base.nck; c += 32) P.base.ck_time[c] = kI64Max;
   __syncwarp();
-  if (S.row_has_bad_device(P.place)) {
-    if (lane == 0) B.status[0] = GMG_SIM_BADDEV;
-    return;
-  }
-  S.reset_common();
-  S.ck = 0;
-  S.next_ck = 0;
-  // checkpoint 0: the initial state, valid for every resume time >= 0
-  S.maybe_checkpoint(0);
-  S.run();
-  if (lane == 0) B.status[0] = S.status;
-  if (S.status != GMG_SIM_OK) return;
-  int32_t miss = 0;
-  for (int r = lane; r < S.g.R; r += 32) {
-    const int64_t c = S.creq()[r];
-    B.res_creq[r] = c;
-    miss += c > __ldg(S.g.deadline + r) ? 1 : 0;
-  }
-  miss = (int32_t)__reduce_add_sync(kFullMask, (unsigned)miss);
-  S.dv.write_peak(B.res_peak);
-  const int64_t makespan = S.dv.max_busy(S.g);
-  const int64_t score = warp_sum_i64(S.score);
-  if (lane == 0) {
-    int64_t* rs = B.res_scalars;
-    rs[0] = makespan;
-    rs[1] = S.vflag ? kI64Max : score;
-    rs[2] = S.vflag;
-    rs[3] = S.vop;
-    rs[4] = S.vdev;
-    rs[5] = S.vt;
-    rs[6] = miss;
-    rs[7] = S.ck;
-  }
+  sweep_base(S, P);
+  write_base(S, P.base);
 }
 
+// The same by two warps, the sweep and the HBM accounting (32-bit times).
+template <bool kNarrow, bool kTypes, int kHot>
+__global__ void __launch_bounds__(64, 1) sim_base_pair_kernel(const __grid_constant__ SimParams P) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  if (threadIdx.x < 32) {
+    Sim<kNarrow, kBase, true, true, kTypes, kHot, !kNarrow, kSweep> S(P);
+    setup_slot(S, P, 0, 0, smem);
+    sweep_base(S, P);
+    S.hand_end();
+    leave_pair(S);
+  } else {
+    Sim<kNarrow, kBase, true, true, kTypes, kHot, !kNarrow, kAccount> S(P);
+    setup_slot(S, P, 0, 0, smem);
+    warp_prefetch_l2(P.g.ws, P.g.ws_bytes);
+    for (int c = lane_id(); c < P.base.nck; c += 32) P.base.ck_time[c] = kI64Max;
+    copy_base_row(P);
+    S.row = P.place;
+    S.reset_common();
+    S.account();
+    write_base(S, P.base);
+    S.done();
+  }
+}
 
 // ---------------------------------------------------------------------------
 // select_best (Algorithm 1, BestRecordedCandidateResult): block argmin of
@@ -135,7 +142,9 @@ __global__ void __launch_bounds__(256) select_final_kernel(const Rank* part, int
 size_t select_rank_bytes() { return sizeof(Rank); }
 
 const void* full_kernel_ptr(const DevGmg& g);  // gmgsim_full.cu
-const void* inc_kernel_ptr(const DevGmg& g);   // gmgsim_inc.cu
+const void* full_pair_kernel_ptr(const DevGmg& g);
+const void* inc_kernel_ptr(const DevGmg& g);  // gmgsim_inc.cu
+const void* inc_pair_kernel_ptr(const DevGmg& g);
 
 // Instances by (at most 32 accelerators, accelerator id in the event key,
 // 32-bit times, accelerator types; compact records wherever the graph has
@@ -156,6 +165,18 @@ const void* base_kernel_ptr(const DevGmg& g) {
   const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
   return g.D <= 32 ? base_ptr_n<true>(key, t32, types, hot) : base_ptr_n<false>(key, t32, types, hot);
 }
+// Two warps: graphs with 32-bit times.
+const void* base_pair_kernel_ptr(const DevGmg& g) {
+  const bool types = g.ntypes >= 2;
+  if (g.hot_ok)
+    return g.D <= 32 ? (const void*)sim_base_pair_kernel<true, false, kHotGlobal>
+                     : (const void*)sim_base_pair_kernel<false, false, kHotGlobal>;
+  if (g.D <= 32)
+    return types ? (const void*)sim_base_pair_kernel<true, true, kHotNone>
+                 : (const void*)sim_base_pair_kernel<true, false, kHotNone>;
+  return types ? (const void*)sim_base_pair_kernel<false, true, kHotNone>
+               : (const void*)sim_base_pair_kernel<false, false, kHotNone>;
+}
 
 cudaError_t set_smem_limits(int smem) {
   DevGmg g{};
@@ -165,7 +186,8 @@ cudaError_t set_smem_limits(int smem) {
     g.t32 = (c >> 2) & 1;
     g.ntypes = c & 8 ? 2 : 0;
     g.hot_ok = (c >> 4) & 1;
-    const void* fns[] = {full_kernel_ptr(g), inc_kernel_ptr(g), base_kernel_ptr(g)};
+    const void* fns[] = {full_kernel_ptr(g),      inc_kernel_ptr(g),      base_kernel_ptr(g),
+                         full_pair_kernel_ptr(g), inc_pair_kernel_ptr(g), base_pair_kernel_ptr(g)};
     for (const void* f : fns) {
       const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
       if (e != cudaSuccess) return e;
@@ -182,19 +204,17 @@ static cudaError_t launch_ptr(const void* fn, const SimParams& P, int grid, int 
   return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, st);
 }
 
-cudaError_t launch_full(const SimParams& P, int grid, int block, size_t smem, cudaStream_t st) {
-  return launch_ptr(full_kernel_ptr(P.g), P, grid, block,
-                    smem, st);
+// pair: two warps per candidate, a block of their own.
+cudaError_t launch_full(bool pair, const SimParams& P, int grid, int block, size_t smem, cudaStream_t st) {
+  return launch_ptr(pair ? full_pair_kernel_ptr(P.g) : full_kernel_ptr(P.g), P, grid, block, smem, st);
 }
 
-cudaError_t launch_inc(const SimParams& P, int grid, int block, size_t smem, cudaStream_t st) {
-  return launch_ptr(inc_kernel_ptr(P.g), P, grid, block,
-                    smem, st);
+cudaError_t launch_inc(bool pair, const SimParams& P, int grid, int block, size_t smem, cudaStream_t st) {
+  return launch_ptr(pair ? inc_pair_kernel_ptr(P.g) : inc_kernel_ptr(P.g), P, grid, block, smem, st);
 }
 
-cudaError_t launch_base(const SimParams& P, size_t smem, cudaStream_t st) {
-  return launch_ptr(base_kernel_ptr(P.g), P, 1, 32, smem,
-                    st);
+cudaError_t launch_base(bool pair, const SimParams& P, size_t smem, cudaStream_t st) {
+  return launch_ptr(pair ? base_pair_kernel_ptr(P.g) : base_kernel_ptr(P.g), P, 1, pair ? 64 : 32, smem, st);
 }
 
 cudaError_t launch_select(const int32_t* status, const int32_t* viol, const int64_t* score,

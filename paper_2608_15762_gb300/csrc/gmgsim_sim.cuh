@@ -310,14 +310,17 @@ struct Devices {
     pk = kPkShared ? lv + D : pk_global;  // a compile-time fact of the instance
     fr = reinterpret_cast<TM*>(lv + (kPkShared ? 2 * D : D));
   }
-  __device__ void reset(const DevGmg& g) {
+  __device__ void reset_free(const DevGmg& g) {
+    for (int d = lane_id(); d < D; d += 32) fr[d] = (TM)g.avail0[d];
+    __syncwarp();
+  }
+  __device__ void reset_bytes(const DevGmg& g) {
     const unsigned l = lane_id();
     for (int d = l; d < D; d += 32) {
       lv[d] = g.base[d];
       pk[d] = g.base[d];
       if (kPkShared)
         for (int w = 0; w < 4; ++w) reinterpret_cast<uint4*>(acc)[4 * d + w] = make_uint4(0u, 0u, 0u, 0u);
-      fr[d] = (TM)g.avail0[d];
     }
     __syncwarp();
   }
@@ -339,18 +342,21 @@ struct Devices {
     if (lane_id() == 0) lv[d] = v;
     __syncwarp();
   }
-  __device__ void save(int64_t* dst) const {
-    const unsigned l = lane_id();
-    for (int d = l; d < D; d += 32) {
-      dst[d] = (int64_t)fr[d];
+  __device__ void save_free(int64_t* dst) const {
+    for (int d = lane_id(); d < D; d += 32) dst[d] = (int64_t)fr[d];
+  }
+  __device__ void save_bytes(int64_t* dst) const {
+    for (int d = lane_id(); d < D; d += 32) {
       dst[D + d] = lv[d];
-      dst[2 * D + d] = pk[d];
+      dst[2 * D + d] = kPkShared ? pk[d] : __ldcg(pk + d);
     }
   }
-  __device__ void load(const int64_t* src) {
-    const unsigned l = lane_id();
-    for (int d = l; d < D; d += 32) {
-      fr[d] = (TM)src[d];
+  __device__ void load_free(const int64_t* src) {
+    for (int d = lane_id(); d < D; d += 32) fr[d] = (TM)src[d];
+    __syncwarp();
+  }
+  __device__ void load_bytes(const int64_t* src) {
+    for (int d = lane_id(); d < D; d += 32) {
       lv[d] = src[D + d];
       pk[d] = src[2 * D + d];
       if (kPkShared)
@@ -395,7 +401,7 @@ __device__ __forceinline__ WarpSmem carve_smem(uint8_t* smem, const SimParams& P
   const size_t side = P.no_side ? 0 : 1;
   const size_t head = align16((size_t)P.pool * 9 + (size_t)P.qs * 8 + (size_t)P.ms * (8 + side) +
                               (size_t)P.sortcap * (8 + side) + (size_t)P.opcap * 4);
-  const size_t per = head + (size_t)P.dev_bytes;
+  const size_t per = head + (size_t)P.dev_bytes + (size_t)P.pair_bytes;
   uint8_t* b = smem + per * wib;
   WarpSmem w;
   w.pool = reinterpret_cast<uint64_t*>(b);
@@ -426,15 +432,53 @@ __device__ __forceinline__ WarpSmem carve_smem(uint8_t* smem, const SimParams& P
 // read-only path, kHotShared from the CTA's shared-memory copy (staged by
 // sim_full_staged_kernel).
 constexpr int kHotNone = 0, kHotGlobal = 1, kHotShared = 2;
+// kRole: a candidate may have two warps (few candidates: what counts is then the
+// time of one simulation, and nothing in the sweep depends on the HBM
+// accounting).  kSweep starts the ops and hands them over in batches, kAccount
+// generates and applies their HBM events and writes the results; kBoth does
+// both in one warp.
+constexpr int kBoth = 0, kSweep = 1, kAccount = 2;
+
+// What the sweep hands over: n started ops (in the buffer of the same index) and
+// what to do once their events are generated.
+struct Hand {
+  int64_t t;       // drain limit, time of the checkpoint, or the candidate
+  int64_t score, nev;
+  int32_t n, flags;
+  int32_t iters, status;
+  int32_t ck, pad;
+};
+constexpr int kHandDrain = 1, kHandEnd = 2, kHandCheckpoint = 4, kHandKeep = 8, kHandResume = 16, kHandQuit = 32;
+
+// Named barriers of a pair, a block of 64 threads: full 0, full 1, empty 0, empty
+// 1.  The ids are immediates: an id in a register would make every block claim
+// all 16 barriers, and an SM has 64 (measured: 4 blocks instead of 14).
+__device__ __forceinline__ void pair_sync(int id) {
+  __syncwarp();
+  if (id == 0) asm volatile("barrier.sync 0, 64;" ::: "memory");
+  else if (id == 1) asm volatile("barrier.sync 1, 64;" ::: "memory");
+  else if (id == 2) asm volatile("barrier.sync 2, 64;" ::: "memory");
+  else asm volatile("barrier.sync 3, 64;" ::: "memory");
+}
+__device__ __forceinline__ void pair_arrive(int id) {
+  __threadfence_block();
+  __syncwarp();
+  if (id == 0) asm volatile("barrier.arrive 0, 64;" ::: "memory");
+  else if (id == 1) asm volatile("barrier.arrive 1, 64;" ::: "memory");
+  else if (id == 2) asm volatile("barrier.arrive 2, 64;" ::: "memory");
+  else asm volatile("barrier.arrive 3, 64;" ::: "memory");
+}
+
 template <bool kNarrow, int kMode, bool kKey, bool kT32 = false, bool kTypes = false, int kHot = kHotNone,
-          bool kPool = !kNarrow>
+          bool kPool = !kNarrow, int kRole = kBoth>
 struct Sim {
   static_assert(kHot == kHotNone || (kT32 && !kTypes), "compact records: 32-bit times, one type");
   using tm_t = typename std::conditional<kT32, int32_t, int64_t>::type;
   const SimParams& P;
   const DevGmg& g;
   static constexpr int kSlots = kReadyPoolWide / 32;  // pool slots per lane (kPool)
-  static constexpr bool kCompact = kHot != kHotNone;
+  static constexpr bool kCompact = kHot != kHotNone, kKeyed = kKey, kPooled = kPool;
+  static constexpr int kRoleOf = kRole;
   static constexpr tm_t kNever = (tm_t)(~(typename std::make_unsigned<tm_t>::type)0 >> 1);
   struct Pending {
     tm_t r, e, dur;  // ready time, earliest finish (both kNever: empty), duration
@@ -447,13 +491,17 @@ struct Sim {
   Pending pd;       // !kPool: this lane's pending op
   uint64_t* pool;   // kPool: shared [32 * kSlots], pending READY keys (kKeyMax = empty)
   uint8_t* fstk;    // shared [32 * kSlots]: the empty slots, a stack of nfree
+  uint64_t* bounce; // kPool: shared [48], a batch's keys and slots on their way to its lanes (the sort
+                    // area, free between drains; of a pair's sweep its own)
   int nfree;
   MemLog log;
   uint64_t* sortk;
   uint8_t* sortd;
   static constexpr int kWindows = 4;
   tm_t drained;     // every event before this time is applied, none after it
-  uint32_t* oplog;  // ops started since the last HBM-event generation
+  uint32_t* oplog;  // ops started since the last HBM-event generation (a pair: two buffers, oplog and hands of index hb)
+  Hand* hands;      // shared [2]
+  int hb;
   int opn;
   Devices<kNarrow, tm_t> dv;
   const uint8_t* row;
@@ -606,23 +654,28 @@ struct Sim {
 
   __device__ void reset_common() {
     const unsigned lane = lane_id();
-    zero_fin();
-    for (int r = lane; r < g.R; r += 32) creq()[r] = 0;
-    dv.reset(g);
-    q.size = 0;
-    if constexpr (kPool) empty_pool(0);
-    else pd.r = pd.e = kNever;
-    log.n = 0;
-    drained = 0;
+    if constexpr (kRole != kAccount) {
+      zero_fin();
+      for (int r = lane; r < g.R; r += 32) creq()[r] = 0;
+      dv.reset_free(g);
+      q.size = 0;
+      if constexpr (kPool) empty_pool(0);
+      else pd.r = pd.e = kNever;
+      rootptr = 0;
+      load_root();
+      score = 0;
+      iters = nev = readypops = 0;
+      last_t = -1;
+    }
+    if constexpr (kRole != kSweep) {
+      dv.reset_bytes(g);
+      log.n = 0;
+      drained = 0;
+      vflag = 0;
+      vop = vdev = -1;
+      vt = -1;
+    }
     opn = 0;
-    rootptr = 0;
-    load_root();
-    score = 0;
-    iters = nev = readypops = 0;
-    last_t = -1;
-    vflag = 0;
-    vop = vdev = -1;
-    vt = -1;
     status = GMG_SIM_OK;
     __syncwarp();
   }
@@ -1233,6 +1286,7 @@ struct Sim {
   }
 
   __device__ void maybe_checkpoint(int64_t next_t, uint64_t held = kKeyMax);
+  __device__ void save_accounts(int c, int64_t tn, bool keep);
 
   // -------------------------------------------------------------------------
   // The event loop (Sec. 3.3.3), many READY keys at a time.  Let lim be the
@@ -1265,6 +1319,75 @@ struct Sim {
       q.pop();
     }
   }
+  // ---- a candidate's two warps ------------------------------------------------
+  // The sweep owns buffer hb; handing it over, it waits until the other one is
+  // free (two batches ahead at most).
+  __device__ __forceinline__ void hand_over(int64_t t, int flags, int n) {
+    if (lane_id() == 0) {
+      Hand& h = hands[hb];
+      h.t = t;
+      h.flags = flags;
+      h.n = n;
+      h.ck = ck;
+    }
+    pair_arrive(hb);
+    opn = 0;
+    if (flags & kHandQuit) return;
+    hb ^= 1;
+    oplog += hb ? P.opcap : -P.opcap;
+    pair_sync(2 + hb);
+  }
+  // The candidate's end: the other warp finishes it from these results.
+  __device__ __forceinline__ void hand_end() {
+    const int64_t sc = warp_sum_i64(score), ne = warp_sum_i64(nev);
+    if (lane_id() == 0) {
+      Hand& h = hands[hb];
+      h.t = kI64Max;
+      h.flags = kHandEnd;
+      h.n = opn;
+      h.score = sc;
+      h.nev = ne;
+      h.iters = iters;
+      h.status = status;
+    }
+    pair_arrive(hb);
+    pair_sync(2 + hb);  // the buffer stays this warp's
+  }
+  // One batch handed over (kAccount); returns its flags.
+  __device__ __forceinline__ int take_hand(Hand& h) {
+    pair_sync(hb);
+    h = hands[hb];
+    return h.flags;
+  }
+  __device__ __forceinline__ void free_hand() {
+    pair_arrive(2 + hb);
+    hb ^= 1;
+    oplog += hb ? P.opcap : -P.opcap;
+  }
+  // Everything handed over up to the candidate's end, whose results are then
+  // this warp's.
+  __device__ __forceinline__ void account() {
+    while (true) {
+      Hand h;
+      const int flags = take_hand(h);
+      const bool end = (flags & kHandEnd) != 0;
+      opn = h.n;
+      if (end && h.status != GMG_SIM_OK) status = h.status;
+      if (status == GMG_SIM_OK) generate();
+      opn = 0;
+      if (kMode == kBase && (flags & kHandCheckpoint)) save_accounts(h.ck, h.t, (flags & kHandKeep) != 0);
+      if (!end) free_hand();
+      if (status == GMG_SIM_OK && (flags & (kHandDrain | kHandEnd))) drain_log(h.t);
+      if (end) {
+        score = lane_id() == 0 ? h.score : 0;
+        nev = lane_id() == 0 ? h.nev : 0;
+        iters = h.iters;
+        return;
+      }
+    }
+  }
+  __device__ __forceinline__ void done() { pair_arrive(2 + hb); }
+
   __device__ void run() {
     if (status) return;
     if constexpr (kPool) run_pool();
@@ -1609,7 +1732,9 @@ struct Sim {
       const bool end = lim == kNever && o.r == kNever;
       if (end || opn >= P.drain_trigger) {  // the only copy of this code: it is large
         const tm_t t = warp_min_t(pd.r);
-        drain(end ? kI64Max : (int64_t)(t < o.r ? t : o.r));
+        const int64_t tn = end ? kI64Max : (int64_t)(t < o.r ? t : o.r);
+        if constexpr (kRole == kBoth) drain(tn);
+        else if (!end) hand_over(tn, kHandDrain, opn);
         if (end || status) break;
       }
       Batch B;
@@ -1743,15 +1868,15 @@ struct Sim {
         m += __popc(b[s]);
       }
     }
-    // one key per lane, through the sort area (free between drains)
+    // one key per lane, through shared memory
     int at = 0;
     __syncwarp();
 #pragma unroll
     for (int s = 0; s < kSlots; ++s) {
       if ((b[s] >> lane) & 1u) {
         const int pos = at + __popc(b[s] & lanes_below());
-        sortk[pos] = k[s];
-        reinterpret_cast<uint32_t*>(sortk + 32)[pos] = (uint32_t)(32 * s) + lane;
+        bounce[pos] = k[s];
+        reinterpret_cast<uint32_t*>(bounce + 32)[pos] = (uint32_t)(32 * s) + lane;
       }
       at += __popc(b[s]);
     }
@@ -1759,8 +1884,8 @@ struct Sim {
     key = kKeyMax;
     slot = 0;
     if ((int)lane < m) {
-      key = sortk[lane];
-      slot = (int)reinterpret_cast<const uint32_t*>(sortk + 32)[lane];
+      key = bounce[lane];
+      slot = (int)reinterpret_cast<const uint32_t*>(bounce + 32)[lane];
     }
     return m;
   }
@@ -1856,7 +1981,9 @@ struct Sim {
       }
       const bool end = nfree == 32 * kSlots && outside_min() == kKeyMax;
       if (end || opn >= P.drain_trigger) {  // the only copy of this code: it is large
-        drain(end ? kI64Max : rq.time(next_key()));
+        const int64_t tn = end ? kI64Max : rq.time(next_key());
+        if constexpr (kRole == kBoth) drain(tn);
+        else if (!end) hand_over(tn, kHandDrain, opn);
         if (end || status) break;
       }
       uint64_t key;
@@ -1938,7 +2065,7 @@ struct Sim {
     const unsigned lane = lane_id();
     int32_t miss = 0;
     for (int r = lane; r < g.R; r += 32) {
-      const int64_t c = creq()[r];
+      const int64_t c = __ldcg(creq() + r);  // raised by atomics
       miss += c > __ldg(g.deadline + r) ? 1 : 0;
       if (o.req_done) o.req_done[k * g.R + r] = c;
     }
@@ -1999,21 +2126,22 @@ struct Sim {
 // READY heap, event log, partial results; the ops started by then are those
 // with base ready time < T_c.  An incremental candidate whose resume time T0
 // is >= T_c restarts there.
-template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool>
-__device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool>::maybe_checkpoint(int64_t tn, uint64_t held) {
+template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool, int kRole>
+__device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>::maybe_checkpoint(int64_t tn, uint64_t held) {
   if (kMode != kBase) return;
   const DevBase& B = P.base;
   if (ck >= B.nck || readypops < next_ck) return;
   if (tn <= (int64_t)last_t) return;
   const unsigned lane = lane_id();
-  generate();
+  if constexpr (kRole == kBoth) generate();
   // the pool's keys (or the keys that the lanes hold) follow the heap's
   const uint32_t hm = __ballot_sync(kFullMask, held != kKeyMax);
   const int nready = q.size + (kPool ? 32 * kSlots - nfree : __popc(hm));
-  if (nready <= B.ckq && log.n <= B.ckm) {
+  const bool keep = nready <= B.ckq;
+  if (keep) {
     int64_t* sc = B.ck_scalars + (int64_t)ck * 8;
     uint64_t* qk = B.ck_qkey + (int64_t)ck * B.ckq;
-    if (kPool) {
+    if constexpr (kPool) {
       int at = q.size;
 #pragma unroll
       for (int s = 0; s < kSlots; ++s) {
@@ -2027,33 +2155,78 @@ __device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool>::maybe_chec
     }
     const int64_t total = warp_sum_i64(score);
     if (lane == 0) {
-      B.ck_time[ck] = tn;
       sc[0] = nready;
       sc[1] = rootptr;
       sc[2] = total;
+    }
+    dv.save_free(B.ck_dev + (int64_t)ck * 3 * g.D);
+    for (int r = lane; r < g.R; r += 32) B.ck_creq[(int64_t)ck * g.R + r] = __ldcg(creq() + r);
+    for (int x = lane; x < q.size; x += 32) qk[x] = *q.kp(x);
+  }
+  if constexpr (kRole == kBoth) save_accounts(ck, tn, keep);
+  else hand_over(tn, kHandCheckpoint | (keep ? kHandKeep : 0), opn);
+  ++ck;
+  next_ck += B.stride_pops;
+  __syncwarp();
+}
+
+// The accounting's part of checkpoint c at time tn (keep: the sweep's part is
+// saved): live and peak bytes, the event log, the first violation.
+template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool, int kRole>
+__device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>::save_accounts(int c, int64_t tn, bool keep) {
+  const DevBase& B = P.base;
+  const unsigned lane = lane_id();
+  if (keep && log.n <= B.ckm) {
+    int64_t* sc = B.ck_scalars + (int64_t)c * 8;
+    if (lane == 0) {
+      B.ck_time[c] = tn;
       sc[3] = (int64_t)drained;
       sc[4] = vflag;
       sc[5] = vt;
       sc[6] = ((int64_t)vop << 32) | (uint32_t)vdev;
       sc[7] = log.n;
     }
-    dv.save(B.ck_dev + (int64_t)ck * 3 * g.D);
-    for (int r = lane; r < g.R; r += 32) B.ck_creq[(int64_t)ck * g.R + r] = creq()[r];
-    for (int x = lane; x < q.size; x += 32) qk[x] = *q.kp(x);
+    dv.save_bytes(B.ck_dev + (int64_t)c * 3 * g.D);
     for (int x = lane; x < log.n; x += 32) {
-      B.ck_mkey[(int64_t)ck * B.ckm + x] = *log.kp(x);
-      if (!kKey) B.ck_mdev[(int64_t)ck * B.ckm + x] = *log.dp(x);
+      B.ck_mkey[(int64_t)c * B.ckm + x] = *log.kp(x);
+      if (!kKey) B.ck_mdev[(int64_t)c * B.ckm + x] = *log.dp(x);
     }
   } else if (lane == 0) {
-    B.ck_time[ck] = kI64Max;
+    B.ck_time[c] = kI64Max;
   }
-  ++ck;
-  next_ck += B.stride_pops;
   __syncwarp();
 }
 
-template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool>
-__device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool>& S, const SimParams& P, unsigned wib,
+// Results of the base placement (after its last drain).
+template <class S_>
+__device__ __forceinline__ void write_base(S_& S, const DevBase& B) {
+  const unsigned lane = lane_id();
+  if (lane == 0) B.status[0] = S.status;
+  if (S.status != GMG_SIM_OK) return;
+  int32_t miss = 0;
+  for (int r = lane; r < S.g.R; r += 32) {
+    const int64_t c = __ldcg(S.creq() + r);
+    B.res_creq[r] = c;
+    miss += c > __ldg(S.g.deadline + r) ? 1 : 0;
+  }
+  miss = (int32_t)__reduce_add_sync(kFullMask, (unsigned)miss);
+  S.dv.write_peak(B.res_peak);
+  const int64_t makespan = S.dv.max_busy(S.g);
+  const int64_t score = warp_sum_i64(S.score);
+  if (lane == 0) {
+    int64_t* rs = B.res_scalars;
+    rs[0] = makespan;
+    rs[1] = S.vflag ? kI64Max : score;
+    rs[2] = S.vflag;
+    rs[3] = S.vop;
+    rs[4] = S.vdev;
+    rs[5] = S.vt;
+    rs[6] = miss;
+  }
+}
+
+template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool, int kRole>
+__device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>& S, const SimParams& P, unsigned wib,
                            int64_t slot, uint8_t* smem) {
   uint8_t* sl = P.scratch + slot * P.slot_bytes;
   const WarpSmem w = carve_smem(smem, P, wib);
@@ -2068,16 +2241,31 @@ __device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool>&
   S.log.sd = w.logd;
   S.log.n = 0;
   S.sortk = w.sortk;
+  S.bounce = w.sortk;
   S.sortd = w.sortd;
   S.oplog = w.oplog;
   S.opn = 0;
-  using tm_t = typename Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool>::tm_t;
+  using tm_t = typename Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>::tm_t;
   S.fbuf = reinterpret_cast<tm_t*>(sl + P.off_f);
   S.sl = sl;
   S.dv.setup(P.g, w.dev, P.off_pk >= 0 ? reinterpret_cast<int64_t*>(sl + P.off_pk) : nullptr);
   S.T0 = -1;
   S.Tc = 0;
+  S.ck = 0;
+  S.hb = 0;
+  if constexpr (kRole != kBoth) {  // behind the accelerator state: the second buffer is P.opcap entries after the first
+    uint8_t* c = w.dev + P.dev_bytes;
+    S.hands = reinterpret_cast<Hand*>(c);
+    S.oplog = reinterpret_cast<uint32_t*>(c + 2 * sizeof(Hand) + 8 * 48);
+    S.bounce = reinterpret_cast<uint64_t*>(c + 2 * sizeof(Hand));
+    // buffer 1 starts free
+    if (kRole == kAccount) pair_arrive(3);
+  }
 }
+
+// Leaving: the sweep takes the last arrival that nothing has waited for.
+template <class S_>
+__device__ __forceinline__ void leave_pair(S_& S) { pair_sync(2 + (S.hb ^ 1)); }
 
 }  // namespace
 }  // namespace gsim

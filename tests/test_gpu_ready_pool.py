@@ -85,14 +85,15 @@ def test_pending_ops_and_accounting(D, kw):
     compare(inc.to_numpy(), *O.incremental_batch(d, base, mv))
 
 
-@pytest.mark.parametrize("K", [32, 33])
-def test_default_staging_rule_gives_the_same(K):
-    """The staged copy and the L1 path on the two sides of the default's line."""
+@pytest.mark.parametrize("K", [1, 130])
+def test_two_warps_one_warp_and_staged_give_the_same(K):
+    """Two warps per candidate (the default for few), one warp and the staged copy."""
     wl = W.config2()
     rows = wl.full_rows(range(K))
     g = G.gmg_create(wl.desc)
-    outs = [G.sim_batch(g, torch_place(rows), req_done=True, gmg_staging=m)
-            for m in (G.GMG_STAGING_DEFAULT, G.GMG_STAGING_SHARED, G.GMG_STAGING_L1)]
+    place = torch_place(rows)
+    outs = [G.sim_batch(g, place, req_done=True, **kw)
+            for kw in ({}, dict(warps_per_block=4), dict(gmg_staging=G.GMG_STAGING_SHARED))]
     torch.cuda.synchronize()
     for o in outs:
         compare(o.to_numpy(), *oracle_rows(wl.desc, rows))
@@ -119,3 +120,23 @@ def test_arbitrated_events_at_one_time(D, kw):
     torch.cuda.synchronize()
     compare(out.to_numpy(), *O.simulate_batch(d, rows, arbitrated=True))
     compare(inc.to_numpy(), *O.incremental_batch(d, base, mv, arbitrated=True), check_events=D > 32)
+
+
+@pytest.mark.parametrize("D", [8, 64])
+@pytest.mark.parametrize("more", [0, 1])
+def test_both_sides_of_the_two_warp_line(D, more):
+    """As many candidates as fit with two warps each, and one more."""
+    d = _chains(27, D=D, chains=5, length=4, fan=2, bytes_lo=1 << 18, cap=6 << 20)
+    g = G.gmg_create(d)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    K = 14 * sms + more
+    rows = _rows(28, K, d.n_ops, D)
+    out = G.sim_batch(g, torch_place(rows), req_done=True)
+    base = rows[0, :d.n_ops].copy()
+    mv = W.random_moves(29, K, base, D, max_moves=4)
+    mv.dev[mv.off[2]:mv.off[3]] = D               # written without the second warp
+    b = G.base_create(g, torch.from_numpy(base).cuda())
+    inc = G.sim_incremental(g, b, *G.moves_to_device(mv, "cuda"), req_done=True)
+    torch.cuda.synchronize()
+    compare(out.to_numpy(), *oracle_rows(d, rows))
+    compare(inc.to_numpy(), *O.incremental_batch(d, base, mv))
