@@ -869,10 +869,10 @@ def main():
     props = torch.cuda.get_device_properties(device)
     issue_peak = props.multi_processor_count * 4 * pk["sm_max_mhz"] * 1e6 / 1e9  # Ginst/s
     arb_kern = "sim_arb_kernel" if D <= 32 else "sim_arbw_kernel"
-    # the library's default: two warps per candidate while all fit (14 blocks of 64 threads per SM), then
+    # the library's default: two warps per candidate while all fit (14 blocks of 64 threads per SM, 10 with 64-bit times), then
     # the staged kernel for graphs whose copy takes 16 KB at most, else one warp per candidate
-    pair = p.g.info["t32"] == 1 and p.staging != 1 and not p.arb
-    pairs = 14 * props.multi_processor_count
+    pair = p.staging != 1 and not p.arb
+    pairs = (14 if p.g.info["t32"] == 1 else 10) * props.multi_processor_count
     staged_run = p.staging == 1 or (p.staging == 0 and p.g.info["stageable"] == 1 and not p.arb and
                                     not (pair and p.n_full <= pairs) and
                                     20 * wl.desc.n_ops + 8 * wl.desc.n_edges <= 16 << 10)
@@ -882,7 +882,7 @@ def main():
              "inc": ("sim_arb_inc_kernel" if p.arb_base else arb_kern if p.arb else
                      "sim_inc_pair_kernel" if pair and p.n_inc <= pairs else "sim_inc_kernel"),
              "base": ("sim_arb_base_kernel" if p.arb_base else
-                      "sim_base_pair_kernel" if p.g.info["t32"] == 1 else "sim_base_kernel")}
+                      "sim_base_pair_kernel")}
     kcount = {"full": p.n_full, "inc": p.n_inc, "base": 1}
     out_bytes_per_cand = 8 + 8 + 4 + 4 + 4 + 4 + 8 + 4 + 8 + 8 * D
     alg_bytes = {"full": p.n_full * (W_ld(N) + out_bytes_per_cand),

@@ -125,8 +125,8 @@ typedef struct gmg_base gmg_base_t; /* opaque; base schedule snapshot for increm
  * within the CTA's shared memory, else GMG_EINVAL.  GMG_STAGING_L1: 4-warp
  * CTAs read the records through the read-only L1 path.
  * GMG_STAGING_DEFAULT takes the fastest measured: batches of up to about 14
- * candidates per SM run with two warps per candidate by the L1 path (32-bit
- * times), larger ones are staged where staging applies and the copy takes 16 KB
+ * candidates per SM (10 with times beyond 2^32) run with two warps per candidate
+ * by the L1 path, larger ones are staged where staging applies and the copy takes 16 KB
  * at most, and take the L1 path elsewhere; sim_batch_noalloc always
  * takes the L1 path (and refuses GMG_STAGING_SHARED). */
 #define GMG_STAGING_DEFAULT 0
@@ -178,7 +178,7 @@ typedef struct {
                             pool in shared memory (more than 32 accelerators and keys with 5 bits
                             of room; with at most 32 accelerators lanes hold them).  Either way
                             every op whose start the others cannot change starts at once */
-  int32_t t32;           /* 1 if the kernels carry times as 32-bit integers (time_bound < 2^31) */
+  int32_t t32;           /* 1 if the kernels carry times as 32-bit integers (time_bound < 2^32 - 1) */
   int32_t stageable;     /* 1 if sim_batch can stage this graph's hot fields in shared memory on
                             the current device (one accelerator type, uniform links, 32-bit times,
                             at most 32 accelerators, and the copy fits beside one warp's areas);

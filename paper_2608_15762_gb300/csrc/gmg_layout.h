@@ -97,7 +97,7 @@ struct DevGmg {
   uint64_t keymask;           // key part of a log entry: 2^ds - 1
   int32_t tb;                 // time bits needed (every time < 2^tb)
   int32_t dev_key;            // 1 if an accelerator id fits above (time, class, op) in 64 bits
-  int32_t t32;                // 1 if every time is below 2^31 (the kernels then use int32 times)
+  int32_t t32;                // 1 if every time is below 2^32 - 1 (the kernels then use uint32 times)
   int32_t ntypes;             // accelerator types; >= 2: durations from durt by dtype
   const int64_t* durt;        // [N*ntypes] duration of op i on type t at i*ntypes + t
   const uint8_t* dtype;       // [D] type of each accelerator
@@ -106,9 +106,9 @@ struct DevGmg {
   int32_t qb;                 // bits of the earliest finish in a READY pool key (0, or 6 to kMaxQB)
   // The hot fields in a compact form, read by the sweep wherever the graph has
   // it (hot_ok) and staged into shared memory by sim_full_staged_kernel
-  // (stage_ok: also at most 32 accelerators).
+  // (stage_ok: also at most 32 accelerators and times below 2^31).
   const uint4* st_hot;        // [N] {dur, xq | flags << 29, succ_off | nsucc << 24, pred_off | npred << 24}
-  const int32_t* st_rel;      // [N] release
+  const uint32_t* st_rel;     // [N] release
   int32_t hot_ok;             // 1: 32-bit times, one type, uniform links, lists and sizes fit the fields
   int32_t stage_ok;
   int32_t n_edges;
@@ -129,6 +129,8 @@ inline int64_t stage_smem_bytes(int64_t n, int64_t E) {
 // Resident 4-warp blocks per SM the simulation kernels are compiled for (their
 // register budget).
 constexpr int kBlocksPerSM = 7;
+// Blocks of two warps per SM (72 registers a thread; with 64-bit times 96).
+constexpr int kPairsPerSM = 14, kPairsPerSM64 = 10;
 
 // Slots of the READY pool on more than 32 accelerators (a multiple of 32, at
 // most 256; compile-time overridable for tuning sweeps).

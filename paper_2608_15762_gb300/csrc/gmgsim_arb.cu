@@ -367,7 +367,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode, kHot>, Sim<true, kMode, tr
           fu = uh < 0 ? kNever : this->fin((uint32_t)uh);
         }
         arbitrate(tx);
-        if (kMode == kBase) this->last_t = tx;
+        if (kMode == kBase) this->last_t = (int64_t)tx;
       }
       if (status) break;
     }
@@ -386,7 +386,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode, kHot>, Sim<true, kMode, tr
     if (this->ck >= B.nck || this->readypops < this->next_ck) return;
     const tm_t r = warp_min_t(pd.r);
     const tm_t tn = r < o.r ? r : o.r;
-    if (tn <= this->last_t) return;
+    if ((int64_t)tn <= this->last_t) return;
     generate();  // the simulation checkpoint then finds no started op left to generate
     this->template arrivals<kDevBits>();
     const int c = this->ck;

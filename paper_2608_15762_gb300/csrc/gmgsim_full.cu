@@ -28,13 +28,13 @@ __global__ void __launch_bounds__(128, kBlocksPerSM) sim_full_kernel(const __gri
 }
 
 // Few candidates: two warps each, the sweep and the HBM accounting.
-template <bool kNarrow, bool kTypes, int kHot>
-__global__ void __launch_bounds__(64, 2 * kBlocksPerSM) sim_full_pair_kernel(const __grid_constant__ SimParams P) {
+template <bool kNarrow, bool kT32, bool kTypes, int kHot>
+__global__ void __launch_bounds__(64, kT32 ? kPairsPerSM : kPairsPerSM64) sim_full_pair_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int64_t slot = blockIdx.x;
   const int64_t nslots = gridDim.x;
   if (threadIdx.x < 32u) {
-    Sim<kNarrow, kFull, true, true, kTypes, kHot, !kNarrow, kSweep> S(P);
+    Sim<kNarrow, kFull, true, kT32, kTypes, kHot, !kNarrow, kSweep> S(P);
     setup_slot(S, P, 0, slot, smem);
     for (int64_t k = slot; k < P.K; k += nslots) {
       S.row = P.place + k * P.ld;
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(64, 2 * kBlocksPerSM) sim_full_pair_kernel(con
     }
     leave_pair(S);
   } else {
-    Sim<kNarrow, kFull, true, true, kTypes, kHot, !kNarrow, kAccount> S(P);
+    Sim<kNarrow, kFull, true, kT32, kTypes, kHot, !kNarrow, kAccount> S(P);
     setup_slot(S, P, 0, slot, smem);
     for (int64_t k = slot; k < P.K; k += nslots) {
       S.row = P.place + k * P.ld;
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(32 * kStageMaxWarps, 1) sim_full_staged_kernel
   Sim<true, kFull, true, true, false, kHotShared> S(P);
   setup_slot(S, P, wib, slot, smem + P.stage_bytes);
   S.sh_hot = reinterpret_cast<const uint4*>(s_hot);
-  S.sh_rel = reinterpret_cast<const int32_t*>(s_rel);
+  S.sh_rel = reinterpret_cast<const uint32_t*>(s_rel);
   S.sh_succ = reinterpret_cast<const uint32_t*>(s_succ);
   S.sh_pred = reinterpret_cast<const uint32_t*>(s_pred);
   for (int64_t k = slot; k < P.K; k += nslots) {
@@ -173,17 +173,17 @@ const void* full_kernel_ptr(const DevGmg& g) {
   const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
   return g.D <= 32 ? full_ptr_n<true>(key, t32, types, hot) : full_ptr_n<false>(key, t32, types, hot);
 }
-// Two warps per candidate: graphs with 32-bit times.
-const void* full_pair_kernel_ptr(const DevGmg& g) {
-  const bool types = g.ntypes >= 2;
-  if (g.hot_ok)
-    return g.D <= 32 ? (const void*)sim_full_pair_kernel<true, false, kHotGlobal>
-                     : (const void*)sim_full_pair_kernel<false, false, kHotGlobal>;
-  if (g.D <= 32)
-    return types ? (const void*)sim_full_pair_kernel<true, true, kHotNone>
-                 : (const void*)sim_full_pair_kernel<true, false, kHotNone>;
-  return types ? (const void*)sim_full_pair_kernel<false, true, kHotNone>
-               : (const void*)sim_full_pair_kernel<false, false, kHotNone>;
+// Two warps per candidate: graphs whose accelerator ids fit into the event key.
+template <bool N, bool T32>
+const void* full_pair_ptr(bool types) {
+  return types ? (const void*)sim_full_pair_kernel<N, T32, true, kHotNone>
+               : (const void*)sim_full_pair_kernel<N, T32, false, kHotNone>;
 }
+template <bool N>
+const void* full_pair_ptr_n(const DevGmg& g) {
+  if (g.hot_ok) return (const void*)sim_full_pair_kernel<N, true, false, kHotGlobal>;
+  return g.t32 ? full_pair_ptr<N, true>(g.ntypes >= 2) : full_pair_ptr<N, false>(g.ntypes >= 2);
+}
+const void* full_pair_kernel_ptr(const DevGmg& g) { return g.D <= 32 ? full_pair_ptr_n<true>(g) : full_pair_ptr_n<false>(g); }
 
 }  // namespace gsim

@@ -40,6 +40,7 @@ constexpr int64_t kI64Max = 0x7fffffffffffffffll;
 constexpr int kMaxOpsLog2 = 28;          // op ids must fit the packed key
 constexpr int kDefaultWarpsPerBlock = 4;
 constexpr int kSharedOverflowEntries = 33;  // behind the READY pool: the root and its children
+constexpr int64_t kMaxTime32 = 0xffffffff;  // times below this fit the 32-bit instances (about 71 minutes)
 constexpr int64_t kDefaultQueueCap = 1 << 16;
 constexpr int kSharedLogEntries = 192, kSharedLogEntriesWide = 112;
 constexpr int64_t kDefaultLogCap = 1 << 17;
@@ -75,7 +76,7 @@ struct Built {
   // compact hot records for a CTA's staged copy (sim_opts_t.gmg_staging = 1)
   bool stage_ready = false;
   std::vector<uint32_t> st_hot;  // [4n]
-  std::vector<int32_t> st_rel;   // [n]
+  std::vector<uint32_t> st_rel;  // [n]
   Layout L{};
 };
 
@@ -411,9 +412,9 @@ int build(const gmg_desc_t* d, Built& b) {
   std::sort(b.roots.begin(), b.roots.end());
   b.nroots = (int)b.roots.size();
   // compact records for the staged copy: one accelerator type, uniform links,
-  // every time below 2^31, lists addressable in 24 bits with fewer than 256
+  // 32-bit times, lists addressable in 24 bits with fewer than 256
   // entries per op, transfer sizes (xq) below 2^29
-  b.stage_ready = !b.T && b.uniform && b.time_bound < (int64_t(1) << 31) && b.E < (1 << 24);
+  b.stage_ready = !b.T && b.uniform && b.time_bound < kMaxTime32 && b.E < (1 << 24);
   for (int i = 0; i < n && b.stage_ready; ++i) {
     const OpRec& r = b.ops[i];
     b.stage_ready = r.nsucc < 256 && r.npred < 256 && r.xq < (int64_t(1) << 29);
@@ -427,7 +428,7 @@ int build(const gmg_desc_t* d, Built& b) {
       b.st_hot[4 * (size_t)i + 1] = (uint32_t)r.xq | ((r.flags & 7u) << 29);
       b.st_hot[4 * (size_t)i + 2] = r.succ_off | (r.nsucc << 24);
       b.st_hot[4 * (size_t)i + 3] = r.pred_off | (r.npred << 24);
-      b.st_rel[i] = (int32_t)r.release;
+      b.st_rel[i] = (uint32_t)r.release;
     }
   }
   plan(b);
@@ -580,10 +581,11 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
 
 // Two warps per candidate where all candidates fit on the GPU at once that way
 // (and the caller has not set the warps per block): the sweep of a candidate
-// does not wait for its HBM accounting.  Graphs with 32-bit times.
+// does not wait for its HBM accounting.  Graphs whose accelerator ids fit into
+// the event key.
 int plan_pair(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& L) {
   const DevGmg& G = g->dg;
-  if (!G.t32 || (o && o->warps_per_block > 0)) return GMG_EINVAL;
+  if (!G.dev_key || (o && o->warps_per_block > 0)) return GMG_EINVAL;
   const int rc = plan_launch(g, K, o, inc, L);
   if (rc) return rc;
   SimParams& P = L.P;
@@ -860,7 +862,7 @@ int plan_base(const gmg* g, const sim_opts_t* o, BasePlan& B) {
   if (rc) return rc;
   L.wpb = 1;
   if (B.arb) L.P.dev_bytes = dev_smem_bytes(G.D, 8);  // the arbitrated base keeps 64-bit times
-  L.pair = !B.arb && G.t32;
+  L.pair = !B.arb && G.dev_key != 0;
   if (L.pair) L.P.pair_bytes = pair_bytes(L.P);
   L.smem = smem_per_warp(L.P);
   if (B.arb) {
@@ -1047,15 +1049,14 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   G.dev_key = dev_key ? 1 : 0;
   G.qb = qb;
   G.st_hot = reinterpret_cast<const uint4*>(w + L.off_st_hot);
-  G.st_rel = reinterpret_cast<const int32_t*>(w + L.off_st_rel);
+  G.st_rel = reinterpret_cast<const uint32_t*>(w + L.off_st_rel);
   G.n_edges = b.E;
   G.ws = w;
   G.ws_bytes = (int64_t)L.total;
-  // every time < 2^tb fits int32; the 32-bit instances also take the
-  // accelerator id from the event key
-  G.t32 = (G.tb <= 31 && G.dev_key) ? 1 : 0;
+  // the 32-bit instances also take the accelerator id from the event key
+  G.t32 = (b.time_bound < kMaxTime32 && G.dev_key) ? 1 : 0;
   G.hot_ok = (b.stage_ready && G.t32) ? 1 : 0;
-  G.stage_ok = (G.hot_ok && G.D <= 32) ? 1 : 0;
+  G.stage_ok = (G.hot_ok && G.D <= 32 && b.time_bound < (int64_t(1) << 31)) ? 1 : 0;
   G.uniform = b.uniform ? 1 : 0;
   gmg_info_t& I = g->info;
   std::memset(&I, 0, sizeof(I));

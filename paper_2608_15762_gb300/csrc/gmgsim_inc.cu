@@ -351,13 +351,13 @@ __global__ void __launch_bounds__(128, kBlocksPerSM) sim_inc_kernel(const __grid
 }
 
 // Few candidates: two warps each, the sweep and the HBM accounting.
-template <bool kNarrow, bool kTypes, int kHot>
-__global__ void __launch_bounds__(64, 2 * kBlocksPerSM) sim_inc_pair_kernel(const __grid_constant__ SimParams P) {
+template <bool kNarrow, bool kT32, bool kTypes, int kHot>
+__global__ void __launch_bounds__(64, kT32 ? kPairsPerSM : kPairsPerSM64) sim_inc_pair_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int64_t slot = blockIdx.x;
   uint8_t* crow = P.scratch + slot * P.slot_bytes + P.off_row;
   if (threadIdx.x < 32u) {
-    Sim<kNarrow, kInc, true, true, kTypes, kHot, !kNarrow, kSweep> S(P);
+    Sim<kNarrow, kInc, true, kT32, kTypes, kHot, !kNarrow, kSweep> S(P);
     setup_slot(S, P, 0, slot, smem);
     S.rb = P.base.rb;
     S.fb = P.base.fb;
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(64, 2 * kBlocksPerSM) sim_inc_pair_kernel(cons
     S.hand_over(0, kHandQuit, 0);
     leave_pair(S);
   } else {
-    Sim<kNarrow, kInc, true, true, kTypes, kHot, !kNarrow, kAccount> S(P);
+    Sim<kNarrow, kInc, true, kT32, kTypes, kHot, !kNarrow, kAccount> S(P);
     setup_slot(S, P, 0, slot, smem);
     S.rb = P.base.rb;
     S.fb = P.base.fb;
@@ -409,17 +409,17 @@ const void* inc_kernel_ptr(const DevGmg& g) {
   const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
   return g.D <= 32 ? inc_ptr_n<true>(key, t32, types, hot) : inc_ptr_n<false>(key, t32, types, hot);
 }
-// Two warps per candidate: graphs with 32-bit times.
-const void* inc_pair_kernel_ptr(const DevGmg& g) {
-  const bool types = g.ntypes >= 2;
-  if (g.hot_ok)
-    return g.D <= 32 ? (const void*)sim_inc_pair_kernel<true, false, kHotGlobal>
-                     : (const void*)sim_inc_pair_kernel<false, false, kHotGlobal>;
-  if (g.D <= 32)
-    return types ? (const void*)sim_inc_pair_kernel<true, true, kHotNone>
-                 : (const void*)sim_inc_pair_kernel<true, false, kHotNone>;
-  return types ? (const void*)sim_inc_pair_kernel<false, true, kHotNone>
-               : (const void*)sim_inc_pair_kernel<false, false, kHotNone>;
+// Two warps per candidate: graphs whose accelerator ids fit into the event key.
+template <bool N, bool T32>
+const void* inc_pair_ptr(bool types) {
+  return types ? (const void*)sim_inc_pair_kernel<N, T32, true, kHotNone>
+               : (const void*)sim_inc_pair_kernel<N, T32, false, kHotNone>;
 }
+template <bool N>
+const void* inc_pair_ptr_n(const DevGmg& g) {
+  if (g.hot_ok) return (const void*)sim_inc_pair_kernel<N, true, false, kHotGlobal>;
+  return g.t32 ? inc_pair_ptr<N, true>(g.ntypes >= 2) : inc_pair_ptr<N, false>(g.ntypes >= 2);
+}
+const void* inc_pair_kernel_ptr(const DevGmg& g) { return g.D <= 32 ? inc_pair_ptr_n<true>(g) : inc_pair_ptr_n<false>(g); }
 
 }  // namespace gsim

@@ -41,18 +41,18 @@ __global__ void __launch_bounds__(32, 1) sim_base_kernel(const __grid_constant__
   write_base(S, P.base);
 }
 
-// The same by two warps, the sweep and the HBM accounting (32-bit times).
-template <bool kNarrow, bool kTypes, int kHot>
+// The same by two warps, the sweep and the HBM accounting.
+template <bool kNarrow, bool kT32, bool kTypes, int kHot>
 __global__ void __launch_bounds__(64, 1) sim_base_pair_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
   if (threadIdx.x < 32) {
-    Sim<kNarrow, kBase, true, true, kTypes, kHot, !kNarrow, kSweep> S(P);
+    Sim<kNarrow, kBase, true, kT32, kTypes, kHot, !kNarrow, kSweep> S(P);
     setup_slot(S, P, 0, 0, smem);
     sweep_base(S, P);
     S.hand_end();
     leave_pair(S);
   } else {
-    Sim<kNarrow, kBase, true, true, kTypes, kHot, !kNarrow, kAccount> S(P);
+    Sim<kNarrow, kBase, true, kT32, kTypes, kHot, !kNarrow, kAccount> S(P);
     setup_slot(S, P, 0, 0, smem);
     warp_prefetch_l2(P.g.ws, P.g.ws_bytes);
     for (int c = lane_id(); c < P.base.nck; c += 32) P.base.ck_time[c] = kI64Max;
@@ -165,18 +165,18 @@ const void* base_kernel_ptr(const DevGmg& g) {
   const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
   return g.D <= 32 ? base_ptr_n<true>(key, t32, types, hot) : base_ptr_n<false>(key, t32, types, hot);
 }
-// Two warps: graphs with 32-bit times.
-const void* base_pair_kernel_ptr(const DevGmg& g) {
-  const bool types = g.ntypes >= 2;
-  if (g.hot_ok)
-    return g.D <= 32 ? (const void*)sim_base_pair_kernel<true, false, kHotGlobal>
-                     : (const void*)sim_base_pair_kernel<false, false, kHotGlobal>;
-  if (g.D <= 32)
-    return types ? (const void*)sim_base_pair_kernel<true, true, kHotNone>
-                 : (const void*)sim_base_pair_kernel<true, false, kHotNone>;
-  return types ? (const void*)sim_base_pair_kernel<false, true, kHotNone>
-               : (const void*)sim_base_pair_kernel<false, false, kHotNone>;
+// Two warps: graphs whose accelerator ids fit into the event key.
+template <bool N, bool T32>
+const void* base_pair_ptr(bool types) {
+  return types ? (const void*)sim_base_pair_kernel<N, T32, true, kHotNone>
+               : (const void*)sim_base_pair_kernel<N, T32, false, kHotNone>;
 }
+template <bool N>
+const void* base_pair_ptr_n(const DevGmg& g) {
+  if (g.hot_ok) return (const void*)sim_base_pair_kernel<N, true, false, kHotGlobal>;
+  return g.t32 ? base_pair_ptr<N, true>(g.ntypes >= 2) : base_pair_ptr<N, false>(g.ntypes >= 2);
+}
+const void* base_pair_kernel_ptr(const DevGmg& g) { return g.D <= 32 ? base_pair_ptr_n<true>(g) : base_pair_ptr_n<false>(g); }
 
 cudaError_t set_smem_limits(int smem) {
   DevGmg g{};

@@ -419,8 +419,8 @@ __device__ __forceinline__ WarpSmem carve_smem(uint8_t* smem, const SimParams& P
 // ---------------------------------------------------------------------------
 // One warp's simulator.
 // ---------------------------------------------------------------------------
-// kT32: every time of the graph is below 2^31 (the host's bound), so ready,
-// start, finish, free and arrival times are carried as int32 (bytes, scores
+// kT32: every time of the graph is below 2^32 - 1 (the host's bound), so ready,
+// start, finish, free and arrival times are carried as uint32 (bytes, scores
 // and outputs stay int64).
 // kTypes: the graph has several accelerator types (durations per (type, op)).
 // kNarrow: at most 32 accelerators.
@@ -473,13 +473,13 @@ template <bool kNarrow, int kMode, bool kKey, bool kT32 = false, bool kTypes = f
           bool kPool = !kNarrow, int kRole = kBoth>
 struct Sim {
   static_assert(kHot == kHotNone || (kT32 && !kTypes), "compact records: 32-bit times, one type");
-  using tm_t = typename std::conditional<kT32, int32_t, int64_t>::type;
+  using tm_t = typename std::conditional<kT32, uint32_t, int64_t>::type;
   const SimParams& P;
   const DevGmg& g;
   static constexpr int kSlots = kReadyPoolWide / 32;  // pool slots per lane (kPool)
   static constexpr bool kCompact = kHot != kHotNone, kKeyed = kKey, kPooled = kPool;
   static constexpr int kRoleOf = kRole;
-  static constexpr tm_t kNever = (tm_t)(~(typename std::make_unsigned<tm_t>::type)0 >> 1);
+  static constexpr tm_t kNever = kT32 ? (tm_t)0xffffffffu : (tm_t)kI64Max;  // later than every time
   struct Pending {
     tm_t r, e, dur;  // ready time, earliest finish (both kNever: empty), duration
     uint32_t op;
@@ -520,14 +520,14 @@ struct Sim {
   int64_t score, nev;   // each lane's share, summed at the end
   int64_t readypops;
   int32_t iters;        // ops started (loop guard; the event count of a full run)
-  tm_t last_t;          // latest READY time handled, kept in base mode only (checkpoints)
+  int64_t last_t;       // latest READY time handled, kept in base mode only (checkpoints)
   int32_t vflag, vop, vdev, status;
   int64_t vt;
   // base checkpoints
   int ck, next_ck;
   // staged GMG (kHotShared): shared copies
   const uint4* sh_hot;      // per op {dur, xq | flags << 29, succ_off | nsucc << 24, pred_off | npred << 24}
-  const int32_t* sh_rel;    // per op release
+  const uint32_t* sh_rel;   // per op release
   const uint32_t* sh_succ;  // successor lists
   const uint32_t* sh_pred;  // predecessor lists (hold bits included)
 
@@ -536,10 +536,12 @@ struct Sim {
 
   // Started ops are those with a finish time: every finish time is >= 1, the
   // finish array is zeroed per candidate, and the sweep marks a join whose READY
-  // key is queued with -1.
+  // key is queued with kQueued.
+  static constexpr tm_t kQueued = (tm_t)-1;
+  static __device__ __forceinline__ bool started(tm_t f) { return kT32 ? (uint32_t)f - 1u < 0xfffffffeu : f > 0; }
   // The low 32 bits of a base-snapshot time (little-endian int64).
   static __device__ __forceinline__ tm_t base_time(const int64_t* a, uint32_t x) {
-    if (kT32) return (tm_t)__ldg(reinterpret_cast<const int32_t*>(a) + 2 * (size_t)x);
+    if (kT32) return (tm_t)__ldg(reinterpret_cast<const uint32_t*>(a) + 2 * (size_t)x);
     return (tm_t)__ldg(a + x);
   }
   // Duration of op i on accelerator d: by the accelerator's type when the
@@ -585,7 +587,7 @@ struct Sim {
 
 
   __device__ __forceinline__ tm_t warp_min_t(tm_t v) const {
-    if (kT32) return (tm_t)__reduce_min_sync(kFullMask, (int)v);
+    if (kT32) return (tm_t)__reduce_min_sync(kFullMask, (unsigned)v);
     return (tm_t)warp_min_u64((uint64_t)v);  // times are >= 0
   }
 
@@ -750,7 +752,7 @@ struct Sim {
       if (row[sb & ~kSibLater] != d) return true;
       if (sb & kSibLater) return false;  // the other consumer finishes later
       const tm_t fs = fin(sb);
-      return fs > 0 && fs < f;
+      return started(fs) && fs < f;
     }
     const uint32_t p = ps.x & kIdMask;
     const XqSucc px = op_xqsucc(g.ops, p);
@@ -761,7 +763,7 @@ struct Sim {
     for (uint32_t w = 0; w < nl; ++w) {
       const uint32_t c = __ldg(lst + w);
       const tm_t fc = c != x ? fin(c) : 0;
-      if (c != x && row[c] == d && !(fc > 0 && fc < f)) return false;
+      if (c != x && row[c] == d && !(started(fc) && fc < f)) return false;
     }
     return true;
   }
@@ -1478,7 +1480,7 @@ struct Sim {
       const tm_t a = fin(p);
       const int dp = row[p];
       const tm_t b = a + (dp != x.d ? sends(p, dp, x.d) : (tm_t)0);
-      x.rdy = a > 0 && fj == 0;
+      x.rdy = started(a) && fj == 0;
       x.r = b > x.r ? b : x.r;
     } else if (x.join) {
       const tm_t fj = fin(x.j);
@@ -1487,7 +1489,7 @@ struct Sim {
         if (p == i) continue;
         tm_t a = fin(p);
         const int dp = row[p];
-        if (a <= 0) {
+        if (!started(a)) {
           x.rdy = false;
           break;
         }
@@ -1506,7 +1508,7 @@ struct Sim {
       const uint32_t grp = __match_any_sync(kFullMask, x.rdy && x.join ? x.j : ~lane_id());
       if (x.join && __ffs(grp) - 1 != (int)lane_id()) x.rdy = false;
     }
-    if (x.rdy && x.join) fbuf[x.j] = (tm_t)-1;
+    if (x.rdy && x.join) fbuf[x.j] = kQueued;
     __syncwarp();
   }
   // Op i of this lane started, ready at r and ending at f (act: the lanes that
@@ -1528,7 +1530,7 @@ struct Sim {
     }
     opn += __popc(act);
     if (kMode == kBase) {
-      const tm_t lt = (tm_t)warp_max_u64(v ? (uint64_t)r : 0ull);
+      const int64_t lt = (int64_t)warp_max_u64(v ? (uint64_t)r : 0ull);
       last_t = lt > last_t ? lt : last_t;
       readypops += __popc(act);
     }
@@ -2131,7 +2133,7 @@ __device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>::may
   if (kMode != kBase) return;
   const DevBase& B = P.base;
   if (ck >= B.nck || readypops < next_ck) return;
-  if (tn <= (int64_t)last_t) return;
+  if (tn <= last_t) return;
   const unsigned lane = lane_id();
   if constexpr (kRole == kBoth) generate();
   // the pool's keys (or the keys that the lanes hold) follow the heap's
@@ -2249,7 +2251,7 @@ __device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, 
   S.fbuf = reinterpret_cast<tm_t*>(sl + P.off_f);
   S.sl = sl;
   S.dv.setup(P.g, w.dev, P.off_pk >= 0 ? reinterpret_cast<int64_t*>(sl + P.off_pk) : nullptr);
-  S.T0 = -1;
+  S.T0 = 0;
   S.Tc = 0;
   S.ck = 0;
   S.hb = 0;

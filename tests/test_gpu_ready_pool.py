@@ -64,6 +64,7 @@ def _rows(seed, K, n, D):
     dict(chains=20, length=6, bytes_lo=1 << 18, cap=6 << 20),    # capacities that bind
     dict(chains=5, length=5, bytes_lo=1 << 48, bytes_hi=1 << 50),  # sizes beyond 48 bits
     dict(chains=30, length=6, dur_hi=1 << 29),                   # 64-bit times
+    dict(chains=30, length=6, release_hi=3_900_000_000),         # 32-bit times beyond 2^31
 ])
 def test_pending_ops_and_accounting(D, kw):
     d = _chains(7, D=D, **kw)
@@ -105,6 +106,7 @@ def test_two_warps_one_warp_and_staged_give_the_same(K):
     dict(chains=80, length=4, dur_hi=1, release_hi=2, bytes_lo=0, bytes_hi=1 << 12),
     dict(chains=9, length=4, fan=5),                                       # several destinations per op
     dict(chains=40, length=4, dur_hi=1 << 29),                             # 64-bit times
+    dict(chains=40, length=4, release_hi=3_900_000_000),                   # 32-bit times beyond 2^31
 ])
 def test_arbitrated_events_at_one_time(D, kw):
     """More pending ops than lanes, and more completions and intents at one time
