@@ -389,6 +389,7 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode, kHot>, Sim<true, kMode, tr
     if ((int64_t)tn <= this->last_t) return;
     generate();  // the simulation checkpoint then finds no started op left to generate
     this->template arrivals<kDevBits>();
+    this->drain_log((int64_t)tn);
     const int c = this->ck;
     this->maybe_checkpoint((int64_t)tn, this->held_key());
     if (this->ck > c && B.ck_time[c] != kI64Max) save_arb(c);

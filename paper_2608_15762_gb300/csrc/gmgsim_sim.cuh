@@ -1377,9 +1377,9 @@ struct Sim {
       if (end && h.status != GMG_SIM_OK) status = h.status;
       if (status == GMG_SIM_OK) generate();
       opn = 0;
-      if (kMode == kBase && (flags & kHandCheckpoint)) save_accounts(h.ck, h.t, (flags & kHandKeep) != 0);
       if (!end) free_hand();
-      if (status == GMG_SIM_OK && (flags & (kHandDrain | kHandEnd))) drain_log(h.t);
+      if (status == GMG_SIM_OK) drain_log(h.t);
+      if (kMode == kBase && (flags & kHandCheckpoint)) save_accounts(h.ck, h.t, (flags & kHandKeep) != 0);
       if (end) {
         score = lane_id() == 0 ? h.score : 0;
         nev = lane_id() == 0 ? h.nev : 0;
@@ -2127,7 +2127,11 @@ struct Sim {
 // time next_t handled yet), save the complete simulator state -- accelerator state,
 // READY heap, event log, partial results; the ops started by then are those
 // with base ready time < T_c.  An incremental candidate whose resume time T0
-// is >= T_c restarts there.
+// is >= T_c restarts there.  The events before T_c are applied first: what is
+// left in the log is small.  (Checkpoints every few ops generate events before
+// the sweep's own drain is due; without a drain of their own the log of an 8 x
+// 32-layer graph, one checkpoint per 12 ops, kept every event: 24 ms for the base
+// and 21 ms for a late candidate instead of 2.7 and 0.09.)
 template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool, int kRole>
 __device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>::maybe_checkpoint(int64_t tn, uint64_t held) {
   if (kMode != kBase) return;
@@ -2135,7 +2139,10 @@ __device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>::may
   if (ck >= B.nck || readypops < next_ck) return;
   if (tn <= last_t) return;
   const unsigned lane = lane_id();
-  if constexpr (kRole == kBoth) generate();
+  if constexpr (kRole == kBoth) {
+    generate();
+    drain_log(tn);
+  }
   // the pool's keys (or the keys that the lanes hold) follow the heap's
   const uint32_t hm = __ballot_sync(kFullMask, held != kKeyMax);
   const int nready = q.size + (kPool ? 32 * kSlots - nfree : __popc(hm));
