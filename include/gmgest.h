@@ -62,7 +62,7 @@ size_t est_update_tmp_bytes(int32_t n_est, int32_t n_feat, int64_t n_samples);
  *   d_tmp              caller buffer of est_update_tmp_bytes bytes, 256-byte
  *                      aligned (GMG_EWS if smaller); scratch, contents lost
  * The coefficients and flags are read back with est_coefficients.  Sums have
- * a fixed order (128-row chunks reduced by a fixed tree, chunks added in
+ * a fixed order (chunks of rows reduced by a fixed tree, chunks added in
  * order), so results are reproducible run to run. */
 int est_update(void* d_state, int32_t n_est, int32_t n_feat, const int32_t* d_off, const double* d_x,
                const double* d_y, int64_t n_samples, void* d_tmp, size_t tmp_bytes, gmg_stream_t stream);

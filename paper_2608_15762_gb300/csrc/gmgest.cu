@@ -2,20 +2,27 @@
 // executor feedback and the integer duration / link tables they produce for
 // the simulation.  The C ABI is declared in include/gmgest.h.
 //
-// est_update, in three launches:
-//  1. chunk counts: every estimator's samples are cut into chunks of kChunk
-//     rows; one block computes the exclusive prefix of the chunk counts;
-//  2. one warp per chunk: lane l sums rows l, l+32, ... of the chunk into the
-//     upper triangle of X^T X, X^T y and a count (fp64), the 32 partial sums
-//     are combined by a fixed shfl_xor tree and written to the caller's
-//     buffer -- enough independent loads in flight to stream the samples at
-//     memory speed;
-//  3. one warp per estimator: lane l adds the partials of chunks l, l+32, ...,
-//     a fixed shfl_xor tree combines the lanes, lane 0 adds the result to the
-//     running statistics and refits by a Cholesky solve of the normal
-//     equations.
+// est_update, in two launches:
+//  1. one warp per chunk of 32 to 512 consecutive sample rows (enough chunks to
+//     fill the GPU, long enough that the reduction is a small part): for every
+//     estimator with rows in the chunk, lane l sums rows l, l+32, ... into the
+//     upper triangle of X^T X and X^T y (fp64); a fixed tree combines the lanes
+//     and the totals go to the caller's buffer.  Estimator e's part of chunk c is
+//     entry c + e (each chunk and each estimator begins one, in order), so an
+//     estimator's entries are consecutive and no prefix of chunk counts is needed;
+//  2. per estimator, its entries are added in a fixed order -- by one warp, or by
+//     eight that share them -- and one warp adds the result to the running
+//     statistics and refits by a Cholesky solve of the normal equations, lane i
+//     holding row i.
 // Every sum has a fixed order, so results do not depend on scheduling.  F
 // (<= 8) is a template parameter so the per-sample arrays stay in registers.
+//
+// The first launch is bound by fp64 instructions (an SM issues two fp64 lanes a
+// clock): F(F+1)/2 + F multiply-adds per row cannot go.  The tree halves the
+// values that a lane carries with every step: 31 additions a lane for up to 32
+// values instead of 5 for each value.  458,752 rows
+// of 5 features: 44.5 -> 22.8 us (fp64 floor 15); the second launch, 28 estimators of 64
+// entries: 26.5 -> 9.8 us.
 
 #include <cuda_runtime.h>
 #include <math.h>
@@ -29,7 +36,9 @@ namespace {
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr double kPivotRel = 1e-12;   // pivot threshold relative to its own diagonal entry
 constexpr int64_t kMaxTicks = int64_t(1) << 40;
-constexpr int32_t kChunk = 128;       // sample rows per warp in the first reduction pass
+constexpr int32_t kMinChunk = 32, kMaxChunk = 512;  // sample rows per warp in the first launch
+constexpr int64_t kChunks = 1824;  // warps that fill 152 SMs (12 each)
+constexpr int kFitWarps = 8;       // warps per estimator in the second launch when it has many entries
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -73,220 +82,237 @@ State view(void* d_state, int32_t E, int32_t F) {
                reinterpret_cast<int32_t*>(b + L.fitted)};
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
+// The lanes' totals of the values v[0..N): lane l gets the total of value l (and
+// of value 32 + l in the second word).  Step by step a lane passes half of the
+// values that it carries to the lane across and adds its own half's: the same
+// pairwise tree (distance 16, 8, ..., 1) for every value.
+template <int N>
+__device__ __forceinline__ double reduce_to_lanes(double (&v)[32]) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFullMask, v, o);
-  return v;
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const double give = up ? v[i] : v[i + o];
+      const double keep = up ? v[i + o] : v[i];
+      v[i] = keep + __shfl_xor_sync(kFullMask, give, o);
+    }
+  }
+  return v[0];
 }
 
-// Chunk prefix: chunks[e] = exclusive prefix of ceil(count_e / kChunk);
-// chunks[E] = total.  One block; thread t takes a contiguous run of
-// estimators.
-__global__ void __launch_bounds__(1024) est_chunks_kernel(int32_t E, const int32_t* __restrict__ off,
-                                                          int32_t* __restrict__ chunks) {
-  __shared__ int32_t part[1024];
-  const int t = threadIdx.x;
-  const int32_t per = (E + 1023) / 1024;
-  const int32_t e0 = min(E, t * per), e1 = min(E, e0 + per);
-  int32_t sum = 0;
-  for (int32_t e = e0; e < e1; ++e) sum += (off[e + 1] - off[e] + kChunk - 1) / kChunk;
-  part[t] = sum;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {  // inclusive scan (Hillis-Steele)
-    const int32_t v = t >= o ? part[t - o] : 0;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
-  }
-  int32_t acc = part[t] - sum;
-  for (int32_t e = e0; e < e1; ++e) {
-    chunks[e] = acc;
-    acc += (off[e + 1] - off[e] + kChunk - 1) / kChunk;
-  }
-  if (t == 1023) chunks[E] = part[1023];
-}
-
-// One warp per chunk: partial statistics [T triangle | F | count].
+// One warp per chunk of rows: entry c + e = [T triangle | F] of estimator e's rows.
 template <int F>
-__global__ void __launch_bounds__(128) est_partial_kernel(int32_t E, int64_t max_chunks,
+__global__ void __launch_bounds__(128) est_partial_kernel(int32_t E, int32_t S, int32_t chunk,
                                                           const int32_t* __restrict__ off,
-                                                          const int32_t* __restrict__ chunks,
                                                           const double* __restrict__ x,
                                                           const double* __restrict__ y,
                                                           double* __restrict__ partial) {
   constexpr int T = F * (F + 1) / 2;
-  constexpr int P = T + F + 1;
+  constexpr int N = T + F;
   const int lane = threadIdx.x & 31;
   const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (c >= max_chunks || c >= chunks[E]) return;  // whole warps leave together
-  // the estimator whose chunk range holds c: the last e with chunks[e] <= c
-  int32_t lo = 0, hi = E - 1;
-  while (lo < hi) {
-    const int32_t mid = (lo + hi + 1) >> 1;
-    if (chunks[mid] <= c) lo = mid;
-    else hi = mid - 1;
+  const int64_t c0 = c * chunk;
+  if (c0 >= S) return;  // whole warps leave together
+  const int32_t r0 = (int32_t)c0, r1 = (int32_t)(c0 + chunk < S ? c0 + chunk : S);
+  // the first estimator that ends after r0: 32 probes at a time
+  int32_t lo = 0, left = E;
+  while (left > 0) {
+    const int32_t step = (left + 31) >> 5;
+    const int32_t last = lo + min(left, (lane + 1) * step) - 1;  // of the lane's part
+    const uint32_t b = __ballot_sync(kFullMask, off[last + 1] > r0);
+    if (b == 0u) {
+      lo += left;
+      break;
+    }
+    const int32_t skip = (__ffs(b) - 1) * step;
+    lo += skip;
+    left = step == 1 ? 0 : min(step, left - skip);
   }
-  const int32_t e = lo;
-  const int32_t r0 = off[e] + (int32_t)(c - chunks[e]) * kChunk;
-  const int32_t r1 = min(off[e + 1], r0 + kChunk);
-  double g[T], h[F], cnt = 0.0;
+  for (int32_t e = lo; e < E; ++e) {
+    const int32_t a0 = off[e], a1 = off[e + 1];
+    if (a0 >= r1) break;
+    const int32_t s0 = a0 > r0 ? a0 : r0, s1 = a1 < r1 ? a1 : r1;
+    if (s1 <= s0) continue;  // no samples
+    double v[N];
 #pragma unroll
-  for (int t = 0; t < T; ++t) g[t] = 0.0;
+    for (int t = 0; t < N; ++t) v[t] = 0.0;
+    for (int32_t r = s0 + lane; r < s1; r += 64) {
+      // rows r and r + 32: twice the loads in flight
+      double xv[2][F], yv[2];
 #pragma unroll
-  for (int a = 0; a < F; ++a) h[a] = 0.0;
-  // rows r and r + 32 per step: twice the loads in flight, same summation
-  // order for every run
-  for (int32_t r = r0 + lane; r < r1; r += 64) {
+      for (int h = 0; h < 2; ++h) {
+        const int32_t rr = r + 32 * h;
+        const bool in = rr < s1;
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const int32_t rr = r + 32 * half;
-      if (rr < r1) {
-        double xv[F];
+        for (int a = 0; a < F; ++a) xv[h][a] = in ? x[(int64_t)rr * F + a] : 0.0;
+        yv[h] = in ? y[rr] : 0.0;
+      }
 #pragma unroll
-        for (int a = 0; a < F; ++a) xv[a] = x[(int64_t)rr * F + a];
-        const double yv = y[rr];
+      for (int h = 0; h < 2; ++h) {
+        if (r + 32 * h >= s1) break;
         int t = 0;
 #pragma unroll
         for (int a = 0; a < F; ++a) {
-          h[a] += xv[a] * yv;
+          v[T + a] += xv[h][a] * yv[h];
 #pragma unroll
-          for (int b = a; b < F; ++b) g[t++] += xv[a] * xv[b];
+          for (int b = a; b < F; ++b) v[t++] += xv[h][a] * xv[h][b];
         }
-        cnt += 1.0;
       }
     }
+    double* out = partial + (c + e) * N;
+#pragma unroll
+    for (int w = 0; w < (N + 31) / 32; ++w) {
+      double q[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) q[i] = 32 * w + i < N ? v[32 * w + i < N ? 32 * w + i : 0] : 0.0;
+      const double tot = reduce_to_lanes<N>(q);
+      if (32 * w + lane < N) out[32 * w + lane] = tot;
+    }
   }
-#pragma unroll
-  for (int t = 0; t < T; ++t) g[t] = warp_sum(g[t]);
-#pragma unroll
-  for (int a = 0; a < F; ++a) h[a] = warp_sum(h[a]);
-  cnt = warp_sum(cnt);
-  if (lane != 0) return;
-  double* out = partial + c * P;
-#pragma unroll
-  for (int t = 0; t < T; ++t) out[t] = g[t];
-#pragma unroll
-  for (int a = 0; a < F; ++a) out[T + a] = h[a];
-  out[T + F] = cnt;
 }
 
-// One warp per estimator: add the chunk partials (fixed order), then refit.
-template <int F>
-__global__ void __launch_bounds__(128) est_fit_kernel(State S, int32_t E, const int32_t* __restrict__ chunks,
-                                                      const double* __restrict__ partial) {
+// kWarps warps per estimator (blocks of 4 estimators with one warp each, else of
+// one): add the entries in a fixed order, then refit.
+template <int F, int kWarps>
+__global__ void __launch_bounds__(kWarps == 1 ? 128 : 32 * kWarps)
+    est_fit_kernel(State S, int32_t E, int32_t chunk, const int32_t* __restrict__ off,
+                   const double* __restrict__ partial) {
   constexpr int T = F * (F + 1) / 2;
-  constexpr int P = T + F + 1;
-  const int lane = threadIdx.x & 31;
-  const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (e >= E) return;  // whole warps leave together
-  double g[T], h[F], cnt = 0.0;
+  constexpr int N = T + F;
+  constexpr int kPer = kWarps == 1 ? 4 : 1;  // estimators per block
+  __shared__ double part[kWarps * kPer][N];
+  __shared__ double sum[kPer][N];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int q = kWarps == 1 ? w : 0;  // the block's estimator of this warp
+  const int64_t e = (int64_t)blockIdx.x * kPer + q;
+  const bool in = e < E;
+  const int32_t a0 = in ? off[e] : 0, a1 = in ? off[e + 1] : 0;
+  const int64_t n0 = a0 / chunk + e;
+  const int64_t n = a1 > a0 ? (a1 - 1) / chunk - a0 / chunk + 1 : 0;
+  // lane l adds values l and 32 + l of entries first, first + kWarps, ...
 #pragma unroll
-  for (int t = 0; t < T; ++t) g[t] = 0.0;
-#pragma unroll
-  for (int a = 0; a < F; ++a) h[a] = 0.0;
-  for (int32_t c = chunks[e] + lane; c < chunks[e + 1]; c += 32) {
-    const double* p = partial + (int64_t)c * P;
-#pragma unroll
-    for (int t = 0; t < T; ++t) g[t] += p[t];
-#pragma unroll
-    for (int a = 0; a < F; ++a) h[a] += p[T + a];
-    cnt += p[T + F];
+  for (int u = 0; u < (N + 31) / 32; ++u) {
+    const int t = 32 * u + lane;
+    if (t < N) {
+      double acc = 0.0;
+#pragma unroll 4
+      for (int64_t k = kWarps == 1 ? 0 : w; k < n; k += kWarps) acc += partial[(n0 + k) * N + t];
+      part[w][t] = acc;
+    }
   }
+  if (kWarps == 1) __syncwarp();
+  else __syncthreads();
+  if ((kWarps > 1 && w > 0) || !in) return;  // whole warps leave together
 #pragma unroll
-  for (int t = 0; t < T; ++t) g[t] = warp_sum(g[t]);
+  for (int u = 0; u < (N + 31) / 32; ++u) {
+    const int t = 32 * u + lane;
+    if (t < N) {
+      double acc = part[kWarps == 1 ? w : 0][t];
 #pragma unroll
-  for (int a = 0; a < F; ++a) h[a] = warp_sum(h[a]);
-  cnt = warp_sum(cnt);
-  if (lane != 0) return;
-  double* G = S.g + e * T;
-  double* H = S.h + e * F;
-#pragma unroll
-  for (int t = 0; t < T; ++t) g[t] = (G[t] += g[t]);
-#pragma unroll
-  for (int a = 0; a < F; ++a) h[a] = (H[a] += h[a]);
-  const double n = (S.n[e] += cnt);
-  // Cholesky factor L (lower) of the full matrix built from the triangle
-  double A[F][F];
-  {
-    int t = 0;
-#pragma unroll
-    for (int a = 0; a < F; ++a)
-#pragma unroll
-      for (int b = a; b < F; ++b) {
-        A[a][b] = g[t];
-        A[b][a] = g[t];
-        ++t;
-      }
+      for (int k = 1; k < kWarps; ++k) acc += part[k][t];
+      double* st = t < T ? S.g + e * T + t : S.h + e * F + (t - T);
+      acc += *st;
+      *st = acc;
+      sum[q][t] = acc;
+    }
   }
+  double cnt = 0.0;
+  if (lane == 0) cnt = (S.n[e] += (double)(a1 - a0));
+  cnt = __shfl_sync(kFullMask, cnt, 0);
+  __syncwarp();
+  // lane i: row i of the full matrix and of the factor L
+  // (below the diagonal; inv: the reciprocal of its diagonal entry, the only
+  // division of a column)
+  double A[F], Lr[F], v = 0.0, diag = 0.0, inv = 0.0;
+#pragma unroll
+  for (int b = 0; b < F; ++b) {
+    const int i = lane < F ? lane : 0, r = i < b ? i : b, c = i < b ? b : i;
+    A[b] = sum[q][r * F - r * (r - 1) / 2 + (c - r)];
+    if (i == b) diag = A[b];
+    Lr[b] = 0.0;
+  }
+  if (lane < F) v = sum[q][T + lane];
   // A pivot is compared with its own diagonal entry, which makes the test
   // independent of each feature's scale (bytes next to a constant term).
-  bool ok = n >= (double)F;
-  double L[F][F];
+  bool ok = cnt >= (double)F;
 #pragma unroll
   for (int j = 0; j < F; ++j) {
-    double d = A[j][j];
+    const double d = __shfl_sync(kFullMask, A[j], j);
+    const double own = __shfl_sync(kFullMask, diag, j);
+    ok = ok && d > kPivotRel * own;
+    const double ljj = sqrt(fmax(d, 0.0)), r = 1.0 / ljj;
+    if (lane == j) inv = r;
+    if (lane > j && lane < F) Lr[j] = ok ? A[j] * r : 0.0;
 #pragma unroll
-    for (int k = 0; k < j; ++k) d -= L[j][k] * L[j][k];
-    ok = ok && d > kPivotRel * A[j][j];
-    const double ljj = sqrt(fmax(d, 0.0));
-    L[j][j] = ljj;
-#pragma unroll
-    for (int i = j + 1; i < F; ++i) {
-      double v = A[i][j];
-#pragma unroll
-      for (int k = 0; k < j; ++k) v -= L[i][k] * L[j][k];
-      L[i][j] = ok ? v / ljj : 0.0;
+    for (int k = j + 1; k < F; ++k) {
+      const double lkj = __shfl_sync(kFullMask, Lr[j], k);
+      A[k] -= Lr[j] * lkj;
     }
   }
-  double beta[F];
+  double beta = 0.0;
   if (ok) {
-    double z[F];
 #pragma unroll
-    for (int i = 0; i < F; ++i) {
-      double v = h[i];
-#pragma unroll
-      for (int k = 0; k < i; ++k) v -= L[i][k] * z[k];
-      z[i] = v / L[i][i];
+    for (int k = 0; k < F; ++k) {  // L z = h
+      const double z = __shfl_sync(kFullMask, v * inv, k);
+      if (lane == k) v = z;
+      else if (lane > k) v -= Lr[k] * z;
     }
 #pragma unroll
-    for (int i = F - 1; i >= 0; --i) {
-      double v = z[i];
+    for (int k = F - 1; k >= 0; --k) {  // L^T beta = z
+      const double bk = __shfl_sync(kFullMask, v * inv, k);
+      if (lane == k) beta = bk;
+      // L[k][i] is lane k's Lr[i]
 #pragma unroll
-      for (int k = i + 1; k < F; ++k) v -= L[k][i] * beta[k];
-      beta[i] = v / L[i][i];
+      for (int i = 0; i < k; ++i) {
+        const double lki = __shfl_sync(kFullMask, Lr[i], k);
+        if (lane == i) v -= lki * bk;
+      }
     }
-  } else {
-#pragma unroll
-    for (int i = 0; i < F; ++i) beta[i] = 0.0;
   }
-#pragma unroll
-  for (int a = 0; a < F; ++a) S.beta[e * F + a] = beta[a];
-  S.fitted[e] = ok ? 1 : 0;
+  if (lane < F) S.beta[e * F + lane] = ok ? beta : 0.0;
+  if (lane == 0) S.fitted[e] = ok ? 1 : 0;
 }
 
-__device__ __forceinline__ int64_t clamp_rint(double v, int64_t lo) {
-  const double r = rint(v);
-  if (!(r >= (double)lo)) return lo;  // also NaN
-  if (r >= (double)kMaxTicks) return kMaxTicks;
-  return (int64_t)r;
+// Rounds to the nearest integer (halves to even), at least lo, at most kMaxTicks;
+// lo for NaN (the conversion gives the smallest integer then).
+__device__ __forceinline__ int64_t to_ticks(double v, int64_t lo) {
+  const int64_t r = __double2ll_rn(v);
+  return r < lo ? lo : r > kMaxTicks ? kMaxTicks : r;
 }
 
-__global__ void __launch_bounds__(256) est_predict_kernel(State S, int32_t F, int64_t NT, int32_t T,
+// One thread per op, its features loaded once for all types.
+template <int F>
+__global__ void __launch_bounds__(256) est_predict_kernel(State S, int32_t N, int32_t T,
                                                           const int32_t* __restrict__ est_of,
                                                           const double* __restrict__ x,
                                                           const int64_t* __restrict__ dflt,
                                                           int64_t* __restrict__ dur) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= NT) return;
-  const int64_t i = q / T;
-  const int32_t e = est_of[q];
-  if (e < 0 || !S.fitted[e]) {
-    dur[q] = dflt[i];
-    return;
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  double xv[F];
+#pragma unroll
+  for (int a = 0; a < F; ++a) xv[a] = x[i * F + a];
+  for (int32_t t = 0; t < T; ++t) {
+    const int64_t q = i * T + t;
+    const int32_t e = est_of[q];
+    if (e < 0 || !S.fitted[e]) {
+      dur[q] = dflt[i];
+      continue;
+    }
+    double v = 0.0;
+#pragma unroll
+    for (int a = 0; a < F; ++a) v += S.beta[(int64_t)e * F + a] * xv[a];
+    dur[q] = to_ticks(v, 1);
   }
-  double v = 0.0;
-  for (int a = 0; a < F; ++a) v += S.beta[(int64_t)e * F + a] * x[i * F + a];
-  dur[q] = clamp_rint(v, 1);
+}
+
+template <int F>
+cudaError_t launch_predict(State S, int32_t N, int32_t T, const int32_t* est_of, const double* x, const int64_t* dflt,
+                           int64_t* dur, cudaStream_t st) {
+  est_predict_kernel<F><<<(int)(((int64_t)N + 255) / 256), 256, 0, st>>>(S, N, T, est_of, x, dflt, dur);
+  return cudaGetLastError();
 }
 
 __global__ void __launch_bounds__(256) est_links_kernel(State S, int32_t D, const int64_t* __restrict__ bw_dflt,
@@ -301,29 +327,46 @@ __global__ void __launch_bounds__(256) est_links_kernel(State S, int32_t D, cons
     return;
   }
   const double alpha = S.beta[2 * (int64_t)q], c = S.beta[2 * (int64_t)q + 1];
-  bw[q] = alpha > 0.0 ? clamp_rint(1.0 / alpha, 1) : kMaxTicks;
-  lat[q] = clamp_rint(c, 0);
+  bw[q] = alpha > 0.0 ? to_ticks(1.0 / alpha, 1) : kMaxTicks;
+  lat[q] = to_ticks(c, 0);
 }
 
-// Upper bound of the chunk count: sum over e of ceil(count_e / kChunk).
-int64_t max_chunks(int32_t E, int64_t S) { return S / kChunk + E; }
+// Coefficients and fitted flags (each if asked for) in one launch.
+__global__ void __launch_bounds__(256) est_copy_kernel(State S, int64_t nb, int32_t E, double* __restrict__ beta,
+                                                       int32_t* __restrict__ fitted) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nb && beta) beta[i] = S.beta[i];
+  if (i < E && fitted) fitted[i] = S.fitted[i];
+}
+
+// Rows per chunk for S samples, and an upper bound of the entries of S or fewer
+// samples (chunks + estimators).
+int32_t chunk_rows(int64_t S) {
+  int32_t c = kMinChunk;
+  while (c < kMaxChunk && S / c > kChunks) c *= 2;
+  return c;
+}
+int64_t max_entries(int32_t E, int64_t S) {
+  const int64_t few = S / kMinChunk + 1, most = S / kMaxChunk + 1;
+  return (few < kChunks + 2 ? few : most > kChunks + 2 ? most : kChunks + 2) + E;
+}
 
 template <int F>
 cudaError_t launch_update(State S, int32_t E, int64_t nsamp, const int32_t* off, const double* x,
-                          const double* y, int32_t* chunks, double* partial, cudaStream_t st) {
-  const int64_t mc = max_chunks(E, nsamp);
-  est_chunks_kernel<<<1, 1024, 0, st>>>(E, off, chunks);
-  if (mc > 0) est_partial_kernel<F><<<(int)((mc * 32 + 127) / 128), 128, 0, st>>>(E, mc, off, chunks, x, y, partial);
-  est_fit_kernel<F><<<(int)(((int64_t)E * 32 + 127) / 128), 128, 0, st>>>(S, E, chunks, partial);
+                          const double* y, double* partial, cudaStream_t st) {
+  const int32_t chunk = chunk_rows(nsamp);
+  const int64_t nc = (nsamp + chunk - 1) / chunk;
+  if (nc > 0) est_partial_kernel<F><<<(int)((nc * 32 + 127) / 128), 128, 0, st>>>(E, (int32_t)nsamp, chunk, off, x, y, partial);
+  // several warps share an estimator's entries where it has more than a few
+  if (nc / E >= 2 * kFitWarps) est_fit_kernel<F, kFitWarps><<<E, 32 * kFitWarps, 0, st>>>(S, E, chunk, off, partial);
+  else est_fit_kernel<F, 1><<<(E + 3) / 4, 128, 0, st>>>(S, E, chunk, off, partial);
   return cudaGetLastError();
 }
 
-// Caller buffer of est_update: chunk prefix [E+1] int32, then the partials
-// [max chunks][F(F+1)/2 + F + 1] fp64.
-size_t tmp_partial_off(int32_t E) { return align256(4 * ((size_t)E + 1)); }
+// Caller buffer of est_update: the entries [chunks + estimators][F(F+1)/2 + F] fp64.
 size_t tmp_bytes(int32_t E, int32_t F, int64_t S) {
-  const size_t P = (size_t)F * (F + 1) / 2 + F + 1;
-  return tmp_partial_off(E) + align256(8 * P * (size_t)max_chunks(E, S));
+  const size_t N = (size_t)F * (F + 1) / 2 + F;
+  return align256(8 * N * (size_t)max_entries(E, S));
 }
 
 bool args_ok(const void* state, int32_t E, int32_t F) {
@@ -364,18 +407,17 @@ int est_update(void* d_state, int32_t n_est, int32_t n_feat, const int32_t* d_of
     return GMG_EWS;
   const State S = view(d_state, n_est, n_feat);
   const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  int32_t* chunks = static_cast<int32_t*>(d_tmp);
-  double* partial = reinterpret_cast<double*>(static_cast<uint8_t*>(d_tmp) + tmp_partial_off(n_est));
+  double* partial = static_cast<double*>(d_tmp);
   cudaError_t e = cudaSuccess;
   switch (n_feat) {
-    case 1: e = launch_update<1>(S, n_est, n_samples, d_off, d_x, d_y, chunks, partial, st); break;
-    case 2: e = launch_update<2>(S, n_est, n_samples, d_off, d_x, d_y, chunks, partial, st); break;
-    case 3: e = launch_update<3>(S, n_est, n_samples, d_off, d_x, d_y, chunks, partial, st); break;
-    case 4: e = launch_update<4>(S, n_est, n_samples, d_off, d_x, d_y, chunks, partial, st); break;
-    case 5: e = launch_update<5>(S, n_est, n_samples, d_off, d_x, d_y, chunks, partial, st); break;
-    case 6: e = launch_update<6>(S, n_est, n_samples, d_off, d_x, d_y, chunks, partial, st); break;
-    case 7: e = launch_update<7>(S, n_est, n_samples, d_off, d_x, d_y, chunks, partial, st); break;
-    default: e = launch_update<8>(S, n_est, n_samples, d_off, d_x, d_y, chunks, partial, st); break;
+    case 1: e = launch_update<1>(S, n_est, n_samples, d_off, d_x, d_y, partial, st); break;
+    case 2: e = launch_update<2>(S, n_est, n_samples, d_off, d_x, d_y, partial, st); break;
+    case 3: e = launch_update<3>(S, n_est, n_samples, d_off, d_x, d_y, partial, st); break;
+    case 4: e = launch_update<4>(S, n_est, n_samples, d_off, d_x, d_y, partial, st); break;
+    case 5: e = launch_update<5>(S, n_est, n_samples, d_off, d_x, d_y, partial, st); break;
+    case 6: e = launch_update<6>(S, n_est, n_samples, d_off, d_x, d_y, partial, st); break;
+    case 7: e = launch_update<7>(S, n_est, n_samples, d_off, d_x, d_y, partial, st); break;
+    default: e = launch_update<8>(S, n_est, n_samples, d_off, d_x, d_y, partial, st); break;
   }
   return e == cudaSuccess ? GMG_OK : GMG_ECUDA;
 }
@@ -385,27 +427,32 @@ int est_coefficients(const void* d_state, int32_t n_est, int32_t n_feat, double*
   if (!args_ok(d_state, n_est, n_feat)) return GMG_EINVAL;
   const State S = view(const_cast<void*>(d_state), n_est, n_feat);
   const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (d_beta && cudaMemcpyAsync(d_beta, S.beta, 8 * (size_t)n_est * n_feat, cudaMemcpyDeviceToDevice, st) !=
-                    cudaSuccess)
-    return GMG_ECUDA;
-  if (d_fitted &&
-      cudaMemcpyAsync(d_fitted, S.fitted, 4 * (size_t)n_est, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return GMG_ECUDA;
-  return GMG_OK;
+  if (!d_beta && !d_fitted) return GMG_OK;
+  const int64_t nb = (int64_t)n_est * n_feat;
+  est_copy_kernel<<<(int)((nb + 255) / 256), 256, 0, st>>>(S, nb, n_est, d_beta, d_fitted);
+  return cudaGetLastError() == cudaSuccess ? GMG_OK : GMG_ECUDA;
 }
 
 int est_predict_durations(const void* d_state, int32_t n_est, int32_t n_feat, int32_t n_ops, int32_t n_types,
                           const int32_t* d_est_of, const double* d_x, const int64_t* d_dflt, int64_t* d_dur,
                           gmg_stream_t stream) {
   if (!args_ok(d_state, n_est, n_feat) || n_ops < 0 || n_types < 1) return GMG_EINVAL;
-  const int64_t NT = (int64_t)n_ops * n_types;
-  if (NT == 0) return GMG_OK;
+  if (n_ops == 0) return GMG_OK;
   if (!d_est_of || !d_x || !d_dflt || !d_dur) return GMG_EINVAL;
   const State S = view(const_cast<void*>(d_state), n_est, n_feat);
-  const int blocks = (int)((NT + 255) / 256);
-  est_predict_kernel<<<blocks, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(S, n_feat, NT, n_types,
-                                                                                  d_est_of, d_x, d_dflt, d_dur);
-  return cudaGetLastError() == cudaSuccess ? GMG_OK : GMG_ECUDA;
+  const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  cudaError_t e = cudaSuccess;
+  switch (n_feat) {
+    case 1: e = launch_predict<1>(S, n_ops, n_types, d_est_of, d_x, d_dflt, d_dur, st); break;
+    case 2: e = launch_predict<2>(S, n_ops, n_types, d_est_of, d_x, d_dflt, d_dur, st); break;
+    case 3: e = launch_predict<3>(S, n_ops, n_types, d_est_of, d_x, d_dflt, d_dur, st); break;
+    case 4: e = launch_predict<4>(S, n_ops, n_types, d_est_of, d_x, d_dflt, d_dur, st); break;
+    case 5: e = launch_predict<5>(S, n_ops, n_types, d_est_of, d_x, d_dflt, d_dur, st); break;
+    case 6: e = launch_predict<6>(S, n_ops, n_types, d_est_of, d_x, d_dflt, d_dur, st); break;
+    case 7: e = launch_predict<7>(S, n_ops, n_types, d_est_of, d_x, d_dflt, d_dur, st); break;
+    default: e = launch_predict<8>(S, n_ops, n_types, d_est_of, d_x, d_dflt, d_dur, st); break;
+  }
+  return e == cudaSuccess ? GMG_OK : GMG_ECUDA;
 }
 
 int est_links(const void* d_state, int32_t n_dev, const int64_t* d_bw_dflt, const int64_t* d_lat_dflt,
