@@ -316,7 +316,8 @@ size_t select_best_tmp_bytes(int32_t K);
  * (score, k) (score_mode 0) or (sla_miss, score, k) (mode 1) over candidates
  * with status 0 and viol_flag 0, or -1 if none; d_best[1] = its score
  * (INT64_MAX if none).  Reads status, viol_flag, score, sla_miss of d_out.
- * Two launches: per-block argmin, then a final argmin. */
+ * Two launches (per-block argmin, then a final argmin), or one up to 4,096
+ * candidates. */
 int select_best(const sim_out_t* d_out, int32_t K, int32_t score_mode, int64_t* d_best,
                 void* d_tmp, size_t tmp_bytes, gmg_stream_t stream);
 

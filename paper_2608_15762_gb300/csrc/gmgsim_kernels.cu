@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(64, 1) sim_base_pair_kernel(const __grid_const
 // ---------------------------------------------------------------------------
 // select_best (Algorithm 1, BestRecordedCandidateResult): block argmin of
 // (mode ? sla_miss : 0, score, k) over eligible candidates, then a one-block
-// final argmin.
+// final argmin; one block alone for few candidates.
 // ---------------------------------------------------------------------------
 struct Rank {
   int64_t a;  // sla_miss (mode 1) or 0; INT64_MAX = not eligible
@@ -108,9 +108,8 @@ __device__ Rank block_argmin(Rank r) {
   return r;
 }
 
-__global__ void __launch_bounds__(256) select_partial_kernel(const int32_t* status, const int32_t* viol,
-                                                             const int64_t* score, const int32_t* miss,
-                                                             int32_t K, int32_t mode, Rank* part) {
+__device__ __forceinline__ Rank best_of(const int32_t* status, const int32_t* viol, const int64_t* score,
+                                        const int32_t* miss, int32_t K, int32_t mode) {
   Rank r{kI64Max, kI64Max, kI64Max};
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < K;
        k += (int64_t)gridDim.x * blockDim.x) {
@@ -118,7 +117,19 @@ __global__ void __launch_bounds__(256) select_partial_kernel(const int32_t* stat
     const Rank c{mode ? (int64_t)miss[k] : 0, score[k], k};
     if (rank_less(c, r)) r = c;
   }
-  r = block_argmin(r);
+  return block_argmin(r);
+}
+
+__device__ __forceinline__ void write_best(const Rank& r, int64_t* best) {
+  const bool none = r.k == kI64Max;
+  best[0] = none ? -1 : r.k;
+  best[1] = none ? kI64Max : r.s;
+}
+
+__global__ void __launch_bounds__(256) select_partial_kernel(const int32_t* status, const int32_t* viol,
+                                                             const int64_t* score, const int32_t* miss,
+                                                             int32_t K, int32_t mode, Rank* part) {
+  const Rank r = best_of(status, viol, score, miss, K, mode);
   if (threadIdx.x == 0) part[blockIdx.x] = r;
 }
 
@@ -127,12 +138,18 @@ __global__ void __launch_bounds__(256) select_final_kernel(const Rank* part, int
   for (int i = threadIdx.x; i < nparts; i += blockDim.x)
     if (rank_less(part[i], r)) r = part[i];
   r = block_argmin(r);
-  if (threadIdx.x == 0) {
-    const bool none = r.k == kI64Max;
-    best[0] = none ? -1 : r.k;
-    best[1] = none ? kI64Max : r.s;
-  }
+  if (threadIdx.x == 0) write_best(r, best);
 }
+
+// Up to kSelectOne candidates: one block does both (a second launch costs more
+// than the few rows that each thread goes through).
+__global__ void __launch_bounds__(1024) select_one_kernel(const int32_t* status, const int32_t* viol,
+                                                          const int64_t* score, const int32_t* miss, int32_t K,
+                                                          int32_t mode, int64_t* best) {
+  const Rank r = best_of(status, viol, score, miss, K, mode);
+  if (threadIdx.x == 0) write_best(r, best);
+}
+constexpr int32_t kSelectOne = 4096;
 
 }  // namespace
 
@@ -220,6 +237,11 @@ cudaError_t launch_base(bool pair, const SimParams& P, size_t smem, cudaStream_t
 cudaError_t launch_select(const int32_t* status, const int32_t* viol, const int64_t* score,
                           const int32_t* miss, int32_t K, int32_t mode, void* tmp, int nparts,
                           int64_t* best, cudaStream_t st) {
+  if (K <= kSelectOne) {
+    const int threads = K <= 32 ? 32 : (K + 31) / 32 * 32;
+    select_one_kernel<<<1, threads < 1024 ? threads : 1024, 0, st>>>(status, viol, score, miss, K, mode, best);
+    return cudaGetLastError();
+  }
   Rank* part = reinterpret_cast<Rank*>(tmp);
   select_partial_kernel<<<nparts, 256, 0, st>>>(status, viol, score, miss, K, mode, part);
   cudaError_t e = cudaGetLastError();

@@ -142,3 +142,18 @@ def test_both_sides_of_the_two_warp_line(D, more):
     torch.cuda.synchronize()
     compare(out.to_numpy(), *oracle_rows(d, rows))
     compare(inc.to_numpy(), *O.incremental_batch(d, base, mv))
+
+
+@pytest.mark.parametrize("K", [1, 32, 33, 1024, 1025, 4096, 4097])
+def test_select_best_on_both_sides_of_one_block(K):
+    g = np.random.default_rng(K)
+    out = G.SimOut.empty(K, 1, 1, "cuda")
+    st = (g.random(K) < 0.2).astype(np.int32)
+    vf = (g.random(K) < 0.3).astype(np.int32)
+    sc, ms = g.integers(0, max(2, K // 2), K), g.integers(0, 3, K).astype(np.int32)
+    for t, a in ((out.status, st), (out.viol_flag, vf), (out.score, sc), (out.sla_miss, ms)):
+        t.copy_(torch.from_numpy(np.ascontiguousarray(a)))
+    for mode in (0, 1):
+        ok = [(int(ms[k]) if mode else 0, int(sc[k]), k) for k in range(K) if st[k] == 0 and vf[k] == 0]
+        want = [min(ok)[2], min(ok)[1]] if ok else [-1, np.iinfo(np.int64).max]
+        assert G.select_best(out, score_mode=mode).cpu().tolist() == want
