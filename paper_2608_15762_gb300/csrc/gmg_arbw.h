@@ -17,6 +17,7 @@ struct ArbWParams {
   int32_t shared_links;   // 1 if two ordered pairs share a link id
   int32_t xcap;           // transfers per candidate (sum over ops of min(successors, D-1))
   int32_t smem_arb;       // shared bytes of the arbitration state per warp
+  int32_t few;            // 1: the instance with more registers and fewer blocks per SM
   int64_t smem_std;       // shared bytes of the simulation state of all warps of a block
   // byte offsets inside a warp's scratch slot
   int64_t off_cnt;        // int32 [N]  inputs present (joins)
@@ -29,7 +30,7 @@ struct ArbWParams {
 };
 
 cudaError_t set_arbw_smem_limit();
-const void* arbw_kernel_ptr(const DevGmg& g);
+const void* arbw_kernel_ptr(const DevGmg& g, bool few);
 cudaError_t launch_arbw(const ArbWParams& A, int grid, int block, size_t smem,
                         cudaStream_t st);
 

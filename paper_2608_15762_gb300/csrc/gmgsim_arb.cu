@@ -785,8 +785,13 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode, kHot>, Sim<true, kMode, tr
   }
 };
 
+// 96 registers a thread, 5 blocks per SM: at 72 and 7 blocks the spills cost more
+// than the two blocks give (prefill graph, ms, 7 blocks / 5: 2,048 placements
+// 12.7 / 9.6, 3,000 15.0 / 10.6, 4,096 18.4 / 18.6).
+constexpr int kArbBlocks = 5;
+
 template <bool kT32, bool kTypes, int kHot>
-__global__ void __launch_bounds__(128, 7) sim_arb_kernel(const __grid_constant__ ArbParams A) {
+__global__ void __launch_bounds__(128, kArbBlocks) sim_arb_kernel(const __grid_constant__ ArbParams A) {
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
@@ -846,7 +851,7 @@ __global__ void __launch_bounds__(32, 1) sim_arb_base_kernel(const __grid_consta
 
 // Incremental candidates resumed from the arbitrated base snapshot.
 template <bool kT32, bool kTypes, int kHot>
-__global__ void __launch_bounds__(128, 7) sim_arb_inc_kernel(const __grid_constant__ ArbParams A) {
+__global__ void __launch_bounds__(128, kArbBlocks) sim_arb_inc_kernel(const __grid_constant__ ArbParams A) {
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;

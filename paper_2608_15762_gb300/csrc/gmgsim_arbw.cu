@@ -368,8 +368,11 @@ struct ArbWSim : ArbEvents<ArbWSim<kT32, kTypes, kHot>, Sim<false, kFull, true, 
   }
 };
 
-template <bool kT32, bool kTypes, int kHot>
-__global__ void __launch_bounds__(128, 6) sim_arbw_kernel(const __grid_constant__ ArbWParams A) {
+// kBlocks per SM: 4 (128 registers a thread) while that holds all candidates,
+// else 6 (80).  Ms on 64 accelerators, 6,208 ops, 6 blocks / 4: 1,024 placements
+// 46.4 / 40.6, 2,400 52.1 / 45.7, 3,600 60.8 / 86.7.
+template <bool kT32, bool kTypes, int kHot, int kBlocks>
+__global__ void __launch_bounds__(128, kBlocks) sim_arbw_kernel(const __grid_constant__ ArbWParams A) {
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
@@ -400,14 +403,16 @@ __global__ void __launch_bounds__(128, 6) sim_arbw_kernel(const __grid_constant_
 
 // Instances by (32-bit times, accelerator types; compact records wherever the
 // graph has them).
-const void* arbw_kernel_ptr(const DevGmg& g) {
-  if (g.hot_ok) return (const void*)sim_arbw_kernel<true, false, kHotGlobal>;
+template <int kBlocks>
+const void* arbw_ptr(const DevGmg& g) {
+  if (g.hot_ok) return (const void*)sim_arbw_kernel<true, false, kHotGlobal, kBlocks>;
   if (g.t32)
-    return g.ntypes >= 2 ? (const void*)sim_arbw_kernel<true, true, kHotNone>
-                         : (const void*)sim_arbw_kernel<true, false, kHotNone>;
-  return g.ntypes >= 2 ? (const void*)sim_arbw_kernel<false, true, kHotNone>
-                       : (const void*)sim_arbw_kernel<false, false, kHotNone>;
+    return g.ntypes >= 2 ? (const void*)sim_arbw_kernel<true, true, kHotNone, kBlocks>
+                         : (const void*)sim_arbw_kernel<true, false, kHotNone, kBlocks>;
+  return g.ntypes >= 2 ? (const void*)sim_arbw_kernel<false, true, kHotNone, kBlocks>
+                       : (const void*)sim_arbw_kernel<false, false, kHotNone, kBlocks>;
 }
+const void* arbw_kernel_ptr(const DevGmg& g, bool few) { return few ? arbw_ptr<4>(g) : arbw_ptr<6>(g); }
 
 // Every instance may ask for the shared memory that the device has.
 cudaError_t set_arbw_smem_limit() {
@@ -415,18 +420,18 @@ cudaError_t set_arbw_smem_limit() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   DevGmg g{};
-  for (int c = 0; c < 8 && e == cudaSuccess; ++c) {
+  for (int c = 0; c < 16 && e == cudaSuccess; ++c) {
     g.hot_ok = c & 1;
     g.t32 = (c >> 1) & 1;
     g.ntypes = c & 4 ? 2 : 0;
-    e = cudaFuncSetAttribute(arbw_kernel_ptr(g), cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    e = cudaFuncSetAttribute(arbw_kernel_ptr(g, (c & 8) != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
   }
   return e;
 }
 
 cudaError_t launch_arbw(const ArbWParams& A, int grid, int block, size_t smem, cudaStream_t st) {
   void* args[] = {const_cast<ArbWParams*>(&A)};
-  return cudaLaunchKernel(arbw_kernel_ptr(A.P.g), dim3(grid), dim3(block), args, smem, st);
+  return cudaLaunchKernel(arbw_kernel_ptr(A.P.g, A.few != 0), dim3(grid), dim3(block), args, smem, st);
 }
 
 }  // namespace gsim

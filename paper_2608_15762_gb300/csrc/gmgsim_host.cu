@@ -809,11 +809,15 @@ int plan_arbw(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbWParam
   }
   const int sms = device_sms();
   if (sms <= 0) return GMG_ECUDA;
-  int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, arbw_kernel_ptr(G), 32 * L.wpb,
-                                                    L.smem) != cudaSuccess)
+  // few candidates: the instance with more registers, if it holds them all at
+  // once or the other one holds no more (shared memory)
+  int bps = 0, many = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, arbw_kernel_ptr(G, true), 32 * L.wpb, L.smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&many, arbw_kernel_ptr(G, false), 32 * L.wpb, L.smem) !=
+          cudaSuccess)
     return GMG_ECUDA;
-  bps = std::max(bps, 1);
+  A.few = K <= (int64_t)sms * bps * L.wpb || many <= bps ? 1 : 0;
+  bps = std::max(A.few ? bps : many, 1);
   const int64_t need = (std::max<int64_t>(K, 1) + L.wpb - 1) / L.wpb;
   L.grid = (int)std::min<int64_t>(need, (int64_t)sms * bps);
   L.slots = (int64_t)L.grid * L.wpb;

@@ -144,6 +144,19 @@ def test_both_sides_of_the_two_warp_line(D, more):
     compare(inc.to_numpy(), *O.incremental_batch(d, base, mv))
 
 
+@pytest.mark.parametrize("more", [0, 1])
+def test_both_sides_of_the_wide_arbitrated_line(more):
+    """As many candidates as the instance with four blocks per SM holds, and one more."""
+    d = _chains(30, D=33, chains=5, length=4, fan=2, bytes_lo=1 << 18, cap=6 << 20)
+    g = G.gmg_create(d)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    K = 16 * sms + more
+    rows = _rows(31, K, d.n_ops, 33)
+    out = G.sim_batch(g, torch_place(rows), req_done=True, arbitrated=True)
+    torch.cuda.synchronize()
+    compare(out.to_numpy(), *O.simulate_batch(d, rows, arbitrated=True))
+
+
 @pytest.mark.parametrize("K", [1, 32, 33, 1024, 1025, 4096, 4097])
 def test_select_best_on_both_sides_of_one_block(K):
     g = np.random.default_rng(K)
