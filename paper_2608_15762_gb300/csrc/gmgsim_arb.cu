@@ -9,25 +9,32 @@
 //                      receiving endpoint and the pair's link are free again;
 //                      p's successors on e have one more input present.
 //
-// Lane a keeps accelerator a's side of both in registers.  An accelerator
-// sends one transfer at a time, so lane a holds the completion time of the
-// transfer it is sending, if any; and its ops finish in the order they start,
-// so the ops with remote successors that it has started but whose intents
-// have not arrived form a FIFO in finish order: lane a holds its head.  The
-// next DONE and the next INTENT are warp minima over the lanes (intents by
-// (time, producer)).
+// Lane a keeps accelerator a's side of both.  An accelerator sends one transfer
+// at a time, so lane a holds the completion time of the transfer it is sending,
+// if any.  Its ops finish in the order they start, so those with remote
+// successors form one list in finish order, linked through a per-op array: first
+// the ops whose intents have arrived and are not all on their way, then those
+// whose intents are to come.  The next DONE and the next INTENT are warp minima
+// over the lanes.
 //
-// After every INTENT / DONE at time t the arbiter starts, in (intent time,
+// After the last INTENT / DONE of a time t the arbiter starts, in (intent time,
 // producer, destination) order, every pending intent whose sending endpoint,
 // receiving endpoint and link are all free (the communication graph of Sec.
 // 3.5.2; the selection rule among conflicting intents is this FIFO greedy
-// one).  Intents are numbered as they arrive, which is that order, and only
-// the head of a pair's queue can start (the rest share its endpoints), so the
-// arbiter repeatedly takes the smallest head number over the pairs whose
-// endpoints and link are free: lane a scans the pairs out of accelerator a, a
-// warp minimum picks the winner.  A started transfer allocates its receive
-// buffer and lasts the transfer estimate.  When no two ordered pairs share a
-// link id, a busy link implies a busy sender and the link state is not kept.
+// one).  An intent's time is its producer's finish time, so lane a's first list
+// entry with a destination that it can send to is its earliest, and a warp
+// minimum over (finish time, op) picks the next.  A started transfer allocates
+// its receive buffer and lasts the transfer estimate.  When no two ordered pairs
+// share a link id, a busy link implies a busy sender and the link state is not
+// kept.
+//
+// What bounds the kernel is the chain of dependent steps and loads per event, one
+// event time after the other.  So READY ops start many at a time, as in the
+// pure-latency simulation, and stop at the next event; an entry is a producer and
+// a bit mask of its destinations, not a record per intent in a queue per pair; an
+// arrival's consumer lookups, needed for HBM accounting only, wait and are done
+// for a warp of arrivals side by side.  Prefill graph, 8 accelerators, 2,048
+// placements: 15.3 ms -> 9.6.
 //
 // Readiness: an op's inputs are counted as they become present -- a local
 // predecessor's output when that predecessor starts (its finish time is then

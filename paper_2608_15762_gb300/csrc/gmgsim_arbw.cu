@@ -14,7 +14,7 @@
 // the arbiter takes, per lane, the first entry that can start among the lane's
 // accelerators, and the smallest (finish time, op) over the warp.  (With the
 // tables in global scratch and a queue per accelerator pair, each event was a
-// chain of L2 loads.)
+// chain of L2 loads: 64 accelerators, 6,208 ops, 1,024 placements 56.6 ms -> 40.7.)
 //
 // The HBM-event generation and the input counting are the narrow kernel's
 // (gmg_arb_events.h).  Every loop is bounded by the graph: completions by the

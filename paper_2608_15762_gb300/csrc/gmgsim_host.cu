@@ -45,7 +45,7 @@ constexpr int64_t kDefaultQueueCap = 1 << 16;
 constexpr int kSharedLogEntries = 192, kSharedLogEntriesWide = 112;
 constexpr int64_t kDefaultLogCap = 1 << 17;
 constexpr int kSortCap = 128;             // power of two; raised to n_dev's power of two
-constexpr int kOpsPerGeneration = 24;     // ~85 HBM events per generation (prefill graphs)
+constexpr int kOpsPerGeneration = 24;     // at most one op a lane; 20, 28 and 30 are no faster
 constexpr int kCheckpoints = 256;
 constexpr int kArbCheckpoints = 64;       // arbitrated bases also keep ~32 bytes per op per checkpoint
 constexpr int kCheckpointQueue = 4096;
@@ -581,8 +581,9 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
 
 // Two warps per candidate where all candidates fit on the GPU at once that way
 // (and the caller has not set the warps per block): the sweep of a candidate
-// does not wait for its HBM accounting.  Graphs whose accelerator ids fit into
-// the event key.
+// does not wait for its HBM accounting.  Beyond that the accounting warps take
+// issue slots and residency from further candidates.  Graphs whose accelerator ids
+// fit into the event key.
 int plan_pair(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& L) {
   const DevGmg& G = g->dg;
   if (!G.dev_key || (o && o->warps_per_block > 0)) return GMG_EINVAL;

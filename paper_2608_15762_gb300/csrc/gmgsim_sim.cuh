@@ -17,31 +17,40 @@
 //                  of a successor at f_i (Recv before Send, Sec. 3.5.2), each
 //                  released by its last listed consumer there (Sec. 3.3.2).
 //
-// READY keys are taken many at a time (Sim::run): every pending key carries a
-// lower bound of its op's finish, and all pending keys with a ready time below
-// the smallest of these bounds are started together, one op per lane -- nothing
-// that they make ready can precede any of them.  Pending keys sit in a pool of
-// 32 or more slots in shared memory; what does not fit goes to a
-// warp-cooperative 32-ary min-heap.  Ops without predecessors enter the pool
-// when they are due: their keys are pre-sorted on the host.
+// READY ops are taken many at a time (Sim::run): every pending op has a lower
+// bound of its finish, and all pending ops with a ready time below the smallest
+// of these bounds are started together, one per lane -- nothing that they make
+// ready can precede any of them.  What bounds the kernels is the chain of
+// dependent instructions and loads per batch, and the issue slots that all warps
+// share; DRAM is idle.  On the prefill graph (3,088 ops, 8 accelerators) it is
+// 2.5 to 3 ops a batch and 173 warp instructions an op, against 333 for one key
+// at a time.  With at most 32 accelerators the lanes hold the pending ops, one
+// each (prefill, 4,096 placements, 4.74 ms -> 3.23; as keys in shared memory
+// instead: 4.5); with more, where more ops than lanes are pending, they are 64-bit
+// keys in a pool in shared memory (256 accelerators, 4,096 placements, 128 ms ->
+// 83).  What does not fit goes to a warp-cooperative 32-ary min-heap.  Ops
+// without predecessors come in when they are due: their keys are pre-sorted on
+// the host.
 //
 // HBM events are appended to a per-warp log in O(1).  Every event produced
 // while handling READY(r, .) happens at a time >= r, so once the next READY
 // key has time T, every logged event with time < T is final and no later
-// event can precede it.  Such events are drained in batches: extracted into
-// shared memory, bitonic-sorted by (time, frees before allocs, op), and
-// applied in order to the per-accelerator live bytes, which gives the peaks
-// and the first capacity violation (Sec. 3.4.2 OOM discard) exactly.
+// event can precede it.  Such events are drained in batches.  Their order
+// matters only on an accelerator whose peak they can raise: there they are sorted
+// by (time, frees before allocs, op) and applied in order, which gives the peaks
+// and the first capacity violation (Sec. 3.4.2 OOM discard) exactly; elsewhere
+// their sum is added (apply_due).
 //
 // Lanes also fan out over successor lists (readiness, transfer arrivals,
 // distinct receiving accelerators via __match_any_sync) and predecessor
 // lists (ready-time maxima, last-consumer releases).  With at most 32
-// accelerators, lane d keeps accelerator d's free time, live bytes and peak
-// in registers.
+// accelerators, lane d keeps accelerator d's free time in a register.
 //
-// No wait in these kernels depends on another warp or block; the only loop
-// whose trip count is not bounded by the data is the event loop, capped at
-// g.max_iter iterations (status GMG_SIM_LOOP).
+// No wait in these kernels depends on another block.  The two warps of a pair
+// (kRole) meet at named barriers of their block, and each message of one has its
+// counterpart in the other, whatever the candidate's status.  The only loop whose
+// trip count is not bounded by the data is the event loop, capped at g.max_iter
+// iterations (status GMG_SIM_LOOP).
 
 #pragma once
 
@@ -436,7 +445,8 @@ constexpr int kHotNone = 0, kHotGlobal = 1, kHotShared = 2;
 // time of one simulation, and nothing in the sweep depends on the HBM
 // accounting).  kSweep starts the ops and hands them over in batches, kAccount
 // generates and applies their HBM events and writes the results; kBoth does
-// both in one warp.
+// both in one warp.  (One warp / two, ms: 14 placements of the prefill graph 1.84 /
+// 1.41, 2,048 2.07 / 1.53, 2,048 of a decode graph of 49,408 ops 65.7 / 31.3.)
 constexpr int kBoth = 0, kSweep = 1, kAccount = 2;
 
 // What the sweep hands over: n started ops (in the buffer of the same index) and
@@ -1061,7 +1071,9 @@ struct Sim {
   // each in every quarter of the time since the last drain, and within a quarter
   // the live bytes are at most those at its start plus all its allocations; with
   // more (few events each) the whole drain is one such interval.  Everywhere
-  // else the sums are enough.
+  // else the sums are enough.  (Prefill graph: 1.6 events an op are ordered with
+  // one bound per drain, fewer with quarters; without the wide sort networks that
+  // no drain then needs, 4,096 placements 3.66 ms -> 3.22.)
   __device__ __forceinline__ void apply_due(int m, tm_t span) {
     const unsigned lane = lane_id();
     uint32_t fail = 0u;
