@@ -173,6 +173,19 @@ __global__ void __launch_bounds__(128) est_partial_kernel(int32_t E, int32_t S, 
   }
 }
 
+__device__ __forceinline__ double tree8(const double (&a)[8]) {
+  return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+}
+
+// a / d from r = 1 / d: the product, corrected once by its residual (without that
+// the coefficients' error against exact sums grows by a sixth; with a division
+// each, 15 in a row, the kernel takes 7 us more).  d and r are finite and positive
+// wherever the result is used.
+__device__ __forceinline__ double quotient(double a, double d, double r) {
+  const double q = a * r, e = fma(-q, d, a);
+  return e == e ? fma(e, r, q) : q;  // an infinite q has no residual
+}
+
 // kWarps warps per estimator (blocks of 4 estimators with one warp each, else of
 // one): add the entries in a fixed order, then refit.
 template <int F, int kWarps>
@@ -196,10 +209,17 @@ __global__ void __launch_bounds__(kWarps == 1 ? 128 : 32 * kWarps)
   for (int u = 0; u < (N + 31) / 32; ++u) {
     const int t = 32 * u + lane;
     if (t < N) {
-      double acc = 0.0;
-#pragma unroll 4
-      for (int64_t k = kWarps == 1 ? 0 : w; k < n; k += kWarps) acc += partial[(n0 + k) * N + t];
-      part[w][t] = acc;
+      // eight sums side by side: their loads overlap, and short sums and a tree
+      // lose less than one long sum
+      double a[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) a[c] = 0.0;
+      for (int64_t k = kWarps == 1 ? 0 : w; k < n; k += 8 * kWarps) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          if (k + c * kWarps < n) a[c] += partial[(n0 + k + c * kWarps) * N + t];
+      }
+      part[w][t] = tree8(a);
     }
   }
   if (kWarps == 1) __syncwarp();
@@ -210,8 +230,12 @@ __global__ void __launch_bounds__(kWarps == 1 ? 128 : 32 * kWarps)
     const int t = 32 * u + lane;
     if (t < N) {
       double acc = part[kWarps == 1 ? w : 0][t];
+      if (kWarps == 8) {
+        double a[8];
 #pragma unroll
-      for (int k = 1; k < kWarps; ++k) acc += part[k][t];
+        for (int c = 0; c < 8; ++c) a[c] = part[c % kWarps][t];
+        acc = tree8(a);
+      }
       double* st = t < T ? S.g + e * T + t : S.h + e * F + (t - T);
       acc += *st;
       *st = acc;
@@ -223,9 +247,8 @@ __global__ void __launch_bounds__(kWarps == 1 ? 128 : 32 * kWarps)
   cnt = __shfl_sync(kFullMask, cnt, 0);
   __syncwarp();
   // lane i: row i of the full matrix and of the factor L
-  // (below the diagonal; inv: the reciprocal of its diagonal entry, the only
-  // division of a column)
-  double A[F], Lr[F], v = 0.0, diag = 0.0, inv = 0.0;
+  // (below the diagonal; own_l, inv: its diagonal entry and the reciprocal)
+  double A[F], Lr[F], v = 0.0, diag = 0.0, own_l = 1.0, inv = 1.0;
 #pragma unroll
   for (int b = 0; b < F; ++b) {
     const int i = lane < F ? lane : 0, r = i < b ? i : b, c = i < b ? b : i;
@@ -243,8 +266,11 @@ __global__ void __launch_bounds__(kWarps == 1 ? 128 : 32 * kWarps)
     const double own = __shfl_sync(kFullMask, diag, j);
     ok = ok && d > kPivotRel * own;
     const double ljj = sqrt(fmax(d, 0.0)), r = 1.0 / ljj;
-    if (lane == j) inv = r;
-    if (lane > j && lane < F) Lr[j] = ok ? A[j] * r : 0.0;
+    if (lane == j) {
+      own_l = ljj;
+      inv = r;
+    }
+    if (lane > j && lane < F) Lr[j] = ok ? quotient(A[j], ljj, r) : 0.0;
 #pragma unroll
     for (int k = j + 1; k < F; ++k) {
       const double lkj = __shfl_sync(kFullMask, Lr[j], k);
@@ -255,13 +281,13 @@ __global__ void __launch_bounds__(kWarps == 1 ? 128 : 32 * kWarps)
   if (ok) {
 #pragma unroll
     for (int k = 0; k < F; ++k) {  // L z = h
-      const double z = __shfl_sync(kFullMask, v * inv, k);
+      const double z = __shfl_sync(kFullMask, quotient(v, own_l, inv), k);
       if (lane == k) v = z;
       else if (lane > k) v -= Lr[k] * z;
     }
 #pragma unroll
     for (int k = F - 1; k >= 0; --k) {  // L^T beta = z
-      const double bk = __shfl_sync(kFullMask, v * inv, k);
+      const double bk = __shfl_sync(kFullMask, quotient(v, own_l, inv), k);
       if (lane == k) beta = bk;
       // L[k][i] is lane k's Lr[i]
 #pragma unroll
