@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <functional>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -62,7 +63,7 @@ struct Layout {
 struct Built {
   int n = 0, E = 0, D = 0, R = 0, Ec = 0, nroots = 0, ib = 1, T = 0;
   bool uniform = true;
-  int64_t bw0 = 1, lat0 = 0, time_bound = 0, max_iter = 0, queue_bound = 0, log_bound = 0;
+  int64_t bw0 = 1, lat0 = 0, time_bound = 0, max_iter = 0, queue_bound = 0, log_bound = 0, burst = 0;
   std::vector<OpRec> ops;
   std::vector<uint32_t> succ, pred, sib, cons;
   std::vector<uint64_t> roots;
@@ -405,6 +406,16 @@ int build(const gmg_desc_t* d, Built& b) {
   b.max_iter = (int64_t)iters;
   b.queue_bound = (int64_t)qb;
   b.log_bound = (int64_t)lb;
+  {
+    // the most HBM events that starting 32 ops logs: their own copies and those they
+    // send, and the inputs they release
+    std::vector<int64_t> ev(n);
+    for (int i = 0; i < n; ++i)
+      ev[i] = 2 + 2 * (int64_t)std::min<uint32_t>(b.ops[i].nsucc, (uint32_t)(D - 1)) + b.ops[i].npred;
+    const int m = std::min(n, 32);
+    std::partial_sort(ev.begin(), ev.begin() + m, ev.end(), std::greater<int64_t>());
+    for (int i = 0; i < m; ++i) b.burst += ev[i];
+  }
   // roots, by (release, id)
   for (int i = 0; i < n; ++i)
     if (b.ops[i].npred == 0)
@@ -449,6 +460,7 @@ struct gmg {
   gmg_info_t info;
   int64_t queue_bound;
   int64_t log_bound;
+  int64_t burst;           // HBM events that starting 32 ops logs at most
   const uint16_t* linkid;  // device [D*D]
   int32_t shared_links;    // 1 if two distinct ordered pairs share a link id
   int64_t xfer_bound;
@@ -480,10 +492,18 @@ int queue_cap(const gmg* g, const sim_opts_t* o) {
   return (int)std::max<int64_t>(c, 1);
 }
 
+// HBM events that a candidate's log holds: twice the caller's queue_cap, and never
+// fewer than a warp may hold in shared memory on any graph, else what the graph can
+// log (up to a default).  Up to 32 ops more than kOpsPerGeneration start before their
+// events are generated, and the arbitrated kernels keep arrivals back until then:
+// the log has room for these as well.
 int log_cap(const gmg* g, const sim_opts_t* o) {
-  const int64_t c = (o && o->queue_cap > 0) ? 2 * (int64_t)o->queue_cap
-                                           : std::min<int64_t>(g->log_bound, kDefaultLogCap);
-  return (int)std::max<int64_t>(c, 1);
+  const int64_t more = g->burst + 2 * kArbArrivals;
+  const int64_t c = (o && o->queue_cap > 0)
+                        ? std::min(std::max<int64_t>(2 * (int64_t)o->queue_cap, kSharedLogEntries) + more,
+                                   g->log_bound + g->dg.n)
+                        : std::min(g->log_bound, kDefaultLogCap + more);
+  return (int)std::min<int64_t>(std::max<int64_t>(c, 1), INT32_MAX);
 }
 
 size_t smem_per_warp(const SimParams& P) {
@@ -1076,6 +1096,7 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   I.time_bound = b.time_bound;
   g->queue_bound = b.queue_bound;
   g->log_bound = b.log_bound;
+  g->burst = b.burst;
   g->linkid = b.linkid.empty() ? nullptr : reinterpret_cast<const uint16_t*>(w + L.off_linkid);
   g->xfer_bound = b.xfer_bound;
   g->shared_links = b.shared_links ? 1 : 0;
