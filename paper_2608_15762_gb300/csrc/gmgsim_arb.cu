@@ -347,9 +347,13 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode, kHot>, Sim<true, kMode, tr
         if (end || status) break;
       }
       lim = lim < tx ? lim : tx;
+      if (kMode == kBase && this->readypops >= this->next_ck) {
+        // READY ops start now (the next comes before every transfer event)
+        const tm_t r = warp_min_t(pd.r);
+        if ((r < o.r ? r : o.r) < tx) arb_checkpoint(o);
+      }
       const bool act = this->starts(lim, tx, o);
       if (__any_sync(kFullMask, act)) {
-        if (kMode == kBase && this->readypops >= this->next_ck) arb_checkpoint(o);
         Batch B;
         if (!this->start_held(act, B)) break;
         start_ops(B, o);

@@ -1587,7 +1587,9 @@ struct Sim {
   // Whether this lane's pending op starts now: those before lim, the smallest
   // earliest finish (and `until`, a time that no start may pass).  Keys outside
   // the lanes that are due (rare: every root once, the heap only after the lanes
-  // were all taken) come into empty lanes first.
+  // were all taken) come into empty lanes first.  Each lowers lim by its own bound,
+  // so all that come in start now: no root waits in a lane, where it would take the
+  // place of an op that the caller's queue_cap counts.
   __device__ __forceinline__ bool starts(tm_t lim, tm_t until, Outside& o) {
     if (o.r >= lim) return pd.r < lim;
     uint32_t fm = __ballot_sync(kFullMask, pd.r == kNever);
@@ -1600,6 +1602,8 @@ struct Sim {
         pd.op = rq.op(o.k);
         fresh = true;
       }
+      const tm_t e = (tm_t)rq.bound(o.k);
+      lim = e < lim ? e : lim;
       take_outside(o.k);
       look_outside(o);
     }
@@ -1608,7 +1612,8 @@ struct Sim {
     lim = lim < until ? lim : until;
     bool act = pd.r < lim;
     if (o.r < lim) {
-      // no empty lane: only keys before the next outside one; if there is none
+      // no empty lane (or a bound below the finish that it stands for): only keys
+      // before the next outside one; if there is none
       // it changes places with the last key of the lanes
       act = act && precedes(pd.r, pd.op, o.r, rq.op(o.k));
       if (!__any_sync(kFullMask, act)) {
@@ -1808,23 +1813,29 @@ struct Sim {
     lim = warp_min_t(lim);
     lim = lim < until ? lim : until;
     // keys outside the pool that are due come in (rare: the roots once each,
-    // the heap only after the pool was full)
+    // the heap only after the pool was full), as far as they are among the 32 that
+    // can start now: no root waits in the pool, where it would count as one of the
+    // ops that the caller's queue_cap limits
     uint64_t x = outside_min();
     uint64_t kb = kKeyMax;  // keys below kb are started
+    uint64_t in = 0;        // one above the last key that came in
     if (key_time(x) < lim) {
       __syncwarp();
       while (key_time(x) < lim) {
+        int c = 0;  // the pool's keys before x
+#pragma unroll
+        for (int s = 0; s < kSlots; ++s) c += __popc(__ballot_sync(kFullMask, pool[32 * s + lane] < x));
+        if (c >= 32 || (nfree == 0 && c > 0)) {
+          kb = x;
+          break;
+        }
         int slot;
         if (nfree > 0) {
           slot = fstk[--nfree];
           take_outside(x);
         } else {
-          // full: x waits unless it is the next key of all; it then changes
-          // places with the pool's last key
-          if (x > pool_min()) {
-            kb = x;
-            break;
-          }
+          // full, and x is the next key of all: it changes places with the pool's
+          // last key
           uint64_t mx = 0;
           int ms = 0;
 #pragma unroll
@@ -1841,6 +1852,7 @@ struct Sim {
           q.push(last);  // the heap keeps one entry beyond its limit for this
         }
         if (lane == 0) pool[slot] = x;
+        in = x + 1;
         __syncwarp();
         const tm_t e = (tm_t)rq.bound(x);
         lim = e < lim ? e : lim;
@@ -1859,9 +1871,9 @@ struct Sim {
       m += __popc(b[s]);
     }
     if (m > 32) {
-      // more keys than lanes: a bound with 16 to 32 keys below it (or at
-      // least one)
-      uint64_t lo = pool_min() + 1, hi = kb;
+      // more keys than lanes: those up to the last that came in (32 at most), else
+      // a bound with 16 to 32 keys below it (or at least one)
+      uint64_t lo = in ? in : pool_min() + 1, hi = in ? in : kb;
       m = 0;
       while (m < 16 && hi - lo > 1) {
         const uint64_t mid = lo + (hi - lo) / 2;
@@ -1974,7 +1986,6 @@ struct Sim {
       rest &= rest - 1;
       if (!q.push(__shfl_sync(kFullMask, nk, src))) status = GMG_SIM_QUEUE;
     }
-    if (32 * kSlots - nfree + q.size > P.pend_cap) status = GMG_SIM_QUEUE;
     __syncwarp();
   }
   __device__ __forceinline__ void free_slots(bool gone, int slot) {
@@ -1989,11 +2000,18 @@ struct Sim {
 
   __device__ void run_pool() {
     while (true) {
+      // counted between batches: the started ops' slots are free again, or their
+      // successors'
+      const int pending = 32 * kSlots - nfree + q.size;
+      if (pending > P.pend_cap) {
+        status = GMG_SIM_QUEUE;
+        break;
+      }
       if (kMode == kBase && readypops >= next_ck) {
         const uint64_t nk = next_key();
         if (nk != kKeyMax) maybe_checkpoint(rq.time(nk));
       }
-      const bool end = nfree == 32 * kSlots && outside_min() == kKeyMax;
+      const bool end = pending == 0 && rkey == kKeyMax;
       if (end || opn >= P.drain_trigger) {  // the only copy of this code: it is large
         const int64_t tn = end ? kI64Max : rq.time(next_key());
         if constexpr (kRole == kBoth) drain(tn);

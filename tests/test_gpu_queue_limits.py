@@ -56,3 +56,37 @@ def test_the_log_holds_what_a_generation_adds(D, preds, lat, arb):
     d = mk(preds, [1 + i % 3 for i in range(n)], [64 + i for i in range(n)], n_dev=D, bw=100, lat=lat)
     for got, want in _run(d, 1, arb):
         compare(got, *want)
+
+
+@pytest.mark.parametrize("arb", [False, True])
+@pytest.mark.parametrize("D", [1, 8, 33, 256])
+@pytest.mark.parametrize("roots,gap,succ", [
+    (40, 10 ** 6, 5),    # roots far in the future
+    (40, 10 ** 6, 33),   # as many pending ops as may wait beside them
+    (90, 0, 0),          # more roots at once than ops may wait
+    (90, 0, 20),
+    (40, 3, 20),         # roots that come in while others run
+])
+def test_ops_without_predecessors_do_not_count_before_they_start(D, roots, gap, succ, arb):
+    preds = [[] for _ in range(roots)] + [[0]] * succ
+    n = len(preds)
+    d = mk(preds, [5] * n, [1] * n, n_dev=D, bw=1, lat=1, release=[i * gap for i in range(roots)] + [0] * succ)
+    for got, want in _run(d, 1, arb):
+        compare(got, *want)
+
+
+@pytest.mark.parametrize("D", [1, 8, 32])
+def test_resumed_where_roots_start(D):
+    """Arbitrated bases take checkpoints right before ops without predecessors
+    start; moves of ops on both sides of them, with the base's queue_cap."""
+    preds = [[] for _ in range(40)] + [[i] for i in range(40)]
+    n = len(preds)
+    d = mk(preds, [5] * n, [3] * n, n_dev=D, bw=1, lat=1, release=[i * 4 for i in range(40)] + [0] * 40)
+    base = np.arange(n, dtype=np.uint8) % D
+    mv = W.random_moves(3, 40, base, D, max_moves=3)
+    g = G.gmg_create(d)
+    for arb in (False, True):
+        b = G.base_create(g, torch.from_numpy(base).cuda(), queue_cap=40, arbitrated=arb)
+        inc = G.sim_incremental(g, b, *G.moves_to_device(mv, "cuda"), req_done=True, queue_cap=40, arbitrated=arb)
+        torch.cuda.synchronize()
+        compare(inc.to_numpy(), *O.incremental_batch(d, base, mv, arbitrated=arb, resumed=arb))
