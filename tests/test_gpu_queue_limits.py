@@ -2,7 +2,8 @@
 queue_cap ops that became ready may wait, and a call beyond that answers
 GMG_SIM_QUEUE; within it every result is the oracle's.  Ops without
 predecessors do not count before they start, and the log of HBM events has room
-for what one generation adds."""
+for what one generation adds.  (With at most 32 accelerators and in the arbitrated
+kernels one op more may wait, where a root's successor took the root's place.)"""
 import numpy as np
 import pytest
 
@@ -90,3 +91,76 @@ def test_resumed_where_roots_start(D):
         inc = G.sim_incremental(g, b, *G.moves_to_device(mv, "cuda"), req_done=True, queue_cap=40, arbitrated=arb)
         torch.cuda.synchronize()
         compare(inc.to_numpy(), *O.incremental_batch(d, base, mv, arbitrated=arb, resumed=arb))
+
+
+def _late(queue_cap, late, D, successor=True):
+    """32 ops at time 0, the first with as many successors as may wait, all
+    released at 1e6; then `late` ops without predecessors, each with one more
+    such successor (or none)."""
+    preds = [[] for _ in range(32)] + [[0]] * (32 + queue_cap)
+    rel = [0] * 32 + [10 ** 6] * (32 + queue_cap)
+    for t in range(late):
+        preds.append([])
+        rel.append(1000 + 10 * t)
+        if successor:
+            preds.append([len(preds) - 1])
+            rel.append(10 ** 6)
+    n = len(preds)
+    return mk(preds, [1] * n, [1] * n, n_dev=D, bw=1, lat=1, release=rel)
+
+
+@pytest.mark.parametrize("arb", [False, True])
+@pytest.mark.parametrize("D", [1, 8, 32, 33, 256])
+@pytest.mark.parametrize("queue_cap", [1, 3, 100, 200])
+@pytest.mark.parametrize("late,successor", [(0, True), (3, False), (1, True), (2, True), (40, True)])
+def test_pending_ops_beyond_the_limit_are_never_dropped(D, queue_cap, late, successor, arb):
+    """Ops that wait outside while all places are taken change places with the
+    last pending one; none is lost."""
+    d = _late(queue_cap, late, D, successor)
+    spare = 1 if D <= 32 or arb else 0
+    for got, want in _run(d, queue_cap, arb):
+        if successor and late > spare:
+            assert (got["status"] == G.SIM_QUEUE).all()
+        elif successor and late:
+            ok = got["status"] == 0
+            assert ((got["status"] == G.SIM_QUEUE) | ok).all()
+            if ok.any():
+                compare(got, *(w[ok] for w in want), ks=np.flatnonzero(ok))
+        else:
+            compare(got, *want)
+    for got, want in _run(d, queue_cap + late, arb):
+        compare(got, *want)
+
+
+@pytest.mark.parametrize("arb", [False, True])
+@pytest.mark.parametrize("D", [1, 8, 33])
+@pytest.mark.parametrize("late", [0, 1, 3])
+def test_resumed_candidates_at_the_limit(D, late, arb):
+    """The same against a base with room: moves of the late ops' successors, of
+    the first op's and of the first op itself."""
+    if arb and D > 32:
+        pytest.skip("candidates of an arbitrated base: at most 32 accelerators")
+    q = 100
+    d = _late(q, late, D)
+    n = d.n_ops
+    base = np.arange(n, dtype=np.uint8) % D
+    ops = [0, 40, n - 1]
+    mv = W.Moves(np.arange(len(ops) + 1, dtype=np.int32), np.array(ops, np.int32),
+                 ((base[ops] + 1) % D).astype(np.uint8))
+    g = G.gmg_create(d)
+    b = G.base_create(g, torch.from_numpy(base).cuda(), arbitrated=arb)
+    dev = G.moves_to_device(mv, "cuda")
+    at, room = [G.sim_incremental(g, b, *dev, queue_cap=c, arbitrated=arb) for c in (q, q + 50)]
+    torch.cuda.synchronize()
+    want = O.incremental_batch(d, base, mv, arbitrated=arb, resumed=arb)
+    compare(room.to_numpy(), *want[:2])
+    st = at.to_numpy()["status"]
+    if D == 1:                            # no move has an effect: the base's results
+        assert (st == 0).all()
+    elif late == 0:
+        assert st[0] == 0
+    elif late > 1 or D > 32:
+        assert (st == G.SIM_QUEUE).all()
+    ok = st == 0
+    for f in ("makespan", "score", "events"):
+        assert (at.to_numpy()[f][ok] == want[0][f][ok]).all()
