@@ -14,6 +14,7 @@
 #include "gmg_access.h"
 #include "gmg_arb.h"
 #include "gmg_arbw.h"
+#include "gmg_once.h"
 
 namespace gsim {
 // launchers (gmgsim_kernels.cu)
@@ -446,9 +447,16 @@ int build(const gmg_desc_t* d, Built& b) {
   return GMG_OK;
 }
 
+// The current device, or -1.
+int current_device() {
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess ? dev : -1;
+}
+
 int device_sms() {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return -1;
+  const int dev = current_device();
+  int sms = 0;
+  if (dev < 0) return -1;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
   return sms;
 }
@@ -526,7 +534,7 @@ int dev_smem_bytes(int D, size_t tbytes) {
 // lists of ops.
 int pair_bytes(const SimParams& P) { return (int)align_up(2 * 48 + 8 * 48 + 2 * (size_t)P.opcap * 4, 16); }
 
-bool g_smem_set = false;
+OncePerDevice g_smem_set;
 
 // Slot layout and grid for K candidates of kind `inc`.
 int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& L) {
@@ -573,7 +581,7 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
   P.slot_bytes = (int64_t)o2;
   const int sms = device_sms();
   if (sms <= 0) return GMG_ECUDA;
-  if (!g_smem_set) {
+  const bool limits = g_smem_set.done(current_device(), [&] {
     // the largest per-block request: 4 warps with 256 accelerators
     SimParams big = P;
     big.g.D = 256;
@@ -584,9 +592,9 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
     big.dev_bytes = 32 + 24 * 256;
     big.no_side = 0;
     big.pair_bytes = pair_bytes(big);
-    if (set_smem_limits(4 * (int)smem_per_warp(big)) != cudaSuccess) return GMG_ECUDA;
-    g_smem_set = true;
-  }
+    return set_smem_limits(4 * (int)smem_per_warp(big)) == cudaSuccess;
+  });
+  if (!limits) return GMG_ECUDA;
   int bps = 0;
   const void* fn = inc ? inc_kernel_ptr(G) : full_kernel_ptr(G);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, 32 * L.wpb, L.smem) != cudaSuccess)
@@ -656,7 +664,7 @@ int check_out(const sim_out_t* o, const sim_opts_t* opts) {
 bool staged(const sim_opts_t* o) { return o && o->gmg_staging == GMG_STAGING_SHARED; }
 bool l1_path(const sim_opts_t* o) { return o && o->gmg_staging == GMG_STAGING_L1; }
 
-bool g_stage_smem_set = false;
+OncePerDevice g_stage_smem_set;
 constexpr int64_t kStageSmallBytes = 16 << 10;
 
 // sim_batch with the GMG staged in shared memory: one CTA per SM with as many
@@ -666,8 +674,9 @@ int plan_staged(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L) {
   if (!G.stage_ok || (o && o->transfer_mode != GMG_TRANSFER_LATENCY)) return GMG_EINVAL;
   int rc = plan_launch(g, K, o, false, L);
   if (rc) return rc;
-  int dev = 0, optin = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
+  const int dev = current_device();
+  int optin = 0;
+  if (dev < 0 ||
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
     return GMG_ECUDA;
   SimParams& P = L.P;
@@ -681,12 +690,11 @@ int plan_staged(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L) {
   const int sms = device_sms();
   if (sms <= 0) return GMG_ECUDA;
   const int w = (int)std::min<int64_t>(fit, std::max<int64_t>(1, ((int64_t)std::max(K, 1) + sms - 1) / sms));
-  if (!g_stage_smem_set) {
-    if (cudaFuncSetAttribute(full_staged_kernel_ptr(), cudaFuncAttributeMaxDynamicSharedMemorySize, optin) !=
-        cudaSuccess)
-      return GMG_ECUDA;
-    g_stage_smem_set = true;
-  }
+  if (!g_stage_smem_set.done(dev, [&] {
+        return cudaFuncSetAttribute(full_staged_kernel_ptr(), cudaFuncAttributeMaxDynamicSharedMemorySize, optin) ==
+               cudaSuccess;
+      }))
+    return GMG_ECUDA;
   L.wpb = w;
   L.smem = (size_t)P.stage_bytes + (size_t)w * spw;
   L.grid = (int)std::min<int64_t>(sms, ((int64_t)std::max(K, 1) + w - 1) / w);
@@ -786,7 +794,7 @@ int plan_arb(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbParams&
   return GMG_OK;
 }
 
-bool g_arbw_smem_set = false;
+OncePerDevice g_arbw_smem_set;
 
 // Arbitrated transfers on 33..256 accelerators: per-accelerator transfer
 // state in tables.  Op ids below 2^24 (an intent packs op << 8 | destination).
@@ -823,11 +831,8 @@ int plan_arbw(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbWParam
   A.smem_arb = (int32_t)align_up((2 * tsz + 20) * D + 32 + (4 + tsz) * kArbArrivals, 16);
   A.smem_std = (int64_t)L.smem;
   L.smem += (size_t)L.wpb * (size_t)A.smem_arb;
-  if (!g_arbw_smem_set) {
-    // a block of four warps on 256 accelerators asks for most
-    if (set_arbw_smem_limit() != cudaSuccess) return GMG_ECUDA;
-    g_arbw_smem_set = true;
-  }
+  // a block of four warps on 256 accelerators asks for most
+  if (!g_arbw_smem_set.done(current_device(), [] { return set_arbw_smem_limit() == cudaSuccess; })) return GMG_ECUDA;
   const int sms = device_sms();
   if (sms <= 0) return GMG_ECUDA;
   // few candidates: the instance with more registers, if it holds them all at

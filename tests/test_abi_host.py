@@ -150,3 +150,37 @@ def test_nvtx_ranges_are_opt_in_and_balanced(monkeypatch):
         probe(True)
     assert calls == [("push", "gmgsim.probe"), ("pop",), ("push", "gmgsim.probe"), ("pop",)]
     assert G.sim_batch.__name__ == "sim_batch" and G.sim_incremental.__wrapped__ is not None
+
+
+def test_set_up_runs_once_on_every_device(tmp_path):
+    """Shared-memory limits are set for the current device only: the library asks
+    once per device, again where it failed, and from several threads."""
+    import subprocess
+    src = tmp_path / "once.cpp"
+    src.write_text(r"""
+#include <atomic>
+#include <cstdio>
+#include <thread>
+#include <vector>
+#include "gmg_once.h"
+int main() {
+  gsim::OncePerDevice o;
+  std::atomic<int> calls{0};
+  auto yes = [&] { ++calls; return true; };
+  auto no = [&] { ++calls; return false; };
+  std::vector<std::thread> ts;
+  for (int t = 0; t < 8; ++t) ts.emplace_back([&] { for (int d = 0; d < 4; ++d) o.done(d, yes); });
+  for (auto& t : ts) t.join();
+  const int four = calls;
+  const bool failed = o.done(9, no), again = o.done(9, yes), kept = o.done(9, no);
+  const int nine = calls - four;
+  const bool none = o.done(-1, yes), beyond = o.done(1000, yes);
+  std::printf("%d %d %d %d %d %d %d", four, failed, again, kept, nine, none, beyond);
+}
+""")
+    exe = tmp_path / "once"
+    subprocess.check_call(["g++", "-std=c++17", "-pthread", "-I",
+                           os.path.join(ROOT, "paper_2608_15762_gb300", "csrc"), str(src), "-o", str(exe)])
+    assert subprocess.check_output([str(exe)]).decode() == "4 0 1 1 2 0 1"
+    host = open(os.path.join(ROOT, "paper_2608_15762_gb300", "csrc", "gmgsim_host.cu")).read()
+    assert not re.search(r"^\s*(static )?bool g_\w+", host, re.M), "a process-wide flag"
