@@ -183,7 +183,7 @@ __device__ __forceinline__ double tree8(const double (&a)[8]) {
 // wherever the result is used.
 __device__ __forceinline__ double quotient(double a, double d, double r) {
   const double q = a * r, e = fma(-q, d, a);
-  return e == e ? fma(e, r, q) : q;  // an infinite q has no residual
+  return isfinite(e) ? fma(e, r, q) : q;  // an infinite q (or a) has no residual
 }
 
 // kWarps warps per estimator (blocks of 4 estimators with one warp each, else of

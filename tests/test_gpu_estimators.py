@@ -185,3 +185,22 @@ def test_empty_batches_one_type_and_one_accelerator():
     tr = G.Estimators(1, 2)                                     # one accelerator: only the diagonal
     bw, lat = tr.links(1, _dev(np.array([9]), np.int64), _dev(np.array([4]), np.int64))
     assert bw.cpu().tolist() == [9] and lat.cpu().tolist() == [4]
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_a_coefficient_beyond_the_range_is_infinite(sign):
+    """sum(x y) / sum(x x) = 1e350: the quotient of a division, and durations at
+    the ends of their range, not those of an undefined number."""
+    n = 40
+    est = G.Estimators(2, 1)
+    x = np.full((2 * n, 1), 1e-100)
+    y = np.full(2 * n, sign * 1e250)
+    x[n:], y[n:] = 2.0, 6.0
+    est.update(_dev([0, n, 2 * n], np.int32), _dev(x, np.float64), _dev(y, np.float64))
+    beta, fitted = est.coefficients()
+    assert fitted.cpu().tolist() == [1, 1]
+    assert beta.cpu().numpy()[:, 0].tolist() == [sign * np.inf, 3.0]
+    est_of = np.array([[0], [0], [1]], np.int32)
+    d = est.predict_durations(_dev(est_of, np.int32), _dev([[1.0], [-1.0], [4.0]], np.float64),
+                              _dev([9, 9, 9], np.int64)).cpu().numpy()[:, 0]
+    assert d.tolist() == ([OE.MAX_TICKS, 1, 12] if sign > 0 else [1, OE.MAX_TICKS, 12])
