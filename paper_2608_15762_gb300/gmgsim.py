@@ -147,8 +147,12 @@ def _stream_handle(stream) -> Optional[int]:
     import torch
     if stream is not None:
         return int(stream.cuda_stream) or None
-    # the current stream's handle without a Stream object: 0.4 us a call instead of 3
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
+    # the current stream's handle without a Stream object, where this torch has that:
+    # 0.4 us a call instead of 3
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return int(torch.cuda.current_stream().cuda_stream) or None
+    return raw(torch.cuda.current_device()) or None
 
 
 def _np_ptr(a):

@@ -184,3 +184,21 @@ int main() {
     assert subprocess.check_output([str(exe)]).decode() == "4 0 1 1 2 0 1"
     host = open(os.path.join(ROOT, "paper_2608_15762_gb300", "csrc", "gmgsim_host.cu")).read()
     assert not re.search(r"^\s*(static )?bool g_\w+", host, re.M), "a process-wide flag"
+
+
+@pytest.mark.parametrize("raw", [True, False])
+def test_the_current_stream_with_and_without_its_raw_handle(monkeypatch, raw):
+    torch = pytest.importorskip("torch")
+
+    class Stream:
+        cuda_stream = 0x50
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    if raw:
+        monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda dev: 0x40 + dev, raising=False)
+    else:
+        monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    assert G._stream_handle(None) == (0x43 if raw else 0x50)
+    assert G._stream_handle(Stream) == 0x50
+    monkeypatch.setattr(Stream, "cuda_stream", 0)                # the default stream
+    assert G._stream_handle(Stream) is None
