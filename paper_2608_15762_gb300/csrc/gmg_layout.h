@@ -133,14 +133,11 @@ constexpr int kBlocksPerSM = 7;
 constexpr int kPairsPerSM = 14, kPairsPerSM64 = 10;
 
 // Slots of the READY pool on more than 32 accelerators (a multiple of 32, at
-// most 256; compile-time overridable for tuning sweeps).  160: with 128 slots a
+// most 256).  160: with 128 slots a
 // batch scans less (4,096 placements on 256 accelerators 80 ms -> 79), but graphs
 // with more pending ops spill into the heap (213,568 ops, 65,536 candidates with
 // a longer log in the room gained: 5.06 s -> 5.78).
-#ifndef GMG_POOL_WIDE
-#define GMG_POOL_WIDE 160
-#endif
-constexpr int kReadyPoolWide = GMG_POOL_WIDE;
+constexpr int kReadyPoolWide = 160;
 
 // The staged-GMG kernel's largest CTA (one per SM; 72 registers a thread).
 constexpr int kStageMaxWarps = 28;

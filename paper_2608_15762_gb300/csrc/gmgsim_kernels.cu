@@ -28,10 +28,10 @@ __device__ __forceinline__ void sweep_base(S_& S, const SimParams& P) {
   S.run();
 }
 
-template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
+template <bool kNarrow, bool kTypes>
 __global__ void __launch_bounds__(32, 1) sim_base_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
-  Sim<kNarrow, kBase, kKey, kT32, kTypes, kHot> S(P);
+  Sim<kNarrow, kBase, false, false, kTypes, kHotNone> S(P);
   setup_slot(S, P, 0, 0, smem);
   warp_prefetch_l2(P.g.ws, P.g.ws_bytes);
   copy_base_row(P);
@@ -41,7 +41,8 @@ __global__ void __launch_bounds__(32, 1) sim_base_kernel(const __grid_constant__
   write_base(S, P.base);
 }
 
-// The same by two warps, the sweep and the HBM accounting.
+// The same by two warps, the sweep and the HBM accounting: graphs whose accelerator
+// ids fit into the event key.
 template <bool kNarrow, bool kT32, bool kTypes, int kHot>
 __global__ void __launch_bounds__(64, 1) sim_base_pair_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
@@ -163,26 +164,17 @@ const void* full_pair_kernel_ptr(const DevGmg& g);
 const void* inc_kernel_ptr(const DevGmg& g);  // gmgsim_inc.cu
 const void* inc_pair_kernel_ptr(const DevGmg& g);
 
-// Instances by (at most 32 accelerators, accelerator id in the event key,
-// 32-bit times, accelerator types; compact records wherever the graph has
-// them).  32-bit times are only chosen with the accelerator id in the key,
-// compact records only with 32-bit times.
-template <bool N, bool K, bool T32>
-const void* base_ptr(bool types) {
-  return types ? (const void*)sim_base_kernel<N, K, T32, true, kHotNone>
-               : (const void*)sim_base_kernel<N, K, T32, false, kHotNone>;
-}
+// One warp (64-bit times): graphs whose accelerator ids do not fit into the event
+// key.
 template <bool N>
-const void* base_ptr_n(bool key, bool t32, bool types, bool hot) {
-  if (!key) return base_ptr<N, false, false>(types);
-  if (hot) return (const void*)sim_base_kernel<N, true, true, false, kHotGlobal>;
-  return t32 ? base_ptr<N, true, true>(types) : base_ptr<N, true, false>(types);
+const void* base_ptr(bool types) {
+  return types ? (const void*)sim_base_kernel<N, true> : (const void*)sim_base_kernel<N, false>;
 }
 const void* base_kernel_ptr(const DevGmg& g) {
-  const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
-  return g.D <= 32 ? base_ptr_n<true>(key, t32, types, hot) : base_ptr_n<false>(key, t32, types, hot);
+  return g.D <= 32 ? base_ptr<true>(g.ntypes >= 2) : base_ptr<false>(g.ntypes >= 2);
 }
-// Two warps: graphs whose accelerator ids fit into the event key.
+// Two warps: all others, by (at most 32 accelerators, 32-bit times, accelerator
+// types; compact records wherever the graph has them, only with 32-bit times).
 template <bool N, bool T32>
 const void* base_pair_ptr(bool types) {
   return types ? (const void*)sim_base_pair_kernel<N, T32, true, kHotNone>
