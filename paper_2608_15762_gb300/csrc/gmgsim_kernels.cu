@@ -143,14 +143,16 @@ __global__ void __launch_bounds__(256) select_final_kernel(const Rank* part, int
 }
 
 // Up to kSelectOne candidates: one block does both (a second launch costs more
-// than the few rows that each thread goes through).
+// than the few rows that each thread goes through: one / two launches in a graph,
+// us, 256 candidates 2.4 / 4.4, 1,024 3.4 / 4.6, 2,048 4.0 / 4.4, 4,096 5.3 / 4.7,
+// 8,192 7.4 / 4.7).
 __global__ void __launch_bounds__(1024) select_one_kernel(const int32_t* status, const int32_t* viol,
                                                           const int64_t* score, const int32_t* miss, int32_t K,
                                                           int32_t mode, int64_t* best) {
   const Rank r = best_of(status, viol, score, miss, K, mode);
   if (threadIdx.x == 0) write_best(r, best);
 }
-constexpr int32_t kSelectOne = 4096;
+constexpr int32_t kSelectOne = 2048;
 
 }  // namespace
 

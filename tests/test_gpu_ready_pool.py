@@ -170,3 +170,41 @@ def test_select_best_on_both_sides_of_one_block(K):
         ok = [(int(ms[k]) if mode else 0, int(sc[k]), k) for k in range(K) if st[k] == 0 and vf[k] == 0]
         want = [min(ok)[2], min(ok)[1]] if ok else [-1, np.iinfo(np.int64).max]
         assert G.select_best(out, score_mode=mode).cpu().tolist() == want
+
+
+@pytest.mark.parametrize("D", [33, 64, 256])
+@pytest.mark.parametrize("kw", [
+    dict(chains=40, length=5),
+    dict(chains=170, length=2),                                   # more pending ops than pool slots
+    dict(chains=9, length=4, fan=5, bytes_lo=1 << 18, cap=6 << 20),  # joins, capacities that bind
+    dict(chains=30, length=5, release_hi=1 << 41),
+])
+def test_wide_graphs_whose_keys_leave_no_room_for_the_accelerator(D, kw):
+    """Times so wide that an HBM event's accelerator is kept beside its key:
+    the pool with events applied one at a time, full placements and moves."""
+    d = _chains(41, D=D, dur_hi=1 << 40, **kw)
+    rows = _rows(42, 9, d.n_ops, D)
+    g = G.gmg_create(d)
+    assert g.info["batched_sweep"] == 0 and g.info["t32"] == 0
+    tk = torch.tensor([0, 8], dtype=torch.int32, device="cuda")
+    out = G.sim_batch(g, torch_place(rows), req_done=True, trace_k=tk)
+    base = rows[0, :d.n_ops].copy()
+    mv = W.random_moves(43, 24, base, D, max_moves=5)
+    b = G.base_create(g, torch.from_numpy(base).cuda())
+    inc = G.sim_incremental(g, b, *G.moves_to_device(mv, "cuda"), req_done=True)
+    torch.cuda.synchronize()
+    got = out.to_numpy()
+    compare(got, *oracle_rows(d, rows))
+    for slot, k in enumerate((0, 8)):
+        r = O.simulate(d, rows[k])
+        assert np.array_equal(got["trace_start"][slot], r["start"])
+        assert np.array_equal(got["trace_finish"][slot], r["finish"])
+    compare(inc.to_numpy(), *O.incremental_batch(d, base, mv))
+    with pytest.raises(G.GmgError) as e:
+        G.sim_batch(g, torch_place(rows), arbitrated=True)
+    assert e.value.code == G.GMG_ERANGE
+
+
+@pytest.mark.parametrize("K", [2048, 2049])
+def test_select_best_at_the_line(K):
+    test_select_best_on_both_sides_of_one_block(K)
