@@ -871,7 +871,9 @@ def main():
     arb_kern = "sim_arb_kernel" if D <= 32 else "sim_arbw_kernel"
     # the library's default: two warps per candidate while all fit (14 blocks of 64 threads per SM, 10 with 64-bit times), then
     # the staged kernel for graphs whose copy takes 16 KB at most, else one warp per candidate
-    pair = p.staging != 1 and not p.arb
+    # an HBM event's key holds its accelerator
+    dev_key = int(p.g.info["time_bound"]).bit_length() + p.g.info["id_bits"] <= 53
+    pair = p.staging != 1 and not p.arb and dev_key
     pairs = (14 if p.g.info["t32"] == 1 else 10) * props.multi_processor_count
     staged_run = p.staging == 1 or (p.staging == 0 and p.g.info["stageable"] == 1 and not p.arb and
                                     not (pair and p.n_full <= pairs) and
@@ -882,7 +884,7 @@ def main():
              "inc": ("sim_arb_inc_kernel" if p.arb_base else arb_kern if p.arb else
                      "sim_inc_pair_kernel" if pair and p.n_inc <= pairs else "sim_inc_kernel"),
              "base": ("sim_arb_base_kernel" if p.arb_base else
-                      "sim_base_pair_kernel")}
+                      "sim_base_pair_kernel" if dev_key else "sim_base_kernel")}
     kcount = {"full": p.n_full, "inc": p.n_inc, "base": 1}
     out_bytes_per_cand = 8 + 8 + 4 + 4 + 4 + 4 + 8 + 4 + 8 + 8 * D
     alg_bytes = {"full": p.n_full * (W_ld(N) + out_bytes_per_cand),

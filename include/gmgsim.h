@@ -123,7 +123,8 @@ typedef struct gmg_base gmg_base_t; /* opaque; base schedule snapshot for increm
  * lists into shared memory with bulk copies; needs one accelerator type,
  * uniform links, every time below 2^31, at most 32 accelerators and the copy
  * within the CTA's shared memory, else GMG_EINVAL.  GMG_STAGING_L1: 4-warp
- * CTAs read the records through the read-only L1 path.
+ * CTAs (with few candidates two warps for each, unless warps_per_block is set) read
+ * the records through the read-only L1 path.
  * GMG_STAGING_DEFAULT takes the fastest measured: batches of up to about 14
  * candidates per SM (10 with times beyond 2^32) run with two warps per candidate
  * by the L1 path, larger ones are staged where staging applies and the copy takes 16 KB
@@ -141,7 +142,9 @@ typedef struct {
   int32_t score_mode;       /* select_best: 0 = score, 1 = (sla_miss, score) */
   int32_t n_trace;          /* number of candidates whose per-op schedule is written */
   const int32_t* d_trace_k; /* device [n_trace]: candidate indices to trace (distinct) */
-  int32_t queue_cap;        /* per-candidate event-queue entries; 0 = library default */
+  int32_t queue_cap;        /* per-candidate event-queue entries: 32 more ops may be ready and wait, and
+                               the log of HBM events holds at least twice as many (0 = library default);
+                               a candidate that needs more ends with GMG_SIM_QUEUE */
   int32_t warps_per_block;  /* 0 = library default (tuning knob) */
   int32_t transfer_mode;    /* GMG_TRANSFER_*; 0 = GMG_TRANSFER_LATENCY */
   int32_t gmg_staging;      /* GMG_STAGING_*; sim_batch with pure-latency transfers only */
@@ -174,10 +177,12 @@ typedef struct {
   int32_t uniform_links; /* 1 if every off-diagonal link has the same bw and latency */
   int64_t time_bound;    /* proven upper bound of every simulated time */
   int64_t default_queue_cap;
-  int32_t batched_sweep; /* 1 if the simulation kernels keep the pending ops of this graph in a
-                            pool in shared memory (more than 32 accelerators and keys with 5 bits
-                            of room; with at most 32 accelerators lanes hold them).  Either way
-                            every op whose start the others cannot change starts at once */
+  int32_t batched_sweep; /* 1 on more than 32 accelerators if an HBM event's key also holds its
+                            accelerator (id_bits and the bits of time_bound: 53 at most): events
+                            are then applied in batches, else one at a time.  Whatever its value, pending ops are in
+                            a pool in shared memory there (lanes hold them with at most 32
+                            accelerators and under arbitrated transfers), and every op whose
+                            start the others cannot change starts at once */
   int32_t t32;           /* 1 if the kernels carry times as 32-bit integers (time_bound < 2^32 - 1) */
   int32_t stageable;     /* 1 if sim_batch can stage this graph's hot fields in shared memory on
                             the current device (one accelerator type, uniform links, 32-bit times,
@@ -316,7 +321,7 @@ size_t select_best_tmp_bytes(int32_t K);
  * (score, k) (score_mode 0) or (sla_miss, score, k) (mode 1) over candidates
  * with status 0 and viol_flag 0, or -1 if none; d_best[1] = its score
  * (INT64_MAX if none).  Reads status, viol_flag, score, sla_miss of d_out.
- * Two launches (per-block argmin, then a final argmin), or one up to 4,096
+ * Two launches (per-block argmin, then a final argmin), or one up to 2,048
  * candidates. */
 int select_best(const sim_out_t* d_out, int32_t K, int32_t score_mode, int64_t* d_best,
                 void* d_tmp, size_t tmp_bytes, gmg_stream_t stream);

@@ -708,9 +708,14 @@ int plan_staged(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L) {
 // staged kernel for small graphs, whose copy leaves the L1 cache to the
 // candidates' own arrays, else one warp per candidate.  *stg tells which.
 // (Measured, two warps / staged / one warp: the 50-op graph 55 / 65 / 67 us for
-// 256 candidates, - / 90 / 98 us for 4,096; the prefill graph, N = 3088, a 90 KB
-// copy, 1.41 / 1.80 / 1.84 ms for 14, 1.61 / 2.11 / 2.07 ms for 2,048, - / 3.39 /
-// 3.11 ms for 4,096.)
+// 256 candidates; the prefill graph, N = 3088, a 90 KB copy, 1.41 / 1.80 / 1.84 ms
+// for 14, 1.61 / 2.11 / 2.07 ms for 2,048.  Where two warps are not chosen, staged /
+// one warp, for 2,129, 4,096 and 16,384 candidates: a copy of 1.4 KB 82 / 86, 101 /
+// 107 and 364 / 380 us; 5.6 KB 257 / 255, 336 / 344 and 1,356 / 1,307; 11 KB 472 /
+// 460, 621 / 630 and 2,511 / 2,405; 17 KB 585 / 556, 816 / 786 and 3,302 / 3,020; 44
+// KB 1,320 / 1,222, 1,869 / 1,735 and 7,603 / 6,832; 88 KB 2,275 / 2,168, 3,641 /
+// 3,212 and 14,987 / 13,366.  Up to 3 KB staging always wins, from 17 KB never, in
+// between either by 4% at most.)
 int plan_full(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, bool* stg) {
   *stg = false;
   if (!staged(o)) {
@@ -1106,7 +1111,7 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   g->xfer_bound = b.xfer_bound;
   g->shared_links = b.shared_links ? 1 : 0;
   I.default_queue_cap = std::min<int64_t>(b.queue_bound, kDefaultQueueCap);
-  I.batched_sweep = b.D > 32 && dev_key && tb + b.ib + 2 + 5 <= 63 ? 1 : 0;
+  I.batched_sweep = b.D > 32 && dev_key ? 1 : 0;
   I.t32 = G.t32;
   // staged only where the copy also fits beside a warp's areas on this device
   I.stageable = 0;

@@ -43,8 +43,7 @@
 //
 // Lanes also fan out over successor lists (readiness, transfer arrivals,
 // distinct receiving accelerators via __match_any_sync) and predecessor
-// lists (ready-time maxima, last-consumer releases).  With at most 32
-// accelerators, lane d keeps accelerator d's free time in a register.
+// lists (ready-time maxima, last-consumer releases).
 //
 // No wait in these kernels depends on another block.  The two warps of a pair
 // (kRole) meet at named barriers of their block, and each message of one has its
