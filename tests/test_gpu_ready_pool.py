@@ -208,3 +208,24 @@ def test_wide_graphs_whose_keys_leave_no_room_for_the_accelerator(D, kw):
 @pytest.mark.parametrize("K", [2048, 2049])
 def test_select_best_at_the_line(K):
     test_select_best_on_both_sides_of_one_block(K)
+
+
+@pytest.mark.parametrize("D", [1, 2, 3, 32])
+@pytest.mark.parametrize("kw", [
+    dict(chains=1, length=40),                                    # one op at a time
+    dict(chains=1, length=12, fan=40),                            # one op with more successors than lanes
+    dict(chains=3, length=10, fan=3, bytes_lo=1 << 18, cap=6 << 20),  # capacities that bind
+    dict(chains=33, length=6),
+])
+def test_staged_and_one_warp_on_few_accelerators(D, kw):
+    """One warp per candidate, staged and through L1: batches of one op, and drains
+    ordered without sums on one or two accelerators."""
+    d = _chains(34, D=D, **kw)
+    rows = _rows(35, 40, d.n_ops, D)
+    g = G.gmg_create(d)
+    place = torch_place(rows)
+    outs = [G.sim_batch(g, place, req_done=True, **o)
+            for o in (dict(warps_per_block=4), dict(gmg_staging=G.GMG_STAGING_SHARED))]
+    torch.cuda.synchronize()
+    for o in outs:
+        compare(o.to_numpy(), *oracle_rows(d, rows))
