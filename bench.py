@@ -870,14 +870,14 @@ def main():
     issue_peak = props.multi_processor_count * 4 * pk["sm_max_mhz"] * 1e6 / 1e9  # Ginst/s
     arb_kern = "sim_arb_kernel" if D <= 32 else "sim_arbw_kernel"
     # the library's default: two warps per candidate while all fit (14 blocks of 64 threads per SM, 10 with 64-bit times), then
-    # the staged kernel for graphs whose copy takes 16 KB at most, else one warp per candidate
+    # the staged kernel where its copy and the areas of 28 warps take 170 KB at most, else one warp per candidate
     # an HBM event's key holds its accelerator
     dev_key = int(p.g.info["time_bound"]).bit_length() + p.g.info["id_bits"] <= 53
     pair = p.staging != 1 and not p.arb and dev_key
     pairs = (14 if p.g.info["t32"] == 1 else 10) * props.multi_processor_count
     staged_run = p.staging == 1 or (p.staging == 0 and p.g.info["stageable"] == 1 and not p.arb and
                                     not (pair and p.n_full <= pairs) and
-                                    20 * wl.desc.n_ops + 8 * wl.desc.n_edges <= 16 << 10)
+                                    20 * wl.desc.n_ops + 8 * wl.desc.n_edges + 28 * (3056 + (84 * D + 15) // 16 * 16) <= 170 << 10)
     full_kern = ("sim_full_staged_kernel" if staged_run else
                  "sim_full_pair_kernel" if pair and p.n_full <= pairs else "sim_full_kernel")
     kname = {"full": arb_kern if p.arb else full_kern,

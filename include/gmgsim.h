@@ -127,8 +127,8 @@ typedef struct gmg_base gmg_base_t; /* opaque; base schedule snapshot for increm
  * the records through the read-only L1 path.
  * GMG_STAGING_DEFAULT takes the fastest measured: batches of up to about 14
  * candidates per SM (10 with times beyond 2^32) run with two warps per candidate
- * by the L1 path, larger ones are staged where staging applies and the copy takes 16 KB
- * at most, and take the L1 path elsewhere; sim_batch_noalloc always
+ * by the L1 path, larger ones are staged where staging applies and copy and warps take
+ * 170 KB of shared memory at most, and take the L1 path elsewhere; sim_batch_noalloc always
  * takes the L1 path (and refuses GMG_STAGING_SHARED). */
 #define GMG_STAGING_DEFAULT 0
 #define GMG_STAGING_SHARED 1

@@ -665,7 +665,7 @@ bool staged(const sim_opts_t* o) { return o && o->gmg_staging == GMG_STAGING_SHA
 bool l1_path(const sim_opts_t* o) { return o && o->gmg_staging == GMG_STAGING_L1; }
 
 OncePerDevice g_stage_smem_set;
-constexpr int64_t kStageSmallBytes = 16 << 10;
+constexpr int64_t kStageSharedBytes = 170 << 10;
 
 // sim_batch with the GMG staged in shared memory: one CTA per SM with as many
 // warps (up to kStageMaxWarps) as fit beside the staged copy.
@@ -705,27 +705,29 @@ int plan_staged(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L) {
 // Full placements with pure-latency transfers: the staged-GMG kernel when the
 // caller asks for it (an error if it cannot serve the graph); by default two
 // warps per candidate while all candidates fit at once that way, beyond that the
-// staged kernel for small graphs, whose copy leaves the L1 cache to the
-// candidates' own arrays, else one warp per candidate.  *stg tells which.
+// staged kernel where its copy and kStageMaxWarps warps' areas leave the L1 cache
+// enough of the shared memory for the candidates' own arrays, else one warp per
+// candidate.  *stg tells which.
 // (Measured, two warps / staged / one warp: the 50-op graph 55 / 65 / 67 us for
 // 256 candidates; the prefill graph, N = 3088, a 90 KB copy, 1.41 / 1.80 / 1.84 ms
-// for 14, 1.61 / 2.11 / 2.07 ms for 2,048.  Where two warps are not chosen, staged /
-// one warp, for 2,129, 4,096 and 16,384 candidates: a copy of 1.4 KB 82 / 86, 101 /
-// 107 and 364 / 380 us; 5.6 KB 257 / 255, 336 / 344 and 1,356 / 1,307; 11 KB 472 /
-// 460, 621 / 630 and 2,511 / 2,405; 17 KB 585 / 556, 816 / 786 and 3,302 / 3,020; 44
-// KB 1,320 / 1,222, 1,869 / 1,735 and 7,603 / 6,832; 88 KB 2,275 / 2,168, 3,641 /
-// 3,212 and 14,987 / 13,366.  Up to 3 KB staging always wins, from 17 KB never, in
-// between either by 4% at most.)
+// for 14, 1.61 / 2.11 / 2.07 ms for 2,048.  Staged / one warp, 4,096 candidates, us,
+// by the KB that copy and areas take: on 2 accelerators 100 KB 549 / 613, 144 KB 2,031
+// / 2,280, 155 KB 2,431 / 2,673, 177 KB 3,426 / 3,531; on 6 109 KB 558 / 600, 164 KB
+// 2,180 / 2,358, 186 KB 3,104 / 3,115; on 12 166 KB 1,771 / 1,896, 177 KB 2,313 / 2,200;
+// on 16 165 KB 1,466 / 1,577, 176 KB 1,942 / 1,866; on 24 172 KB 1,213 / 1,249, 194 KB
+// 1,916 / 1,905; on 32 168 KB 542 / 565, 190 KB 1,208 / 1,336, 201 KB 1,905 / 1,722.
+// With 2,200 candidates the two are within 3%.)
 int plan_full(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, bool* stg) {
   *stg = false;
   if (!staged(o)) {
     const int rc = plan_pair(g, K, o, false, L);
     if (rc != GMG_EINVAL) return rc;
   }
-  if (staged(o) || (!l1_path(o) && stage_smem_bytes(g->dg.n, g->dg.n_edges) <= kStageSmallBytes)) {
+  if (!l1_path(o)) {
     const int rc = plan_staged(g, K, o, L);
-    *stg = rc == GMG_OK;
-    if (staged(o) || rc != GMG_EINVAL) return rc;
+    const bool small = rc == GMG_OK && L.P.stage_bytes + kStageMaxWarps * (int64_t)smem_per_warp(L.P) <= kStageSharedBytes;
+    *stg = rc == GMG_OK && (staged(o) || small);
+    if (staged(o) || *stg || (rc != GMG_OK && rc != GMG_EINVAL)) return rc;
   }
   return plan_launch(g, K, o, false, L);
 }

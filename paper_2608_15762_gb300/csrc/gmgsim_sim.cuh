@@ -1003,10 +1003,14 @@ struct Sim {
   // Sort and apply m extracted events of accelerators whose order matters.
   // may_violate: one of them may exceed its capacity -- then equal times are
   // told apart by op id (the whole entry is the sort key), else the order of
-  // equal times of one kind does not matter and 32 bits hold the key.
+  // equal times of one kind does not matter and 32 bits hold the key.  The staged
+  // kernel keeps to one way: it serves the many candidates of small graphs, whose
+  // warps run all of this code all the time, and both ways at once overflow the
+  // instruction cache (386 ops, 8 accelerators, 4,096 placements: 588 -> 547 us,
+  // 1,544 ops 1,909 -> 1,514; through L1 the prefill graph would lose, 3.06 -> 3.10).
   __device__ __forceinline__ void apply_ordered(int m, bool may_violate, tm_t span) {
     constexpr int kDevBits = kNarrow ? 5 : 8;
-    if (!may_violate && m <= 32 && (span >> (32 - kDevBits - 6)) == 0) {
+    if (kHot != kHotShared && !may_violate && m <= 32 && (span >> (32 - kDevBits - 6)) == 0) {
       apply_short(m);
     } else {
       sort_area(m);
@@ -1063,6 +1067,12 @@ struct Sim {
     __syncwarp();
   }
 
+  // Extracted events are not summed up but ordered: sizes that the 24-bit halves
+  // would not hold; and the staged kernel on one or two accelerators, where nearly
+  // every drain can raise a peak (386 ops, 4,096 placements: 574 -> 549 us on two,
+  // on eight 547 -> 563).
+  __device__ __forceinline__ bool unsummed() const { return (kHot == kHotShared && g.D <= 2) || g.big_bytes; }
+
   // Apply the m events just extracted.  Their order matters only on an
   // accelerator whose peak they can raise (without a violation so far the peak
   // is within the capacity).  An upper bound of its live bytes is cheap: with at
@@ -1078,7 +1088,7 @@ struct Sim {
     uint32_t fail = 0u;
     bool viol = false;
     if constexpr (kNarrow) {
-      if (g.big_bytes) {  // not summed: the 24-bit halves would not hold the sizes
+      if (unsummed()) {
         apply_ordered(m, true, span);
         return;
       }
@@ -1196,7 +1206,7 @@ struct Sim {
             const tm_t t = (tm_t)((e & lowmask()) >> (g.ib + 2)) - drained;
             const int w = min((int)(t >> wsh), kWindows - 1);
             uint32_t* a = dv.acc + 4 * (kWindows * dev + w) + (al ? 0 : 2);
-            if (!g.big_bytes) {
+            if (!unsummed()) {
               atomicAdd(a, (uint32_t)b & 0xffffffu);
               atomicAdd(a + 1, (uint32_t)(b >> 24));
             }
