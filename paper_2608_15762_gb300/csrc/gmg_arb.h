@@ -29,6 +29,7 @@ struct ArbParams {
   int32_t shared_links;   // 1 if two ordered pairs share a link id (else the sender check covers links)
   int32_t xcap;           // transfers per candidate (sum over ops of min(successors, D-1))
   int32_t smem_arb;       // shared bytes of the arbitration state per warp
+  int32_t blocks;         // blocks per SM of the instance that sim_batch launches (kArbBlocks and more)
   int64_t smem_std;       // shared bytes of the simulation state of all warps of a block
   // byte offsets inside a warp's scratch slot
   int64_t off_cnt;        // int32 [N]  inputs present (joins)
@@ -47,8 +48,13 @@ cudaError_t launch_expand_moves(const uint8_t* base_row, const int32_t* base_sta
                                 int32_t D, const int32_t* off, const int32_t* op, const uint8_t* dev, int32_t K,
                                 uint8_t* rows, int32_t* status, cudaStream_t st);
 
+// Blocks per SM of the arbitrated kernels on at most 32 accelerators; how many ops
+// and accelerators a graph may have that takes 7.
+constexpr int kArbBlocks = 5;
+constexpr int kArbSevenOps = 1024, kArbSevenDevices = 12;
+
 // Kernel entry of one instance (for occupancy queries) and the launcher.
-const void* arb_kernel_ptr(const DevGmg& g);
+const void* arb_kernel_ptr(const DevGmg& g, int blocks);
 cudaError_t launch_arb(const ArbParams& A, int grid, int block, size_t smem, cudaStream_t st);
 
 // The arbitrated base snapshot (one warp) and the incremental candidates

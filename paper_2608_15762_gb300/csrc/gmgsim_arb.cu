@@ -796,13 +796,18 @@ struct ArbSim : ArbEvents<ArbSim<kT32, kTypes, kMode, kHot>, Sim<true, kMode, tr
   }
 };
 
-// 96 registers a thread, 5 blocks per SM: at 72 and 7 blocks the spills cost more
-// than the two blocks give (prefill graph, ms, 7 blocks / 5: 2,048 placements
-// 12.7 / 9.6, 3,000 15.0 / 10.6, 4,096 18.4 / 18.6).
-constexpr int kArbBlocks = 5;
-
-template <bool kT32, bool kTypes, int kHot>
-__global__ void __launch_bounds__(128, kArbBlocks) sim_arb_kernel(const __grid_constant__ ArbParams A) {
+// 96 registers a thread, 5 blocks per SM (kArbBlocks): at 72 and 7 blocks the
+// spills cost more than the two blocks give (prefill graph, ms, 7 blocks / 5: 2,048
+// placements 12.7 / 9.6, 3,000 15.0 / 10.6) -- unless they save a second wave: 6
+// blocks where they hold all placements and 5 do not (5 / 6, 3,500 placements: 98
+// ops on 2 accelerators 0.49 / 0.33 ms, 3,088 ops on 8 17.8 / 12.1), 7 where 6 do not
+// and the graph has 1,024 ops and 12 accelerators at most (5 / 7, 4,096 placements:
+// 386 ops on 8 accelerators 2.24 / 2.00, 772 4.41 / 4.17, 3,088 18.7 / 19.2, 392 in
+// four requests 2.28 / 2.27; 392 and 772 ops on 16 accelerators 2.35 / 2.47 and 4.55 /
+// 4.58, 386 on 32 2.33 / 2.65).  Resumed candidates are handed out one by one and gain
+// nothing from it (3,500 on 8 accelerators, 3,088 ops, 5 / 6 / 7: 10.6 / 13.5 / 14.2).
+template <bool kT32, bool kTypes, int kHot, int kBlocks>
+__global__ void __launch_bounds__(128, kBlocks) sim_arb_kernel(const __grid_constant__ ArbParams A) {
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
@@ -927,22 +932,33 @@ cudaError_t launch_expand_moves(const uint8_t* base_row, const int32_t* base_sta
 
 // Instances by (32-bit times, accelerator types; compact records wherever the
 // graph has them).
-#define ARB_PTR(kernel)                                                       \
-  if (G.hot_ok) return (const void*)kernel<true, false, kHotGlobal>;          \
-  if (G.t32)                                                                  \
-    return G.ntypes >= 2 ? (const void*)kernel<true, true, kHotNone>          \
-                         : (const void*)kernel<true, false, kHotNone>;        \
-  return G.ntypes >= 2 ? (const void*)kernel<false, true, kHotNone> : (const void*)kernel<false, false, kHotNone>
-const void* arb_kernel_ptr(const DevGmg& G) { ARB_PTR(sim_arb_kernel); }
-const void* arb_inc_kernel_ptr(const DevGmg& G) { ARB_PTR(sim_arb_inc_kernel); }
-#undef ARB_PTR
+template <int kBlocks>
+const void* arb_ptr(const DevGmg& g) {
+  if (g.hot_ok) return (const void*)sim_arb_kernel<true, false, kHotGlobal, kBlocks>;
+  if (g.t32)
+    return g.ntypes >= 2 ? (const void*)sim_arb_kernel<true, true, kHotNone, kBlocks>
+                         : (const void*)sim_arb_kernel<true, false, kHotNone, kBlocks>;
+  return g.ntypes >= 2 ? (const void*)sim_arb_kernel<false, true, kHotNone, kBlocks>
+                       : (const void*)sim_arb_kernel<false, false, kHotNone, kBlocks>;
+}
+const void* arb_kernel_ptr(const DevGmg& g, int blocks) {
+  return blocks == 7 ? arb_ptr<7>(g) : blocks == 6 ? arb_ptr<6>(g) : arb_ptr<kArbBlocks>(g);
+}
+const void* arb_inc_kernel_ptr(const DevGmg& g) {
+  if (g.hot_ok) return (const void*)sim_arb_inc_kernel<true, false, kHotGlobal>;
+  if (g.t32)
+    return g.ntypes >= 2 ? (const void*)sim_arb_inc_kernel<true, true, kHotNone>
+                         : (const void*)sim_arb_inc_kernel<true, false, kHotNone>;
+  return g.ntypes >= 2 ? (const void*)sim_arb_inc_kernel<false, true, kHotNone>
+                       : (const void*)sim_arb_inc_kernel<false, false, kHotNone>;
+}
 const void* arb_base_kernel_ptr(bool types) {
   return types ? (const void*)sim_arb_base_kernel<true> : (const void*)sim_arb_base_kernel<false>;
 }
 
 cudaError_t launch_arb(const ArbParams& A, int grid, int block, size_t smem, cudaStream_t st) {
   void* args[] = {const_cast<ArbParams*>(&A)};
-  return cudaLaunchKernel(arb_kernel_ptr(A.P.g), dim3(grid), dim3(block), args, smem, st);
+  return cudaLaunchKernel(arb_kernel_ptr(A.P.g, A.blocks), dim3(grid), dim3(block), args, smem, st);
 }
 
 cudaError_t launch_arb_base(bool types, const ArbParams& A, size_t smem, cudaStream_t st) {

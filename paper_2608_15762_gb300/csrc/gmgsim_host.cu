@@ -790,9 +790,21 @@ int plan_arb(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbParams&
   const int sms = device_sms();
   if (sms <= 0) return GMG_ECUDA;
   int bps = 0;
-  const void* fn = mode == kInc ? arb_inc_kernel_ptr(G) : arb_kernel_ptr(G);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, 32 * L.wpb, L.smem) != cudaSuccess)
-    return GMG_ECUDA;
+  A.blocks = kArbBlocks;
+  auto resident = [&](const void* fn, int* n) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, fn, 32 * L.wpb, L.smem) == cudaSuccess;
+  };
+  if (!resident(mode == kInc ? arb_inc_kernel_ptr(G) : arb_kernel_ptr(G, A.blocks), &bps)) return GMG_ECUDA;
+  // more blocks per SM where they save a second wave (reasons at the kernel)
+  for (int more = 6; mode == kFull && more <= 7 && K > (int64_t)sms * bps * L.wpb; ++more) {
+    int n = 0;
+    if (more == 7 && (G.n > kArbSevenOps || G.D > kArbSevenDevices)) break;
+    if (!resident(arb_kernel_ptr(G, more), &n)) return GMG_ECUDA;
+    if (K <= (int64_t)sms * n * L.wpb) {
+      A.blocks = more;
+      bps = n;
+    }
+  }
   bps = std::max(bps, 1);
   const int64_t need = (std::max<int64_t>(K, 1) + L.wpb - 1) / L.wpb;
   L.grid = (int)std::min<int64_t>(need, (int64_t)sms * bps);

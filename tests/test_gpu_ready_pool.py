@@ -229,3 +229,17 @@ def test_staged_and_one_warp_on_few_accelerators(D, kw):
     torch.cuda.synchronize()
     for o in outs:
         compare(o.to_numpy(), *oracle_rows(d, rows))
+
+
+@pytest.mark.parametrize("D", [2, 8])
+@pytest.mark.parametrize("blocks,more", [(5, 0), (5, 1), (6, 0), (6, 1), (7, 0), (7, 1)])
+def test_both_sides_of_the_arbitrated_lines(D, blocks, more):
+    """As many candidates as the instances with 5, 6 and 7 blocks per SM hold, and
+    one more."""
+    d = _chains(32, D=D, chains=3, length=4, fan=2)
+    g = G.gmg_create(d)
+    K = 4 * blocks * torch.cuda.get_device_properties(0).multi_processor_count + more
+    rows = _rows(33, K, d.n_ops, D)
+    out = G.sim_batch(g, torch_place(rows), req_done=True, arbitrated=True)
+    torch.cuda.synchronize()
+    compare(out.to_numpy(), *O.simulate_batch(d, rows, arbitrated=True))
