@@ -522,11 +522,12 @@ size_t smem_per_warp(const SimParams& P) {
 }
 
 // Shared bytes of accelerator state per warp: live bytes; peaks and a drain's
-// sums, or (more than 32 accelerators: the peaks are in global scratch) a bit
+// sums (16 bytes a part), or (more than 32 accelerators: the peaks are in global scratch) a bit
 // set of the accelerators whose order matters; free times (of tbytes each).
-int dev_smem_bytes(int D, size_t tbytes) {
+int dev_smem_bytes(const DevGmg& G, size_t tbytes) {
+  const int D = G.D;
   const bool narrow = D <= 32;
-  return (int)align_up((size_t)D * 8 + (narrow ? (size_t)D * 72 : 32) + (size_t)D * tbytes, 16);
+  return (int)align_up((size_t)D * 8 + (narrow ? (size_t)D * (8 + ((size_t)16 << G.parts_log)) : 32) + (size_t)D * tbytes, 16);
 }
 
 // Shared bytes that a candidate's two warps hand started ops over in: two
@@ -558,7 +559,7 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
   while (P.sortcap < G.D) P.sortcap <<= 1;
   P.drain_trigger = kOpsPerGeneration;
   P.opcap = kOpsPerGeneration + 32;
-  P.dev_bytes = dev_smem_bytes(G.D, G.t32 ? 4 : 8);
+  P.dev_bytes = dev_smem_bytes(G, G.t32 ? 4 : 8);
   P.no_side = G.dev_key ? 1 : 0;  // the accelerator is inside the log entry
   L.smem = (size_t)L.wpb * smem_per_warp(P);
   size_t o2 = 0;
@@ -910,7 +911,7 @@ int plan_base(const gmg* g, const sim_opts_t* o, BasePlan& B) {
   int rc = B.arb ? plan_arb(g, 1, o, L, B.A, kBase) : plan_launch(g, 1, o, false, L);
   if (rc) return rc;
   L.wpb = 1;
-  if (B.arb) L.P.dev_bytes = dev_smem_bytes(G.D, 8);  // the arbitrated base keeps 64-bit times
+  if (B.arb) L.P.dev_bytes = dev_smem_bytes(G, 8);  // the arbitrated base keeps 64-bit times
   L.pair = !B.arb && G.dev_key != 0;
   if (L.pair) L.P.pair_bytes = pair_bytes(L.P);
   L.smem = smem_per_warp(L.P);
@@ -1105,6 +1106,7 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   // the 32-bit instances also take the accelerator id from the event key
   G.t32 = (b.time_bound < kMaxTime32 && G.dev_key) ? 1 : 0;
   G.hot_ok = (b.stage_ready && G.t32) ? 1 : 0;
+  G.parts_log = drain_parts_log(G.D, G.hot_ok != 0);
   G.stage_ok = (G.hot_ok && G.D <= 32 && b.time_bound < (int64_t(1) << 31)) ? 1 : 0;
   G.uniform = b.uniform ? 1 : 0;
   gmg_info_t& I = g->info;

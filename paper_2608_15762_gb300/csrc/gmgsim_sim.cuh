@@ -297,19 +297,23 @@ struct MemLog {
 // array in the warp's global scratch (only raised by atomicMax and read where an
 // allocation may exceed it).
 // ---------------------------------------------------------------------------
-template <bool kPkShared, typename TM>
+// kFour: a drain's sums cover four parts of its time (a constant of the instances
+// with compact records, else 2^g.parts_log).
+template <bool kPkShared, typename TM, bool kFour>
 struct Devices {
   TM* fr;       // shared [D]
   int64_t* lv;  // shared [D]
   int64_t* pk;  // [D], shared or global
-  uint32_t* acc;   // shared [16 * D], zero between drains (kPkShared)
+  uint32_t* acc;   // shared [(4 << parts()) * D], zero between drains (kPkShared)
   uint32_t* over;  // shared [8] (!kPkShared)
-  int D;
+  int D, plog;
+  __device__ __forceinline__ int parts() const { return kFour ? kPartsLog : plog; }
   __device__ void setup(const DevGmg& g, uint8_t* sm, int64_t* pk_global) {
     D = g.D;
+    plog = g.parts_log;
     if (kPkShared) {  // sums of a drain by accelerator, else a bit set of accelerators
       acc = reinterpret_cast<uint32_t*>(sm);
-      sm += 64 * (size_t)D;
+      sm += (16 << parts()) * (size_t)D;
     } else {
       over = reinterpret_cast<uint32_t*>(sm);
       sm += 32;
@@ -328,7 +332,7 @@ struct Devices {
       lv[d] = g.base[d];
       pk[d] = g.base[d];
       if (kPkShared)
-        for (int w = 0; w < 4; ++w) reinterpret_cast<uint4*>(acc)[4 * d + w] = make_uint4(0u, 0u, 0u, 0u);
+        for (int w = 0; w < 1 << parts(); ++w) reinterpret_cast<uint4*>(acc)[(d << parts()) + w] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncwarp();
   }
@@ -368,7 +372,7 @@ struct Devices {
       lv[d] = src[D + d];
       pk[d] = src[2 * D + d];
       if (kPkShared)
-        for (int w = 0; w < 4; ++w) reinterpret_cast<uint4*>(acc)[4 * d + w] = make_uint4(0u, 0u, 0u, 0u);
+        for (int w = 0; w < 1 << parts(); ++w) reinterpret_cast<uint4*>(acc)[(d << parts()) + w] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncwarp();
   }
@@ -506,13 +510,12 @@ struct Sim {
   MemLog log;
   uint64_t* sortk;
   uint8_t* sortd;
-  static constexpr int kWindows = 4;
   tm_t drained;     // every event before this time is applied, none after it
   uint32_t* oplog;  // ops started since the last HBM-event generation (a pair: two buffers, oplog and hands of index hb)
   Hand* hands;      // shared [2]
   int hb;
   int opn;
-  Devices<kNarrow, tm_t> dv;
+  Devices<kNarrow, tm_t, kHot != kHotNone> dv;
   const uint8_t* row;
   tm_t* fbuf;       // finish times (scratch)
   uint8_t* sl;      // the warp's scratch slot (the less used arrays in it are found from the launch parameters)
@@ -1094,11 +1097,12 @@ struct Sim {
       }
       bool over = false;
       if ((int)lane < g.D) {
-        uint4* q4 = reinterpret_cast<uint4*>(dv.acc) + kWindows * lane;
+        uint4* q4 = reinterpret_cast<uint4*>(dv.acc) + (lane << dv.parts());
         const int64_t l0 = dv.lv[lane], peak = dv.pk[lane];
         int64_t l = l0, top = 0;
 #pragma unroll
-        for (int w = 0; w < kWindows; ++w) {
+        for (int w = 0; w < 1 << kPartsLog; ++w) {
+          if (w >> dv.parts()) break;
           const uint4 x = q4[w];
           q4[w] = make_uint4(0u, 0u, 0u, 0u);
           const int64_t most = l + (int64_t)(((uint64_t)x.y << 24) + x.x);
@@ -1204,8 +1208,8 @@ struct Sim {
           const int dev = (int)(e >> g.ds);
           if constexpr (kNarrow) {
             const tm_t t = (tm_t)((e & lowmask()) >> (g.ib + 2)) - drained;
-            const int w = min((int)(t >> wsh), kWindows - 1);
-            uint32_t* a = dv.acc + 4 * (kWindows * dev + w) + (al ? 0 : 2);
+            const int w = min((int)(t >> wsh), (1 << dv.parts()) - 1);
+            uint32_t* a = dv.acc + 4 * ((dev << dv.parts()) + w) + (al ? 0 : 2);
             if (!unsummed()) {
               atomicAdd(a, (uint32_t)b & 0xffffffu);
               atomicAdd(a + 1, (uint32_t)(b >> 24));
@@ -1269,7 +1273,7 @@ struct Sim {
     // has one interval)
     const tm_t span = t_next == kI64Max ? kNever : (tm_t)t_next - drained;
     int wsh = 8 * (int)sizeof(tm_t) - 1;
-    if (span < ((tm_t)1 << 30)) wsh = max(0, 32 - __clz((uint32_t)span) - 2);
+    if (span < ((tm_t)1 << 30)) wsh = max(0, 32 - __clz((uint32_t)span) - dv.parts());
     while (log.n > 0) {
       uint64_t kmax = lim;
       if (log.n > P.sortcap) {

@@ -243,3 +243,24 @@ def test_both_sides_of_the_arbitrated_lines(D, blocks, more):
     out = G.sim_batch(g, torch_place(rows), req_done=True, arbitrated=True)
     torch.cuda.synchronize()
     compare(out.to_numpy(), *O.simulate_batch(d, rows, arbitrated=True))
+
+
+@pytest.mark.parametrize("D", [16, 17, 32])
+@pytest.mark.parametrize("kw", [dict(n_types=2), dict(link_hetero=True), dict(n_types=2, dur_hi=1 << 30)])
+def test_drains_summed_in_one_part_and_in_four(D, kw):
+    """Graphs without compact records on both sides of 16 accelerators, with a
+    capacity that binds."""
+    d = W.random_desc(51, 400, D, window=80, **kw)
+    rows = _rows(52, 24, d.n_ops, D)
+    d.cap[:] = int(np.median(oracle_rows(d, rows)[1].max(axis=1)))   # half of the placements exceed it
+    g = G.gmg_create(d)
+    outs = [G.sim_batch(g, torch_place(rows), req_done=True, warps_per_block=w) for w in (0, 4)]
+    base = rows[0, :d.n_ops].copy()
+    mv = W.random_moves(53, 24, base, D, max_moves=5)
+    b = G.base_create(g, torch.from_numpy(base).cuda())
+    inc = G.sim_incremental(g, b, *G.moves_to_device(mv, "cuda"), req_done=True)
+    torch.cuda.synchronize()
+    want = oracle_rows(d, rows)
+    for o in outs:
+        compare(o.to_numpy(), *want)
+    compare(inc.to_numpy(), *O.incremental_batch(d, base, mv))
