@@ -23,12 +23,12 @@
 // ready can precede any of them.  What bounds the kernels is the chain of
 // dependent instructions and loads per batch, and the issue slots that all warps
 // share; DRAM is idle.  On the prefill graph (3,088 ops, 8 accelerators) it is
-// 2.5 to 3 ops a batch and 173 warp instructions an op, against 333 for one key
+// 2.5 to 3 ops a batch and 172 warp instructions an op, against 333 for one key
 // at a time.  With at most 32 accelerators the lanes hold the pending ops, one
-// each (prefill, 4,096 placements, 4.74 ms -> 3.23; as keys in shared memory
+// each (prefill, 4,096 placements, 4.74 ms -> 3.09; as keys in shared memory
 // instead: 4.5); with more, where more ops than lanes are pending, they are 64-bit
 // keys in a pool in shared memory (256 accelerators, 4,096 placements, 128 ms ->
-// 83).  What does not fit goes to a warp-cooperative 32-ary min-heap.  Ops
+// 81).  What does not fit goes to a warp-cooperative 32-ary min-heap.  Ops
 // without predecessors come in when they are due: their keys are pre-sorted on
 // the host.
 //
@@ -1080,7 +1080,7 @@ struct Sim {
   // accelerator whose peak they can raise (without a violation so far the peak
   // is within the capacity).  An upper bound of its live bytes is cheap: with at
   // most 32 accelerators extract() has summed up what is allocated and freed on
-  // each in every quarter of the time since the last drain, and within a quarter
+  // each in every part (kPartsLog) of the time since the last drain, and within one
   // the live bytes are at most those at its start plus all its allocations; with
   // more (few events each) the whole drain is one such interval.  Everywhere
   // else the sums are enough.  (Prefill graph: 1.6 events an op are ordered with
@@ -1172,8 +1172,8 @@ struct Sim {
   // Move the logged events whose key part is < kmax to the sort area (their
   // number is known to fit) and compact the rest; returns their number.  Sums
   // them up for apply_due on the way: with at most 32 accelerators what is
-  // allocated and freed per accelerator and quarter of the time since the last
-  // drain (quarters of 2^wsh), each as sums of the low 24 and of the higher 24
+  // allocated and freed per accelerator and part of the time since the last
+  // drain (parts of 2^wsh), each as sums of the low 24 and of the higher 24
   // bits of the sizes (32-bit shared atomics; at most 256 events), with more the
   // allocations into the live bytes.
   __device__ int extract(uint64_t kmax, int wsh) {
@@ -1269,8 +1269,8 @@ struct Sim {
   }
   __device__ __forceinline__ void drain_log(int64_t t_next) {
     const uint64_t lim = t_next == kI64Max ? kKeyMax : kc.time_floor(t_next);
-    // the time since the last drain, and quarters of it (the last drain of all
-    // has one interval)
+    // the time since the last drain, and parts of it (the last drain of all has one
+    // interval)
     const tm_t span = t_next == kI64Max ? kNever : (tm_t)t_next - drained;
     int wsh = 8 * (int)sizeof(tm_t) - 1;
     if (span < ((tm_t)1 << 30)) wsh = max(0, 32 - __clz((uint32_t)span) - dv.parts());
