@@ -113,7 +113,6 @@ struct DevGmg {
   int32_t stage_ok;
   int32_t n_edges;
   int32_t big_bytes;          // 1: some output has 2^48 bytes or more
-  int32_t parts_log;          // a drain's sums cover 2^parts_log parts of its time (at most 32 accelerators)
   const uint8_t* ws;          // the whole device copy (every array above), for L2 prefetches
   int64_t ws_bytes;
 };
@@ -156,14 +155,14 @@ constexpr uint32_t kReady = 0, kFree = 1, kAlloc = 2;
 constexpr int kArbArrivals = 64;
 
 // log2 of the parts of a drain's time that are summed up by themselves on at most
-// 32 accelerators: 16 bytes of shared memory each per accelerator and warp.  Four
-// with compact records (their instances have it as a constant) and up to 16
-// accelerators; else one, which leaves the L1 cache to the records and the
-// candidates' arrays (4,096 placements on 32 accelerators, four parts / one: 772 ops,
-// links by node, 1.72 / 1.43 ms, 3,088 ops 6.11 / 5.16, on two accelerator types 4.55
-// / 3.98).
+// 32 accelerators: 16 bytes of shared memory each per accelerator and warp.
 constexpr int kPartsLog = 2;
-inline int drain_parts_log(int D, bool compact) { return compact || D <= 16 ? kPartsLog : 0; }
+// Where the one-warp kernels of full placements and move lists take one part: on 17
+// to 32 accelerators without compact records, which leaves the L1 cache to the records
+// and the candidates' arrays (4,096 placements on 32 accelerators, four parts / one: 772
+// ops, links by node, 1.72 / 1.43 ms, 3,088 ops 6.11 / 5.16, on two accelerator types
+// 4.55 / 3.98).
+inline bool one_part(const DevGmg& g) { return g.D > 16 && g.D <= 32 && g.dev_key && !g.hot_ok; }
 
 // Candidate simulation modes.
 enum Mode : int { kFull = 0, kInc = 1, kBase = 2 };

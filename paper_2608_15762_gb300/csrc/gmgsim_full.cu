@@ -7,13 +7,13 @@ namespace {
 // ---------------------------------------------------------------------------
 // sim_batch: K full placements.
 // ---------------------------------------------------------------------------
-template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
+template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot, int kParts = kPartsLog>
 __global__ void __launch_bounds__(128, kBlocksPerSM) sim_full_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
   const int64_t nslots = (int64_t)gridDim.x * (blockDim.x >> 5);
-  Sim<kNarrow, kFull, kKey, kT32, kTypes, kHot> S(P);
+  Sim<kNarrow, kFull, kKey, kT32, kTypes, kHot, !kNarrow, kBoth, kParts> S(P);
   setup_slot(S, P, wib, slot, smem);
   for (int64_t k = slot; k < P.K; k += nslots) {
     S.row = P.place + k * P.ld;
@@ -158,10 +158,10 @@ cudaError_t launch_full_staged(const SimParams& P, int grid, int block, size_t s
 // 32-bit times, accelerator types; compact records wherever the graph has
 // them).  32-bit times are only chosen with the accelerator id in the key,
 // compact records only with 32-bit times.
-template <bool N, bool K, bool T32>
+template <bool N, bool K, bool T32, int kParts = kPartsLog>
 const void* full_ptr(bool types) {
-  return types ? (const void*)sim_full_kernel<N, K, T32, true, kHotNone>
-               : (const void*)sim_full_kernel<N, K, T32, false, kHotNone>;
+  return types ? (const void*)sim_full_kernel<N, K, T32, true, kHotNone, kParts>
+               : (const void*)sim_full_kernel<N, K, T32, false, kHotNone, kParts>;
 }
 template <bool N>
 const void* full_ptr_n(bool key, bool t32, bool types, bool hot) {
@@ -171,6 +171,7 @@ const void* full_ptr_n(bool key, bool t32, bool types, bool hot) {
 }
 const void* full_kernel_ptr(const DevGmg& g) {
   const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
+  if (one_part(g)) return t32 ? full_ptr<true, true, true, 0>(types) : full_ptr<true, true, false, 0>(types);
   return g.D <= 32 ? full_ptr_n<true>(key, t32, types, hot) : full_ptr_n<false>(key, t32, types, hot);
 }
 // Two warps per candidate: graphs whose accelerator ids fit into the event key.

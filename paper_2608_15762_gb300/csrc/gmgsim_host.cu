@@ -524,10 +524,9 @@ size_t smem_per_warp(const SimParams& P) {
 // Shared bytes of accelerator state per warp: live bytes; peaks and a drain's
 // sums (16 bytes a part), or (more than 32 accelerators: the peaks are in global scratch) a bit
 // set of the accelerators whose order matters; free times (of tbytes each).
-int dev_smem_bytes(const DevGmg& G, size_t tbytes) {
-  const int D = G.D;
+int dev_smem_bytes(int D, size_t tbytes, int parts_log = kPartsLog) {
   const bool narrow = D <= 32;
-  return (int)align_up((size_t)D * 8 + (narrow ? (size_t)D * (8 + ((size_t)16 << G.parts_log)) : 32) + (size_t)D * tbytes, 16);
+  return (int)align_up((size_t)D * 8 + (narrow ? (size_t)D * (8 + ((size_t)16 << parts_log)) : 32) + (size_t)D * tbytes, 16);
 }
 
 // Shared bytes that a candidate's two warps hand started ops over in: two
@@ -559,7 +558,7 @@ int plan_launch(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& 
   while (P.sortcap < G.D) P.sortcap <<= 1;
   P.drain_trigger = kOpsPerGeneration;
   P.opcap = kOpsPerGeneration + 32;
-  P.dev_bytes = dev_smem_bytes(G, G.t32 ? 4 : 8);
+  P.dev_bytes = dev_smem_bytes(G.D, G.t32 ? 4 : 8, one_part(G) ? 0 : kPartsLog);
   P.no_side = G.dev_key ? 1 : 0;  // the accelerator is inside the log entry
   L.smem = (size_t)L.wpb * smem_per_warp(P);
   size_t o2 = 0;
@@ -619,6 +618,7 @@ int plan_pair(const gmg* g, int32_t K, const sim_opts_t* o, bool inc, Launch& L)
   const int rc = plan_launch(g, K, o, inc, L);
   if (rc) return rc;
   SimParams& P = L.P;
+  P.dev_bytes = dev_smem_bytes(G.D, G.t32 ? 4 : 8);
   P.pair_bytes = pair_bytes(P);
   L.pair = true;
   L.wpb = 1;
@@ -770,6 +770,8 @@ int plan_arb(const gmg* g, int32_t K, const sim_opts_t* o, Launch& L, ArbParams&
   if (rc) return rc;
   std::memset(&A, 0, sizeof(A));
   SimParams& P = L.P;
+  P.dev_bytes = dev_smem_bytes(G.D, G.t32 ? 4 : 8);
+  L.smem = (size_t)L.wpb * smem_per_warp(P);
   size_t o2 = (size_t)P.slot_bytes;
   auto take = [&](size_t bytes) {
     const size_t at = o2;
@@ -911,7 +913,8 @@ int plan_base(const gmg* g, const sim_opts_t* o, BasePlan& B) {
   int rc = B.arb ? plan_arb(g, 1, o, L, B.A, kBase) : plan_launch(g, 1, o, false, L);
   if (rc) return rc;
   L.wpb = 1;
-  if (B.arb) L.P.dev_bytes = dev_smem_bytes(G, 8);  // the arbitrated base keeps 64-bit times
+  L.P.dev_bytes = dev_smem_bytes(G.D, G.t32 ? 4 : 8);
+  if (B.arb) L.P.dev_bytes = dev_smem_bytes(G.D, 8);  // the arbitrated base keeps 64-bit times
   L.pair = !B.arb && G.dev_key != 0;
   if (L.pair) L.P.pair_bytes = pair_bytes(L.P);
   L.smem = smem_per_warp(L.P);
@@ -1106,7 +1109,6 @@ int gmg_create(const gmg_desc_t* desc, void* d_ws, size_t ws_bytes, gmg_stream_t
   // the 32-bit instances also take the accelerator id from the event key
   G.t32 = (b.time_bound < kMaxTime32 && G.dev_key) ? 1 : 0;
   G.hot_ok = (b.stage_ready && G.t32) ? 1 : 0;
-  G.parts_log = drain_parts_log(G.D, G.hot_ok != 0);
   G.stage_ok = (G.hot_ok && G.D <= 32 && b.time_bound < (int64_t(1) << 31)) ? 1 : 0;
   G.uniform = b.uniform ? 1 : 0;
   gmg_info_t& I = g->info;

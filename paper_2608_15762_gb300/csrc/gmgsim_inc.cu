@@ -333,12 +333,12 @@ __device__ void regen(S_& S, uint32_t p) {
   S.log_event(lane == 0, S.kc.make(m > hm ? m : hm, kFree, p), dp);
 }
 
-template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot>
+template <bool kNarrow, bool kKey, bool kT32, bool kTypes, int kHot, int kParts = kPartsLog>
 __global__ void __launch_bounds__(128, kBlocksPerSM) sim_inc_kernel(const __grid_constant__ SimParams P) {
   extern __shared__ __align__(16) uint8_t smem[];
   const unsigned wib = threadIdx.x >> 5;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
-  Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot> S(P);
+  Sim<kNarrow, kInc, kKey, kT32, kTypes, kHot, !kNarrow, kBoth, kParts> S(P);
   setup_slot(S, P, wib, slot, smem);
   S.rb = P.base.rb;
   S.fb = P.base.fb;
@@ -394,10 +394,10 @@ __global__ void __launch_bounds__(64, kT32 ? kPairsPerSM : kPairsPerSM64) sim_in
 // 32-bit times, accelerator types; compact records wherever the graph has
 // them).  32-bit times are only chosen with the accelerator id in the key,
 // compact records only with 32-bit times.
-template <bool N, bool K, bool T32>
+template <bool N, bool K, bool T32, int kParts = kPartsLog>
 const void* inc_ptr(bool types) {
-  return types ? (const void*)sim_inc_kernel<N, K, T32, true, kHotNone>
-               : (const void*)sim_inc_kernel<N, K, T32, false, kHotNone>;
+  return types ? (const void*)sim_inc_kernel<N, K, T32, true, kHotNone, kParts>
+               : (const void*)sim_inc_kernel<N, K, T32, false, kHotNone, kParts>;
 }
 template <bool N>
 const void* inc_ptr_n(bool key, bool t32, bool types, bool hot) {
@@ -407,6 +407,7 @@ const void* inc_ptr_n(bool key, bool t32, bool types, bool hot) {
 }
 const void* inc_kernel_ptr(const DevGmg& g) {
   const bool key = g.dev_key != 0, t32 = g.t32 != 0, types = g.ntypes >= 2, hot = g.hot_ok != 0;
+  if (one_part(g)) return t32 ? inc_ptr<true, true, true, 0>(types) : inc_ptr<true, true, false, 0>(types);
   return g.D <= 32 ? inc_ptr_n<true>(key, t32, types, hot) : inc_ptr_n<false>(key, t32, types, hot);
 }
 // Two warps per candidate: graphs whose accelerator ids fit into the event key.

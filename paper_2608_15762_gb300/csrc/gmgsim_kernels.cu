@@ -191,12 +191,12 @@ const void* base_pair_kernel_ptr(const DevGmg& g) { return g.D <= 32 ? base_pair
 
 cudaError_t set_smem_limits(int smem) {
   DevGmg g{};
-  for (int c = 0; c < 32; ++c) {
-    g.D = c & 1 ? 32 : 33;
-    g.dev_key = (c >> 1) & 1;
-    g.t32 = (c >> 2) & 1;
-    g.ntypes = c & 8 ? 2 : 0;
-    g.hot_ok = (c >> 4) & 1;
+  for (int c = 0; c < 48; ++c) {
+    g.D = c % 3 == 0 ? 16 : c % 3 == 1 ? 32 : 33;
+    g.dev_key = (c / 3) & 1;
+    g.t32 = (c / 6) & 1;
+    g.ntypes = (c / 12) & 1 ? 2 : 0;
+    g.hot_ok = (c / 24) & 1;
     const void* fns[] = {full_kernel_ptr(g),      inc_kernel_ptr(g),      base_kernel_ptr(g),
                          full_pair_kernel_ptr(g), inc_pair_kernel_ptr(g), base_pair_kernel_ptr(g)};
     for (const void* f : fns) {

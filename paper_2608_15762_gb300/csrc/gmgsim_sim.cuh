@@ -297,23 +297,20 @@ struct MemLog {
 // array in the warp's global scratch (only raised by atomicMax and read where an
 // allocation may exceed it).
 // ---------------------------------------------------------------------------
-// kFour: a drain's sums cover four parts of its time (a constant of the instances
-// with compact records, else 2^g.parts_log).
-template <bool kPkShared, typename TM, bool kFour>
+// kParts: a drain's sums cover 2^kParts parts of its time.
+template <bool kPkShared, typename TM, int kParts>
 struct Devices {
   TM* fr;       // shared [D]
   int64_t* lv;  // shared [D]
   int64_t* pk;  // [D], shared or global
-  uint32_t* acc;   // shared [(4 << parts()) * D], zero between drains (kPkShared)
+  uint32_t* acc;   // shared [(4 << kParts) * D], zero between drains (kPkShared)
   uint32_t* over;  // shared [8] (!kPkShared)
-  int D, plog;
-  __device__ __forceinline__ int parts() const { return kFour ? kPartsLog : plog; }
+  int D;
   __device__ void setup(const DevGmg& g, uint8_t* sm, int64_t* pk_global) {
     D = g.D;
-    plog = g.parts_log;
     if (kPkShared) {  // sums of a drain by accelerator, else a bit set of accelerators
       acc = reinterpret_cast<uint32_t*>(sm);
-      sm += (16 << parts()) * (size_t)D;
+      sm += (16 << kParts) * (size_t)D;
     } else {
       over = reinterpret_cast<uint32_t*>(sm);
       sm += 32;
@@ -332,7 +329,7 @@ struct Devices {
       lv[d] = g.base[d];
       pk[d] = g.base[d];
       if (kPkShared)
-        for (int w = 0; w < 1 << parts(); ++w) reinterpret_cast<uint4*>(acc)[(d << parts()) + w] = make_uint4(0u, 0u, 0u, 0u);
+        for (int w = 0; w < 1 << kParts; ++w) reinterpret_cast<uint4*>(acc)[(d << kParts) + w] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncwarp();
   }
@@ -372,7 +369,7 @@ struct Devices {
       lv[d] = src[D + d];
       pk[d] = src[2 * D + d];
       if (kPkShared)
-        for (int w = 0; w < 1 << parts(); ++w) reinterpret_cast<uint4*>(acc)[(d << parts()) + w] = make_uint4(0u, 0u, 0u, 0u);
+        for (int w = 0; w < 1 << kParts; ++w) reinterpret_cast<uint4*>(acc)[(d << kParts) + w] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncwarp();
   }
@@ -439,6 +436,7 @@ __device__ __forceinline__ WarpSmem carve_smem(uint8_t* smem, const SimParams& P
 // kPool: pending READY ops are keys in a pool in shared memory (the pure-latency
 // kernels of more than 32 accelerators, where more ops are pending than a warp
 // has lanes), else each lane holds one.
+// kParts: a drain's sums cover 2^kParts parts of its time (at most 32 accelerators).
 // kHot: the sweep reads compact 16-byte records (duration, transfer time, flags,
 // both CSR lists) instead of the 64-byte ones -- kHotGlobal through the
 // read-only path, kHotShared from the CTA's shared-memory copy (staged by
@@ -483,7 +481,7 @@ __device__ __forceinline__ void pair_arrive(int id) {
 }
 
 template <bool kNarrow, int kMode, bool kKey, bool kT32 = false, bool kTypes = false, int kHot = kHotNone,
-          bool kPool = !kNarrow, int kRole = kBoth>
+          bool kPool = !kNarrow, int kRole = kBoth, int kParts = kPartsLog>
 struct Sim {
   static_assert(kHot == kHotNone || (kT32 && !kTypes), "compact records: 32-bit times, one type");
   using tm_t = typename std::conditional<kT32, uint32_t, int64_t>::type;
@@ -515,7 +513,7 @@ struct Sim {
   Hand* hands;      // shared [2]
   int hb;
   int opn;
-  Devices<kNarrow, tm_t, kHot != kHotNone> dv;
+  Devices<kNarrow, tm_t, kParts> dv;
   const uint8_t* row;
   tm_t* fbuf;       // finish times (scratch)
   uint8_t* sl;      // the warp's scratch slot (the less used arrays in it are found from the launch parameters)
@@ -1080,7 +1078,7 @@ struct Sim {
   // accelerator whose peak they can raise (without a violation so far the peak
   // is within the capacity).  An upper bound of its live bytes is cheap: with at
   // most 32 accelerators extract() has summed up what is allocated and freed on
-  // each in every part (kPartsLog) of the time since the last drain, and within one
+  // each in every part (2^kParts of them) of the time since the last drain, and within one
   // the live bytes are at most those at its start plus all its allocations; with
   // more (few events each) the whole drain is one such interval.  Everywhere
   // else the sums are enough.  (Prefill graph: 1.6 events an op are ordered with
@@ -1097,12 +1095,11 @@ struct Sim {
       }
       bool over = false;
       if ((int)lane < g.D) {
-        uint4* q4 = reinterpret_cast<uint4*>(dv.acc) + (lane << dv.parts());
+        uint4* q4 = reinterpret_cast<uint4*>(dv.acc) + (lane << kParts);
         const int64_t l0 = dv.lv[lane], peak = dv.pk[lane];
         int64_t l = l0, top = 0;
 #pragma unroll
-        for (int w = 0; w < 1 << kPartsLog; ++w) {
-          if (w >> dv.parts()) break;
+        for (int w = 0; w < 1 << kParts; ++w) {
           const uint4 x = q4[w];
           q4[w] = make_uint4(0u, 0u, 0u, 0u);
           const int64_t most = l + (int64_t)(((uint64_t)x.y << 24) + x.x);
@@ -1208,8 +1205,8 @@ struct Sim {
           const int dev = (int)(e >> g.ds);
           if constexpr (kNarrow) {
             const tm_t t = (tm_t)((e & lowmask()) >> (g.ib + 2)) - drained;
-            const int w = min((int)(t >> wsh), (1 << dv.parts()) - 1);
-            uint32_t* a = dv.acc + 4 * ((dev << dv.parts()) + w) + (al ? 0 : 2);
+            const int w = min((int)(t >> wsh), (1 << kParts) - 1);
+            uint32_t* a = dv.acc + 4 * ((dev << kParts) + w) + (al ? 0 : 2);
             if (!unsummed()) {
               atomicAdd(a, (uint32_t)b & 0xffffffu);
               atomicAdd(a + 1, (uint32_t)(b >> 24));
@@ -1273,7 +1270,7 @@ struct Sim {
     // interval)
     const tm_t span = t_next == kI64Max ? kNever : (tm_t)t_next - drained;
     int wsh = 8 * (int)sizeof(tm_t) - 1;
-    if (span < ((tm_t)1 << 30)) wsh = max(0, 32 - __clz((uint32_t)span) - dv.parts());
+    if (span < ((tm_t)1 << 30)) wsh = max(0, 32 - __clz((uint32_t)span) - kParts);
     while (log.n > 0) {
       uint64_t kmax = lim;
       if (log.n > P.sortcap) {
@@ -1573,7 +1570,8 @@ struct Sim {
   // parallel start one op at a time: one request of 386 ops on 2 accelerators,
   // 4,096 placements, 634 -> 603 us; the prefill graph 3.21 -> 3.06 ms.  Where all
   // warps have room to wait the exchange costs more than it gives: the sweep warps
-  // of pairs, decode 31.2 -> 31.7 ms, and the pool, wide 81.6 -> 84.5 ms, do without.)
+  // of pairs, decode 31.2 -> 31.7 ms, and the pool, wide 81.6 -> 84.5 ms, do without;
+  // so do the 64-byte records, two types on 16 accelerators 3.82 -> 3.96 ms.)
   template <class B_>
   __device__ __forceinline__ void spread(B_& B, int src, uint32_t& u, uint32_t& step) const {
     B.i = __shfl_sync(kFullMask, B.i, src);
@@ -1795,7 +1793,7 @@ struct Sim {
       Batch B;
       if (!start_held(starts(lim, kNever, o), B)) break;
       uint32_t u = 0, step = 1;
-      const bool one = kRole == kBoth && (B.b & (B.b - 1u)) == 0u;
+      const bool one = kRole == kBoth && kCompact && (B.b & (B.b - 1u)) == 0u;
       if (one) spread(B, __ffs(B.b) - 1, u, step);
       for (; __any_sync(kFullMask, u < B.s.nsucc); u += step) {
         Reached x;
@@ -2201,8 +2199,8 @@ struct Sim {
 // the sweep's own drain is due; without a drain of their own the log of an 8 x
 // 32-layer graph, one checkpoint per 12 ops, kept every event: 24 ms for the base
 // and 21 ms for a late candidate instead of 2.7 and 0.09.)
-template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool, int kRole>
-__device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>::maybe_checkpoint(int64_t tn, uint64_t held) {
+template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool, int kRole, int kParts>
+__device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole, kParts>::maybe_checkpoint(int64_t tn, uint64_t held) {
   if (kMode != kBase) return;
   const DevBase& B = P.base;
   if (ck >= B.nck || readypops < next_ck) return;
@@ -2250,8 +2248,8 @@ __device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>::may
 
 // The accounting's part of checkpoint c at time tn (keep: the sweep's part is
 // saved): live and peak bytes, the event log, the first violation.
-template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool, int kRole>
-__device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>::save_accounts(int c, int64_t tn, bool keep) {
+template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool, int kRole, int kParts>
+__device__ void Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole, kParts>::save_accounts(int c, int64_t tn, bool keep) {
   const DevBase& B = P.base;
   const unsigned lane = lane_id();
   if (keep && log.n <= B.ckm) {
@@ -2303,8 +2301,8 @@ __device__ __forceinline__ void write_base(S_& S, const DevBase& B) {
   }
 }
 
-template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool, int kRole>
-__device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>& S, const SimParams& P, unsigned wib,
+template <bool kNarrow, int kMode, bool kKey, bool kT32, bool kTypes, int kHot, bool kPool, int kRole, int kParts>
+__device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole, kParts>& S, const SimParams& P, unsigned wib,
                            int64_t slot, uint8_t* smem) {
   uint8_t* sl = P.scratch + slot * P.slot_bytes;
   const WarpSmem w = carve_smem(smem, P, wib);
@@ -2323,7 +2321,7 @@ __device__ void setup_slot(Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, 
   S.sortd = w.sortd;
   S.oplog = w.oplog;
   S.opn = 0;
-  using tm_t = typename Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole>::tm_t;
+  using tm_t = typename Sim<kNarrow, kMode, kKey, kT32, kTypes, kHot, kPool, kRole, kParts>::tm_t;
   S.fbuf = reinterpret_cast<tm_t*>(sl + P.off_f);
   S.sl = sl;
   S.dv.setup(P.g, w.dev, P.off_pk >= 0 ? reinterpret_cast<int64_t*>(sl + P.off_pk) : nullptr);
